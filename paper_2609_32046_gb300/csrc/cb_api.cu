@@ -59,13 +59,12 @@ struct cb_ctx {
     int num_sms = 0;
     int G = 1;
     bool use_tc = false;
+    bool tc_stage_must = false;     // paged senders must be staged (the shapes score_kernel = 2 takes)
     float scale = 0.f;
-    int64_t n_chunk1_max = 0;
-    float2* stats = nullptr;
+    float* scratch = nullptr;       // per sender: pass-1 partials, then pass-2 partials in their place
     float* offs = nullptr;
     uint16_t* ext = nullptr;        // tcgen05 passes: per-row offset terms [S][nS][R_pad][16] bf16
     uint16_t* ones = nullptr;       // tcgen05 passes: [128][16] bf16 block of ones columns
-    float* part = nullptr;
     float* span_keys = nullptr;
     uint16_t* stage = nullptr;      // tcgen05 passes: contiguous copies of paged senders' K (on demand)
     int64_t stage_elems = 0;
@@ -161,6 +160,17 @@ cb_status check_source_ptr(cb_ctx* ctx, const void* p, const char* what, int i, 
 }
 
 bool stride_ok(int64_t s) { return s > 0 && (s % 8) == 0; }
+
+// Small senders of head dimension 64 keep to the mma.sync passes: up to two waves of their blocks
+// (128 positions x 16 tokens of one group, two resident on an SM) they take less time than the
+// tcgen05 passes, whose CTAs set up barriers and tensor memory and whose tensor maps the host
+// encodes (2 layers x 2 KV heads, m = 16: 16 against 18 us at T = 512 and 18 against 21 at 8192;
+// 24 layers x 8, T = 300, m = 8: 25 against 27; beyond the line, 16 x 8, T = 1024, m = 16: 49
+// against 27).  The rule reads the sender alone, so its scores do not depend on the call's others.
+bool small_sender(const cb_ctx* ctx, int64_t T, int32_t m) {
+    const int64_t nS = (int64_t)ctx->cfg.n_layers * ctx->cfg.n_kv_heads;
+    return ctx->cfg.head_dim == 64 && m <= 64 && nS * ((T + 127) / 128) * ((m + 15) / 16) <= 4 * (int64_t)ctx->num_sms;
+}
 
 // The optional block table of a sender (paged layout).
 cb_status check_pages(cb_ctx* ctx, const cb_kv& s, int i) {
@@ -272,8 +282,10 @@ cb_status cb_create(const cb_config* cfg, cb_ctx** out) {
         return fail(nullptr, CB_EINVAL, "span_width %d not in [1, %d]", c.span_width, cbk::kMaxSpanWidth);
     if (c.n_sink < 0 || c.n_latent < 0) return fail(nullptr, CB_EINVAL, "n_sink and n_latent must be >= 0");
     if (c.score_kernel < 0 || c.score_kernel > 2) return fail(nullptr, CB_EINVAL, "score_kernel must be 0, 1 or 2");
-    const bool tc_ok = cbk::tc_path_supported(c.head_dim, G, c.pool_width / 2, c.max_query_tokens);
-    if (c.score_kernel == 2 && !tc_ok)
+    const bool tc_ok = cbk::tc_path_supported(c.head_dim, G, c.pool_width / 2);
+    // score_kernel = 2 takes the shapes it has always taken
+    const bool tc_asked_ok = tc_ok && c.head_dim == 128 && c.max_query_tokens * G <= 512;
+    if (c.score_kernel == 2 && !tc_asked_ok)
         return fail(nullptr, CB_ESHAPE, "tcgen05 score passes need head_dim 128, pool_width <= 7 and "
                     "max_query_tokens * G <= 512");
 
@@ -285,18 +297,17 @@ cb_status cb_create(const cb_config* cfg, cb_ctx** out) {
     ctx->device = dev;
     ctx->G = G;
     ctx->use_tc = c.score_kernel == 2 || (c.score_kernel == 0 && tc_ok);
+    ctx->tc_stage_must = tc_asked_ok;
     ctx->scale = c.softmax_scale > 0.f ? c.softmax_scale : 1.f / std::sqrt((float)c.head_dim);
     cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, dev);
 
     const int64_t nS = (int64_t)c.n_layers * c.n_kv_heads;
     const int64_t S = c.max_senders;
-    ctx->n_chunk1_max = cbk::stats_slots(c.max_positions);
     const int64_t rows = (int64_t)c.max_query_tokens * G;
     ctx->keys_per_sender = (c.max_positions + c.span_width - 1) / c.span_width;
     int64_t total = 0;
-    e = alloc(&ctx->stats, (size_t)(S * nS * ctx->n_chunk1_max * rows), &total);
+    e = alloc(&ctx->scratch, (size_t)(S * cbk::score_scratch_floats(nS, rows, c.max_positions)), &total);
     if (e == cudaSuccess) e = alloc(&ctx->offs, (size_t)(S * nS * rows), &total);
-    if (e == cudaSuccess) e = alloc(&ctx->part, (size_t)(S * 3 * nS * c.max_positions), &total);
     if (e == cudaSuccess) e = alloc(&ctx->span_keys, (size_t)(S * ctx->keys_per_sender), &total);
     if (e == cudaSuccess && ctx->use_tc) {
         e = alloc(&ctx->ext, (size_t)(S * nS * cbk::rows_pad128(rows) * cbk::kExtCols), &total);
@@ -326,11 +337,10 @@ void cb_destroy(cb_ctx* ctx) {
     {
         DeviceGuard dg(ctx->device);
         cudaDeviceSynchronize();
-        cudaFree(ctx->stats);
+        cudaFree(ctx->scratch);
         cudaFree(ctx->offs);
         cudaFree(ctx->ext);
         cudaFree(ctx->ones);
-        cudaFree(ctx->part);
         cudaFree(ctx->span_keys);
         cudaFree(ctx->stage);
         cudaFree(ctx->err);
@@ -388,7 +398,7 @@ cb_status cb_score(cb_ctx* ctx, int32_t n, const cb_kv* senders, const cb_query*
         // room for the largest one, and for the rest up to kStageBudget elements per sub-batch
         int64_t largest = 0, sum = 0;
         for (int i = 0; i < n; ++i)
-            if (senders[i].pages) {
+            if (senders[i].pages && !small_sender(ctx, senders[i].T, queries[i].m)) {
                 const int64_t e = (int64_t)nS * senders[i].T * c.head_dim;
                 largest = e > largest ? e : largest;
                 sum += e;
@@ -396,21 +406,37 @@ cb_status cb_score(cb_ctx* ctx, int32_t n, const cb_kv* senders, const cb_query*
         const int64_t want = largest > (sum < cbk::kStageBudget ? sum : cbk::kStageBudget)
                                  ? largest : (sum < cbk::kStageBudget ? sum : cbk::kStageBudget);
         if (want > ctx->stage_elems) {
-            cudaFree(ctx->stage);   // waits for work still using it
-            ctx->scratch_bytes -= ctx->stage_elems * 2;
-            ctx->stage = nullptr;
-            ctx->stage_elems = 0;
-            if (cudaMalloc(reinterpret_cast<void**>(&ctx->stage), (size_t)want * 2) != cudaSuccess) {
-                cudaGetLastError();
+            // Shapes that score_kernel = 2 does not name can also read pages directly (the mma.sync
+            // passes), so they neither allocate inside a stream capture nor fail for want of memory.
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            if (!ctx->tc_stage_must && cudaStreamIsCapturing(strm, &cap) != cudaSuccess) cudaGetLastError();
+            if (ctx->tc_stage_must || cap == cudaStreamCaptureStatusNone) {
+                cudaFree(ctx->stage);   // waits for work still using it
+                ctx->scratch_bytes -= ctx->stage_elems * 2;
                 ctx->stage = nullptr;
-                return fail(ctx, CB_ENOMEM, "cannot allocate %lld bytes to stage paged caches", (long long)want * 2);
+                ctx->stage_elems = 0;
+                if (cudaMalloc(reinterpret_cast<void**>(&ctx->stage), (size_t)want * 2) == cudaSuccess) {
+                    ctx->stage_elems = want;
+                    ctx->scratch_bytes += want * 2;
+                } else {
+                    cudaGetLastError();
+                    ctx->stage = nullptr;
+                    if (ctx->tc_stage_must)
+                        return fail(ctx, CB_ENOMEM, "cannot allocate %lld bytes to stage paged caches", (long long)want * 2);
+                }
             }
-            ctx->stage_elems = want;
-            ctx->scratch_bytes += want * 2;
         }
     }
-    for (int b0 = 0; b0 < n; b0 += cbk::kMaxBatch) {
-        const int nb = n - b0 < cbk::kMaxBatch ? n - b0 : cbk::kMaxBatch;
+    // the senders of the tcgen05 passes, then those of the mma.sync passes
+    std::vector<int32_t> order(n);
+    int n_tc = 0, n_small = 0;
+    for (int i = 0; i < n; ++i)
+        if (ctx->use_tc && !small_sender(ctx, senders[i].T, queries[i].m)) order[n_tc++] = i;
+    for (int i = 0; i < n; ++i)
+        if (!ctx->use_tc || small_sender(ctx, senders[i].T, queries[i].m)) order[n_tc + n_small++] = i;
+    for (int b0 = 0; b0 < n;) {
+        const bool tc = b0 < n_tc;
+        const int left = (tc ? n_tc : n) - b0, nb = left < cbk::kMaxBatch ? left : cbk::kMaxBatch;
         cbk::ScoreBatch* bt = new cbk::ScoreBatch();
         bt->n = nb;
         bt->n_layers = c.n_layers;
@@ -422,26 +448,26 @@ cb_status cb_score(cb_ctx* ctx, int32_t n, const cb_kv* senders, const cb_query*
         bt->p_inf = std::isinf(c.p) ? 1 : 0;
         bt->alpha = c.alpha;
         bt->pool_half = c.pool_width / 2;
-        bt->use_tc = ctx->use_tc ? 1 : 0;
+        bt->use_tc = tc ? 1 : 0;
         bt->timer = ctx->timer;
         bt->err = ctx->err;
-        bt->stats = ctx->stats;
+        bt->stats = reinterpret_cast<float2*>(ctx->scratch);
+        bt->part = ctx->scratch;
         bt->offs = ctx->offs;
-        bt->ext = ctx->use_tc ? ctx->ext : nullptr;
+        bt->ext = tc ? ctx->ext : nullptr;
         bt->ones = ctx->ones;
-        bt->part = ctx->part;
         bt->stage = ctx->stage;
         bt->stage_elems = ctx->stage_elems;
         bt->wait_ns = (uint64_t)ctx->wait_ns;
-        bt->stall = b0 == 0 ? ctx->stall_next : 0;
-        int64_t so = 0, oo = 0, eo = 0, po = 0, b1 = 0, b2 = 0;
+        bt->stall = b0 == 0 ? ctx->stall_next : 0;   // (of the tcgen05 passes)
+        int64_t so = 0, oo = 0, eo = 0, b1 = 0, b2 = 0;
         for (int k = 0; k < nb; ++k) {
-            const cb_kv& s = senders[b0 + k];
-            const cb_query& q = queries[b0 + k];
+            const cb_kv& s = senders[order[b0 + k]];
+            const cb_query& q = queries[order[b0 + k]];
             cbk::ScoreSender& d = bt->s[k];
             d.k = static_cast<const uint16_t*>(s.k);
             d.q = static_cast<const uint16_t*>(q.q);
-            d.scores = scores[b0 + k];
+            d.scores = scores[order[b0 + k]];
             d.T = s.T;
             d.ks_l = s.s_layer; d.ks_h = s.s_head; d.ks_p = s.s_pos;
             d.pm = page_map(s);
@@ -451,18 +477,21 @@ cb_status cb_score(cb_ctx* ctx, int32_t n, const cb_kv* senders, const cb_query*
             d.m = q.m;
             d.n_chunk1 = (int32_t)((s.T + cbk::kStatsChunk - 1) / cbk::kStatsChunk);
             d.n_chunk2 = (int32_t)((s.T + cbk::kAccumChunk - 1) / cbk::kAccumChunk);
-            d.stats_off = so; so += (int64_t)nS * cbk::stats_slots(s.T) * q.m * ctx->G;
+            d.stats_off = so / 2;
+            d.part_off = so;
+            d.n_rc = 1;
+            so += cbk::score_scratch_floats(nS, (int64_t)q.m * ctx->G, s.T);
             d.offs_off = oo; oo += (int64_t)nS * q.m * ctx->G;
             d.ext_off = eo; eo += (int64_t)nS * cbk::rows_pad128((int64_t)q.m * ctx->G) * cbk::kExtCols;
-            d.part_off = po; po += (int64_t)3 * nS * s.T;
             d.blk1_begin = b1; b1 += (int64_t)nS * d.n_chunk1;
             d.blk2_begin = b2; b2 += (int64_t)nS * d.n_chunk2;
         }
         int path = 0;
         const int sms = ctx->score_sms > 0 && ctx->score_sms < ctx->num_sms ? ctx->score_sms : ctx->num_sms;
         cudaError_t e = cbk::launch_score(*bt, strm, sms, &path);
-        ctx->score_path = path;
+        ctx->score_path = b0 > 0 && ctx->score_path > path ? ctx->score_path : path;
         delete bt;
+        b0 += nb;
         if (e != cudaSuccess) return fail(ctx, CB_ECUDA, "score launch failed: %s", cudaGetErrorString(e));
     }
     ctx->stall_next = 0;

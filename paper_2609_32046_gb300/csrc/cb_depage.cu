@@ -17,7 +17,6 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kUnroll = 4;
-constexpr int kPieces = 16;   // 16-byte pieces of a d = 128 row
 
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
     uint4 v;
@@ -28,13 +27,15 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
 }
 
 // Grid: x = slice of (position, head, piece) triples, y = sender, z = layer.
+template <int D>
 __global__ void __launch_bounds__(kThreads) k_depage(const __grid_constant__ DepageBatch db) {
+    constexpr int kPieces = D / 8;   // 16-byte pieces of a row
     const DepageSender& sd = db.s[blockIdx.y];
     const int l = blockIdx.z;
     const int Hkv = db.n_kv_heads;
     const int64_t total = sd.T * Hkv * kPieces;
     const uint16_t* src = sd.k + (int64_t)l * sd.ks_l;
-    uint16_t* dst = sd.out + (int64_t)l * Hkv * sd.T * 128;
+    uint16_t* dst = sd.out + (int64_t)l * Hkv * sd.T * D;
     const int64_t stride = (int64_t)gridDim.x * kThreads;
     for (int64_t e0 = (int64_t)blockIdx.x * kThreads + threadIdx.x; e0 < total; e0 += stride * kUnroll) {
         uint4 v[kUnroll];
@@ -45,7 +46,7 @@ __global__ void __launch_bounds__(kThreads) k_depage(const __grid_constant__ Dep
             at[u] = -1;
             if (e >= total) continue;
             const int piece = (int)(e & (kPieces - 1));
-            const int64_t rest = e >> 4;
+            const int64_t rest = e / kPieces;
             int g;
             int64_t t;
             if (rest <= 0xffffffffll) {   // 32-bit division where it suffices
@@ -55,7 +56,7 @@ __global__ void __launch_bounds__(kThreads) k_depage(const __grid_constant__ Dep
                 g = (int)(rest % Hkv);
                 t = rest / Hkv;
             }
-            at[u] = ((int64_t)g * sd.T + t) * 128 + piece * 8;
+            at[u] = ((int64_t)g * sd.T + t) * D + piece * 8;
             const int64_t ro = row_offset(sd.pm, sd.ks_p, t);
             if (ro < 0) {
                 if (piece == 0) atomicOr(db.err, kErrPageIndex);
@@ -76,7 +77,7 @@ cudaError_t launch_depage(const DepageBatch& b, cudaStream_t st, int num_sms) {
     if (b.n == 0) return cudaSuccess;
     int64_t maxT = 0;
     for (int i = 0; i < b.n; ++i) maxT = b.s[i].T > maxT ? b.s[i].T : maxT;
-    const int64_t pieces = maxT * b.n_kv_heads * kPieces;
+    const int64_t pieces = maxT * b.n_kv_heads * (b.head_dim / 8);
     // about 48 blocks per SM over the whole grid (six waves of eight resident blocks): more,
     // shorter blocks kept more of the copy in flight than one wave of long ones
     int64_t x = ((int64_t)num_sms * 48) / ((int64_t)b.n * b.n_layers);
@@ -84,7 +85,8 @@ cudaError_t launch_depage(const DepageBatch& b, cudaStream_t st, int num_sms) {
     if (x > need) x = need;
     if (x < 1) x = 1;
     dim3 grid((unsigned)x, (unsigned)b.n, (unsigned)b.n_layers);
-    k_depage<<<grid, kThreads, 0, st>>>(b);
+    if (b.head_dim == 128) k_depage<128><<<grid, kThreads, 0, st>>>(b);
+    else k_depage<64><<<grid, kThreads, 0, st>>>(b);
     return cudaGetLastError();
 }
 

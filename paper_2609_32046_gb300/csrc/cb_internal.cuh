@@ -17,11 +17,24 @@ inline int64_t stats_slots(int64_t T) {
     const int64_t b = 4 * ((T + kStatsChunkTc - 1) / kStatsChunkTc);
     return a > b ? a : b;
 }
+
+// Length of a partial row of T positions: a multiple of four, so that every row is 16-byte aligned.
+__host__ __device__ inline int64_t part_row(int64_t T) { return (T + 3) & ~int64_t(3); }
+
+// Floats of score scratch of a sender with R query rows: the pass-1 partials (float2 per slot and
+// row of each of nS groups), whose place the pass-2 partials take once the combine kernel has read
+// them, and 3 T more a group.  The pass-2 partials, two rows of part_row(T) floats for each of up
+// to ceil(R / 256) row chunks, always fit: 8 (T + 3) (R / 256 + 1) bytes a group are no more
+// than 8 R slots + 12 T with slots >= max(T / 256, 4).  Rounded to 16 bytes.
+inline int64_t score_scratch_floats(int64_t nS, int64_t R, int64_t T) {
+    const int64_t f = nS * (2 * stats_slots(T) * R + 3 * T);
+    return (f + 3) & ~int64_t(3);
+}
 constexpr int kAccumChunk = 128;     // output positions per pass-2 block
 constexpr int kHalo = 8;             // extra positions each side of a pass-2 block (>= pool_width/2)
 constexpr int kMaxPoolWidth = 15;
 constexpr int kMaxSpanWidth = 256;
-constexpr int kFinSlices = 16;        // finalize: groups summed in 16 fixed slices
+constexpr int kFinSlices = 32;        // finalize: groups summed in 32 fixed slices
 constexpr int kMaxQueryTokens = 1024;
 
 // Device error word bits (set by kernels' own bounds checks).
@@ -71,7 +84,8 @@ struct ScoreSender {
     int64_t stats_off;        // float2 offset of this sender's pass-1 partials
     int64_t offs_off;         // float offset of this sender's per-row softmax offsets
     int64_t ext_off;          // bf16 offset of this sender's [nS][R_pad][16] offset rows (tcgen05 passes)
-    int64_t part_off;         // float offset of this sender's [3][nS][T] partials
+    int64_t part_off;         // float offset of this sender's [n_rc][2][nS][part_row(T)] partials
+    int32_t n_rc;             // row chunks the second pass left partials of (1 on the mma.sync path)
     int64_t blk1_begin;       // first pass-1 block of this sender
     int64_t blk2_begin;       // first pass-2 block of this sender
 };
@@ -91,7 +105,7 @@ struct ScoreBatch {
     uint16_t* ext;            // tcgen05 passes: -offset / scale_log2e per row as three bf16 terms
                               // (hi, mid, lo, then 13 zeros; -1e30 on padding rows), else null
     const uint16_t* ones;     // tcgen05 passes: [128][16] bf16, columns 0-2 = 1, the rest 0
-    float* part;              // per-group U_s, N_s, D_s partials
+    float* part;              // per-group partials: sums over tokens of b and of Pool(b)^p
     uint16_t* stage;          // tcgen05 passes: contiguous copies of paged senders' K
     int64_t stage_elems;      // its capacity (bf16 elements)
     uint64_t wait_ns;         // tcgen05 passes: limit of one bounded mbarrier wait
@@ -106,12 +120,12 @@ struct DepageSender {
     int64_t ks_l, ks_h, ks_p;
     PageMap pm;
     int64_t T;
-    uint16_t* out;            // [nL][Hkv][T][128]
+    uint16_t* out;            // [nL][Hkv][T][d]
 };
 
 struct DepageBatch {
     int32_t n;
-    int32_t n_layers, n_kv_heads;
+    int32_t n_layers, n_kv_heads, head_dim;
     uint32_t* err;
     DepageSender s[kMaxDepage];
 };
@@ -182,18 +196,15 @@ struct GatherBatch {
 // Records the message cb_last_error(NULL) returns (entry points without a context).
 void set_context_free_error(const char* msg);
 
-// Finalize tiles of a sender of T positions, and the floats of its slice sums.
-
 // True when the tcgen05 score passes handle this shape.
-bool tc_path_supported(int head_dim, int G, int pool_half, int max_query_tokens);
+bool tc_path_supported(int head_dim, int G, int pool_half);
 
 // Launchers (return the launch error, if any).
 // *path_out: 2 when the tcgen05 passes ran, 1 for the mma.sync passes.
-cudaError_t launch_score(const ScoreBatch& b, cudaStream_t st, int num_sms, int* path_out);
+cudaError_t launch_score(ScoreBatch& b, cudaStream_t st, int num_sms, int* path_out);
 cudaError_t launch_select(const SelectBatch& b, cudaStream_t st);
 cudaError_t launch_compact(const CompactBatch& b, cudaStream_t st, int num_sms);
 cudaError_t launch_gather(const GatherBatch& b, cudaStream_t st, int num_sms);
-// head_dim = 128 only (the tcgen05 passes' shape).
 cudaError_t launch_depage(const DepageBatch& b, cudaStream_t st, int num_sms);
 // Staging elements the tcgen05 passes want for paged senders (0 when none is paged): enough
 // for the largest paged sender and for paged sub-batches up to kStageBudget elements.

@@ -4,10 +4,11 @@
 //                       sum of exp of the logits of every (query token r, head h)
 //   combine k_combine   per (sender, s): chunk partials -> one log2 offset per row
 //   pass 2  k_accum     per (sender, s, 128-position chunk + 8-position halo):
-//                       a/G = exp2(z - offset), b = sum over the group's heads,
-//                       N_s = sum_r Pool(b_r)^p, bsum = sum_r b  ->  U_s, N_s, D_s
-//   k_finalize          per (sender, 240-position tile, slice of the groups): fixed-order
-//                       sums over s, Q = Pool(U), C = (N/D)^(1/(p-1)), S = Q * C^alpha
+//                       a/G = exp2(z - offset), b = sum over the group's heads
+//                       -> sum_r b and sum_r Pool(b_r)^p per position
+//   k_finalize          per (sender, 56-position tile): U_s, N_s and D_s = Pool(mean_r b)^p from
+//                       those, fixed-order sums over s, Q = Pool(U), C = (N/D)^(1/(p-1)),
+//                       S = Q * C^alpha
 //
 // Both logit passes use the bf16 tensor cores through mma.sync m16n8k16 with fp32
 // accumulation.  Rows of one m16 tile are (8 query tokens) x (2 heads of the
@@ -595,19 +596,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_accum(const __grid_constant__ S
     if (threadIdx.x < kAccumChunk) {
         const int64_t t = t0 + threadIdx.x;
         if (t < T) {
-            const int col = threadIdx.x + kHalo;
-            const float inv_m = 1.f / (float)sd.m;
-            float mx = bsum[col - ph];
-            for (int u = -ph + 1; u <= ph; ++u) mx = fmaxf(mx, bsum[col + u]);
-            // p = infinity: the largest pooled token value and the pooled token mean itself
             const float Nv = bt.p_inf ? fmaxf(nred[threadIdx.x], nred[kAccumChunk + threadIdx.x])
-                                      : (nred[threadIdx.x] + nred[kAccumChunk + threadIdx.x]) * inv_m;
-            const float Dv = bt.p_inf ? mx * inv_m : powp(mx * inv_m, bt.p, p2);
-            const float Uv = bsum[col] * inv_m / (float)bt.n_kv_heads;
+                                      : nred[threadIdx.x] + nred[kAccumChunk + threadIdx.x];
+            const int64_t Tp = part_row(T);
             float* part = bt.part + sd.part_off;
-            part[((int64_t)0 * nS + s) * T + t] = Uv;
-            part[((int64_t)1 * nS + s) * T + t] = Nv;
-            part[((int64_t)2 * nS + s) * T + t] = Dv;
+            part[(int64_t)s * Tp + t] = bsum[threadIdx.x + kHalo];
+            part[((int64_t)nS + s) * Tp + t] = Nv;
         }
     }
 }
@@ -615,122 +609,147 @@ __global__ void __launch_bounds__(kThreads, 2) k_accum(const __grid_constant__ S
 // ---------------------------------------------------------------------------
 // finalize: fixed-order sums over the groups, Pool(U), C, S -- one launch
 // ---------------------------------------------------------------------------
-// Block (64-position tile, sender); thread (slice k, quad q) sums slice k of the groups
-// (s = k, k + 16, ... in increasing order) for the four consecutive positions of quad q:
-// quads 2..17 are the tile (U, N and D), quads 0, 1 and 18, 19 the kHalo positions on each
-// side (U only, for Pool).  A batch of groups' loads is issued before they are added (the partials
-// mostly come from DRAM, so the kernel needs many bytes in flight), with one 16-byte load per
-// quad where the sender's partial rows are 16-byte aligned.  The 16 slice sums of every
-// position are then added in slice order in shared memory, U is pooled and C and S written.
-// Each sum has a fixed order, so the scores are deterministic.
-constexpr int kFinPos = 64;                          // output positions per block
-constexpr int kFinQuads = kFinPos / 4 + kHalo / 2;   // 16 tile quads + 2 on each side
-constexpr int kFinSpan = 4 * kFinQuads;              // positions whose U is summed
-constexpr int kFinThreads = kFinSlices * kFinQuads;  // 320
+// Block (tile of positions, sender); thread (slice k, quad q) sums slice k of the groups
+// (s = k, k + 32, ... in increasing order) for the four consecutive positions of quad q, whose
+// partial rows it reads with 16-byte loads: per group the sums over all query tokens of b and of
+// Pool(b)^p (row chunks added up first).  D_s = Pool(mean_r b)^p needs the neighbouring quads'
+// values, which come by shuffles from the neighbouring lanes, so the first and last HQ quads of a
+// tile (HQ = 1 for pool widths up to 9, else 2) are its Pool margin: 16 quads read, 56 (48)
+// positions written.  A batch of groups' loads is issued before they are added: the partials come
+// mostly from DRAM, so the kernel needs many bytes in flight, and with 288 groups a thread has
+// all of its nine groups' loads in flight at once.  The 32 slice sums of every position are then
+// added as a tree in shared memory (the rounding of these sums is most of a score's error: 4.5e-7
+// with the slices added in turn), U is pooled and C and S written.  Each sum has a fixed order, so
+// the scores are deterministic.
+constexpr int kFinQuads = 16;
+constexpr int kFinSpan = 4 * kFinQuads;
+constexpr int kFinThreads = kFinSlices * kFinQuads;  // 512
 
-// BATCH: groups of a slice loaded before they are added (9 for 288 groups; fewer groups, e.g. 64,
-// take a smaller batch, whose smaller register footprint fits several blocks an SM)
-template <int BATCH>
+constexpr int fin_out(int HQ) { return kFinSpan - 8 * HQ; }   // output positions per block
+
+// Window max over positions -ph .. ph of the four positions x, whose neighbours are in the lanes
+// of the same 16 lanes before and after (values of lanes past either end are not used by outputs).
+template <int HQ>
+__device__ __forceinline__ void pool_quads(const float (&x)[4], int ph, float (&o)[4]) {
+    float y[4 * (2 * HQ + 1)];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        y[4 * HQ + e] = x[e];
+#pragma unroll
+        for (int k = 1; k <= HQ; ++k) {
+            y[4 * (HQ - k) + e] = __shfl_up_sync(0xffffffffu, x[e], k, 16);
+            y[4 * (HQ + k) + e] = __shfl_down_sync(0xffffffffu, x[e], k, 16);
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        o[e] = x[e];
+#pragma unroll
+        for (int v = 1; v <= 4 * HQ; ++v)
+            if (v <= ph) o[e] = fmaxf(o[e], fmaxf(y[4 * HQ + e - v], y[4 * HQ + e + v]));
+    }
+}
+
+// BATCH: groups of a slice loaded before they are added: 9 (all of 288 groups) while the grid is
+// about one block an SM; 3, whose smaller register footprint fits two blocks an SM, so that one
+// block's loads are in flight while the other adds, for more blocks; 2 for up to 64 groups.
+template <int BATCH, int HQ>
 __global__ void __launch_bounds__(kFinThreads) k_finalize(const __grid_constant__ ScoreBatch bt) {
-    constexpr int kFinBatch = BATCH;
     __shared__ float su[kFinSlices][kFinSpan];
-    __shared__ float sn[kFinSlices][kFinPos];
-    __shared__ float sdn[kFinSlices][kFinPos];
-    __shared__ float us[kFinSpan];
+    __shared__ float sn[kFinSlices][kFinSpan];
+    __shared__ float sdn[kFinSlices][kFinSpan];
+    __shared__ float tot[3][kFinSpan];
     const ScoreSender& sd = bt.s[blockIdx.y];
     const int64_t T = sd.T;
-    const int64_t t0 = (int64_t)blockIdx.x * kFinPos;
-    if (t0 >= T) return;
+    const int64_t t0 = (int64_t)blockIdx.x * fin_out(HQ) - 4 * HQ;   // first position read
+    if (t0 + 4 * HQ >= T) return;
     const int sl = threadIdx.x / kFinQuads, q = threadIdx.x % kFinQuads;
     const int nS = bt.n_layers * bt.n_kv_heads;
-    const float* part = bt.part + sd.part_off;
-    const int64_t rN = (int64_t)nS * T, rD = 2 * rN;    // first N and D rows
-    const bool pinf = bt.p_inf;
-    const bool full = q >= kHalo / 4 && q < kHalo / 4 + kFinPos / 4;   // a tile quad: N and D too
-    const int64_t t = t0 - kHalo + 4 * q;
+    const int64_t rs = part_row(T) / 4;                 // row stride in float4
+    const bool pinf = bt.p_inf, p2 = bt.p == 2.f;
+    const int ph = bt.pool_half, n_rc = sd.n_rc;
+    const float inv_m = 1.f / (float)sd.m;
+    const int64_t t = t0 + 4 * q;
+    const bool in = t >= 0 && t < T;
+    const float4* p = reinterpret_cast<const float4*>(bt.part + sd.part_off) + (in ? t / 4 : 0);
     float u[4] = {0.f, 0.f, 0.f, 0.f}, n[4] = {0.f, 0.f, 0.f, 0.f}, d[4] = {0.f, 0.f, 0.f, 0.f};
-    auto add = [&](float (&acc)[4], const float4 v, bool mx) {
-        if (mx) {
-            acc[0] = fmaxf(acc[0], v.x); acc[1] = fmaxf(acc[1], v.y);
-            acc[2] = fmaxf(acc[2], v.z); acc[3] = fmaxf(acc[3], v.w);
-        } else {
-            acc[0] += v.x; acc[1] += v.y; acc[2] += v.z; acc[3] += v.w;
+    for (int s0 = sl; s0 - sl < nS; s0 += kFinSlices * BATCH) {   // the same trips for a warp's two slices
+        float4 a[BATCH], b[BATCH];
+#pragma unroll
+        for (int k = 0; k < BATCH; ++k) {
+            const int s = s0 + k * kFinSlices;
+            a[k] = b[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (s < nS && in) {
+                a[k] = __ldcs(p + (int64_t)s * rs);
+                b[k] = __ldcs(p + (int64_t)(nS + s) * rs);
+            }
         }
-    };
-    if ((T & 3) == 0 && (sd.part_off & 3) == 0) {
-        // 16-byte aligned rows: the quad lies wholly inside or wholly outside [0, T)
-        if (t >= 0 && t < T) {
-            const float4* p = reinterpret_cast<const float4*>(part + t);
-            const int64_t rs = T / 4;   // row stride in float4
-            for (int s0 = sl; s0 < nS; s0 += kFinSlices * kFinBatch) {
-                float4 a[kFinBatch], b[kFinBatch], c[kFinBatch];
+        for (int c = 1; c < n_rc; ++c) {
 #pragma unroll
-                for (int k = 0; k < kFinBatch; ++k) {
-                    const int s = s0 + k * kFinSlices;
-                    if (s < nS) {
-                        a[k] = __ldcs(p + (int64_t)s * rs);
-                        if (full) {
-                            b[k] = __ldcs(p + (rN / 4) + (int64_t)s * rs);
-                            c[k] = __ldcs(p + (rD / 4) + (int64_t)s * rs);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < kFinBatch; ++k) {
-                    if (s0 + k * kFinSlices >= nS) break;
-                    add(u, a[k], false);
-                    if (full) {
-                        add(n, b[k], pinf);   // p = infinity: N and D are maxima over the groups
-                        add(d, c[k], pinf);
+            for (int k = 0; k < BATCH; ++k) {
+                const int s = s0 + k * kFinSlices;
+                if (s < nS && in) {
+                    const float4 x = __ldcs(p + (int64_t)(2 * c * nS + s) * rs);
+                    const float4 y = __ldcs(p + (int64_t)((2 * c + 1) * nS + s) * rs);
+                    a[k].x += x.x; a[k].y += x.y; a[k].z += x.z; a[k].w += x.w;
+                    if (pinf) {
+                        b[k].x = fmaxf(b[k].x, y.x); b[k].y = fmaxf(b[k].y, y.y);
+                        b[k].z = fmaxf(b[k].z, y.z); b[k].w = fmaxf(b[k].w, y.w);
+                    } else {
+                        b[k].x += y.x; b[k].y += y.y; b[k].z += y.z; b[k].w += y.w;
                     }
                 }
             }
         }
-    } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int64_t te = t + e;
-            if (te < 0 || te >= T) continue;   // outside the sender: U = 0 adds nothing to Pool
-            const float* p = part + te;
-            for (int s = sl; s < nS; s += kFinSlices) {
-                u[e] += __ldcs(p + (int64_t)s * T);
-                if (!full) continue;
-                const float b = __ldcs(p + rN + (int64_t)s * T), c = __ldcs(p + rD + (int64_t)s * T);
-                n[e] = pinf ? fmaxf(n[e], b) : n[e] + b;
-                d[e] = pinf ? fmaxf(d[e], c) : d[e] + c;
+        for (int k = 0; k < BATCH; ++k) {
+            if (s0 - sl + k * kFinSlices >= nS) break;   // (groups past the last: zeros, which add nothing)
+            float x[4] = {a[k].x, a[k].y, a[k].z, a[k].w}, y[4] = {b[k].x, b[k].y, b[k].z, b[k].w}, o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (t + e >= T) x[e] = y[e] = 0.f;       // padding of the row (never written)
+            pool_quads<HQ>(x, ph, o);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                u[e] += x[e];
+                const float pm = o[e] * inv_m;           // Pool(mean over tokens of b)
+                if (pinf) {
+                    n[e] = fmaxf(n[e], y[e]);            // p = infinity: N and D are maxima over the groups
+                    d[e] = fmaxf(d[e], pm);
+                } else {
+                    n[e] += y[e];
+                    d[e] += powp(pm, bt.p, p2);
+                }
             }
         }
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         su[sl][4 * q + e] = u[e];
-        if (full) {
-            sn[sl][4 * q - kHalo + e] = n[e];
-            sdn[sl][4 * q - kHalo + e] = d[e];
-        }
+        sn[sl][4 * q + e] = n[e];
+        sdn[sl][4 * q + e] = d[e];
     }
     __syncthreads();
-    const int x = threadIdx.x;
-    if (x < kFinSpan) {
-        float U = 0.f;
+    if (threadIdx.x < 3 * kFinSpan) {
+        const int w = threadIdx.x / kFinSpan, x = threadIdx.x % kFinSpan;
+        const float(*src)[kFinSpan] = w == 0 ? su : (w == 1 ? sn : sdn);
+        const bool mx = w > 0 && pinf;
+        float v[kFinSlices];
 #pragma unroll
-        for (int k = 0; k < kFinSlices; ++k) U += su[k][x];
-        us[x] = U;
-    }
-    float Nv = 0.f, Dv = 0.f;
-    if (x < kFinPos) {
+        for (int k = 0; k < kFinSlices; ++k) v[k] = src[k][x];
 #pragma unroll
-        for (int k = 0; k < kFinSlices; ++k) {
-            Nv = pinf ? fmaxf(Nv, sn[k][x]) : Nv + sn[k][x];
-            Dv = pinf ? fmaxf(Dv, sdn[k][x]) : Dv + sdn[k][x];
-        }
+        for (int h = kFinSlices / 2; h > 0; h /= 2)
+#pragma unroll
+            for (int k = 0; k < h; ++k) v[k] = mx ? fmaxf(v[k], v[k + h]) : v[k] + v[k + h];
+        tot[w][x] = v[0];
     }
     __syncthreads();
-    if (x < kFinPos && t0 + x < T) {
-        const int ph = bt.pool_half;
-        const int c = x + kHalo;
-        float Q = us[c - ph];
-        for (int v = -ph + 1; v <= ph; ++v) Q = fmaxf(Q, us[c + v]);
+    const int x = threadIdx.x + 4 * HQ;
+    if (threadIdx.x < fin_out(HQ) && t0 + x < T) {
+        float Q = tot[0][x];
+        for (int v = 1; v <= ph; ++v) Q = fmaxf(Q, fmaxf(tot[0][x - v], tot[0][x + v]));
+        Q *= inv_m / (float)bt.n_kv_heads;
+        const float Nv = pinf ? tot[1][x] : tot[1][x] * inv_m, Dv = tot[2][x];
         const float C = Dv > FLT_MIN ? (pinf ? Nv / Dv : powf(Nv / Dv, 1.f / (bt.p - 1.f))) : 1.f;
         sd.scores[t0 + x] = bt.alpha == 0.f ? Q : Q * powf(C, bt.alpha);
     }
@@ -740,16 +759,26 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(const __grid_constant_
 
 namespace {
 
-cudaError_t launch_finalize(const ScoreBatch& b, cudaStream_t st) {
-    int64_t maxT = 0;
-    for (int i = 0; i < b.n; ++i) maxT = b.s[i].T > maxT ? b.s[i].T : maxT;
-    dim3 grid((unsigned)((maxT + kFinPos - 1) / kFinPos), (unsigned)b.n);
-    const int per_slice = (b.n_layers * b.n_kv_heads + kFinSlices - 1) / kFinSlices;
-    if (per_slice <= 4)
-        k_finalize<4><<<grid, kFinThreads, 0, st>>>(b);
+template <int BATCH>
+cudaError_t launch_finalize_b(const ScoreBatch& b, int64_t maxT, cudaStream_t st) {
+    const int out = b.pool_half <= 4 ? fin_out(1) : fin_out(2);
+    const dim3 grid((unsigned)((maxT + out - 1) / out), (unsigned)b.n);
+    if (b.pool_half <= 4)
+        k_finalize<BATCH, 1><<<grid, kFinThreads, 0, st>>>(b);
     else
-        k_finalize<9><<<grid, kFinThreads, 0, st>>>(b);
+        k_finalize<BATCH, 2><<<grid, kFinThreads, 0, st>>>(b);
     return cudaGetLastError();
+}
+
+cudaError_t launch_finalize(const ScoreBatch& b, cudaStream_t st, int num_sms) {
+    int64_t maxT = 0, tiles = 0;
+    for (int i = 0; i < b.n; ++i) {
+        maxT = b.s[i].T > maxT ? b.s[i].T : maxT;
+        tiles += (b.s[i].T + fin_out(1) - 1) / fin_out(1);
+    }
+    const int per_slice = (b.n_layers * b.n_kv_heads + kFinSlices - 1) / kFinSlices;
+    if (per_slice <= 2) return launch_finalize_b<2>(b, maxT, st);
+    return tiles <= num_sms + num_sms / 4 ? launch_finalize_b<9>(b, maxT, st) : launch_finalize_b<3>(b, maxT, st);
 }
 
 // Rows of all senders of a batch; few rows (long senders, few groups) take four threads a row.
@@ -797,7 +826,7 @@ size_t accum_smem(int max_rows) {
 }
 
 template <int D, int G>
-cudaError_t launch_dg(const ScoreBatch& b, cudaStream_t st) {
+cudaError_t launch_dg(const ScoreBatch& b, cudaStream_t st, int num_sms) {
     int64_t nblk1 = 0, nblk2 = 0;
     int max_rows = 0;
     const int nS = b.n_layers * b.n_kv_heads;
@@ -819,7 +848,7 @@ cudaError_t launch_dg(const ScoreBatch& b, cudaStream_t st) {
     stage_mark(b.timer, kStageCombine, st);
     k_accum<D, G><<<(unsigned)nblk2, kThreads, smem2, st>>>(b);
     stage_mark(b.timer, kStageAccum, st);
-    launch_finalize(b, st);
+    launch_finalize(b, st, num_sms);
     stage_mark(b.timer, kStageFinalize, st);
     return cudaGetLastError();
 }
@@ -829,39 +858,32 @@ cudaError_t launch_dg(const ScoreBatch& b, cudaStream_t st) {
 cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_t* err,
                             cudaError_t (*combine)(const ScoreBatch&, cudaStream_t));
 
-cudaError_t launch_score(const ScoreBatch& b_in, cudaStream_t st, int num_sms, int* path_out) {
-    const int G = b_in.n_q_heads / b_in.n_kv_heads;
-    const ScoreBatch& b = b_in;
+cudaError_t launch_score(ScoreBatch& b, cudaStream_t st, int num_sms, int* path_out) {
+    const int G = b.n_q_heads / b.n_kv_heads;
     if (b.use_tc) {
-        ScoreBatch* w = new ScoreBatch(b);
-        cudaError_t e = launch_score_tc(*w, st, num_sms, b.err, launch_combine);
-        if (e == cudaErrorNotSupported) {
-            // the driver rejected a tensor map for these strides: use the mma.sync passes
-            delete w;
-            ScoreBatch* v = new ScoreBatch(b);
-            v->use_tc = 0;
-            e = launch_score(*v, st, num_sms, path_out);
-            delete v;
+        cudaError_t e = launch_score_tc(b, st, num_sms, b.err, launch_combine);
+        if (e != cudaErrorNotSupported) {
+            *path_out = 2;
+            if (e == cudaSuccess) {
+                launch_finalize(b, st, num_sms);
+                stage_mark(b.timer, kStageFinalize, st);
+                e = cudaGetLastError();
+            }
             return e;
         }
-        *path_out = 2;
-        if (e == cudaSuccess) {
-            launch_finalize(*w, st);
-            stage_mark(w->timer, kStageFinalize, st);
-            e = cudaGetLastError();
-        }
-        delete w;
-        return e;
+        // the driver rejected a tensor map for these strides (nothing has been launched), or a paged
+        // sender has no room in the staging buffer: use the mma.sync passes
+        b.use_tc = 0;
     }
     *path_out = 1;
     if (b.head_dim == 128) {
-        if (G == 4) return launch_dg<128, 4>(b, st);
-        if (G == 2) return launch_dg<128, 2>(b, st);
-        if (G == 1) return launch_dg<128, 1>(b, st);
+        if (G == 4) return launch_dg<128, 4>(b, st, num_sms);
+        if (G == 2) return launch_dg<128, 2>(b, st, num_sms);
+        if (G == 1) return launch_dg<128, 1>(b, st, num_sms);
     } else if (b.head_dim == 64) {
-        if (G == 4) return launch_dg<64, 4>(b, st);
-        if (G == 2) return launch_dg<64, 2>(b, st);
-        if (G == 1) return launch_dg<64, 1>(b, st);
+        if (G == 4) return launch_dg<64, 4>(b, st, num_sms);
+        if (G == 2) return launch_dg<64, 2>(b, st, num_sms);
+        if (G == 1) return launch_dg<64, 1>(b, st, num_sms);
     }
     return cudaErrorInvalidValue;
 }

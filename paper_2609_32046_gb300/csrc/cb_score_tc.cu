@@ -9,27 +9,42 @@
 // inside a tile breaks), and both passes read that copy.
 //
 //   k_stats_tc  pass 1, D = Q_s K_tile^T: TMEM lane = row (r, h), column = position.
-//               Each epilogue thread owns one row and keeps its running max and
-//               sum of exp2 over its group's tiles of a 1024-position chunk.
-//   k_accum_tc  pass 2, D = K_tile Q_s^T (+ a ninth K-step of ones x the rows' offset terms,
+//               Each epilogue thread owns one row and one quarter of a tile's positions and keeps
+//               its running max and sum of exp2 over a chunk of positions.
+//   k_accum_tc  pass 2, D = K_tile Q_s^T (+ one more K-step of ones x the rows' offset terms,
 //               so TMEM holds z - offset / scale): TMEM lane = position, column = row (r, h).
-//               Each thread owns one position: exp2 of its logits (a / G), the head mean b
-//               and the sums over tokens stay in registers; Pool over positions runs
-//               across lanes with shuffles.  A tile's four 32-row quarters start 3 positions
-//               before their 26 output positions (104 per tile).
+//               A block of positions is four tiles: tile j holds every fourth position from j on,
+//               so a thread owns four neighbouring positions, one of each tile.  exp2 of its
+//               logits (a / G), the head mean b and the sums over tokens stay in registers; Pool
+//               over positions needs the neighbouring lanes' prefix and suffix maxima only.  A
+//               block's four lane quarters cover 128 positions each, 120 of them outputs (480 a
+//               block).
 //
-// Warp roles (576 threads, one CTA per SM, persistent over a contiguous range of work
-// units): warp 0 producer, warp 1 MMA issuer and TMEM owner, warps 2-17 epilogue (two
-// groups of eight taking alternate tiles; warp w reads TMEM lanes 32*(w%4)..+31).  K tiles
-// flow through a ring of smem stages; TMEM holds four 128-column accumulator buffers.
+// Rows: a group's m * G query rows, padded to 128, are processed in row chunks of up to 512
+// (pass 1) or 256 rows (pass 2) whose Q fits in shared memory; a row chunk is the outermost part
+// of a work unit, and the grid is a multiple of the row-chunk count, so that the CTAs of
+// different row chunks walk the same K tiles at the same time and all but the first read them
+// from L2.
+//
+// Warp roles (640 threads, one CTA per SM, persistent over a contiguous range of work
+// units): warp 0 producer, warps 1 and 2 MMA issuers (warp 1 owns TMEM), warp 3 writes pass
+// 2's sums, warps 4-19 epilogue
+// (warp w reads TMEM lanes 32*(w%4)..+31; the four warps of a lane quarter share a buffer's
+// columns).  K tiles flow through a ring of smem stages; TMEM holds a ring of four 128-column
+// accumulator buffers, each drained by all sixteen epilogue warps: the MMA runs up to four buffers
+// ahead.
 // Every mbarrier wait is bounded (1 s); on a timeout the kernel records kErrTimeout, drains
 // its copies and MMAs, frees TMEM and returns.
+#include <algorithm>
+#include <atomic>
 #include <cfloat>
 #include <cstdint>
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
+#include <memory>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "cb_internal.cuh"
@@ -39,60 +54,75 @@ namespace cbk {
 namespace {
 using namespace sm100;
 
-constexpr int kWarpsTc = 18;                // 0 TMA, 1 MMA, 2..17 epilogue
+constexpr int kWarpsTc = 20;                // 0 TMA, 1 and 2 MMA, 3 pass 2's sums, 4..19 epilogue
 constexpr int kThreadsTc = kWarpsTc * 32;
-constexpr int kMaxStages = 4;
+constexpr int kEpiWarps = 16;
+constexpr int kEpi0 = 4;                    // first epilogue warp (TMEM lane quarter = warp % 4)
+constexpr int kMaxStages = 8;
 constexpr int kTileRows = 128;          // K rows per tile
-constexpr int kTileBytes = kTileRows * 256;   // d = 128: two 64-column swizzled blocks
 constexpr int kChunk1 = kStatsChunkTc;  // pass-1 positions per chunk
-constexpr int kMargin = 3;              // pass-2 lanes before/after the output positions
-constexpr int kOutW = 32 - 2 * kMargin;          // 26 output positions per pass-2 warp
-constexpr int kOut2 = 4 * kOutW;                 // 104 output positions per pass-2 tile
+constexpr int kRowHalf = 128;           // query rows of one accumulator buffer
+constexpr int kHalves1 = 4, kHalves2 = 2;        // most 128-row halves of a row chunk (pass 1, pass 2)
+constexpr int kMargin = 4;              // pass-2 positions before/after a lane quarter's outputs
+constexpr int kOutW = 128 - 2 * kMargin;         // 120 output positions per pass-2 lane quarter
+constexpr int kOut2 = 4 * kOutW;                 // 480 output positions per pass-2 block
 constexpr uint32_t kTmemCols = 512;
 constexpr uint64_t kWaitNs = 1000000000ull;      // 1 s per wait
 constexpr uint32_t kPollNs = 1000000u;           // longest suspension of one poll (woken at completion)
-constexpr int kMaxTcSenders = 32;
+constexpr int kMaxTcSenders = 32;         // their tensor maps fill most of the 32,764 bytes of kernel parameters
+
+struct TcMaps {
+    CUtensorMap k[5];     // pass 1: k[0] = 4D {d, T, Hkv, nL}, box {64, 128, 1, 1}.
+                          // pass 2: k[4] = 5D {d, T / 4, 4, Hkv, nL} (position 4 i + j at (i, j)), box
+                          // {64, 32, 1, 1, 1}; k[j] = 4D positions j, j + 4, ... with every one of them (the
+                          // 5D tensor lacks the last T mod 4), box {64, 32, 1, 1}
+    CUtensorMap q;        // 4D {d, Hq, m, nL}, box {64, G, 128 / G, 1}: 128 rows
+    CUtensorMap e;        // pass 2: 3D {16, R_pad, nS} offset terms, box {16, 128, 1}, 32-byte swizzle
+};
 
 struct TcSender {
-    CUtensorMap kmap;     // 4D {d, T, Hkv, nL}, box {64, 128, 1, 1}
-    CUtensorMap kmap32;   // same tensor, box {64, 32, 1, 1}
-    CUtensorMap qmap;     // 4D {d, Hq, m, nL}, box {64, G, qbox_tok, 1}
-    CUtensorMap emap;     // 3D {16, R_pad, nS} offset terms of pass 2, box {16, ebox_rows, 1}, 32-byte swizzle
     float2* stats;        // this sender's pass-1 partials [nS][n_chunk1][R]
-    const float* offs;    // this sender's per-row offsets [nS][R]
-    float* part;          // this sender's partials [3][nS][T]
-    int64_t T;
-    int32_t m, R, R_pad;
-    int32_t n_chunk1, n_tile2;
-    int32_t qbox_tok, n_qbox;
-    int32_t ebox_rows, n_ebox;
-    float inv_m, inv_mh;  // 1 / m and 1 / (m Hkv)
-    int64_t unit1_begin, unit2_begin;
+    float* part;          // this sender's pass-2 partials [n_rc2][2][nS][T_pad]
+    int64_t T, T_pad;
+    int32_t R, halves;    // m * G query rows; 128-row halves of them
+    int32_t n_chunk1;     // pass-1 partial slots: four per chunk of positions
+    int32_t n_blk2;       // pass-2 blocks of positions
+    int32_t n_rc1, n_rc2; // row chunks of each pass
 };
 
 struct TcBatch {
     CUtensorMap omap;     // 2D {16, 128} block of ones columns, one box, 32-byte swizzle
     int32_t n;
     int32_t nL, Hq, Hkv, G;
-    int32_t stages, rpad_max;
+    int32_t stages1, rows1;       // pass 1: K ring stages, Q rows held
+    int32_t kbufs, rows2;         // pass 2: K blocks in flight (1 or 2, four tiles each), Q rows held
+    int32_t max_rc1, max_rc2;
     float sl2e, p;
-    int32_t p_is_2, p_inf, ph;
-    int64_t units1, units2;
+    int32_t p_inf, ph;
+    int64_t weight1, weight2;     // work of each pass: 128-row halves over all units
     uint64_t wait_ns;     // limit of one bounded mbarrier wait
     int32_t stall;        // 1: CTA 0's pass-1 MMA issuer first waits on a barrier nothing arrives on
     uint32_t* err;
+    TcMaps maps[kMaxTcSenders];   // (apart from the sizes: a tensor map is aligned to 128 bytes)
     TcSender s[kMaxTcSenders];
 };
 
+// One unit of work: sender i, group s, row chunk rc, position chunk (pass 1) or block (pass 2) c.
+struct Unit {
+    int i, s, c, rc;
+};
+
+static_assert(sizeof(TcBatch) <= 32764, "kernel parameters");
+
 struct Ctl {
     uint64_t k_full[kMaxStages], k_empty[kMaxStages];
-    uint64_t t_full[4], t_empty[4];   // TMEM buffers of 128 columns (pass 1: group g owns 2g and 2g + 1;
-                                      // pass 2: buffer 2g + h is column half h of group g)
-    uint64_t q_full, q_empty, drain, o_full;
+    uint64_t t_full[4], t_empty[4];   // ring of TMEM buffers of 128 columns
+    uint64_t q_full, q_empty, drain[2], o_full;
     uint64_t stall;         // failure-detection test: a barrier nothing arrives on
     uint64_t wait_ns;       // limit of one bounded wait
-    uint64_t xb[2][2][4];   // pass 2: column-half exchange [tile parity][group][lane quarter]: written
-    uint64_t xe[2][2][4];   //   and read (half 1 reuses a slot only after half 0 has read it)
+    uint64_t xb, xe;        // pass 2: a block's sums written by the epilogue and read by warp 3
+    int32_t units;          // this CTA's units, the first of which is `first`
+    Unit first;
     uint32_t tmem_base;
     int abort;
 };
@@ -105,9 +135,9 @@ __device__ __forceinline__ uint64_t now_ns() {
 }
 
 // Bounded wait: true when the phase completed, false on abort (set by anyone) or timeout.
-// `tag` names the wait in the device error word (bit 8 + tag) when it times out.
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Ctl* ctl, uint32_t* err, int tag) {
-    if (mbar_try_wait(bar, parity)) return true;
+// `tag` names the wait in the device error word (bit 8 + tag) when it times out.  The polling is
+// out of line: the epilogue loops stay small enough for the instruction cache.
+__device__ __noinline__ bool wait_poll(uint64_t* bar, uint32_t parity, Ctl* ctl, uint32_t* err, int tag) {
     const uint64_t t0 = now_ns();
     for (uint32_t i = 1; i < (1u << 30); ++i) {
         if (mbar_try_wait_hint(bar, parity, kPollNs)) return true;
@@ -125,6 +155,10 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Ctl* ct
     return false;
 }
 
+__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Ctl* ctl, uint32_t* err, int tag) {
+    return mbar_try_wait(bar, parity) || wait_poll(bar, parity, ctl, err, tag);
+}
+
 // Wait used only on the way out (drain): bounded by kWaitNs whatever the configured limit
 // (the copies and MMAs it waits for always complete), ignores the abort flag.
 __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
@@ -137,179 +171,197 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
     return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
 }
 
-struct Unit {
-    int i, s, c;   // sender, group, chunk (pass 1) or tile (pass 2)
-};
+// Row chunk rc of n holds the sender's 128-row halves [rc * halves / n, (rc + 1) * halves / n).
+__device__ __forceinline__ int rc_begin(int halves, int n, int rc) { return rc * halves / n; }
 
-__device__ __forceinline__ Unit decode1(const TcBatch& bt, int64_t u) {
-    int i = 0;
-    while (i + 1 < bt.n && bt.s[i + 1].unit1_begin <= u) ++i;
-    const int64_t local = u - bt.s[i].unit1_begin;
-    const int nch = bt.s[i].n_chunk1 / 4;   // n_chunk1 counts (chunk, group, half) partial slots
-    return Unit{i, (int)(local / nch), (int)(local % nch)};
-}
+template <int PASS>
+__device__ __forceinline__ int n_rc(const TcSender& sd) { return PASS == 1 ? sd.n_rc1 : sd.n_rc2; }
+template <int PASS>
+__device__ __forceinline__ int n_c(const TcSender& sd) { return PASS == 1 ? sd.n_chunk1 / 4 : sd.n_blk2; }
 
-__device__ __forceinline__ Unit decode2(const TcBatch& bt, int64_t u) {
-    int i = 0;
-    while (i + 1 < bt.n && bt.s[i + 1].unit2_begin <= u) ++i;
-    const int64_t local = u - bt.s[i].unit2_begin;
-    return Unit{i, (int)(local / bt.s[i].n_tile2), (int)(local % bt.s[i].n_tile2)};
-}
-
-// Pass-2 units in order without a division per unit: (sender, group, tile) advanced by one.
-__device__ __forceinline__ void next2(const TcBatch& bt, Unit& un) {
-    if (un.i >= bt.n) return;   // past the last unit
-    if (++un.c == bt.s[un.i].n_tile2) {
-        un.c = 0;
-        if (++un.s == bt.nL * bt.Hkv) {
-            un.s = 0;
-            ++un.i;
+// Units are ordered by row chunk, sender, group and position.  One unit weighs as much as its row
+// chunk has halves.  Unit that begins at or after weight `w`, and its place in the order.
+template <int PASS>
+__device__ __forceinline__ int64_t unit_at(const TcBatch& bt, int64_t w, Unit* un) {
+    const int nS = bt.nL * bt.Hkv, max_rc = PASS == 1 ? bt.max_rc1 : bt.max_rc2;
+    int64_t u = 0;
+    for (int rc = 0; rc < max_rc; ++rc)
+        for (int i = 0; i < bt.n; ++i) {
+            const TcSender& sd = bt.s[i];
+            const int n = n_rc<PASS>(sd);
+            if (rc >= n) continue;
+            const int wt = rc_begin(sd.halves, n, rc + 1) - rc_begin(sd.halves, n, rc);
+            const int64_t units = (int64_t)nS * n_c<PASS>(sd);
+            if (w < units * wt) {
+                const int64_t k = (w + wt - 1) / wt;
+                if (k < units) {
+                    *un = Unit{i, (int)(k / n_c<PASS>(sd)), (int)(k % n_c<PASS>(sd)), rc};
+                    return u + k;
+                }
+                w = units * wt;   // rounds up to the next sender's first unit
+            }
+            w -= units * wt;
+            u += units;
         }
-    }
+    return u;
 }
 
-// Pass-1 units likewise (sender, group, chunk).
-__device__ __forceinline__ void next1(const TcBatch& bt, Unit& un) {
-    if (un.i >= bt.n) return;
-    if (++un.c == bt.s[un.i].n_chunk1 / 4) {
-        un.c = 0;
-        if (++un.s == bt.nL * bt.Hkv) {
-            un.s = 0;
-            ++un.i;
+// This CTA's contiguous share of the units (by weight), into shared memory.
+template <int PASS>
+__device__ __forceinline__ void my_units(const TcBatch& bt, Ctl* ctl) {
+    const int64_t total = PASS == 1 ? bt.weight1 : bt.weight2;
+    Unit first{0, 0, 0, 0}, end;
+    const int64_t b = unit_at<PASS>(bt, total * blockIdx.x / gridDim.x, &first);
+    ctl->units = (int32_t)(unit_at<PASS>(bt, total * (blockIdx.x + 1) / gridDim.x, &end) - b);
+    ctl->first = first;
+}
+
+// The next unit in order, without a division.  `nc`: the sender's chunks or blocks, kept by the
+// caller (an indexed read of the kernel parameters for every unit holds a role up).
+template <int PASS>
+__device__ __forceinline__ void next_unit(const TcBatch& bt, Unit& un, int nc) {
+    if (++un.c < nc) return;
+    un.c = 0;
+    if (++un.s < bt.nL * bt.Hkv) return;
+    un.s = 0;
+    const int max_rc = PASS == 1 ? bt.max_rc1 : bt.max_rc2;
+    do {
+        if (++un.i == bt.n) {
+            un.i = 0;
+            if (++un.rc >= max_rc) {   // past the last unit
+                un.rc = 0;
+                return;
+            }
         }
-    }
+    } while (n_rc<PASS>(bt.s[un.i]) <= un.rc);
 }
 
-// Contiguous share of `total` units for this CTA.
-__device__ __forceinline__ void my_range(int64_t total, int64_t* b, int64_t* e) {
-    *b = total * blockIdx.x / gridDim.x;
-    *e = total * (blockIdx.x + 1) / gridDim.x;
-}
-
-// Shared memory: [Q: 2 blocks x rpad x 128 B][offset terms: rpad x 32 B][ones: 4 KB]
-// [K ring: stages x 32 KB][Ctl][epilogue scratch]
+// Shared memory of pass 1: [Q: d / 64 blocks x rows1 x 128 B][K ring][Ctl]; of pass 2:
+// [Q][offset terms: rows2 x 32 B][ones: 4 KB][K blocks of four tiles][Ctl][exchange of sums].
 struct Smem {
     uint8_t* q;
-    uint8_t* ext;     // pass 2: offset terms of Q's rows [rpad][32 B], 32-byte swizzle
+    uint8_t* ext;     // pass 2: offset terms of Q's rows [rows2][32 B], 32-byte swizzle
     uint8_t* ones;    // pass 2: ones columns [128][32 B], 32-byte swizzle
     uint8_t* k;
     Ctl* ctl;
     float* epi;
 };
 
+template <int D, int PASS>
 __device__ __forceinline__ Smem carve(uint8_t* raw, const TcBatch& bt) {
+    constexpr int kTile = kTileRows * D * 2;
     Smem sm;
     uint8_t* base = align1024(raw);
     sm.q = base;
-    sm.ext = base + (size_t)2 * bt.rpad_max * 128;
-    sm.ones = sm.ext + (size_t)bt.rpad_max * 32;
-    sm.k = sm.ones + 128 * 32;
-    sm.ctl = reinterpret_cast<Ctl*>(sm.k + (size_t)bt.stages * kTileBytes);
+    if (PASS == 1) {
+        sm.ext = sm.ones = nullptr;
+        sm.k = base + (size_t)bt.rows1 * D * 2;
+        sm.ctl = reinterpret_cast<Ctl*>(sm.k + (size_t)bt.stages1 * kTile);
+    } else {
+        sm.ext = base + (size_t)bt.rows2 * D * 2;
+        sm.ones = sm.ext + (size_t)bt.rows2 * 32;
+        sm.k = sm.ones + 128 * 32;
+        sm.ctl = reinterpret_cast<Ctl*>(sm.k + (size_t)4 * bt.kbufs * kTile);
+    }
     sm.epi = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(sm.ctl) + 512);
     return sm;
 }
 
-// `releasers`: warps that arrive on a TMEM buffer's empty barrier (pass 1: the eight warps of a
-// group; pass 2: the four warps of one column half).
-__device__ __forceinline__ void init_ctl(Ctl* ctl, int stages, int releasers, uint64_t wait_ns) {
-    for (int k = 0; k < stages; ++k) {
+// `k_releasers`: MMA issuers that arrive on a K slot's empty barrier.
+__device__ __forceinline__ void init_ctl(Ctl* ctl, int k_releasers, uint64_t wait_ns) {
+    for (int k = 0; k < kMaxStages; ++k) {
         mbar_init(&ctl->k_full[k], 1);
-        mbar_init(&ctl->k_empty[k], 1);
+        mbar_init(&ctl->k_empty[k], k_releasers);
     }
     for (int b = 0; b < 4; ++b) {
         mbar_init(&ctl->t_full[b], 1);
-        mbar_init(&ctl->t_empty[b], releasers);
+        mbar_init(&ctl->t_empty[b], kEpiWarps);
     }
+    mbar_init(&ctl->xb, kEpiWarps);
+    mbar_init(&ctl->xe, 1);
     mbar_init(&ctl->q_full, 1);
-    mbar_init(&ctl->q_empty, 1);
-    mbar_init(&ctl->drain, 1);
+    mbar_init(&ctl->q_empty, 2);
+    mbar_init(&ctl->drain[0], 1);
+    mbar_init(&ctl->drain[1], 1);
     mbar_init(&ctl->o_full, 1);
     mbar_init(&ctl->stall, 1);
     ctl->wait_ns = wait_ns;
-    for (int k = 0; k < 16; ++k) {
-        mbar_init(&ctl->xb[k >> 3][(k >> 2) & 1][k & 3], 1);
-        mbar_init(&ctl->xe[k >> 3][(k >> 2) & 1][k & 3], 1);
-    }
     ctl->abort = 0;
     fence_barrier_init();
 }
 
-// Producer: Q of group s (all rows, both column blocks) into the Q region.
-// Pass 2 (with_ext) also brings the rows' offset terms of group s = l * Hkv + g.
-__device__ __forceinline__ void load_q(const TcBatch& bt, const TcSender& sd, const Smem& sm, int l, int g,
-                                       bool with_ext) {
-    const uint32_t bytes = (uint32_t)sd.R_pad * (with_ext ? 256u + 32u : 256u);
-    mbar_arrive_expect_tx(&sm.ctl->q_full, bytes);
-    if (with_ext)
-        for (int b = 0; b < sd.n_ebox; ++b)
-            tma_load_3d(sm.ext + (size_t)b * sd.ebox_rows * 32, &sd.emap, &sm.ctl->q_full, 0, b * sd.ebox_rows,
-                        l * bt.Hkv + g);
-    for (int kb = 0; kb < 2; ++kb)
-        for (int b = 0; b < sd.n_qbox; ++b)
-            tma_load_4d(sm.q + (size_t)kb * bt.rpad_max * 128 + (size_t)b * sd.qbox_tok * bt.G * 128, &sd.qmap,
-                        &sm.ctl->q_full, 64 * kb, g * bt.G, b * sd.qbox_tok, l);
-}
-
-__device__ __forceinline__ void load_k(const TcSender& sd, const Smem& sm, int stage, int l, int g, int32_t t_start) {
-    uint8_t* dst = sm.k + (size_t)stage * kTileBytes;
-    mbar_arrive_expect_tx(&sm.ctl->k_full[stage], kTileBytes);
-    tma_load_4d(dst, &sd.kmap, &sm.ctl->k_full[stage], 0, t_start, g, l);
-    tma_load_4d(dst + kTileBytes / 2, &sd.kmap, &sm.ctl->k_full[stage], 64, t_start, g, l);
-}
-
-// One K = 128 contraction (8 UMMA K-steps).  a_base / b_base: first column block of each
-// operand (rows of 128 B); the second column block sits `a_blk` / `b_blk` bytes later.
-// The descriptors are built once; a K-step only moves the start-address field.
-__device__ __forceinline__ void mma_k128(uint32_t d_tmem, uint32_t a_base, uint32_t a_blk, uint32_t b_base,
-                                        uint32_t b_blk, uint32_t idesc) {
-    const uint64_t ad0 = smem_desc_sw128(a_base), bd0 = smem_desc_sw128(b_base);
-    const uint64_t ad1 = ad0 + (a_blk >> 4), bd1 = bd0 + (b_blk >> 4);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const uint64_t off = (uint64_t)((k & 3) * 2);   // 32 bytes >> 4
-        umma_bf16(d_tmem, (k < 4 ? ad0 : ad1) + off, (k < 4 ? bd0 : bd1) + off, idesc, k > 0 ? 1u : 0u);
+// Producer: the 128-row halves [h0, h0 + nh) of group s's Q (s = l * Hkv + g) into the Q region
+// (column blocks of `rows` rows).  Pass 2 also brings the rows' offset terms.
+template <int D, int PASS>
+__device__ __forceinline__ void load_q(const TcBatch& bt, const TcMaps& mp, const Smem& sm, int s, int h0, int nh) {
+    const int l = s / bt.Hkv, g = s % bt.Hkv;
+    const int rows = PASS == 1 ? bt.rows1 : bt.rows2;
+    mbar_arrive_expect_tx(&sm.ctl->q_full, (uint32_t)nh * kRowHalf * (D * 2 + (PASS == 2 ? 32 : 0)));
+    for (int h = 0; h < nh; ++h) {
+        if (PASS == 2)
+            tma_load_3d(sm.ext + (size_t)h * kRowHalf * 32, &mp.e, &sm.ctl->q_full, 0, (h0 + h) * kRowHalf, s);
+        for (int kb = 0; kb < D / 64; ++kb)
+            tma_load_4d(sm.q + ((size_t)kb * rows + h * kRowHalf) * 128, &mp.q, &sm.ctl->q_full, 64 * kb, g * bt.G,
+                        (h0 + h) * kRowHalf / bt.G, l);
     }
 }
 
-// One 32-column block of pass 1 for this lane's row: running offset m (log2 domain) and
-// sum of exp2(c z - m).  The first block of a chunk (known from the loop indices: testing m
-// instead cost 2%) sets m to its max, or to -FLT_MAX when it holds no position, in which case
-// neither does the rest of the chunk; later blocks reuse m without a check (a per-block test
-// and redo cost 11% of this kernel).  Values up to 2^127 above
-// the first block are exact; a logit so far above it that exp2 or the sum overflows leaves an
-// infinite sum, and the combine kernel recomputes that row's statistics from Q and K.
-__device__ __forceinline__ void stats_block(float (&v)[32], int nvalid, float c, uint64_t cc, float& m, float& sum,
-                                            bool first) {
-    if (nvalid < 32) {
+// Low word of a shared-memory matrix descriptor (the address field); the high word is a constant
+// of the swizzle, so a K-step or another row block only adds to the low word.
+__device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+    return d;
+}
+
+// One contraction over d (d / 16 UMMA K-steps) into d_tmem: operand rows of 128 B in 64-column
+// blocks that lie `a_blk` / `b_blk` (16-byte units) apart.
+template <int D>
+__device__ __forceinline__ void mma_d(uint32_t d_tmem, uint32_t a_lo, uint32_t a_blk, uint32_t b_lo, uint32_t b_blk,
+                                      uint32_t hi, uint32_t idesc) {
 #pragma unroll
-        for (int q = 0; q < 32; ++q) v[q] = q < nvalid ? v[q] : -INFINITY;
-    }
-    if (first) m = fmaxf(max_tree1(v) * c, -FLT_MAX);
-    const uint64_t nm = pack2(-m, -m);
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};   // exp2 results are summed as scalars (no pair packing)
+    for (int k = 0; k < D / 16; ++k)
+        umma_bf16(d_tmem, desc64(a_lo + (k / 4) * a_blk + (k & 3) * 2, hi), desc64(b_lo + (k / 4) * b_blk + (k & 3) * 2, hi),
+                  idesc, k > 0 ? 1u : 0u);
+}
+
+// 32 columns of pass 1 for this lane's row: sum of exp2(c z - m), m the row's offset (log2
+// domain): its first logit of the chunk, or -FLT_MAX where the warp's first block holds no
+// position, in which case neither do the chunk's others.  The sum holds that logit's 1, and any
+// logit up to 2^127 above it is exact; one so far above it that exp2 or the sum overflows leaves
+// an infinite sum, and the combine kernel recomputes that row's statistics from Q and K.  (The
+// maximum of the first block in place of its first logit makes the buffers that hold one wait for
+// the maximum: 788 against 729 cycles a buffer.)  The packed adds leave the loop bound by exp2 (584 cycles for a
+// 128 x 128 buffer, 603 with scalar adds, against 512 for its exp2 alone).
+__device__ __forceinline__ void stats_block(const float (&v)[32], uint64_t cc, uint64_t nm, uint64_t& p0, uint64_t& p1) {
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        float a0, a1;
+    for (int q = 0; q < 16; q += 2) {
+        float a0, a1, b0, b1;
         unpack2(ffma2(pack2(v[2 * q], v[2 * q + 1]), cc, nm), a0, a1);
-        acc[(2 * q) & 3] += ex2(a0);
-        acc[(2 * q + 1) & 3] += ex2(a1);
+        unpack2(ffma2(pack2(v[2 * q + 2], v[2 * q + 3]), cc, nm), b0, b1);
+        p0 = fadd2(p0, pack2(ex2(a0), ex2(a1)));
+        p1 = fadd2(p1, pack2(ex2(b0), ex2(b1)));
     }
-    sum += (acc[0] + acc[1]) + (acc[2] + acc[3]);
 }
 
 // ===========================================================================
 // pass 1
 // ===========================================================================
-// Epilogue: the two groups of four warps take alternate K tiles (tile index within the
-// chunk, even -> group 0).  Thread = TMEM lane = row 128 h + lane of every half h; it keeps
-// the running max and sum of exp2 of its rows over its group's tiles of the chunk and writes
-// them as partial (chunk, group); the combine kernel merges all partials of a group s.
+// Epilogue: thread = TMEM lane = row 128 h + lane of every half h and a quarter of each tile's
+// positions; it keeps the offset and sum of exp2 of its rows over the chunk and writes them as
+// partial (chunk, quarter); the combine kernel merges all partials of a group s.  The two MMA
+// issuers take alternate buffers.
+template <int D, int NH>
 __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constant__ TcBatch bt) {
+    constexpr int kTile = kTileRows * D * 2;
     extern __shared__ uint8_t smem_raw[];
-    const Smem sm = carve(smem_raw, bt);
+    const Smem sm = carve<D, 1>(smem_raw, bt);
     Ctl* ctl = sm.ctl;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) init_ctl(ctl, bt.stages, 8, bt.wait_ns);
+    if (threadIdx.x == 0) {
+        init_ctl(ctl, 2, bt.wait_ns);
+        my_units<1>(bt, ctl);
+    }
     if (warp == 1) {
         tmem_alloc(&ctl->tmem_base, kTmemCols);
         tmem_relinquish();
@@ -318,9 +370,9 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
-    int64_t ub, ue;
-    my_range(bt.units1, &ub, &ue);
-    const int stages = bt.stages;
+    const int n_units = ctl->units;
+    Unit un = ctl->first;
+    const int stages = bt.stages1;
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
@@ -328,24 +380,30 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
             int64_t kt = 0, qn = 0;   // K tiles and Q loads issued
             int st = 0;               // ring slot of the next K tile and its phase parity
             uint32_t ph = 0;
-            int prev = -1;
             bool ok = true;
-            Unit un = decode1(bt, ub);
-            for (int64_t u = ub; u < ue && ok; ++u, next1(bt, un)) {
-                const TcSender& sd = bt.s[un.i];
-                const int l = un.s / bt.Hkv, g = un.s % bt.Hkv;
-                const int key = un.i * 65536 + un.s;
-                if (key != prev) {
+            int nc = 0, l = 0, g = 0;
+            int64_t T = 0;
+            for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
+                const TcMaps& mp = bt.maps[un.i];
+                if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
+                    const TcSender& sd = bt.s[un.i];
+                    nc = n_c<1>(sd);
+                    T = sd.T;
+                    l = un.s / bt.Hkv;
+                    g = un.s % bt.Hkv;
                     if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 0))) break;
-                    load_q(bt, sd, sm, l, g, false);
+                    const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
+                    load_q<D, 1>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0);
                     ++qn;
-                    prev = key;
                 }
                 const int64_t c0 = (int64_t)un.c * kChunk1;
-                const int nt = (int)((min((int64_t)kChunk1, sd.T - c0) + kTileRows - 1) / kTileRows);
+                const int nt = (int)((min((int64_t)kChunk1, T - c0) + kTileRows - 1) / kTileRows);
                 for (int tile = 0; tile < nt; ++tile) {
                     if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 1))) break;
-                    load_k(sd, sm, st, l, g, (int32_t)(c0 + tile * kTileRows));
+                    mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
+                    for (int kb = 0; kb < D / 64; ++kb)
+                        tma_load_4d(sm.k + (size_t)st * kTile + kb * kTileRows * 128, &mp.k[0], &ctl->k_full[st], 64 * kb,
+                                    (int32_t)(c0 + tile * kTileRows), g, l);
                     ++kt;
                     if (++st == stages) { st = 0; ph ^= 1u; }
                 }
@@ -355,110 +413,127 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                 drain_wait(&ctl->k_full[k % stages], (uint32_t)((k / stages) & 1));
             if (qn > 0) drain_wait(&ctl->q_full, (uint32_t)((qn - 1) & 1));
         }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer ----------------
+    } else if (warp <= 2) {
+        // ---------------- MMA issuers ----------------
         if (elect_one()) {
-            int64_t qn = 0, jg0 = 0, jg1 = 0;   // Q loads consumed; items issued per epilogue group
-            int st = 0;                          // ring slot of the next K tile and its phase parity
+            const uint32_t me = (uint32_t)warp - 1;
+            uint32_t qn = 0;          // Q loads consumed
+            uint32_t n = 0;           // accumulator buffers filled by both issuers
+            int st = 0;               // ring slot of the next K tile and its phase parity
             uint32_t ph = 0;
-            int prev = -1;
             bool ok = true;
+            constexpr uint32_t idesc = idesc_bf16_f32(128, 128);
+            const uint64_t qd = smem_desc_sw128(smem_u32(sm.q));
+            const uint32_t hi = (uint32_t)(qd >> 32), q_lo = (uint32_t)qd;
+            const uint32_t k_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.k));
+            const uint32_t q_blk = (uint32_t)bt.rows1 * 128 >> 4;
             // failure-detection test: wait on a barrier that nothing arrives on, so the bounded
             // wait gives up, sets the abort flag and every role of this CTA leaves
             if (bt.stall && blockIdx.x == 0) ok = wait_bar(&ctl->stall, 0, ctl, bt.err, 6);
-            Unit un = decode1(bt, ub);
-            for (int64_t u = ub; u < ue && ok; ++u, next1(bt, un)) {
-                const TcSender& sd = bt.s[un.i];
-                const int key = un.i * 65536 + un.s;
-                if (key != prev) {
-                    if (prev >= 0) umma_commit(&ctl->q_empty);
-                    if (!(ok = wait_bar(&ctl->q_full, (uint32_t)(qn & 1), ctl, bt.err, 2))) break;
-                    tc_fence_after();
+            uint32_t nh = 0;
+            int nc = 0;
+            int64_t T = 0;
+            for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
+                if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
+                    const TcSender& sd = bt.s[un.i];
+                    nc = n_c<1>(sd);
+                    T = sd.T;
+                    nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - rc_begin(sd.halves, sd.n_rc1, un.rc);
+                    if (u > 0) umma_commit(&ctl->q_empty);
+                    if (!(ok = wait_bar(&ctl->q_full, qn & 1, ctl, bt.err, 2))) break;
                     ++qn;
-                    prev = key;
                 }
-                const int halves = sd.R_pad / 128;
                 const int64_t c0 = (int64_t)un.c * kChunk1;
-                const int nt = (int)((min((int64_t)kChunk1, sd.T - c0) + kTileRows - 1) / kTileRows);
-                for (int tile = 0; tile < nt && ok; ++tile) {
+                const int nt = (int)((min((int64_t)kChunk1, T - c0) + kTileRows - 1) / kTileRows);
+                for (int tile = 0; tile < nt; ++tile) {
                     if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
-                    tc_fence_after();
-                    const uint32_t kaddr = smem_u32(sm.k + (size_t)st * kTileBytes);
-                    const int grp = tile & 1;     // epilogue group that owns this tile
-                    for (int h = 0; h < halves; ++h) {
-                        const int64_t j = grp ? jg1++ : jg0++;
-                        const int buf = 2 * grp + (int)(j & 1);
-                        if (!(ok = wait_bar(&ctl->t_empty[buf], (uint32_t)(((j >> 1) & 1) ^ 1), ctl, bt.err, 4))) break;
+                    const uint32_t kt_lo = k_lo + (uint32_t)st * (kTile >> 4);
+                    for (uint32_t h = (n ^ me) & 1; h < nh; h += 2) {   // the tile's buffers n + h of my parity
+                        const uint32_t x = n + h, buf = x & 3;
+                        if (!(ok = wait_bar(&ctl->t_empty[buf], ((x >> 2) & 1) ^ 1, ctl, bt.err, 4))) break;
                         tc_fence_after();
-                        mma_k128(tmem + buf * 128, smem_u32(sm.q) + h * 128 * 128, (uint32_t)bt.rpad_max * 128,
-                                 kaddr, kTileBytes / 2, idesc_bf16_f32(128, 128));
+                        mma_d<D>(tmem + buf * 128, q_lo + h * (kRowHalf * 128 >> 4), q_blk, kt_lo, kTileRows * 128 >> 4, hi,
+                                 idesc);
                         umma_commit(&ctl->t_full[buf]);
                     }
+                    if (!ok) break;
+                    n += nh;
                     umma_commit(&ctl->k_empty[st]);
                     if (++st == stages) { st = 0; ph ^= 1u; }
                 }
             }
-            umma_commit(&ctl->drain);
-            drain_wait(&ctl->drain, 0);
+            umma_commit(&ctl->drain[me]);
+            drain_wait(&ctl->drain[me], 0);
         }
-    } else {
+    } else if (warp >= kEpi0) {
         // ---------------- epilogue: running max / sum per row ----------------
-        // 16 warps: quad = (warp - 2) / 4; group = quad / 2 takes the tiles whose index in the
-        // chunk has its parity, half = quad % 2 takes positions half*64 .. +64 of each tile.
-        const int quad = (warp - 2) >> 2, grp = quad >> 1, hf = quad & 1;
+        const int q = (warp - kEpi0) >> 2;       // column quarter: positions 32 q .. +31 of each tile
         const int sp = warp & 3;                 // TMEM lane quarter
         const int L = sp * 32 + lane;
-        const uint32_t lane_addr = (uint32_t)(sp * 32) << 16;
+        const uint32_t ta = tmem + ((uint32_t)(sp * 32) << 16) + 32 * q;
         const float c = bt.sl2e;
         const uint64_t cc = pack2(c, c);
-        int64_t j = 0;                           // items of this group so far
+        uint32_t n = 0;                          // accumulator buffers consumed
+        float M[NH];                             // per half: offset (log2 domain) and sum of exp2(c z - offset)
+        uint64_t S[NH];
         bool ok = true;
-        Unit un = decode1(bt, ub);
-        for (int64_t u = ub; u < ue && ok; ++u, next1(bt, un)) {
-            const TcSender& sd = bt.s[un.i];
-            const int halves = sd.R_pad / 128;
-            const int64_t c0 = (int64_t)un.c * kChunk1;
-            const int nt = (int)((min((int64_t)kChunk1, sd.T - c0) + kTileRows - 1) / kTileRows);
-            float M[4], S[4];                    // per half: offset (log2 domain) and sum of exp2(c z - offset)
+        // One tile, one buffer a half: load its 32 columns, hand the buffer back, sum.  PART: a tile
+        // with positions past T (`nvalid` of the 32 columns hold one).  The first tile of a chunk
+        // sets the offset to its first logit (to -FLT_MAX where it has none).
+        auto tile = [&](auto part, int nvalid, bool first, int nh) {
+            constexpr bool PART = decltype(part)::value;
 #pragma unroll
-            for (int h = 0; h < 4; ++h) { M[h] = -INFINITY; S[h] = 0.f; }
-            for (int tile = 0; tile < nt && ok; ++tile) {
-                if ((tile & 1) != grp) continue;
-                const int nvalid = (int)min((int64_t)kTileRows, sd.T - (c0 + tile * kTileRows)) - hf * 64;
+            for (int h = 0; h < NH; ++h) {
+                if (h >= nh) break;
+                const uint32_t buf = n & 3;
+                if (!(ok = wait_bar(&ctl->t_full[buf], (n >> 2) & 1, ctl, bt.err, 5))) break;
+                ++n;
+                tc_fence_after();
+                float v[32];
+                tmem_ld32(ta + buf * 128, v);
+                tmem_wait_ld(v);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->t_empty[buf]);
+                if (PART) {
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                    if (h >= halves) break;
-                    const int buf = 2 * grp + (int)(j & 1);
-                    if (!(ok = wait_bar(&ctl->t_full[buf], (uint32_t)((j >> 1) & 1), ctl, bt.err, 5))) break;
-                    ++j;
-                    tc_fence_after();
-                    const uint32_t ta = tmem + lane_addr + buf * 128 + hf * 64;
-                    float m = M[h], sum = S[h];
-#pragma unroll
-                    for (int half32 = 0; half32 < 2; ++half32) {
-                        float v[32];
-                        tmem_ld32(ta + 32 * half32, v);
-                        tmem_wait_ld(v);
-                        if (half32 == 1) {
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(&ctl->t_empty[buf]);   // registers hold the rest
-                        }
-                        stats_block(v, nvalid - 32 * half32, c, cc, m, sum, tile == grp && half32 == 0);
-                    }
-                    M[h] = m;
-                    S[h] = sum;
+                    for (int e = 0; e < 32; ++e) v[e] = e < nvalid ? v[e] : -INFINITY;
                 }
+                if (first) M[h] = fmaxf(v[0] * c, -FLT_MAX);
+                const uint64_t nm = pack2(-M[h], -M[h]);
+                uint64_t p0 = 0, p1 = 0;
+                stats_block(v, cc, nm, p0, p1);
+                S[h] = fadd2(S[h], fadd2(p0, p1));
             }
-            if (!ok) break;
-            // this warp's partial statistics for the chunk: slot 4 c + 2 grp + hf (rows of
-            // tiles it saw none of stay (-inf, 0), rows of positions past T (-FLT_MAX, 0), both
-            // of which add nothing); the combine kernel merges all slots
-            float2* dst = sd.stats + ((int64_t)un.s * sd.n_chunk1 + 4 * un.c + 2 * grp + hf) * sd.R;
+        };
+        float2* dst = nullptr;                   // the current group's partials of this thread's first row
+        int nh = 0, nc = 0, rows = 0, R = 0;     // rows: query rows from the thread's first on
+        int64_t T = 0;
+        for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
+            if (u == 0 || un.c == 0) {
+                const TcSender& sd = bt.s[un.i];
+                const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
+                nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0;
+                nc = n_c<1>(sd);
+                T = sd.T;
+                R = sd.R;
+                rows = R - h0 * kRowHalf - L;
+                dst = sd.stats + ((int64_t)un.s * sd.n_chunk1 + q) * R + h0 * kRowHalf + L;
+            }
+            const int len = (int)min((int64_t)kChunk1, T - (int64_t)un.c * kChunk1);
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                const int row = h * 128 + L;
-                if (h < halves && row < sd.R) dst[row] = make_float2(M[h], S[h]);
+            for (int h = 0; h < NH; ++h) { M[h] = -INFINITY; S[h] = 0; }
+            int t0 = 0;
+            for (; t0 + kTileRows <= len && ok; t0 += kTileRows) tile(std::false_type{}, 32, t0 == 0, nh);
+            if (t0 < len && ok) tile(std::true_type{}, len - t0 - 32 * q, t0 == 0, nh);
+            if (!ok) break;
+            // this warp's partial statistics for the chunk: slot 4 c + q (rows of positions past T
+            // are (-FLT_MAX, 0), which adds nothing); the combine kernel merges all slots
+#pragma unroll
+            for (int h = 0; h < NH; ++h) {
+                float s0, s1;
+                unpack2(S[h], s0, s1);
+                if (h < nh && h * kRowHalf < rows) dst[(int64_t)4 * un.c * R + h * kRowHalf] = make_float2(M[h], s0 + s1);
             }
         }
     }
@@ -470,114 +545,87 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
 // ===========================================================================
 // pass 2
 // ===========================================================================
-// Window max over lanes lane-PH .. lane+PH of x (valid for lanes 3..28, the output lanes).
+// Pool over positions: the thread holds x[0..3], four neighbouring positions; the lane before it
+// the four before, the lane after it the four after.  o[k] = max over positions k - PH .. k + PH.
+// The window of each position is the thread's own part of it and a suffix of the lane before or a
+// prefix of the lane after: six shuffles for four positions (PH = 3).
 template <int PH>
-__device__ __forceinline__ float lane_pool(float x) {
-    if (PH == 0) return x;
-    if (PH == 1) {
-        const float a = __shfl_up_sync(0xffffffffu, x, 1);
-        const float b = __shfl_down_sync(0xffffffffu, x, 1);
-        return fmaxf(x, fmaxf(a, b));
+__device__ __forceinline__ void pool4(const float (&x)[4], float (&o)[4]) {
+    constexpr unsigned kAll = 0xffffffffu;
+    if (PH == 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) o[k] = x[k];
+    } else if (PH == 1) {
+        o[0] = fmax3(__shfl_up_sync(kAll, x[3], 1), x[0], x[1]);
+        o[1] = fmax3(x[0], x[1], x[2]);
+        o[2] = fmax3(x[1], x[2], x[3]);
+        o[3] = fmax3(x[2], x[3], __shfl_down_sync(kAll, x[0], 1));
+    } else if (PH == 2) {
+        const float s23 = fmaxf(x[2], x[3]), p01 = fmaxf(x[0], x[1]);
+        const float all = fmaxf(p01, s23);
+        o[0] = fmax3(__shfl_up_sync(kAll, s23, 1), p01, x[2]);
+        o[1] = fmaxf(__shfl_up_sync(kAll, x[3], 1), all);
+        o[2] = fmaxf(all, __shfl_down_sync(kAll, x[0], 1));
+        o[3] = fmax3(x[1], s23, __shfl_down_sync(kAll, p01, 1));
+    } else {
+        const float s23 = fmaxf(x[2], x[3]), p01 = fmaxf(x[0], x[1]);
+        const float s123 = fmaxf(x[1], s23), p012 = fmaxf(p01, x[2]);
+        const float all = fmaxf(p01, s23);
+        o[0] = fmaxf(__shfl_up_sync(kAll, s123, 1), all);
+        o[1] = fmax3(__shfl_up_sync(kAll, s23, 1), all, __shfl_down_sync(kAll, x[0], 1));
+        o[2] = fmax3(__shfl_up_sync(kAll, x[3], 1), all, __shfl_down_sync(kAll, p01, 1));
+        o[3] = fmaxf(all, __shfl_down_sync(kAll, p012, 1));
     }
-    if (PH == 2) {
-        const float a1 = fmaxf(x, __shfl_down_sync(0xffffffffu, x, 1));        // [l, l+1]
-        const float b1 = __shfl_up_sync(0xffffffffu, a1, 2);                   // [l-2, l-1]
-        return fmaxf(fmaxf(a1, b1), __shfl_down_sync(0xffffffffu, x, 2));      // [l-2, l+2]
-    }
-    const float a1 = fmaxf(x, __shfl_down_sync(0xffffffffu, x, 1));            // [l, l+1]
-    const float a2 = fmaxf(a1, __shfl_down_sync(0xffffffffu, a1, 2));          // [l, l+3]
-    return fmaxf(a2, __shfl_up_sync(0xffffffffu, a2, 3));                      // [l-3, l+3]
 }
 
-template <bool P2>
-__device__ __forceinline__ float pow_p(float x, float p) {
-    if (P2) return x * x;
-    return x > 0.f ? ex2(p * lg2(x)) : 0.f;
+__device__ __forceinline__ float pow_p(float x, float p) { return x > 0.f ? ex2(p * lg2(x)) : 0.f; }
+
+// e0 + .. + e3 as (e0 + e2) + (e1 + e3): one packed add of neighbouring registers, one scalar add.
+__device__ __forceinline__ float sum4(const float* e) {
+    float p, q;
+    unpack2(fadd2(pack2(e[0], e[1]), pack2(e[2], e[3])), p, q);
+    return p + q;
 }
 
-// One 32-column block of pass 2 for this lane's position: a / G = exp2(c z - offset) per
-// column, b = sum over the G heads of each token, then Pool over positions and the sums.
-// Tokens 2i and 2i + 1 share one packed f32x2 add or fma: lane 0 of each pair is the chain of
-// even tokens and lane 1 that of odd tokens, the same order of additions as two scalar chains.
-template <int G, int PH, bool P2>
-__device__ __forceinline__ void accum_block(const float (&v)[32], uint64_t cc, bool valid, bool all_valid, float p,
-                                            bool p_inf, float (&nacc)[2], float (&bsum)[2]) {
-    float e[32];
+// Head sums of C / G tokens from their C columns: a / G = exp2(c z - offset) per column, summed
+// over each token's G heads, as pairs of tokens (2 i, 2 i + 1).
+template <int G, int C>
+__device__ __forceinline__ void head_sums(const float (&v)[C], uint64_t cc, uint64_t* b) {
+    float e[C];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        float a0, a1, a2, a3;
-        unpack2(fmul2(pack2(v[4 * q], v[4 * q + 1]), cc), a0, a1);
-        unpack2(fmul2(pack2(v[4 * q + 2], v[4 * q + 3]), cc), a2, a3);
-        e[4 * q] = ex2(a0);
-        e[4 * q + 1] = ex2(a1);
-        e[4 * q + 2] = ex2(a2);
-        e[4 * q + 3] = ex2(a3);
+    for (int q = 0; q < C / 2; ++q) {
+        float a0, a1;
+        unpack2(fmul2(pack2(v[2 * q], v[2 * q + 1]), cc), a0, a1);
+        e[2 * q] = ex2(a0);
+        e[2 * q + 1] = ex2(a1);
     }
-    constexpr int NP = 16 / G;   // token pairs in these 32 columns
-    uint64_t b[NP];
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
+    for (int i = 0; i < C / (2 * G); ++i) {
         if (G == 1) b[i] = pack2(e[2 * i], e[2 * i + 1]);
-        if (G == 2) b[i] = fadd2(pack2(e[4 * i], e[4 * i + 2]), pack2(e[4 * i + 1], e[4 * i + 3]));
+        if (G == 2) b[i] = pack2(e[4 * i] + e[4 * i + 1], e[4 * i + 2] + e[4 * i + 3]);
         if (G == 4)
-            b[i] = fadd2(fadd2(pack2(e[8 * i], e[8 * i + 4]), pack2(e[8 * i + 1], e[8 * i + 5])),
-                         fadd2(pack2(e[8 * i + 2], e[8 * i + 6]), pack2(e[8 * i + 3], e[8 * i + 7])));
+            b[i] = pack2(sum4(e + 8 * i), sum4(e + 8 * i + 4));
     }
-    if (!all_valid) {
-#pragma unroll
-        for (int i = 0; i < NP; ++i) b[i] = valid ? b[i] : 0ull;
-    }
-    uint64_t bs = pack2(bsum[0], bsum[1]), na = pack2(nacc[0], nacc[1]);
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-        float b0, b1;
-        unpack2(b[i], b0, b1);
-        const float p0 = lane_pool<PH>(b0), p1 = lane_pool<PH>(b1);
-        bs = fadd2(bs, b[i]);
-        if (P2) {
-            const uint64_t pp = pack2(p0, p1);
-            na = ffma2(pp, pp, na);
-        } else if (p_inf) {   // p = infinity: largest pooled value
-            nacc[0] = fmaxf(nacc[0], p0);
-            nacc[1] = fmaxf(nacc[1], p1);
-        } else {
-            nacc[0] += pow_p<false>(p0, p);
-            nacc[1] += pow_p<false>(p1, p);
-        }
-    }
-    unpack2(bs, bsum[0], bsum[1]);
-    if (P2) unpack2(na, nacc[0], nacc[1]);
 }
 
-// Pass 2, G = 4: head sums of the four tokens in 16 columns (exp2(c z - offset) summed over
-// each token's four heads) as the pairs (b0, b1) and (b2, b3); the packed adds keep each
-// token's order (e0 + e1) + (e2 + e3).
-__device__ __forceinline__ void head_sums16(const float (&v)[16], uint64_t cc, uint64_t& b01, uint64_t& b23) {
-    float e[16];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        float a0, a1, a2, a3;
-        unpack2(fmul2(pack2(v[4 * q], v[4 * q + 1]), cc), a0, a1);
-        unpack2(fmul2(pack2(v[4 * q + 2], v[4 * q + 3]), cc), a2, a3);
-        e[4 * q] = ex2(a0);
-        e[4 * q + 1] = ex2(a1);
-        e[4 * q + 2] = ex2(a2);
-        e[4 * q + 3] = ex2(a3);
-    }
-    b01 = fadd2(fadd2(pack2(e[0], e[4]), pack2(e[1], e[5])), fadd2(pack2(e[2], e[6]), pack2(e[3], e[7])));
-    b23 = fadd2(fadd2(pack2(e[8], e[12]), pack2(e[9], e[13])), fadd2(pack2(e[10], e[14]), pack2(e[11], e[15])));
-}
-
-// Epilogue: each warp owns 32 TMEM lanes = positions t0 + 26 w - 3 + lane (w = lane quarter);
-// lanes 3..28 are its output positions, the 3 lanes on each side their Pool margin (the K
-// rows of the four quarters overlap by 6 positions).  The two groups take alternate tiles.
-template <int G, int PH, bool P2>
+// Epilogue: lane quarter w = warp % 4 of a block covers positions 480 c + 120 w - 4 .. + 127; its
+// lane i holds positions 4 i .. 4 i + 3 of them, one in each of the block's four tiles.  Lanes 1
+// to 30 are outputs, lanes 0 and 31 their Pool margin.  The four warps of
+// a lane quarter take 32 columns (query rows) each of every buffer; their sums meet in
+// shared memory at the end of the block, where warp 3 does the adding: an epilogue warp that
+// waited for its three neighbours would hold up the next block's buffers (28 us of this pass).  MMA issuer i fills
+// the buffers of tiles i and i + 2.
+template <int D, int G, int PH, bool P2>
 __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constant__ TcBatch bt) {
+    constexpr int kTile = kTileRows * D * 2;
     extern __shared__ uint8_t smem_raw[];
-    const Smem sm = carve(smem_raw, bt);
+    const Smem sm = carve<D, 2>(smem_raw, bt);
     Ctl* ctl = sm.ctl;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) init_ctl(ctl, bt.stages, 4, bt.wait_ns);
+    if (threadIdx.x == 0) {
+        init_ctl(ctl, 1, bt.wait_ns);
+        my_units<2>(bt, ctl);
+    }
     if (warp == 1) {
         tmem_alloc(&ctl->tmem_base, kTmemCols);
         tmem_relinquish();
@@ -586,261 +634,232 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
-    int64_t ub, ue;
-    my_range(bt.units2, &ub, &ue);
-    const int stages = bt.stages;
+    const int n_units = ctl->units;
+    Unit un = ctl->first;
+    const int slots = 4 * bt.kbufs;
 
     if (warp == 0) {
         if (elect_one()) {
             int64_t kt = 0, qn = 0;   // K tiles and Q loads issued
-            int st = 0;               // ring slot of the next K tile and its phase parity
+            int st = 0;               // slot of the next K tile and its phase parity
             uint32_t ph = 0;
-            int prev = -1;
             bool ok = true;
             // the ones columns of the offset K-step, once per CTA
             mbar_arrive_expect_tx(&ctl->o_full, 128 * 32);
             tma_load_2d(sm.ones, &bt.omap, &ctl->o_full, 0, 0);
-            Unit un = decode2(bt, ub);
-            for (int64_t u = ub; u < ue && ok; ++u, next2(bt, un)) {
-                const TcSender& sd = bt.s[un.i];
-                const int l = un.s / bt.Hkv, g = un.s % bt.Hkv;
-                const int key = un.i * 65536 + un.s;
-                if (key != prev) {
+            int nc = 0, l = 0, g = 0, T = 0;
+            for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
+                const TcMaps& mp = bt.maps[un.i];
+                if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
+                    const TcSender& sd = bt.s[un.i];
+                    nc = sd.n_blk2;
+                    T = (int)sd.T;
+                    l = un.s / bt.Hkv;
+                    g = un.s % bt.Hkv;
                     if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 8))) break;
-                    load_q(bt, sd, sm, l, g, true);
+                    const int h0 = rc_begin(sd.halves, sd.n_rc2, un.rc);
+                    load_q<D, 2>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0);
                     ++qn;
-                    prev = key;
                 }
-                if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 9))) break;
-                // four 32-row boxes: quarter w holds positions t0 + 26 w - 3 .. + 31
-                uint8_t* dst = sm.k + (size_t)st * kTileBytes;
-                mbar_arrive_expect_tx(&ctl->k_full[st], kTileBytes);
-                const int32_t t0 = (int32_t)((int64_t)un.c * kOut2);
-                for (int w = 0; w < 4; ++w)
-                    for (int kb = 0; kb < 2; ++kb)
-                        tma_load_4d(dst + kb * (kTileBytes / 2) + w * 32 * 128, &sd.kmap32, &ctl->k_full[st],
-                                    64 * kb, t0 + kOutW * w - kMargin, g, l);
-                ++kt;
-                if (++st == stages) { st = 0; ph ^= 1u; }
+                const int32_t t0 = un.c * kOut2 - kMargin;
+                // the 5D map serves every tile (a change of map costs the TMA unit time: 150 against
+                // 115 us for the loads of this pass with a map a tile); the maps of the single tiles
+                // are for a last block that ends on one of the last T mod 4 positions
+                const bool whole = t0 + kOut2 + kMargin + 4 <= T / 4 * 4 || T % 4 == 0;
+                for (int j = 0; j < 4; ++j) {
+                    if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 9))) break;
+                    // lane quarter w: positions t0 + 120 w + j + 4 i, i = 0 .. 31 (t0 a multiple of four)
+                    uint8_t* dst = sm.k + (size_t)st * kTile;
+                    mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
+                    for (int w = 0; w < 4; ++w)
+                        for (int kb = 0; kb < D / 64; ++kb) {
+                            uint8_t* box = dst + kb * kTileRows * 128 + w * 32 * 128;
+                            const int32_t i0 = (t0 + kOutW * w) / 4;
+                            if (whole) tma_load_5d(box, &mp.k[4], &ctl->k_full[st], 64 * kb, i0, j, g, l);
+                            else tma_load_4d(box, &mp.k[j], &ctl->k_full[st], 64 * kb, i0, g, l);
+                        }
+                    ++kt;
+                    if (++st == slots) { st = 0; ph ^= 1u; }
+                }
             }
-            for (int64_t k = kt - stages > 0 ? kt - stages : 0; k < kt; ++k)
-                drain_wait(&ctl->k_full[k % stages], (uint32_t)((k / stages) & 1));
+            for (int64_t k = kt - slots > 0 ? kt - slots : 0; k < kt; ++k)
+                drain_wait(&ctl->k_full[k % slots], (uint32_t)((k / slots) & 1));
             if (qn > 0) drain_wait(&ctl->q_full, (uint32_t)((qn - 1) & 1));
             drain_wait(&ctl->o_full, 0);
         }
-    } else if (warp == 1) {
+    } else if (warp <= 2) {
         if (elect_one()) {
-            int64_t qn = 0;              // Q loads consumed
-            uint32_t jpar = 0;           // bit b: parity of the items issued into TMEM buffer b
-            int st = 0;                  // ring slot of the next K tile and its phase parity
+            const int me = warp - 1;
+            uint32_t qn = 0;             // Q loads consumed
+            uint32_t n = 0;              // rounds of the four accumulator buffers issued
+            int st0 = 0;                 // slot of the block's first K tile and its phase parity
             uint32_t ph = 0;
-            int prev = -1;
             bool ok = wait_bar(&ctl->o_full, 0, ctl, bt.err, 15);
-            tc_fence_after();
-            const uint64_t ones_desc = smem_desc_sw32(smem_u32(sm.ones));
-            const uint64_t ext_desc = smem_desc_sw32(smem_u32(sm.ext));
-            Unit un = decode2(bt, ub);
-            for (int64_t u = ub; u < ue && ok; ++u, next2(bt, un)) {
-                const TcSender& sd = bt.s[un.i];
-                const int key = un.i * 65536 + un.s;
-                if (key != prev) {
-                    if (prev >= 0) umma_commit(&ctl->q_empty);
-                    if (!(ok = wait_bar(&ctl->q_full, (uint32_t)(qn & 1), ctl, bt.err, 10))) break;
-                    tc_fence_after();
+            const uint64_t ones_desc = smem_desc_sw32(smem_u32(sm.ones)), ext_desc = smem_desc_sw32(smem_u32(sm.ext));
+            const uint32_t ext_hi = (uint32_t)(ext_desc >> 32), ext_lo = (uint32_t)ext_desc;
+            const uint64_t qd = smem_desc_sw128(smem_u32(sm.q));
+            const uint32_t hi = (uint32_t)(qd >> 32), q_lo = (uint32_t)qd;
+            const uint32_t k_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.k));
+            const uint32_t q_blk = (uint32_t)bt.rows2 * 128 >> 4;
+            constexpr uint32_t idesc = idesc_bf16_f32(128, 128);
+            int nc = 0, nh = 0;
+            for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
+                if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
+                    const TcSender& sd = bt.s[un.i];
+                    nc = sd.n_blk2;
+                    nh = rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - rc_begin(sd.halves, sd.n_rc2, un.rc);
+                    if (u > 0) umma_commit(&ctl->q_empty);
+                    if (!(ok = wait_bar(&ctl->q_full, qn & 1, ctl, bt.err, 10))) break;
                     ++qn;
-                    prev = key;
                 }
-                if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 11))) break;
-                tc_fence_after();
-                const uint32_t kaddr = smem_u32(sm.k + (size_t)st * kTileBytes);
-                const int grp = (int)((u - ub) & 1);   // epilogue group that owns this tile
-                if (sd.R_pad == 256) {
-                    // both halves in one 256-column MMA (faster when the tile has no other rows);
-                    // it waits for both halves' buffers and completes both
-                    const uint32_t jp = (jpar >> (2 * grp)) & 3u;
-                    jpar ^= 3u << (2 * grp);
-                    if (!(ok = wait_bar(&ctl->t_empty[2 * grp], (jp & 1u) ^ 1u, ctl, bt.err, 12))) break;
-                    if (!(ok = wait_bar(&ctl->t_empty[2 * grp + 1], (jp >> 1) ^ 1u, ctl, bt.err, 12))) break;
-                    tc_fence_after();
-                    mma_k128(tmem + grp * 256, kaddr, kTileBytes / 2, smem_u32(sm.q), (uint32_t)bt.rpad_max * 128,
-                             idesc_bf16_f32(128, 256));
-                    // one more K-step: ones (positions) x offset terms (rows) adds -offset / scale to
-                    // every logit, so the epilogue needs only exp2(scale * D)
-                    umma_bf16(tmem + grp * 256, ones_desc, ext_desc, idesc_bf16_f32(128, 256), 1u);
-                    umma_commit(&ctl->t_full[2 * grp]);
-                    umma_commit(&ctl->t_full[2 * grp + 1]);
-                } else {
-                    // one 128-column MMA per column half, each into its own buffer, so that each
-                    // half's warps start as soon as their columns are done and release them on
-                    // their own (the next chunk waits for one half, not for the whole group)
-                    for (int r0 = 0; r0 < sd.R_pad && ok; r0 += 128) {
-                        const int b = 2 * grp + ((r0 >> 7) & 1);
-                        const uint32_t jp = (jpar >> b) & 1u;
-                        jpar ^= 1u << b;
-                        if (!(ok = wait_bar(&ctl->t_empty[b], jp ^ 1u, ctl, bt.err, 12))) break;
+                for (int h = 0; h < nh && ok; ++h, ++n)
+                    for (int j = me; j < 4; j += 2) {
+                        if (h == 0 && !(ok = wait_bar(&ctl->k_full[st0 + j], ph, ctl, bt.err, 11))) break;
+                        if (!(ok = wait_bar(&ctl->t_empty[j], (n & 1) ^ 1, ctl, bt.err, 12))) break;
                         tc_fence_after();
-                        mma_k128(tmem + b * 128, kaddr, kTileBytes / 2, smem_u32(sm.q) + r0 * 128,
-                                 (uint32_t)bt.rpad_max * 128, idesc_bf16_f32(128, 128));
-                        umma_bf16(tmem + b * 128, ones_desc, ext_desc + (uint64_t)((r0 * 32) >> 4),
-                                  idesc_bf16_f32(128, 128), 1u);
-                        umma_commit(&ctl->t_full[b]);
+                        mma_d<D>(tmem + j * 128, k_lo + (uint32_t)(st0 + j) * (kTile >> 4), kTileRows * 128 >> 4,
+                                 q_lo + h * (kRowHalf * 128 >> 4), q_blk, hi, idesc);
+                        // one more K-step: ones (positions) x offset terms (rows) adds -offset / scale to
+                        // every logit, so the epilogue needs only exp2(scale * D)
+                        umma_bf16(tmem + j * 128, ones_desc, desc64(ext_lo + h * (kRowHalf * 32 >> 4), ext_hi), idesc, 1u);
+                        umma_commit(&ctl->t_full[j]);
+                        if (h == nh - 1) umma_commit(&ctl->k_empty[st0 + j]);
                     }
-                }
-                umma_commit(&ctl->k_empty[st]);
-                if (++st == stages) { st = 0; ph ^= 1u; }
+                st0 += 4;
+                if (st0 == slots) { st0 = 0; ph ^= 1u; }
             }
-            umma_commit(&ctl->drain);
-            drain_wait(&ctl->drain, 0);
+            umma_commit(&ctl->drain[me]);
+            drain_wait(&ctl->drain[me], 0);
         }
-    } else {
-        // 16 warps: quad = (warp - 2) / 4; group = quad / 2 takes alternate tiles, half = quad % 2
-        // takes columns half*128 .. +128 of each 256-column chunk (32 tokens when G = 4).
-        const int ew = warp - 2, quad = ew >> 2, grp = quad >> 1, hf = quad & 1, sp = warp & 3;
-        const uint32_t lane_addr = (uint32_t)(sp * 32) << 16;
-        float2* xch = reinterpret_cast<float2*>(sm.epi);   // [parity][grp][sp][32]
-        const float c = bt.sl2e;
-        const uint64_t cc = pack2(c, c);
-        int64_t j = 0, gt = 0;                   // chunks of this warp's buffer and tiles of this group so far
-        int prev = -1;
+    } else if (warp >= kEpi0) {
+        const int q = (warp - kEpi0) >> 2, sp = warp & 3;   // column quarter, TMEM lane quarter
+        const uint32_t ta = tmem + ((uint32_t)(sp * 32) << 16) + 32 * q;
+        float4* xch = reinterpret_cast<float4*>(sm.epi) + q * 256 + sp * 32 + lane;   // [column quarter][U, N][lane quarter][lane]
+        const uint64_t cc = pack2(bt.sl2e, bt.sl2e);
+        const bool p_inf = !P2 && bt.p_inf;
+        uint32_t n = 0, nu = 0;                  // rounds of the four buffers and blocks so far
         bool ok = true;
-        // per-sender values live in registers and are refreshed when the group s changes
-        // (indexed reads of the kernel-parameter block on every tile are slow)
-        float* part = nullptr;                   // U partials of the current group s
-        int64_t nST = 0;                         // distance between the U, N and D partials
-        int64_t T = 0;
-        int nch = 0, n_tile = 1, R_pad = 0;
-        float inv_m = 0.f, inv_mh = 0.f;
-        const int nS = bt.nL * bt.Hkv;
-        Unit un = decode2(bt, ub);
-        n_tile = bt.s[un.i].n_tile2;
-        auto advance = [&]() {   // next unit (sender, group, tile) without parameter reads
-            if (++un.c == n_tile) {
-                un.c = 0;
-                if (++un.s == nS) {
-                    un.s = 0;
-                    ++un.i;
-                    if (un.i < bt.n) n_tile = bt.s[un.i].n_tile2;
-                }
-            }
-        };
-        if (grp == 1 && ub < ue) advance();
-        for (int64_t u = ub + grp; u < ue && ok; u += 2, advance(), advance()) {
-            const int key = un.i * 65536 + un.s;
-            if (key != prev) {
+        int T = 0, nh = 0, R = 0, nc = 0;        // of the current sender and row chunk; R: query rows from its first on
+        for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
+            if (u == 0 || un.c == 0) {
                 const TcSender& sd = bt.s[un.i];
-                R_pad = sd.R_pad;
-                nch = (sd.R_pad + 255) / 256;
-                T = sd.T;
-                inv_m = sd.inv_m;
-                inv_mh = sd.inv_mh;
-                nST = (int64_t)nS * sd.T;
-                part = sd.part + (int64_t)un.s * sd.T;
-                prev = key;
+                const int h0 = rc_begin(sd.halves, sd.n_rc2, un.rc);
+                nh = rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0;
+                R = sd.R - h0 * kRowHalf;
+                T = (int)sd.T;
+                nc = sd.n_blk2;
             }
-            const int64_t pos = (int64_t)un.c * kOut2 + kOutW * sp - kMargin + lane;
-            const bool valid = pos >= 0 && pos < T;
-            const bool all_valid = __all_sync(0xffffffffu, valid);
-            float nacc2[2] = {0.f, 0.f}, bsum2[2] = {0.f, 0.f};   // token partial sums (two chains)
-            for (int ci = 0; ci < nch && ok; ++ci) {
-                // this half's columns (R_pad is a multiple of 128: 0 or 128); a half with none has
-                // no MMA and nothing to wait for
-                const int ncol = min(128, min(256, R_pad - 256 * ci) - hf * 128);
-                if (ncol <= 0) continue;
-                if (!(ok = wait_bar(&ctl->t_full[2 * grp + hf], (uint32_t)(j & 1), ctl, bt.err, 13))) break;
-                ++j;
-                tc_fence_after();
-                const uint32_t ta = tmem + lane_addr + grp * 256 + hf * 128;
-                if (G == 4) {
-                    // head sums of the warp's 32 tokens first, then the buffer goes back to the MMA
-                    // while Pool and the token sums run from registers; each 16-column load is
-                    // issued before the head sums of the one before it
-                    uint64_t b[16];   // (token 2i, token 2i + 1)
-                    {
-                        float va[16], vb[16];
-                        tmem_ld16(ta, va);
+            const int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
+            const bool all_valid = __all_sync(0xffffffffu, pos >= 0 && pos + 3 < T);
+            float us[4] = {0.f, 0.f, 0.f, 0.f}, ns[4] = {0.f, 0.f, 0.f, 0.f};   // per position: sums over tokens
+            for (int h = 0; h < nh && ok; ++h, ++n) {
+                const bool active = h * kRowHalf + 32 * q < R;     // else padding columns only
+                constexpr int kSub = 4 / G;                        // sub-blocks of eight tokens
+#pragma unroll 1
+                for (int sb = 0; sb < kSub; ++sb) {
+                    uint64_t b[4][4];
 #pragma unroll
-                        for (int k = 0; k < 8; k += 2) {
-                            tmem_wait_ld(va);
-                            tmem_ld16(ta + 16 * (k + 1), vb);
-                            head_sums16(va, cc, b[2 * k], b[2 * k + 1]);
-                            tmem_wait_ld(vb);
-                            if (k + 2 < 8) tmem_ld16(ta + 16 * (k + 2), va);
-                            head_sums16(vb, cc, b[2 * k + 2], b[2 * k + 3]);
+                    for (int j = 0; j < 4; ++j) {
+                        if (sb == 0 && !(ok = wait_bar(&ctl->t_full[j], n & 1, ctl, bt.err, 13))) break;
+                        tc_fence_after();
+                        // eight tokens' columns, 16 at a time (8 for G = 1)
+                        constexpr int kCols = G == 1 ? 8 : 16;
+#pragma unroll
+                        for (int x = 0; x < 8 * G; x += kCols) {
+                            float v[kCols];
+                            if (active) {
+                                tmem_ldn(ta + j * 128 + sb * 8 * G + x, v);
+                                tmem_wait_ld(v);
+                            }
+                            if (sb == kSub - 1 && x + kCols == 8 * G) {   // registers hold the rest
+                                tc_fence_before();
+                                __syncwarp();
+                                if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
+                            }
+                            if (active) head_sums<G>(v, cc, b[j] + x / (2 * G));
                         }
                     }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&ctl->t_empty[2 * grp + hf]);
+                    if (!ok) break;
+                    if (!active) continue;
                     if (!all_valid) {
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) b[i] = valid ? b[i] : 0ull;
-                    }
-                    uint64_t bs = pack2(bsum2[0], bsum2[1]), na = pack2(nacc2[0], nacc2[1]);
+                        for (int j = 0; j < 4; ++j) {
+                            const bool valid = pos + j >= 0 && pos + j < T;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        float b0, b1;
-                        unpack2(b[i], b0, b1);
-                        const float p0 = lane_pool<PH>(b0), p1 = lane_pool<PH>(b1);
-                        bs = fadd2(bs, b[i]);
-                        if (P2) {
-                            const uint64_t pp = pack2(p0, p1);
-                            na = ffma2(pp, pp, na);
-                        } else if (bt.p_inf) {
-                            nacc2[0] = fmaxf(nacc2[0], p0);
-                            nacc2[1] = fmaxf(nacc2[1], p1);
-                        } else {
-                            nacc2[0] += pow_p<false>(p0, bt.p);
-                            nacc2[1] += pow_p<false>(p1, bt.p);
+                            for (int i = 0; i < 4; ++i) b[j][i] = valid ? b[j][i] : 0ull;
                         }
                     }
-                    unpack2(bs, bsum2[0], bsum2[1]);
-                    if (P2) unpack2(na, nacc2[0], nacc2[1]);
-                } else {
-                    // 32-column steps; sixteen epilogue warps hide the TMEM load latency
-#pragma unroll 1
-                    for (int col = 0; col < (G == 4 ? 0 : ncol); col += 32) {
-                        float v[32];
-                        tmem_ld32(ta + col, v);
-                        tmem_wait_ld(v);
-                        accum_block<G, PH, P2>(v, cc, valid, all_valid, bt.p, bt.p_inf, nacc2, bsum2);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float x0[4], x1[4], o0[4], o1[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            unpack2(b[j][i], x0[j], x1[j]);
+                            us[j] += x0[j] + x1[j];
+                        }
+                        pool4<PH>(x0, o0);
+                        pool4<PH>(x1, o1);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if (P2) {
+                                ns[j] = fmaf(o0[j], o0[j], fmaf(o1[j], o1[j], ns[j]));
+                            } else if (p_inf) {   // p = infinity: largest pooled value
+                                ns[j] = fmaxf(ns[j], fmaxf(o0[j], o1[j]));
+                            } else {
+                                ns[j] += pow_p(o0[j], bt.p) + pow_p(o1[j], bt.p);
+                            }
+                        }
                     }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&ctl->t_empty[2 * grp + hf]);
                 }
             }
             if (!ok) break;
-            // p = infinity keeps the largest pooled token value instead of the sum of powers
-            const bool p_inf = !P2 && bt.p_inf;
-            float nacc = p_inf ? fmaxf(nacc2[0], nacc2[1]) : nacc2[0] + nacc2[1];
-            float bsum = bsum2[0] + bsum2[1];
-            // the two column halves of the group add up their sums; half tp (the group's tile
-            // parity) writes the results, so the halves take turns waiting for each other
-            const int tp = (int)(gt & 1);
-            float2* xs = xch + ((tp * 2 + grp) * 4 + sp) * 32;
-            uint64_t* xb = &ctl->xb[tp][grp][sp];
-            uint64_t* xe = &ctl->xe[tp][grp][sp];
-            if ((hf ^ tp) == 1) {
-                // the slot was last used two tiles ago: wait until the other half has read it
-                if (!(ok = wait_bar(xe, (uint32_t)(((gt >> 1) & 1) ^ 1), ctl, bt.err, 7))) break;
-                xs[lane] = make_float2(nacc, bsum);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(xb);
-            } else {
-                if (!(ok = wait_bar(xb, (uint32_t)((gt >> 1) & 1), ctl, bt.err, 14))) break;
-                const float2 o = xs[lane];
-                __syncwarp();
-                if (lane == 0) mbar_arrive(xe);
-                nacc = p_inf ? fmaxf(nacc, o.x) : nacc + o.x;
-                bsum += o.y;
-                const float pb = lane_pool<PH>(bsum * inv_m);
-                if (valid && lane >= kMargin && lane < kMargin + kOutW) {
-                    part[pos] = bsum * inv_mh;
-                    part[nST + pos] = p_inf ? nacc : nacc * inv_m;
-                    part[2 * nST + pos] = p_inf ? pb : pow_p<P2>(pb, bt.p);
+            // hand the block's sums to warp 3 (it has read the last block's long ago)
+            if (!(ok = wait_bar(&ctl->xe, (nu & 1) ^ 1, ctl, bt.err, 7))) break;
+            xch[0] = make_float4(us[0], us[1], us[2], us[3]);
+            xch[128] = make_float4(ns[0], ns[1], ns[2], ns[3]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->xb);
+            ++nu;
+        }
+    } else {
+        // ---------------- warp 3: the column quarters' sums of a block, added in a fixed order ----------------
+        const float4* xch = reinterpret_cast<const float4*>(sm.epi) + lane;   // [column quarter][U, N][lane quarter][lane]
+        const bool p_inf = !P2 && bt.p_inf;
+        const int nS = bt.nL * bt.Hkv;
+        bool ok = true;
+        float* part = nullptr;                   // U partials of the current group and row chunk
+        int64_t nST = 0;                         // distance between the U and N partials
+        int T = 0, nc = 0;
+        for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
+            if (u == 0 || un.c == 0) {
+                const TcSender& sd = bt.s[un.i];
+                nST = (int64_t)nS * sd.T_pad;
+                part = sd.part + 2 * un.rc * nST + (int64_t)un.s * sd.T_pad;
+                T = (int)sd.T;
+                nc = sd.n_blk2;
+            }
+            if (!(ok = wait_bar(&ctl->xb, (uint32_t)u & 1, ctl, bt.err, 14))) break;
+#pragma unroll
+            for (int sp = 0; sp < 4; ++sp) {
+                const int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
+                float4 x[4], y[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    x[k] = xch[(8 * k + sp) * 32];
+                    y[k] = xch[(8 * k + 4 + sp) * 32];
+                }
+                auto add = [](float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
+                auto mx = [](float4 a, float4 b) {
+                    return make_float4(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z), fmaxf(a.w, b.w));
+                };
+                if (lane >= 1 && lane <= 30 && pos < T) {   // rows are padded to a multiple of four positions
+                    *reinterpret_cast<float4*>(part + pos) = add(add(x[0], x[1]), add(x[2], x[3]));
+                    *reinterpret_cast<float4*>(part + nST + pos) =
+                        p_inf ? mx(mx(y[0], y[1]), mx(y[2], y[3])) : add(add(y[0], y[1]), add(y[2], y[3]));
                 }
             }
-            ++gt;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->xe);
         }
     }
     tc_fence_before();
@@ -873,7 +892,7 @@ bool encode_nd(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dim
                const cuuint32_t* box, CUtensorMapSwizzle swizzle) {
     auto fn = encoder();
     if (!fn || !base) return false;
-    const cuuint32_t es[4] = {1, 1, 1, 1};
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides_bytes, box,
               es, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -884,40 +903,89 @@ bool encode_4d(CUtensorMap* m, const void* base, const cuuint64_t dims[4], const
     return encode_nd(m, base, 4, dims, strides_bytes, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-size_t smem_bytes(int rpad_max, int stages) {
-    return 1024 + (size_t)2 * rpad_max * 128 + (size_t)rpad_max * 32 + 128 * 32 + (size_t)stages * kTileBytes + 512 +
-           2 * 2 * 4 * 32 * 8;
+constexpr size_t kSmemMax = 227 * 1024;
+
+// Raises a kernel's dynamic shared-memory limit to the SM's, once per device (`done`: a bit each;
+// the call takes about a microsecond of host time, and setting it twice is harmless).
+template <typename K>
+cudaError_t allow_smem(K kernel, std::atomic<uint64_t>& done) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev < 64 ? uint64_t(1) << dev : 0;
+    if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
 }
 
-template <int G, int PH, bool P2>
-cudaError_t launch_accum(const TcBatch& tb, size_t smem, int grid, cudaStream_t st) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_accum_tc<G, PH, P2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+size_t smem1_bytes(int d, int rows, int stages) {
+    return 1024 + (size_t)rows * d * 2 + (size_t)stages * kTileRows * d * 2 + 512;
+}
+
+size_t smem2_bytes(int d, int rows, int kbufs) {
+    return 1024 + (size_t)rows * (d * 2 + 32) + 128 * 32 + (size_t)kbufs * 4 * kTileRows * d * 2 + 512 + 4 * 8 * 128 * 4;
+}
+
+template <int D, int G, int PH, bool P2>
+cudaError_t launch_accum(const TcBatch& tb, int grid, cudaStream_t st) {
+    const size_t smem = smem2_bytes(D, tb.rows2, tb.kbufs);
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = allow_smem(k_accum_tc<D, G, PH, P2>, done);
     if (e != cudaSuccess) return e;
-    k_accum_tc<G, PH, P2><<<grid, kThreadsTc, smem, st>>>(tb);
+    k_accum_tc<D, G, PH, P2><<<grid, kThreadsTc, smem, st>>>(tb);
     return cudaGetLastError();
 }
 
-template <int G, bool P2>
-cudaError_t launch_accum_gp(const TcBatch& tb, size_t smem, int grid, cudaStream_t st) {
+template <int D, int G, bool P2>
+cudaError_t launch_accum_gp(const TcBatch& tb, int grid, cudaStream_t st) {
     switch (tb.ph) {
-        case 0: return launch_accum<G, 0, P2>(tb, smem, grid, st);
-        case 1: return launch_accum<G, 1, P2>(tb, smem, grid, st);
-        case 2: return launch_accum<G, 2, P2>(tb, smem, grid, st);
-        case 3: return launch_accum<G, 3, P2>(tb, smem, grid, st);
+        case 0: return launch_accum<D, G, 0, P2>(tb, grid, st);
+        case 1: return launch_accum<D, G, 1, P2>(tb, grid, st);
+        case 2: return launch_accum<D, G, 2, P2>(tb, grid, st);
+        case 3: return launch_accum<D, G, 3, P2>(tb, grid, st);
     }
     return cudaErrorInvalidValue;
 }
 
-template <int G>
-cudaError_t launch_accum_g(const TcBatch& tb, size_t smem, int grid, cudaStream_t st) {
-    return tb.p_is_2 ? launch_accum_gp<G, true>(tb, smem, grid, st) : launch_accum_gp<G, false>(tb, smem, grid, st);
+template <int D>
+cudaError_t launch_accum_d(const TcBatch& tb, int grid, cudaStream_t st) {
+    const bool p2 = tb.p == 2.f;
+    if (tb.G == 4) return p2 ? launch_accum_gp<D, 4, true>(tb, grid, st) : launch_accum_gp<D, 4, false>(tb, grid, st);
+    if (tb.G == 2) return p2 ? launch_accum_gp<D, 2, true>(tb, grid, st) : launch_accum_gp<D, 2, false>(tb, grid, st);
+    return p2 ? launch_accum_gp<D, 1, true>(tb, grid, st) : launch_accum_gp<D, 1, false>(tb, grid, st);
+}
+
+template <int D, int NH>
+cudaError_t launch_stats(const TcBatch& tb, int grid, cudaStream_t st) {
+    const size_t smem = smem1_bytes(D, tb.rows1, tb.stages1);
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = allow_smem(k_stats_tc<D, NH>, done);
+    if (e != cudaSuccess) return e;
+    k_stats_tc<D, NH><<<grid, kThreadsTc, smem, st>>>(tb);
+    return cudaGetLastError();
+}
+
+template <int D>
+cudaError_t launch_stats_d(const TcBatch& tb, int grid, cudaStream_t st) {
+    if (tb.rows1 <= kRowHalf) return launch_stats<D, 1>(tb, grid, st);
+    if (tb.rows1 <= 2 * kRowHalf) return launch_stats<D, 2>(tb, grid, st);
+    return launch_stats<D, kHalves1>(tb, grid, st);
+}
+
+// CTAs of a pass of `units` units: one an SM, a multiple of the row-chunk count when every sender
+// has the same one (CTAs k, k + grid / n_rc, ... then walk the same K tiles in step, so that a
+// tile comes from DRAM once and from L2 for the other row chunks).
+int pass_grid(int64_t units, int num_sms, int n_rc) {
+    int g = num_sms;
+    if (n_rc > 1 && n_rc <= g) g = g / n_rc * n_rc;
+    return (int)(units < g ? units : g);
 }
 
 }  // namespace
 
-bool tc_path_supported(int head_dim, int G, int pool_half, int max_query_tokens) {
-    return head_dim == 128 && (G == 1 || G == 2 || G == 4) && pool_half <= 3 && max_query_tokens * G <= 512;
+bool tc_path_supported(int head_dim, int G, int pool_half) {
+    return (head_dim == 64 || head_dim == 128) && (G == 1 || G == 2 || G == 4) && pool_half <= 3;
 }
 
 // Pass 1, combine, pass 2 on the tensor cores for senders [0, b.n) of `b`; the caller
@@ -925,26 +993,23 @@ bool tc_path_supported(int head_dim, int G, int pool_half, int max_query_tokens)
 cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_t* err,
                             cudaError_t (*combine)(const ScoreBatch&, cudaStream_t)) {
     const int G = b.n_q_heads / b.n_kv_heads;
-    const int nS = b.n_layers * b.n_kv_heads;
+    const int nS = b.n_layers * b.n_kv_heads, d_head = b.head_dim;
     // Encode every tensor map first: if the driver rejects one (an unusual stride
     // pattern), nothing has been launched and the caller uses the mma.sync passes.
-    std::vector<TcBatch*> batches;
-    auto free_all = [&] { for (TcBatch* p : batches) delete p; };
+    std::vector<std::unique_ptr<TcBatch>> batches;
+    std::vector<std::unique_ptr<TcMaps[]>> maps2;   // pass 2's tensor maps of each sub-batch
     // Sub-batches of at most kMaxTcSenders senders; paged senders are first copied into the
-    // staging buffer (contiguous [nL][Hkv][T][128]), which each sub-batch reuses from its start,
+    // staging buffer (contiguous [nL][Hkv][T][d]), which each sub-batch reuses from its start,
     // so a sub-batch also ends where its paged senders would overflow the staging.
     std::vector<int> firsts;
-    std::vector<DepageBatch*> depages;
-    auto free_depages = [&] { for (DepageBatch* p : depages) delete p; };
+    std::vector<std::unique_ptr<DepageBatch>> depages;
     for (int b0 = 0; b0 < b.n;) {
         int nb = 0;
         int64_t used = 0;
         while (b0 + nb < b.n && nb < kMaxTcSenders) {
             const ScoreSender& s = b.s[b0 + nb];
-            const int64_t e = s.pm.pages ? (int64_t)b.n_layers * b.n_kv_heads * s.T * 128 : 0;
+            const int64_t e = s.pm.pages ? (int64_t)nS * s.T * d_head : 0;
             if (e > 0 && (!b.stage || e > b.stage_elems)) {   // no room: the mma.sync passes read pages
-                free_all();
-                free_depages();
                 return cudaErrorNotSupported;
             }
             if (nb > 0 && used + e > b.stage_elems) break;
@@ -952,13 +1017,16 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             ++nb;
         }
         firsts.push_back(b0);
-        DepageBatch* dp = new DepageBatch();
-        depages.push_back(dp);
+        depages.emplace_back(new DepageBatch);   // (uninitialised, like the next: filled for its senders only)
+        DepageBatch* dp = depages.back().get();
+        dp->n = 0;
         dp->n_layers = b.n_layers;
         dp->n_kv_heads = b.n_kv_heads;
+        dp->head_dim = d_head;
         dp->err = err;
-        TcBatch* tb = new TcBatch();
-        batches.push_back(tb);
+        batches.emplace_back(new TcBatch);
+        maps2.emplace_back(new TcMaps[nb]);
+        TcBatch* tb = batches.back().get();
         tb->n = nb;
         b0 += nb;
         tb->nL = b.n_layers;
@@ -967,16 +1035,18 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
         tb->G = G;
         tb->sl2e = b.scale_log2e;
         tb->p = b.p;
-        tb->p_is_2 = b.p == 2.f;
         tb->p_inf = b.p_inf;
         tb->ph = b.pool_half;
         tb->err = err;
-        int rpad_max = 128;
-        int64_t u1 = 0, u2 = 0, staged = 0;
+        tb->max_rc1 = tb->max_rc2 = 1;
+        tb->weight1 = tb->weight2 = 0;
+        int rows1 = kRowHalf, rows2 = kRowHalf;
+        int64_t staged = 0;
         const int b_first = firsts.back();
         for (int k = 0; k < nb; ++k) {
             const ScoreSender& s = b.s[b_first + k];
             TcSender& d = tb->s[k];
+            TcMaps &mp = tb->maps[k], &mp2 = maps2.back()[k];   // pass 1's and pass 2's maps
             // K as the passes read it: the sender's own tensor, or its staged copy
             const uint16_t* kp = s.k;
             int64_t kl = s.ks_l, kh = s.ks_h, kpos = s.ks_p;
@@ -990,111 +1060,117 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
                 ds.T = s.T;
                 ds.out = b.stage + staged;
                 kp = ds.out;
-                kpos = 128;
-                kh = s.T * 128;
-                kl = (int64_t)b.n_kv_heads * s.T * 128;
+                kpos = d_head;
+                kh = s.T * d_head;
+                kl = (int64_t)b.n_kv_heads * s.T * d_head;
                 staged += kl * b.n_layers;
             }
             d.T = s.T;
-            d.m = s.m;
-            d.inv_m = 1.f / (float)s.m;
-            d.inv_mh = 1.f / ((float)s.m * (float)b.n_kv_heads);
+            d.T_pad = part_row(s.T);
             d.R = s.m * G;
-            d.R_pad = (d.R + 127) / 128 * 128;
-            rpad_max = rpad_max > d.R_pad ? rpad_max : d.R_pad;
-            d.n_chunk1 = (int32_t)(4 * ((s.T + kChunk1 - 1) / kChunk1));   // one partial per (chunk, group, half)
-            d.n_tile2 = (int32_t)((s.T + kOut2 - 1) / kOut2);
+            d.halves = (d.R + kRowHalf - 1) / kRowHalf;
+            d.n_chunk1 = (int32_t)(4 * ((s.T + kChunk1 - 1) / kChunk1));   // one partial per (chunk, column quarter)
+            d.n_blk2 = (int32_t)((s.T + kOut2 - 1) / kOut2);
+            d.n_rc1 = (d.halves + kHalves1 - 1) / kHalves1;
+            d.n_rc2 = (d.halves + kHalves2 - 1) / kHalves2;
             d.stats = b.stats + s.stats_off;
-            d.offs = b.offs + s.offs_off;
             d.part = b.part + s.part_off;
-            d.unit1_begin = u1;
-            u1 += (int64_t)nS * (d.n_chunk1 / 4);
-            d.unit2_begin = u2;
-            u2 += (int64_t)nS * d.n_tile2;
-            // Q arrives in boxes of at most 256 tokens that tile the padded rows exactly
-            // (R_pad is a multiple of 128, so 128-token boxes always divide it for G = 1)
-            const int tok_pad = d.R_pad / G;
-            d.qbox_tok = tok_pad <= 256 ? tok_pad : 128;
-            d.n_qbox = tok_pad / d.qbox_tok;
-            if (d.n_qbox * d.qbox_tok != tok_pad) {
-                free_all();
-                free_depages();
-                return cudaErrorNotSupported;
-            }
-            const cuuint64_t kd[4] = {128, (cuuint64_t)s.T, (cuuint64_t)b.n_kv_heads, (cuuint64_t)b.n_layers};
+            tb->max_rc1 = tb->max_rc1 > d.n_rc1 ? tb->max_rc1 : d.n_rc1;
+            tb->max_rc2 = tb->max_rc2 > d.n_rc2 ? tb->max_rc2 : d.n_rc2;
+            const int r1 = (d.halves + d.n_rc1 - 1) / d.n_rc1 * kRowHalf, r2 = (d.halves + d.n_rc2 - 1) / d.n_rc2 * kRowHalf;
+            rows1 = rows1 > r1 ? rows1 : r1;
+            rows2 = rows2 > r2 ? rows2 : r2;
+            tb->weight1 += (int64_t)nS * (d.n_chunk1 / 4) * d.halves;
+            tb->weight2 += (int64_t)nS * d.n_blk2 * d.halves;
+            const cuuint64_t kd[4] = {(cuuint64_t)d_head, (cuuint64_t)s.T, (cuuint64_t)b.n_kv_heads,
+                                      (cuuint64_t)b.n_layers};
             const cuuint64_t ks[3] = {(cuuint64_t)kpos * 2, (cuuint64_t)kh * 2, (cuuint64_t)kl * 2};
             const cuuint32_t kbox[4] = {64, kTileRows, 1, 1};
-            const cuuint64_t qd[4] = {128, (cuuint64_t)b.n_q_heads, (cuuint64_t)s.m, (cuuint64_t)b.n_layers};
+            const cuuint64_t qd[4] = {(cuuint64_t)d_head, (cuuint64_t)b.n_q_heads, (cuuint64_t)s.m, (cuuint64_t)b.n_layers};
             const cuuint64_t qs[3] = {(cuuint64_t)s.qs_h * 2, (cuuint64_t)s.qs_t * 2, (cuuint64_t)s.qs_l * 2};
-            const cuuint32_t qbox[4] = {64, (cuuint32_t)G, (cuuint32_t)d.qbox_tok, 1};
-            const cuuint32_t kbox32[4] = {64, 32, 1, 1};
-            // offset terms [nS][R_pad][16] written by the combine kernel, boxes of at most 256 rows
-            d.ebox_rows = d.R_pad <= 256 ? d.R_pad : 128;
-            d.n_ebox = d.R_pad / d.ebox_rows;
-            const cuuint64_t ed[3] = {(cuuint64_t)kExtCols, (cuuint64_t)d.R_pad, (cuuint64_t)nS};
-            const cuuint64_t es[2] = {(cuuint64_t)kExtCols * 2, (cuuint64_t)d.R_pad * kExtCols * 2};
-            const cuuint32_t ebox[3] = {(cuuint32_t)kExtCols, (cuuint32_t)d.ebox_rows, 1};
-            if (!encode_4d(&d.kmap, kp, kd, ks, kbox) || !encode_4d(&d.kmap32, kp, kd, ks, kbox32) ||
-                !encode_4d(&d.qmap, s.q, qd, qs, qbox) || d.n_ebox * d.ebox_rows != d.R_pad || !b.ext ||
-                !encode_nd(&d.emap, b.ext + s.ext_off, 3, ed, es, ebox, CU_TENSOR_MAP_SWIZZLE_32B)) {
-                free_all();
-                free_depages();
+            const cuuint32_t qbox[4] = {64, (cuuint32_t)G, (cuuint32_t)(kRowHalf / G), 1};
+            // offset terms [nS][rows padded to 128][16] written by the combine kernel
+            const cuuint64_t rpad = (cuuint64_t)d.halves * kRowHalf;
+            const cuuint64_t ed[3] = {(cuuint64_t)kExtCols, rpad, (cuuint64_t)nS};
+            const cuuint64_t es[2] = {(cuuint64_t)kExtCols * 2, rpad * kExtCols * 2};
+            const cuuint32_t ebox[3] = {(cuuint32_t)kExtCols, kRowHalf, 1};
+            // positions (i, j) = 4 i + j of whole groups of four; and per j every fourth position from j on,
+            // ceil((T - j) / 4) of them (a sender of fewer than four positions has none in its last tiles:
+            // any valid row, masked like all past T)
+            const cuuint64_t k5d[5] = {kd[0], (cuuint64_t)(s.T / 4 > 0 ? s.T / 4 : 1), (cuuint64_t)(s.T < 4 ? s.T : 4),
+                                       kd[2], kd[3]};
+            const cuuint64_t k5s[4] = {4 * ks[0], ks[0], ks[1], ks[2]};
+            const cuuint32_t k5box[5] = {64, 32, 1, 1, 1};
+            bool ok4 = encode_nd(&mp2.k[4], kp, 5, k5d, k5s, k5box, CU_TENSOR_MAP_SWIZZLE_128B);
+            for (int j = 0; j < 4 && s.T % 4 != 0; ++j) {
+                const int64_t first = j < s.T ? j : 0;
+                const cuuint64_t k4d[4] = {kd[0], (cuuint64_t)((s.T - first + 3) / 4), kd[2], kd[3]};
+                const cuuint64_t k4s[3] = {4 * ks[0], ks[1], ks[2]};
+                const cuuint32_t k4box[4] = {64, 32, 1, 1};
+                ok4 = ok4 && encode_4d(&mp2.k[j], kp + first * kpos, k4d, k4s, k4box);
+            }
+            if (!encode_4d(&mp.k[0], kp, kd, ks, kbox) || !ok4 || !encode_4d(&mp.q, s.q, qd, qs, qbox) || !b.ext ||
+                !encode_nd(&mp2.e, b.ext + s.ext_off, 3, ed, es, ebox, CU_TENSOR_MAP_SWIZZLE_32B)) {
                 return cudaErrorNotSupported;
             }
+            mp2.q = mp.q;
         }
         const cuuint64_t od[2] = {(cuuint64_t)kExtCols, 128};
         const cuuint64_t os[1] = {(cuuint64_t)kExtCols * 2};
         const cuuint32_t obox[2] = {(cuuint32_t)kExtCols, 128};
         if (!encode_nd(&tb->omap, b.ones, 2, od, os, obox, CU_TENSOR_MAP_SWIZZLE_32B)) {
-            free_all();
-            free_depages();
             return cudaErrorNotSupported;
         }
-        tb->rpad_max = rpad_max;
-        tb->stages = rpad_max > 256 ? 2 : 4;
-        tb->units1 = u1;
-        tb->units2 = u2;
+        tb->rows1 = rows1;
+        tb->rows2 = rows2;
+        tb->stages1 = 4;
+        while (tb->stages1 > 2 && smem1_bytes(d_head, rows1, tb->stages1) > kSmemMax) --tb->stages1;
+        tb->kbufs = smem2_bytes(d_head, rows2, 2) <= kSmemMax ? 2 : 1;
         tb->wait_ns = b.wait_ns;
         tb->stall = batches.size() == 1 ? b.stall : 0;   // the first launch only
     }
     cudaError_t e = cudaSuccess;
     for (size_t k = 0; k < batches.size() && e == cudaSuccess; ++k) {
-        TcBatch* tb = batches[k];
+        TcBatch* tb = batches[k].get();
         const int b0 = firsts[k];
-        const size_t smem = smem_bytes(tb->rpad_max, tb->stages);
-        e = cudaFuncSetAttribute(k_stats_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) {
-            stage_mark(b.timer, kStageStart, st);
-            e = launch_depage(*depages[k], st, num_sms);   // timed with pass 1
+        // row chunks in step only when all senders have the same number of them
+        int rc1 = tb->max_rc1, rc2 = tb->max_rc2;
+        int64_t units1 = 0, units2 = 0;
+        for (int j = 0; j < tb->n; ++j) {
+            const TcSender& d = tb->s[j];
+            if (d.n_rc1 != tb->max_rc1) rc1 = 1;
+            if (d.n_rc2 != tb->max_rc2) rc2 = 1;
+            units1 += (int64_t)nS * (d.n_chunk1 / 4) * d.n_rc1;
+            units2 += (int64_t)nS * d.n_blk2 * d.n_rc2;
         }
+        stage_mark(b.timer, kStageStart, st);
+        e = launch_depage(*depages[k], st, num_sms);   // timed with pass 1
         if (e == cudaSuccess) {
-            const int g1 = (int)(tb->units1 < num_sms ? tb->units1 : num_sms);
-            k_stats_tc<<<g1, kThreadsTc, smem, st>>>(*tb);
+            const int g1 = pass_grid(units1, num_sms, rc1);
+            e = d_head == 128 ? launch_stats_d<128>(*tb, g1, st) : launch_stats_d<64>(*tb, g1, st);
             stage_mark(b.timer, kStageStats, st);
-            e = cudaGetLastError();
         }
         if (e == cudaSuccess) {
-            // combine reads this batch's chunk counts (512-position chunks)
-            ScoreBatch* sub = new ScoreBatch(b);
-            sub->n = tb->n;
-            for (int j = 0; j < tb->n; ++j) {
-                sub->s[j] = b.s[b0 + j];
-                sub->s[j].n_chunk1 = tb->s[j].n_chunk1;
+            // combine reads this batch's partial-slot counts
+            for (int j = 0; j < tb->n; ++j) b.s[b0 + j].n_chunk1 = tb->s[j].n_chunk1;
+            if (tb->n == b.n) {
+                e = combine(b, st);
+            } else {
+                const std::unique_ptr<ScoreBatch> sub(new ScoreBatch(b));
+                sub->n = tb->n;
+                for (int j = 0; j < tb->n; ++j) sub->s[j] = b.s[b0 + j];
+                e = combine(*sub, st);
             }
-            e = combine(*sub, st);
             stage_mark(b.timer, kStageCombine, st);
-            delete sub;
         }
         if (e == cudaSuccess) {
-            const int g2 = (int)(tb->units2 < num_sms ? tb->units2 : num_sms);
-            if (G == 4) e = launch_accum_g<4>(*tb, smem, g2, st);
-            else if (G == 2) e = launch_accum_g<2>(*tb, smem, g2, st);
-            else e = launch_accum_g<1>(*tb, smem, g2, st);
+            const int g2 = pass_grid(units2, num_sms, rc2);
+            std::copy(maps2[k].get(), maps2[k].get() + tb->n, tb->maps);
+            e = d_head == 128 ? launch_accum_d<128>(*tb, g2, st) : launch_accum_d<64>(*tb, g2, st);
             stage_mark(b.timer, kStageAccum, st);
         }
+        for (int j = 0; j < tb->n; ++j) b.s[b0 + j].n_rc = tb->s[j].n_rc2;   // partials for the finalize kernel
     }
-    free_all();
-    free_depages();
     return e;
 }
 
