@@ -795,8 +795,8 @@ int64_t combine_rows(const ScoreBatch& b) {
 
 template <int TPR>
 cudaError_t launch_combine_t(const ScoreBatch& b, cudaStream_t st) {
-    bool self = false;
-    for (int i = 0; i < b.n; ++i) self = self || b.s[i].kself != nullptr;
+    bool self = false;   // (pass 1 of the tcgen05 path has taken the self keys in)
+    for (int i = 0; i < b.n && !b.use_tc; ++i) self = self || b.s[i].kself != nullptr;
     const int G = b.n_q_heads / b.n_kv_heads;
     const int64_t nS = (int64_t)b.n_layers * b.n_kv_heads;
     constexpr int RPB = kCombThreads / TPR;

@@ -10,7 +10,8 @@
 //
 //   k_stats_tc  pass 1, D = Q_s K_tile^T: TMEM lane = row (r, h), column = position.
 //               Each epilogue thread owns one row and one quarter of a tile's positions and keeps
-//               its running max and sum of exp2 over a chunk of positions.
+//               the sum of exp2 over a chunk of positions.  The query tokens' own keys, where a
+//               call has them, are further tiles of the last chunk under a causal mask.
 //   k_accum_tc  pass 2, D = K_tile Q_s^T (+ one more K-step of ones x the rows' offset terms,
 //               so TMEM holds z - offset / scale): TMEM lane = position, column = row (r, h).
 //               A block of positions is four tiles: tile j holds every fourth position from j on,
@@ -72,7 +73,8 @@ constexpr uint32_t kPollNs = 1000000u;           // longest suspension of one po
 constexpr int kMaxTcSenders = 32;         // their tensor maps fill most of the 32,764 bytes of kernel parameters
 
 struct TcMaps {
-    CUtensorMap k[5];     // pass 1: k[0] = 4D {d, T, Hkv, nL}, box {64, 128, 1, 1}.
+    CUtensorMap k[5];     // pass 1: k[0] = 4D {d, T, Hkv, nL}, box {64, 128, 1, 1}; k[1] the same over the
+                          // query tokens' own keys {d, m, Hkv, nL} (senders that have them).
                           // pass 2: k[4] = 5D {d, T / 4, 4, Hkv, nL} (position 4 i + j at (i, j)), box
                           // {64, 32, 1, 1, 1}; k[j] = 4D positions j, j + 4, ... with every one of them (the
                           // 5D tensor lacks the last T mod 4), box {64, 32, 1, 1}
@@ -88,12 +90,13 @@ struct TcSender {
     int32_t n_chunk1;     // pass-1 partial slots: four per chunk of positions
     int32_t n_blk2;       // pass-2 blocks of positions
     int32_t n_rc1, n_rc2; // row chunks of each pass
+    int32_t m_self;       // query tokens whose own keys join the softmax (m or 0)
 };
 
 struct TcBatch {
     CUtensorMap omap;     // 2D {16, 128} block of ones columns, one box, 32-byte swizzle
     int32_t n;
-    int32_t nL, Hq, Hkv, G;
+    int32_t nL, Hq, Hkv, G, log2g;
     int32_t stages1, rows1;       // pass 1: K ring stages, Q rows held
     int32_t kbufs, rows2;         // pass 2: K blocks in flight (1 or 2, four tiles each), Q rows held
     int32_t max_rc1, max_rc2;
@@ -215,6 +218,9 @@ __device__ __forceinline__ void my_units(const TcBatch& bt, Ctl* ctl) {
     ctl->units = (int32_t)(unit_at<PASS>(bt, total * (blockIdx.x + 1) / gridDim.x, &end) - b);
     ctl->first = first;
 }
+
+// Tiles of the query tokens' own keys, which pass 1 takes after those of a group's last chunk.
+__device__ __forceinline__ int self_tiles(const TcSender& sd) { return (sd.m_self + kTileRows - 1) / kTileRows; }
 
 // The next unit in order, without a division.  `nc`: the sender's chunks or blocks, kept by the
 // caller (an indexed read of the kernel parameters for every unit holds a role up).
@@ -381,13 +387,14 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
             int st = 0;               // ring slot of the next K tile and its phase parity
             uint32_t ph = 0;
             bool ok = true;
-            int nc = 0, l = 0, g = 0;
+            int nc = 0, l = 0, g = 0, n_self = 0;
             int64_t T = 0;
             for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
                 const TcMaps& mp = bt.maps[un.i];
                 if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
                     const TcSender& sd = bt.s[un.i];
                     nc = n_c<1>(sd);
+                    n_self = self_tiles(sd);
                     T = sd.T;
                     l = un.s / bt.Hkv;
                     g = un.s % bt.Hkv;
@@ -398,12 +405,15 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                 }
                 const int64_t c0 = (int64_t)un.c * kChunk1;
                 const int nt = (int)((min((int64_t)kChunk1, T - c0) + kTileRows - 1) / kTileRows);
-                for (int tile = 0; tile < nt; ++tile) {
+                const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
+                for (int tile = 0; tile < n_tiles; ++tile) {
                     if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 1))) break;
                     mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
+                    const bool self = tile >= nt;
+                    const int32_t row = self ? (tile - nt) * kTileRows : (int32_t)(c0 + tile * kTileRows);
                     for (int kb = 0; kb < D / 64; ++kb)
-                        tma_load_4d(sm.k + (size_t)st * kTile + kb * kTileRows * 128, &mp.k[0], &ctl->k_full[st], 64 * kb,
-                                    (int32_t)(c0 + tile * kTileRows), g, l);
+                        tma_load_4d(sm.k + (size_t)st * kTile + kb * kTileRows * 128, &mp.k[self ? 1 : 0],
+                                    &ctl->k_full[st], 64 * kb, row, g, l);
                     ++kt;
                     if (++st == stages) { st = 0; ph ^= 1u; }
                 }
@@ -431,12 +441,13 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
             // wait gives up, sets the abort flag and every role of this CTA leaves
             if (bt.stall && blockIdx.x == 0) ok = wait_bar(&ctl->stall, 0, ctl, bt.err, 6);
             uint32_t nh = 0;
-            int nc = 0;
+            int nc = 0, n_self = 0;
             int64_t T = 0;
             for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
                 if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
                     const TcSender& sd = bt.s[un.i];
                     nc = n_c<1>(sd);
+                    n_self = self_tiles(sd);
                     T = sd.T;
                     nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - rc_begin(sd.halves, sd.n_rc1, un.rc);
                     if (u > 0) umma_commit(&ctl->q_empty);
@@ -444,7 +455,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                     ++qn;
                 }
                 const int64_t c0 = (int64_t)un.c * kChunk1;
-                const int nt = (int)((min((int64_t)kChunk1, T - c0) + kTileRows - 1) / kTileRows);
+                const int nt = (int)((min((int64_t)kChunk1, T - c0) + kTileRows - 1) / kTileRows) +
+                               (un.c + 1 == nc ? n_self : 0);
                 for (int tile = 0; tile < nt; ++tile) {
                     if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
                     const uint32_t kt_lo = k_lo + (uint32_t)st * (kTile >> 4);
@@ -477,11 +489,13 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
         float M[NH];                             // per half: offset (log2 domain) and sum of exp2(c z - offset)
         uint64_t S[NH];
         bool ok = true;
-        // One tile, one buffer a half: load its 32 columns, hand the buffer back, sum.  PART: a tile
-        // with positions past T (`nvalid` of the 32 columns hold one).  The first tile of a chunk
-        // sets the offset to its first logit (to -FLT_MAX where it has none).
-        auto tile = [&](auto part, int nvalid, bool first, int nh) {
-            constexpr bool PART = decltype(part)::value;
+        // One tile, one buffer a half: load its 32 columns, hand the buffer back, sum.  PART: `nvalid` of
+        // the columns hold a position.  SELF: the columns are query tokens' own keys, of which row
+        // (token r, head) has those up to r: `nvalid` there, `tok0` of them for the thread's first row
+        // and one more for each token after its own.  The first tile of a chunk sets the offset to its
+        // first logit, or to -FLT_MAX where it has none (then the first self key of the row sets it).
+        auto tile = [&](auto part, auto self, int nvalid, bool first, int nh, int tok0) {
+            constexpr bool PART = decltype(part)::value, SELF = decltype(self)::value;
 #pragma unroll
             for (int h = 0; h < NH; ++h) {
                 if (h >= nh) break;
@@ -496,10 +510,11 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&ctl->t_empty[buf]);
                 if (PART) {
+                    const int nv = SELF ? min(nvalid, tok0 + (h * kRowHalf >> bt.log2g)) : nvalid;
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) v[e] = e < nvalid ? v[e] : -INFINITY;
+                    for (int e = 0; e < 32; ++e) v[e] = e < nv ? v[e] : -INFINITY;
                 }
-                if (first) M[h] = fmaxf(v[0] * c, -FLT_MAX);
+                if (first || (SELF && M[h] == -FLT_MAX)) M[h] = fmaxf(v[0] * c, -FLT_MAX);
                 const uint64_t nm = pack2(-M[h], -M[h]);
                 uint64_t p0 = 0, p1 = 0;
                 stats_block(v, cc, nm, p0, p1);
@@ -508,6 +523,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
         };
         float2* dst = nullptr;                   // the current group's partials of this thread's first row
         int nh = 0, nc = 0, rows = 0, R = 0;     // rows: query rows from the thread's first on
+        int m_self = 0, tok = 0;                 // tokens with own keys; the thread's first row's token
         int64_t T = 0;
         for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
             if (u == 0 || un.c == 0) {
@@ -518,14 +534,21 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                 T = sd.T;
                 R = sd.R;
                 rows = R - h0 * kRowHalf - L;
+                m_self = sd.m_self;
+                tok = (h0 * kRowHalf + L) >> bt.log2g;
                 dst = sd.stats + ((int64_t)un.s * sd.n_chunk1 + q) * R + h0 * kRowHalf + L;
             }
             const int len = (int)min((int64_t)kChunk1, T - (int64_t)un.c * kChunk1);
 #pragma unroll
             for (int h = 0; h < NH; ++h) { M[h] = -INFINITY; S[h] = 0; }
             int t0 = 0;
-            for (; t0 + kTileRows <= len && ok; t0 += kTileRows) tile(std::false_type{}, 32, t0 == 0, nh);
-            if (t0 < len && ok) tile(std::true_type{}, len - t0 - 32 * q, t0 == 0, nh);
+            constexpr std::false_type no{};
+            constexpr std::true_type yes{};
+            for (; t0 + kTileRows <= len && ok; t0 += kTileRows) tile(no, no, 32, t0 == 0, nh, 0);
+            if (t0 < len && ok) tile(yes, no, len - t0 - 32 * q, t0 == 0, nh, 0);
+            if (m_self > 0 && un.c + 1 == nc)   // the query tokens' own keys join the last chunk
+                for (int u0 = 32 * q; u0 - 32 * q < m_self && ok; u0 += kTileRows)
+                    tile(yes, yes, m_self - u0, false, nh, tok + 1 - u0);
             if (!ok) break;
             // this warp's partial statistics for the chunk: slot 4 c + q (rows of positions past T
             // are (-FLT_MAX, 0), which adds nothing); the combine kernel merges all slots
@@ -1033,6 +1056,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
         tb->Hq = b.n_q_heads;
         tb->Hkv = b.n_kv_heads;
         tb->G = G;
+        tb->log2g = G == 4 ? 2 : G - 1;
         tb->sl2e = b.scale_log2e;
         tb->p = b.p;
         tb->p_inf = b.p_inf;
@@ -1067,6 +1091,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             }
             d.T = s.T;
             d.T_pad = part_row(s.T);
+            d.m_self = s.kself ? s.m : 0;
             d.R = s.m * G;
             d.halves = (d.R + kRowHalf - 1) / kRowHalf;
             d.n_chunk1 = (int32_t)(4 * ((s.T + kChunk1 - 1) / kChunk1));   // one partial per (chunk, column quarter)
@@ -1114,6 +1139,11 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
                 return cudaErrorNotSupported;
             }
             mp2.q = mp.q;
+            if (s.kself) {
+                const cuuint64_t sdm[4] = {kd[0], (cuuint64_t)s.m, kd[2], kd[3]};
+                const cuuint64_t ss[3] = {(cuuint64_t)s.kss_t * 2, (cuuint64_t)s.kss_h * 2, (cuuint64_t)s.kss_l * 2};
+                if (!encode_4d(&mp.k[1], s.kself, sdm, ss, kbox)) return cudaErrorNotSupported;
+            }
         }
         const cuuint64_t od[2] = {(cuuint64_t)kExtCols, 128};
         const cuuint64_t os[1] = {(cuuint64_t)kExtCols * 2};

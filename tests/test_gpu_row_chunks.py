@@ -35,6 +35,8 @@ CASES = [
     ((1, 8, 2, 128), [600], 150, dict(p=float("inf"))),  # maxima over row chunks
     ((1, 8, 2, 64), [333], 65, dict(self_keys=True)),
     ((1, 8, 2, 64), [300], 130, dict(self_keys=True)),  # the self keys fill a tile and part of a second
+    # last chunks of one and six positions: most column quarters of a tile see self keys alone
+    ((1, 8, 2, 128), [1030, 1025, 5, 129], 100, dict(self_keys=True)),
     ((1, 8, 2, 128), [1, 2, 3, 5, 119, 120, 121, 122, 480, 481, 482, 483], 5, {}),
     ((1, 8, 2, 64), [1, 3, 121, 479, 480, 483], 66, dict(pool_width=1)),
 ]
