@@ -4,9 +4,11 @@
 // s = (l, g) with that group's keys K_s = [positions x d] (App. C.1: a_{l,h,r,t} is the
 // softmax over t of scale * <q, k>).  Operands are K-major bf16 tiles in the 128-byte
 // swizzled layout, staged by TMA; one thread issues tcgen05.mma (fp32 accumulation in TMEM);
-// the epilogue warps read TMEM with tcgen05.ld.  A paged sender cache is first copied into a
-// contiguous staging buffer by k_depage (TMA needs a fixed tile shape, which a page boundary
-// inside a tile breaks), and both passes read that copy.
+// the epilogue warps read TMEM with tcgen05.ld.  A paged sender cache (pages of at least 8 rows) is
+// read by pass 1 page by page, and the tiles it has staged go on, by TMA stores out of the ring,
+// into a contiguous copy that pass 2 reads: pass 2's tiles of every fourth position would need a
+// load for every four rows (at least 144 us for the loads alone of qwen8b in 16-position pages,
+// with four issuing warps).  Shorter pages are copied by k_depage first.
 //
 //   k_stats_tc  pass 1, D = Q_s K_tile^T: TMEM lane = row (r, h), column = position.
 //               Each epilogue thread owns one row and one quarter of a tile's positions and keeps
@@ -61,6 +63,7 @@ constexpr int kEpiWarps = 16;
 constexpr int kEpi0 = 4;                    // first epilogue warp (TMEM lane quarter = warp % 4)
 constexpr int kMaxStages = 8;
 constexpr int kTileRows = 128;          // K rows per tile
+constexpr int kMinPageShift = 3;        // shortest pages pass 1 reads itself: 8 rows, one swizzle atom
 constexpr int kChunk1 = kStatsChunkTc;  // pass-1 positions per chunk
 constexpr int kRowHalf = 128;           // query rows of one accumulator buffer
 constexpr int kHalves1 = 4, kHalves2 = 2;        // most 128-row halves of a row chunk (pass 1, pass 2)
@@ -74,7 +77,9 @@ constexpr int kMaxTcSenders = 32;         // their tensor maps fill most of the 
 
 struct TcMaps {
     CUtensorMap k[5];     // pass 1: k[0] = 4D {d, T, Hkv, nL}, box {64, 128, 1, 1}; k[1] the same over the
-                          // query tokens' own keys {d, m, Hkv, nL} (senders that have them).
+                          // query tokens' own keys {d, m, Hkv, nL} (senders that have them).  Of a paged
+                          // sender k[0] = 5D {d, rows of a page, pages, Hkv, nL}, box {64, min(rows, 128), 1, 1, 1},
+                          // and k[2] = the copy, 4D like a strided sender's.
                           // pass 2: k[4] = 5D {d, T / 4, 4, Hkv, nL} (position 4 i + j at (i, j)), box
                           // {64, 32, 1, 1, 1}; k[j] = 4D positions j, j + 4, ... with every one of them (the
                           // 5D tensor lacks the last T mod 4), box {64, 32, 1, 1}
@@ -91,6 +96,8 @@ struct TcSender {
     int32_t n_blk2;       // pass-2 blocks of positions
     int32_t n_rc1, n_rc2; // row chunks of each pass
     int32_t m_self;       // query tokens whose own keys join the softmax (m or 0)
+    const int32_t* pages; // block table of a paged sender that pass 1 reads itself, else null
+    int32_t n_pages, page_shift;
 };
 
 struct TcBatch {
@@ -104,6 +111,7 @@ struct TcBatch {
     int32_t p_inf, ph;
     int64_t weight1, weight2;     // work of each pass: 128-row halves over all units
     uint64_t wait_ns;     // limit of one bounded mbarrier wait
+    int32_t paged;        // some sender has `pages`: warp 3 of pass 1 stores its tiles
     int32_t stall;        // 1: CTA 0's pass-1 MMA issuer first waits on a barrier nothing arrives on
     uint32_t* err;
     TcMaps maps[kMaxTcSenders];   // (apart from the sizes: a tensor map is aligned to 128 bytes)
@@ -273,7 +281,7 @@ __device__ __forceinline__ Smem carve(uint8_t* raw, const TcBatch& bt) {
     return sm;
 }
 
-// `k_releasers`: MMA issuers that arrive on a K slot's empty barrier.
+// `k_releasers`: roles that arrive on a K slot's empty barrier.
 __device__ __forceinline__ void init_ctl(Ctl* ctl, int k_releasers, uint64_t wait_ns) {
     for (int k = 0; k < kMaxStages; ++k) {
         mbar_init(&ctl->k_full[k], 1);
@@ -365,7 +373,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
     Ctl* ctl = sm.ctl;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        init_ctl(ctl, 2, bt.wait_ns);
+        init_ctl(ctl, bt.paged ? 3 : 2, bt.wait_ns);
         my_units<1>(bt, ctl);
     }
     if (warp == 1) {
@@ -389,12 +397,17 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
             bool ok = true;
             int nc = 0, l = 0, g = 0, n_self = 0;
             int64_t T = 0;
+            const int32_t* pages = nullptr;
+            int32_t n_pages = 0, ps = 0;
             for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
                 const TcMaps& mp = bt.maps[un.i];
                 if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
                     const TcSender& sd = bt.s[un.i];
                     nc = n_c<1>(sd);
                     n_self = self_tiles(sd);
+                    pages = sd.pages;
+                    n_pages = sd.n_pages;
+                    ps = sd.page_shift;
                     T = sd.T;
                     l = un.s / bt.Hkv;
                     g = un.s % bt.Hkv;
@@ -407,13 +420,41 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                 const int nt = (int)((min((int64_t)kChunk1, T - c0) + kTileRows - 1) / kTileRows);
                 const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
                 for (int tile = 0; tile < n_tiles; ++tile) {
-                    if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 1))) break;
-                    mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
                     const bool self = tile >= nt;
                     const int32_t row = self ? (tile - nt) * kTileRows : (int32_t)(c0 + tile * kTileRows);
-                    for (int kb = 0; kb < D / 64; ++kb)
-                        tma_load_4d(sm.k + (size_t)st * kTile + kb * kTileRows * 128, &mp.k[self ? 1 : 0],
-                                    &ctl->k_full[st], 64 * kb, row, g, l);
+                    // a tile's block-table entries, all in flight together while its slot is waited for
+                    const int box = ps < 7 ? 1 << ps : kTileRows;
+                    int32_t entry[kTileRows >> kMinPageShift];
+                    if (pages && !self) {
+#pragma unroll
+                        for (int r = 0; r < kTileRows >> kMinPageShift; ++r)
+                            if (r * box < kTileRows && row + r * box < T) entry[r] = __ldg(pages + ((row + r * box) >> ps));
+                    }
+                    if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 1))) break;
+                    mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
+                    if (pages && !self) {
+                        // one box a page (or 128 rows of one); a page past T, or outside the pool (recorded), is
+                        // the coordinate past the last page, which reads as zeros
+#pragma unroll
+                        for (int r = 0; r < kTileRows >> kMinPageShift; ++r) {
+                            if (r * box >= kTileRows) break;
+                            int32_t pg = n_pages;
+                            if (row + r * box < T) {
+                                pg = entry[r];
+                                if (pg < 0 || pg >= n_pages) {
+                                    pg = n_pages;
+                                    atomicOr(bt.err, kErrPageIndex);
+                                }
+                            }
+                            for (int kb = 0; kb < D / 64; ++kb)
+                                tma_load_5d(sm.k + (size_t)st * kTile + (kb * kTileRows + r * box) * 128, &mp.k[0],
+                                            &ctl->k_full[st], 64 * kb, (row + r * box) & ((1 << ps) - 1), pg, g, l);
+                        }
+                    } else {
+                        for (int kb = 0; kb < D / 64; ++kb)
+                            tma_load_4d(sm.k + (size_t)st * kTile + kb * kTileRows * 128, &mp.k[self ? 1 : 0],
+                                        &ctl->k_full[st], 64 * kb, row, g, l);
+                    }
                     ++kt;
                     if (++st == stages) { st = 0; ph ^= 1u; }
                 }
@@ -477,7 +518,51 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
             umma_commit(&ctl->drain[me]);
             drain_wait(&ctl->drain[me], 0);
         }
-    } else if (warp >= kEpi0) {
+    } else if (warp < kEpi0) {
+        // ---------------- paged senders: the staged tiles on into the contiguous copy ----------------
+        if (bt.paged && elect_one()) {
+            int st = 0;               // ring slot of the next K tile and its phase parity
+            uint32_t ph = 0;
+            int prev = -1;            // slot of the tile before, whose stores may still read it
+            bool ok = true;
+            int nc = 0, l = 0, g = 0, n_self = 0;
+            int64_t T = 0;
+            bool store = false;
+            for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
+                if (u == 0 || un.c == 0) {
+                    const TcSender& sd = bt.s[un.i];
+                    nc = n_c<1>(sd);
+                    n_self = self_tiles(sd);
+                    T = sd.T;
+                    l = un.s / bt.Hkv;
+                    g = un.s % bt.Hkv;
+                    store = sd.pages && un.rc == 0;   // once for all row chunks
+                }
+                const int64_t c0 = (int64_t)un.c * kChunk1;
+                const int nt = (int)((min((int64_t)kChunk1, T - c0) + kTileRows - 1) / kTileRows);
+                const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
+                for (int tile = 0; tile < n_tiles; ++tile) {
+                    if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
+                    if (store && tile < nt)
+                        for (int kb = 0; kb < D / 64; ++kb)
+                            tma_store_4d(&bt.maps[un.i].k[2], sm.k + (size_t)st * kTile + kb * kTileRows * 128, 64 * kb,
+                                         (int32_t)(c0 + tile * kTileRows), g, l);
+                    bulk_commit();
+                    if (prev >= 0) {
+                        bulk_wait_read<1>();
+                        mbar_arrive(&ctl->k_empty[prev]);
+                    }
+                    prev = st;
+                    if (++st == stages) { st = 0; ph ^= 1u; }
+                }
+            }
+            if (prev >= 0) {
+                bulk_wait_read<0>();
+                mbar_arrive(&ctl->k_empty[prev]);
+            }
+            bulk_wait<0>();
+        }
+    } else {
         // ---------------- epilogue: running max / sum per row ----------------
         const int q = (warp - kEpi0) >> 2;       // column quarter: positions 32 q .. +31 of each tile
         const int sp = warp & 3;                 // TMEM lane quarter
@@ -1064,6 +1149,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
         tb->err = err;
         tb->max_rc1 = tb->max_rc2 = 1;
         tb->weight1 = tb->weight2 = 0;
+        tb->paged = 0;
         int rows1 = kRowHalf, rows2 = kRowHalf;
         int64_t staged = 0;
         const int b_first = firsts.back();
@@ -1071,19 +1157,27 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             const ScoreSender& s = b.s[b_first + k];
             TcSender& d = tb->s[k];
             TcMaps &mp = tb->maps[k], &mp2 = maps2.back()[k];   // pass 1's and pass 2's maps
-            // K as the passes read it: the sender's own tensor, or its staged copy
+            // K as the passes read it: the sender's own tensor, or its staged copy (which pass 1 writes
+            // itself when the pages are long enough)
             const uint16_t* kp = s.k;
             int64_t kl = s.ks_l, kh = s.ks_h, kpos = s.ks_p;
+            const bool fused = s.pm.pages && s.pm.shift >= kMinPageShift && s.pm.n_pages < INT32_MAX;
+            d.pages = fused ? s.pm.pages : nullptr;
+            d.n_pages = fused ? (int32_t)s.pm.n_pages : 0;
+            d.page_shift = s.pm.shift;
+            tb->paged |= fused;
             if (s.pm.pages) {
-                DepageSender& ds = dp->s[dp->n++];
-                ds.k = s.k;
-                ds.ks_l = s.ks_l;
-                ds.ks_h = s.ks_h;
-                ds.ks_p = s.ks_p;
-                ds.pm = s.pm;
-                ds.T = s.T;
-                ds.out = b.stage + staged;
-                kp = ds.out;
+                if (!fused) {
+                    DepageSender& ds = dp->s[dp->n++];
+                    ds.k = s.k;
+                    ds.ks_l = s.ks_l;
+                    ds.ks_h = s.ks_h;
+                    ds.ks_p = s.ks_p;
+                    ds.pm = s.pm;
+                    ds.T = s.T;
+                    ds.out = b.stage + staged;
+                }
+                kp = b.stage + staged;
                 kpos = d_head;
                 kh = s.T * d_head;
                 kl = (int64_t)b.n_kv_heads * s.T * d_head;
@@ -1134,7 +1228,16 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
                 const cuuint32_t k4box[4] = {64, 32, 1, 1};
                 ok4 = ok4 && encode_4d(&mp2.k[j], kp + first * kpos, k4d, k4s, k4box);
             }
-            if (!encode_4d(&mp.k[0], kp, kd, ks, kbox) || !ok4 || !encode_4d(&mp.q, s.q, qd, qs, qbox) || !b.ext ||
+            bool ok1 = encode_4d(&mp.k[fused ? 2 : 0], kp, kd, ks, kbox);
+            if (fused) {
+                const cuuint64_t rows = (cuuint64_t)1 << s.pm.shift;
+                const cuuint64_t pd[5] = {kd[0], rows, (cuuint64_t)s.pm.n_pages, kd[2], kd[3]};
+                const cuuint64_t pst[4] = {(cuuint64_t)s.ks_p * 2, (cuuint64_t)s.pm.s_page * 2, (cuuint64_t)s.ks_h * 2,
+                                           (cuuint64_t)s.ks_l * 2};
+                const cuuint32_t pbox[5] = {64, (cuuint32_t)(rows < kTileRows ? rows : kTileRows), 1, 1, 1};
+                ok1 = ok1 && encode_nd(&mp.k[0], s.k, 5, pd, pst, pbox, CU_TENSOR_MAP_SWIZZLE_128B);
+            }
+            if (!ok1 || !ok4 || !encode_4d(&mp.q, s.q, qd, qs, qbox) || !b.ext ||
                 !encode_nd(&mp2.e, b.ext + s.ext_off, 3, ed, es, ebox, CU_TENSOR_MAP_SWIZZLE_32B)) {
                 return cudaErrorNotSupported;
             }

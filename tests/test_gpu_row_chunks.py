@@ -121,20 +121,22 @@ def _paged(K, P, seed):
     n = -(-T // P)
     g = torch.Generator().manual_seed(seed)
     table = torch.randperm(n + 3, generator=g)[:n].to(torch.int32).cuda()
-    pool = torch.zeros(nL, n + 3, P, Hkv, d, dtype=K.dtype, device="cuda")
-    full = torch.zeros(nL, n * P, Hkv, d, dtype=K.dtype, device="cuda")
+    pool = torch.full((nL, n + 3, P, Hkv, d), float("nan"), dtype=K.dtype, device="cuda")
+    full = torch.full((nL, n * P, Hkv, d), float("nan"), dtype=K.dtype, device="cuda")   # rows past T
     full[:, :T] = K.permute(0, 2, 1, 3)
     pool[:, table.long()] = full.view(nL, n, P, Hkv, d)
     return cb.PagedKV(pool, pool, table, T)
 
 
-@pytest.mark.parametrize("d,m", [(64, 70), (128, 200)])
-def test_paged_equals_strided(d, m):
-    w = synth.custom_workload(synth.Shape(2, 8, 2, d), [611, 300], m, seed=d, n_planted_spans=2)
+@pytest.mark.parametrize("d,m,P", [(64, 70, 16), (128, 200, 16), (128, 40, 8), (128, 40, 128), (64, 300, 512), (128, 20, 4)])
+def test_paged_equals_strided(d, m, P):
+    """Pages of 8 rows and more go through pass 1's own loads and stores (one box a page, or 128 rows
+    of a longer one), shorter ones through the copy kernel."""
+    w = synth.custom_workload(synth.Shape(2, 8, 2, d), [1100, 300], m, seed=d, n_planted_spans=2)
     Ks, Q = [s.K.cuda() for s in w.senders], w.queries[0].cuda()
-    out = [[torch.empty(t, device="cuda") for t in (611, 300)] for _ in range(2)]
-    for caches, o in zip((Ks, [_paged(K, 16, i) for i, K in enumerate(Ks)]), out):
-        c = make_cb(w.spec.shape, 611, m, 2)
+    out = [[torch.empty(t, device="cuda") for t in (1100, 300)] for _ in range(2)]
+    for caches, o in zip((Ks, [_paged(K, P, i) for i, K in enumerate(Ks)]), out):
+        c = make_cb(w.spec.shape, 1100, m, 2)
         c.score(caches, [Q, Q], o)
         c.sync_status()
         assert c.score_path() == 2
