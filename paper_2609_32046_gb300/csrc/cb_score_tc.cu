@@ -606,42 +606,40 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                 S[h] = fadd2(S[h], fadd2(p0, p1));
             }
         };
-        float2* dst = nullptr;                   // the current group's partials of this thread's first row
-        int nh = 0, nc = 0, rows = 0, R = 0;     // rows: query rows from the thread's first on
-        int m_self = 0, tok = 0;                 // tokens with own keys; the thread's first row's token
-        int64_t T = 0;
-        for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
-            if (u == 0 || un.c == 0) {
-                const TcSender& sd = bt.s[un.i];
-                const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
-                nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0;
-                nc = n_c<1>(sd);
-                T = sd.T;
-                R = sd.R;
-                rows = R - h0 * kRowHalf - L;
-                m_self = sd.m_self;
-                tok = (h0 * kRowHalf + L) >> bt.log2g;
-                dst = sd.stats + ((int64_t)un.s * sd.n_chunk1 + q) * R + h0 * kRowHalf + L;
-            }
-            const int len = (int)min((int64_t)kChunk1, T - (int64_t)un.c * kChunk1);
+        for (int left = n_units; left > 0 && ok;) {
+            // the run of chunks of one group and row chunk (nothing but positions changes in it)
+            const TcSender& sd = bt.s[un.i];
+            const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
+            const int nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0;
+            const int R = sd.R, rows = R - h0 * kRowHalf - L;   // rows: query rows from the thread's first on
+            const int m_self = sd.m_self, tok = (h0 * kRowHalf + L) >> bt.log2g;   // the thread's first row's token
+            const int T = (int)sd.T, nc = n_c<1>(sd), run = min(left, nc - un.c);
+            int c = un.c;
+            float2* dst = sd.stats + ((int64_t)un.s * sd.n_chunk1 + 4 * c + q) * R + h0 * kRowHalf + L;
+            left -= run;
+            un.c += run - 1;
+            next_unit<1>(bt, un, nc);
+            for (int k = 0; k < run && ok; ++k, ++c, dst += 4 * (int64_t)R) {
+                const int len = min(kChunk1, T - c * kChunk1);
 #pragma unroll
-            for (int h = 0; h < NH; ++h) { M[h] = -INFINITY; S[h] = 0; }
-            int t0 = 0;
-            constexpr std::false_type no{};
-            constexpr std::true_type yes{};
-            for (; t0 + kTileRows <= len && ok; t0 += kTileRows) tile(no, no, 32, t0 == 0, nh, 0);
-            if (t0 < len && ok) tile(yes, no, len - t0 - 32 * q, t0 == 0, nh, 0);
-            if (m_self > 0 && un.c + 1 == nc)   // the query tokens' own keys join the last chunk
-                for (int u0 = 32 * q; u0 - 32 * q < m_self && ok; u0 += kTileRows)
-                    tile(yes, yes, m_self - u0, false, nh, tok + 1 - u0);
-            if (!ok) break;
-            // this warp's partial statistics for the chunk: slot 4 c + q (rows of positions past T
-            // are (-FLT_MAX, 0), which adds nothing); the combine kernel merges all slots
+                for (int h = 0; h < NH; ++h) { M[h] = -INFINITY; S[h] = 0; }
+                int t0 = 0;
+                constexpr std::false_type no{};
+                constexpr std::true_type yes{};
+                for (; t0 + kTileRows <= len && ok; t0 += kTileRows) tile(no, no, 32, t0 == 0, nh, 0);
+                if (t0 < len && ok) tile(yes, no, len - t0 - 32 * q, t0 == 0, nh, 0);
+                if (m_self > 0 && c + 1 == nc)   // the query tokens' own keys join the last chunk
+                    for (int u0 = 32 * q; u0 - 32 * q < m_self && ok; u0 += kTileRows)
+                        tile(yes, yes, m_self - u0, false, nh, tok + 1 - u0);
+                if (!ok) break;
+                // this warp's partial statistics for the chunk: slot 4 c + q (rows of positions past T
+                // are (-FLT_MAX, 0), which adds nothing); the combine kernel merges all slots
 #pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                float s0, s1;
-                unpack2(S[h], s0, s1);
-                if (h < nh && h * kRowHalf < rows) dst[(int64_t)4 * un.c * R + h * kRowHalf] = make_float2(M[h], s0 + s1);
+                for (int h = 0; h < NH; ++h) {
+                    float s0, s1;
+                    unpack2(S[h], s0, s1);
+                    if (h < nh && h * kRowHalf < rows) dst[h * kRowHalf] = make_float2(M[h], s0 + s1);
+                }
             }
         }
     }
@@ -845,89 +843,97 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
         float4* xch = reinterpret_cast<float4*>(sm.epi) + q * 256 + sp * 32 + lane;   // [column quarter][U, N][lane quarter][lane]
         const uint64_t cc = pack2(bt.sl2e, bt.sl2e);
         const bool p_inf = !P2 && bt.p_inf;
-        uint32_t n = 0, nu = 0;                  // rounds of the four buffers and blocks so far
+        uint32_t n = 0, nu = 0;                  // parities: rounds of the four buffers, blocks so far
         bool ok = true;
-        int T = 0, nh = 0, R = 0, nc = 0;        // of the current sender and row chunk; R: query rows from its first on
-        for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
-            if (u == 0 || un.c == 0) {
-                const TcSender& sd = bt.s[un.i];
-                const int h0 = rc_begin(sd.halves, sd.n_rc2, un.rc);
-                nh = rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0;
-                R = sd.R - h0 * kRowHalf;
-                T = (int)sd.T;
-                nc = sd.n_blk2;
-            }
-            const int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
-            const bool all_valid = __all_sync(0xffffffffu, pos >= 0 && pos + 3 < T);
-            float us[4] = {0.f, 0.f, 0.f, 0.f}, ns[4] = {0.f, 0.f, 0.f, 0.f};   // per position: sums over tokens
-            for (int h = 0; h < nh && ok; ++h, ++n) {
-                const bool active = h * kRowHalf + 32 * q < R;     // else padding columns only
-                constexpr int kSub = 4 / G;                        // sub-blocks of eight tokens
+        for (int left = n_units; left > 0 && ok;) {
+            // the run of blocks of one group and row chunk (nothing but positions changes in it)
+            const TcSender& sd = bt.s[un.i];
+            const int h0 = rc_begin(sd.halves, sd.n_rc2, un.rc);
+            const int nh = rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0;
+            const int R = sd.R - h0 * kRowHalf;  // query rows from the row chunk's first on
+            const int T = (int)sd.T, nc = sd.n_blk2, run = min(left, nc - un.c);
+            int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
+            left -= run;
+            un.c += run - 1;
+            next_unit<2>(bt, un, nc);
+            for (int k = 0; k < run && ok; ++k, pos += kOut2) {
+                const int first = pos - 4 * lane;
+                const bool all_valid = first >= 0 && first + 128 <= T;
+                float us[4] = {0.f, 0.f, 0.f, 0.f}, ns[4] = {0.f, 0.f, 0.f, 0.f};   // per position: sums over tokens
+                for (int h = 0; h < nh; ++h, n ^= 1) {
+                    if (h * kRowHalf + 32 * q >= R) {   // padding columns only
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if (!(ok = wait_bar(&ctl->t_full[j], n, ctl, bt.err, 13))) break;
+                            if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
+                        }
+                        if (!ok) break;
+                        continue;
+                    }
+                    constexpr int kSub = 4 / G;         // sub-blocks of eight tokens
 #pragma unroll 1
-                for (int sb = 0; sb < kSub; ++sb) {
-                    uint64_t b[4][4];
+                    for (int sb = 0; sb < kSub; ++sb) {
+                        uint64_t b[4][4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        if (sb == 0 && !(ok = wait_bar(&ctl->t_full[j], n & 1, ctl, bt.err, 13))) break;
-                        tc_fence_after();
-                        // eight tokens' columns, 16 at a time (8 for G = 1)
-                        constexpr int kCols = G == 1 ? 8 : 16;
+                        for (int j = 0; j < 4; ++j) {
+                            if (sb == 0 && !(ok = wait_bar(&ctl->t_full[j], n, ctl, bt.err, 13))) break;
+                            tc_fence_after();
+                            // eight tokens' columns, 16 at a time (8 for G = 1)
+                            constexpr int kCols = G == 1 ? 8 : 16;
 #pragma unroll
-                        for (int x = 0; x < 8 * G; x += kCols) {
-                            float v[kCols];
-                            if (active) {
+                            for (int x = 0; x < 8 * G; x += kCols) {
+                                float v[kCols];
                                 tmem_ldn(ta + j * 128 + sb * 8 * G + x, v);
                                 tmem_wait_ld(v);
+                                if (sb == kSub - 1 && x + kCols == 8 * G) {   // registers hold the rest
+                                    tc_fence_before();
+                                    __syncwarp();
+                                    if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
+                                }
+                                head_sums<G>(v, cc, b[j] + x / (2 * G));
                             }
-                            if (sb == kSub - 1 && x + kCols == 8 * G) {   // registers hold the rest
-                                tc_fence_before();
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
+                        }
+                        if (!ok) break;
+                        if (!all_valid) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const bool valid = pos + j >= 0 && pos + j < T;
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) b[j][i] = valid ? b[j][i] : 0ull;
                             }
-                            if (active) head_sums<G>(v, cc, b[j] + x / (2 * G));
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            float x0[4], x1[4], o0[4], o1[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                unpack2(b[j][i], x0[j], x1[j]);
+                                us[j] += x0[j] + x1[j];
+                            }
+                            pool4<PH>(x0, o0);
+                            pool4<PH>(x1, o1);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                if (P2) {
+                                    ns[j] = fmaf(o0[j], o0[j], fmaf(o1[j], o1[j], ns[j]));
+                                } else if (p_inf) {   // p = infinity: largest pooled value
+                                    ns[j] = fmaxf(ns[j], fmaxf(o0[j], o1[j]));
+                                } else {
+                                    ns[j] += pow_p(o0[j], bt.p) + pow_p(o1[j], bt.p);
+                                }
+                            }
                         }
                     }
                     if (!ok) break;
-                    if (!active) continue;
-                    if (!all_valid) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const bool valid = pos + j >= 0 && pos + j < T;
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) b[j][i] = valid ? b[j][i] : 0ull;
-                        }
-                    }
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float x0[4], x1[4], o0[4], o1[4];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            unpack2(b[j][i], x0[j], x1[j]);
-                            us[j] += x0[j] + x1[j];
-                        }
-                        pool4<PH>(x0, o0);
-                        pool4<PH>(x1, o1);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            if (P2) {
-                                ns[j] = fmaf(o0[j], o0[j], fmaf(o1[j], o1[j], ns[j]));
-                            } else if (p_inf) {   // p = infinity: largest pooled value
-                                ns[j] = fmaxf(ns[j], fmaxf(o0[j], o1[j]));
-                            } else {
-                                ns[j] += pow_p(o0[j], bt.p) + pow_p(o1[j], bt.p);
-                            }
-                        }
-                    }
                 }
+                // hand the block's sums to warp 3 (it has read the last block's long ago)
+                if (!ok || !(ok = wait_bar(&ctl->xe, nu ^ 1, ctl, bt.err, 7))) break;
+                xch[0] = make_float4(us[0], us[1], us[2], us[3]);
+                xch[128] = make_float4(ns[0], ns[1], ns[2], ns[3]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->xb);
+                nu ^= 1;
             }
-            if (!ok) break;
-            // hand the block's sums to warp 3 (it has read the last block's long ago)
-            if (!(ok = wait_bar(&ctl->xe, (nu & 1) ^ 1, ctl, bt.err, 7))) break;
-            xch[0] = make_float4(us[0], us[1], us[2], us[3]);
-            xch[128] = make_float4(ns[0], ns[1], ns[2], ns[3]);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&ctl->xb);
-            ++nu;
         }
     } else {
         // ---------------- warp 3: the column quarters' sums of a block, added in a fixed order ----------------
