@@ -138,8 +138,8 @@ def select_noalloc(scores: Sequence, Ts: Sequence[int], budgets: Sequence[int], 
     lib = load_library()
     n = len(scores)
     st = lib.cb_select_noalloc(n, _ptr_array([s.data_ptr() for s in scores]),
-                               _ptr_array([int(t) for t in Ts], ctypes.c_int64),
-                               _ptr_array([int(b) for b in budgets], ctypes.c_int64),
+                               _ptr_array(list(map(int, Ts)), ctypes.c_int64),
+                               _ptr_array(list(map(int, budgets)), ctypes.c_int64),
                                _ptr_array([x.data_ptr() for x in idx]), n_sink, n_latent, span_width,
                                _stream_handle(stream))
     if st != CB_OK:
@@ -156,14 +156,19 @@ def select_noalloc_status(stream=None):
 
 
 def _ptr_array(values, ctype=ctypes.c_void_p):
-    arr = (ctype * len(values))(*values)
-    return arr
+    return (ctype * len(values))(*values)
+
+
+_torch_cuda = None
 
 
 def _stream_handle(stream) -> int:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        global _torch_cuda
+        if _torch_cuda is None:
+            import torch
+            _torch_cuda = torch.cuda
+        return _torch_cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -205,21 +210,23 @@ def kv_desc(K, V=None) -> cb_kv:
     (V ignored: the PagedKV holds both pools)."""
     if isinstance(K, PagedKV):
         return K.desc()
-    assert K.dtype.itemsize == 2 and K.stride(3) == 1
-    if V is not None:
-        assert V.shape == K.shape and V.stride() == K.stride()
-    return cb_kv(K.data_ptr(), V.data_ptr() if V is not None else None, K.shape[2],
-                 K.stride(0), K.stride(1), K.stride(2))
+    st = K.stride()
+    assert K.element_size() == 2 and st[3] == 1
+    if V is None:
+        return cb_kv(K.data_ptr(), None, K.size(2), st[0], st[1], st[2])
+    assert V.stride() == st and V.size() == K.size()
+    return cb_kv(K.data_ptr(), V.data_ptr(), K.size(2), st[0], st[1], st[2])
 
 
 def query_desc(Q, Kself=None) -> cb_query:
     """Q: bf16 [nL][m][Hq][d]; Kself (optional): the query tokens' own keys, bf16 [nL][m][Hkv][d]."""
-    assert Q.dtype.itemsize == 2 and Q.stride(3) == 1
+    st = Q.stride()
+    assert Q.element_size() == 2 and st[3] == 1
     if Kself is None:
-        return cb_query(Q.data_ptr(), Q.shape[1], Q.stride(0), Q.stride(1), Q.stride(2), None, 0, 0, 0)
-    assert Kself.dtype.itemsize == 2 and Kself.stride(3) == 1 and Kself.shape[1] == Q.shape[1]
-    return cb_query(Q.data_ptr(), Q.shape[1], Q.stride(0), Q.stride(1), Q.stride(2), Kself.data_ptr(),
-                    Kself.stride(0), Kself.stride(1), Kself.stride(2))
+        return cb_query(Q.data_ptr(), Q.size(1), st[0], st[1], st[2])   # (the rest: no own keys)
+    ks = Kself.stride()
+    assert Kself.element_size() == 2 and ks[3] == 1 and Kself.size(1) == Q.size(1)
+    return cb_query(Q.data_ptr(), Q.size(1), st[0], st[1], st[2], Kself.data_ptr(), ks[0], ks[1], ks[2])
 
 
 class CacheBack:
@@ -281,8 +288,8 @@ class CacheBack:
     def select(self, scores: Sequence, Ts: Sequence[int], budgets: Sequence[int], idx: Sequence, stream=None):
         n = len(scores)
         sp = _ptr_array([s.data_ptr() for s in scores])
-        Ta = _ptr_array([int(t) for t in Ts], ctypes.c_int64)
-        Ba = _ptr_array([int(b) for b in budgets], ctypes.c_int64)
+        Ta = _ptr_array(list(map(int, Ts)), ctypes.c_int64)
+        Ba = _ptr_array(list(map(int, budgets)), ctypes.c_int64)
         ip = _ptr_array([x.data_ptr() for x in idx])
         self._check(self.lib.cb_select(self.h, n, sp, Ta, Ba, ip, _stream_handle(stream)))
 
@@ -292,11 +299,12 @@ class CacheBack:
         n = len(Ks)
         kv = (cb_kv * n)(*[kv_desc(K, V) for K, V in zip(Ks, Vs)])
         ip = _ptr_array([x.data_ptr() for x in idx])
-        Ba = _ptr_array([int(b) for b in budgets], ctypes.c_int64)
-        Oa = _ptr_array([int(o) for o in offsets], ctypes.c_int64)
-        assert k_out.stride(3) == 1 and k_out.stride(2) == k_out.shape[3] and v_out.stride() == k_out.stride()
+        Ba = _ptr_array(list(map(int, budgets)), ctypes.c_int64)
+        Oa = _ptr_array(list(map(int, offsets)), ctypes.c_int64)
+        ost = k_out.stride()
+        assert ost[3] == 1 and ost[2] == k_out.size(3) and v_out.stride() == ost
         self._check(self.lib.cb_compact(self.h, n, kv, ip, Ba, k_out.data_ptr(), v_out.data_ptr(),
-                                        k_out.shape[2], Oa, k_out.stride(0), k_out.stride(1),
+                                        k_out.size(2), Oa, ost[0], ost[1],
                                         _stream_handle(stream)))
 
     def compact_rope(self, Ks: Sequence, Vs: Sequence, idx: Sequence, budgets: Sequence[int], k_out, v_out,
@@ -306,11 +314,12 @@ class CacheBack:
         n = len(Ks)
         kv = (cb_kv * n)(*[kv_desc(K, V) for K, V in zip(Ks, Vs)])
         ip = _ptr_array([x.data_ptr() for x in idx])
-        Ba = _ptr_array([int(b) for b in budgets], ctypes.c_int64)
-        Oa = _ptr_array([int(o) for o in offsets], ctypes.c_int64)
-        assert k_out.stride(3) == 1 and k_out.stride(2) == k_out.shape[3] and v_out.stride() == k_out.stride()
+        Ba = _ptr_array(list(map(int, budgets)), ctypes.c_int64)
+        Oa = _ptr_array(list(map(int, offsets)), ctypes.c_int64)
+        ost = k_out.stride()
+        assert ost[3] == 1 and ost[2] == k_out.size(3) and v_out.stride() == ost
         self._check(self.lib.cb_compact_rope(self.h, n, kv, ip, Ba, k_out.data_ptr(), v_out.data_ptr(),
-                                             k_out.shape[2], Oa, k_out.stride(0), k_out.stride(1), float(base),
+                                             k_out.size(2), Oa, ost[0], ost[1], float(base),
                                              int(style), int(pos0), _stream_handle(stream)))
 
     def gather(self, tables: Sequence, idx: Sequence, counts: Sequence[int], out, offsets: Sequence[int],
@@ -329,7 +338,7 @@ class CacheBack:
         Ta = _ptr_array([int(t.shape[0]) for t in tables], ctypes.c_int64)
         ip = _ptr_array([x.data_ptr() for x in idx])
         Ca = _ptr_array([int(c) for c in counts], ctypes.c_int64)
-        Oa = _ptr_array([int(o) for o in offsets], ctypes.c_int64)
+        Oa = _ptr_array(list(map(int, offsets)), ctypes.c_int64)
         self._check(self.lib.cb_gather(self.h, n, sp, Ta, src_stride, row_bytes, ip, Ca, out.data_ptr(),
                                        out.shape[0], Oa, out.stride(0) * out.element_size(),
                                        _stream_handle(stream)))
