@@ -57,6 +57,31 @@ def test_three_hop_chain(mode, keep, B_max):
     assert chain.T_old == T_old
 
 
+@pytest.mark.parametrize("form", ["contiguous", "position_major", "different_strides", "offset_rows", "float32"])
+def test_new_rows_join_the_message(form):
+    """Every form of the new rows lands in the chain's buffer: those the compaction kernel takes and
+    those that are copied as tensors."""
+    nL, Hkv, T, d = 2, 2, 130, 64
+    g = torch.Generator(device="cuda").manual_seed(1)
+    c = make_cb(synth.Shape(nL, 4, Hkv, d), 400, 4, 1)
+    chain = cb.Chain(c, 400, keep=0.5, device="cuda")
+    Q = torch.randn(nL, 4, 4, d, generator=g, device="cuda", dtype=torch.bfloat16)
+    for _ in range(2):
+        K, V = (torch.randn(nL, Hkv, T, d, generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+        if form == "position_major":
+            K, V = (x.permute(2, 0, 1, 3).contiguous().permute(1, 2, 0, 3) for x in (K, V))
+        elif form == "different_strides":
+            V = V.permute(1, 0, 2, 3).contiguous().permute(1, 0, 2, 3)
+        elif form == "offset_rows":        # rows that start 8 bytes off a 16-byte boundary
+            K, V = (torch.nn.functional.pad(x, (4, 4))[..., 4:4 + d] for x in (K, V))
+        elif form == "float32":
+            K, V = K.float(), V.float()
+        a = chain.T_old
+        r = chain.hop(Q, K, V)
+        c.sync_status()
+        assert torch.equal(r["K"][:, :, a:].float(), K.float()) and torch.equal(r["V"][:, :, a:].float(), V.float())
+
+
 def test_chain_rejects_overflow():
     shape = (1, 4, 2, 128)
     c = make_cb(synth.Shape(*shape), 200, 4, 1)
