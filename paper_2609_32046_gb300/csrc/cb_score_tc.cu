@@ -21,7 +21,7 @@
 //               logits (a / G), the head mean b and the sums over tokens stay in registers; Pool
 //               over positions needs the neighbouring lanes' prefix and suffix maxima only.  A
 //               block's four lane quarters cover 128 positions each, 120 of them outputs (480 a
-//               block).
+//               block; blocks of two or one quarters where there are few).
 //
 // Rows: a group's m * G query rows, padded to 128, are processed in row chunks of up to 512
 // (pass 1) or 256 rows (pass 2) whose Q fits in shared memory; a row chunk is the outermost part
@@ -69,7 +69,6 @@ constexpr int kRowHalf = 128;           // query rows of one accumulator buffer
 constexpr int kHalves1 = 4, kHalves2 = 2;        // most 128-row halves of a row chunk (pass 1, pass 2)
 constexpr int kMargin = 4;              // pass-2 positions before/after a lane quarter's outputs
 constexpr int kOutW = 128 - 2 * kMargin;         // 120 output positions per pass-2 lane quarter
-constexpr int kOut2 = 4 * kOutW;                 // 480 output positions per pass-2 block
 constexpr uint32_t kTmemCols = 512;
 constexpr uint64_t kWaitNs = 1000000000ull;      // 1 s per wait
 constexpr uint32_t kPollNs = 1000000u;           // longest suspension of one poll (woken at completion)
@@ -106,6 +105,7 @@ struct TcBatch {
     int32_t nL, Hq, Hkv, G, log2g;
     int32_t stages1, rows1;       // pass 1: K ring stages, Q rows held
     int32_t kbufs, rows2;         // pass 2: K blocks in flight (1 or 2, four tiles each), Q rows held
+    int32_t nw;                   // pass 2: lane quarters in use, 120 output positions each (4; fewer when units are few)
     int32_t max_rc1, max_rc2;
     float sl2e, p;
     int32_t p_inf, ph;
@@ -714,14 +714,18 @@ __device__ __forceinline__ void head_sums(const float (&v)[C], uint64_t cc, uint
     }
 }
 
-// Epilogue: lane quarter w = warp % 4 of a block covers positions 480 c + 120 w - 4 .. + 127; its
+// Epilogue: lane quarter w = warp % 4 of block c covers positions 480 c + 120 w - 4 .. + 127; its
 // lane i holds positions 4 i .. 4 i + 3 of them, one in each of the block's four tiles.  Lanes 1
 // to 30 are outputs, lanes 0 and 31 their Pool margin.  The four warps of
 // a lane quarter take 32 columns (query rows) each of every buffer; their sums meet in
 // shared memory at the end of the block, where warp 3 does the adding: an epilogue warp that
 // waited for its three neighbours would hold up the next block's buffers (28 us of this pass).  MMA issuer i fills
 // the buffers of tiles i and i + 2.
-template <int D, int G, int PH, bool P2>
+// P: how N adds up the pooled values.  kPowSquare p = 2, kPowAny another p, kPowInf maxima (an
+// instantiation each: choosing inside the loops spilled registers).
+enum { kPowSquare, kPowAny, kPowInf };
+
+template <int D, int G, int PH, int P>
 __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constant__ TcBatch bt) {
     constexpr int kTile = kTileRows * D * 2;
     extern __shared__ uint8_t smem_raw[];
@@ -742,7 +746,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
     const uint32_t tmem = ctl->tmem_base;
     const int n_units = ctl->units;
     Unit un = ctl->first;
-    const int slots = 4 * bt.kbufs;
+    const int slots = 4 * bt.kbufs, nw = bt.nw;
 
     if (warp == 0) {
         if (elect_one()) {
@@ -767,23 +771,34 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                     load_q<D, 2>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0);
                     ++qn;
                 }
-                const int32_t t0 = un.c * kOut2 - kMargin;
+                const int32_t t0 = un.c * kOutW * nw - kMargin;
                 // the 5D map serves every tile (a change of map costs the TMA unit time: 150 against
                 // 115 us for the loads of this pass with a map a tile); the maps of the single tiles
                 // are for a last block that ends on one of the last T mod 4 positions
-                const bool whole = t0 + kOut2 + kMargin + 4 <= T / 4 * 4 || T % 4 == 0;
+                const int32_t i0 = t0 / 4;
+                const bool whole = t0 + kOutW * nw + 2 * kMargin <= T / 4 * 4 || T % 4 == 0;
                 for (int j = 0; j < 4; ++j) {
                     if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 9))) break;
                     // lane quarter w: positions t0 + 120 w + j + 4 i, i = 0 .. 31 (t0 a multiple of four)
                     uint8_t* dst = sm.k + (size_t)st * kTile;
-                    mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
-                    for (int w = 0; w < 4; ++w)
-                        for (int kb = 0; kb < D / 64; ++kb) {
-                            uint8_t* box = dst + kb * kTileRows * 128 + w * 32 * 128;
-                            const int32_t i0 = (t0 + kOutW * w) / 4;
-                            if (whole) tma_load_5d(box, &mp.k[4], &ctl->k_full[st], 64 * kb, i0, j, g, l);
-                            else tma_load_4d(box, &mp.k[j], &ctl->k_full[st], 64 * kb, i0, g, l);
-                        }
+                    mbar_arrive_expect_tx(&ctl->k_full[st], kTile / 4 * nw);
+                    if (whole && nw == 4) {
+                        // (unrolled, one map: the issue time of these loads is on the path of the next block)
+#pragma unroll
+                        for (int w = 0; w < 4; ++w)
+#pragma unroll
+                            for (int kb = 0; kb < D / 64; ++kb)
+                                tma_load_5d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[4], &ctl->k_full[st], 64 * kb,
+                                            i0 + kOutW / 4 * w, j, g, l);
+                    } else {
+                        for (int w = 0; w < nw; ++w)
+                            for (int kb = 0; kb < D / 64; ++kb) {
+                                uint8_t* box = dst + kb * kTileRows * 128 + w * 32 * 128;
+                                const int32_t iw = i0 + kOutW / 4 * w;
+                                if (whole) tma_load_5d(box, &mp.k[4], &ctl->k_full[st], 64 * kb, iw, j, g, l);
+                                else tma_load_4d(box, &mp.k[j], &ctl->k_full[st], 64 * kb, iw, g, l);
+                            }
+                    }
                     ++kt;
                     if (++st == slots) { st = 0; ph ^= 1u; }
                 }
@@ -842,7 +857,6 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
         const uint32_t ta = tmem + ((uint32_t)(sp * 32) << 16) + 32 * q;
         float4* xch = reinterpret_cast<float4*>(sm.epi) + q * 256 + sp * 32 + lane;   // [column quarter][U, N][lane quarter][lane]
         const uint64_t cc = pack2(bt.sl2e, bt.sl2e);
-        const bool p_inf = !P2 && bt.p_inf;
         uint32_t n = 0, nu = 0;                  // parities: rounds of the four buffers, blocks so far
         bool ok = true;
         for (int left = n_units; left > 0 && ok;) {
@@ -852,77 +866,100 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
             const int nh = rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0;
             const int R = sd.R - h0 * kRowHalf;  // query rows from the row chunk's first on
             const int T = (int)sd.T, nc = sd.n_blk2, run = min(left, nc - un.c);
-            int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
+            int pos = un.c * kOutW * nw + kOutW * sp - kMargin + 4 * lane;
             left -= run;
             un.c += run - 1;
             next_unit<2>(bt, un, nc);
-            for (int k = 0; k < run && ok; ++k, pos += kOut2) {
+            for (int k = 0; k < run && ok; ++k, pos += kOutW * nw) {
                 const int first = pos - 4 * lane;
                 const bool all_valid = first >= 0 && first + 128 <= T;
                 float us[4] = {0.f, 0.f, 0.f, 0.f}, ns[4] = {0.f, 0.f, 0.f, 0.f};   // per position: sums over tokens
+                // N of position j takes two tokens' pooled values
+                auto add_n = [&](int j, float o0, float o1) {
+                    if (P == kPowSquare) ns[j] = fmaf(o0, o0, fmaf(o1, o1, ns[j]));
+                    else if (P == kPowInf) ns[j] = fmaxf(ns[j], fmaxf(o0, o1));
+                    else ns[j] += pow_p(o0, bt.p) + pow_p(o1, bt.p);
+                };
+                // Pool and the sums of two tokens (one pair of each of the four positions)
+                auto pool_pair = [&](const auto& b, int i) {
+                    float x0[4], x1[4], o0[4], o1[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        unpack2(b[j][i], x0[j], x1[j]);
+                        us[j] += x0[j] + x1[j];
+                    }
+                    pool4<PH>(x0, o0);
+                    pool4<PH>(x1, o1);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) add_n(j, o0[j], o1[j]);
+                };
+                // One round of the four buffers.  EDGE: positions outside [0, T) are masked.  For d = 128 a
+                // buffer's 32 columns are read one after the other (eight tokens at a time for G < 4, 16
+                // columns a load) and go back to the MMA, which takes as long as the reading, before the
+                // next buffer's.  For d = 64 the MMA takes half that, so buffers can be held longer: four
+                // tokens' columns at a time, the exp2 of a chunk's four tiles interleaved with Pool of the
+                // chunk before it (143 -> 137 us for d64; d = 128 156 -> 168).  Unpooled sums (PH = 0) need no
+                // neighbours and are taken load by load.
+                auto round = [&](auto edge) {
+                    constexpr bool EDGE = decltype(edge)::value, LAP = D == 64 && PH > 0;
+                    constexpr int kTok = LAP ? 4 : 8, kChunks = 32 / (kTok * G), kPairs = kTok / 2;
+                    constexpr int kCols = kTok * G < 16 ? kTok * G : 16;   // columns of a load
+                    uint64_t b[LAP ? 2 : 1][4][kPairs];
+#pragma unroll(LAP ? kChunks : 1)
+                    for (int c = 0; c < kChunks; ++c) {
+                        auto& bc = b[LAP ? c & 1 : 0];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if (c == 0) {
+                                if (!(ok = wait_bar(&ctl->t_full[j], n, ctl, bt.err, 13))) return;
+                                tc_fence_after();
+                            }
+#pragma unroll
+                            for (int x = 0; x < kTok * G; x += kCols) {
+                                float v[kCols];
+                                tmem_ldn(ta + j * 128 + c * kTok * G + x, v);
+                                if (LAP && c > 0 && (j & 1)) pool_pair(b[LAP ? (c & 1) ^ 1 : 0], j >> 1);
+                                tmem_wait_ld(v);
+                                if (c == kChunks - 1 && x + kCols == kTok * G) {   // registers hold the rest
+                                    tc_fence_before();
+                                    __syncwarp();
+                                    if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
+                                }
+                                uint64_t* bx = bc[j] + x / (2 * G);
+                                head_sums<G>(v, cc, bx);
+                                if (EDGE) {
+                                    const bool valid = pos + j >= 0 && pos + j < T;
+#pragma unroll
+                                    for (int i = 0; i < kCols / (2 * G); ++i) bx[i] = valid ? bx[i] : 0ull;
+                                }
+                                if (PH == 0) {
+#pragma unroll
+                                    for (int i = 0; i < kCols / (2 * G); ++i) {
+                                        float x0, x1;
+                                        unpack2(bx[i], x0, x1);
+                                        us[j] += x0 + x1;
+                                        add_n(j, x0, x1);
+                                    }
+                                }
+                            }
+                        }
+                        if (PH > 0 && (!LAP || c == kChunks - 1)) {
+#pragma unroll
+                            for (int i = 0; i < kPairs; ++i) pool_pair(bc, i);
+                        }
+                    }
+                };
                 for (int h = 0; h < nh; ++h, n ^= 1) {
-                    if (h * kRowHalf + 32 * q >= R) {   // padding columns only
+                    if (h * kRowHalf + 32 * q >= R || sp >= nw) {   // padding columns, or no positions
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             if (!(ok = wait_bar(&ctl->t_full[j], n, ctl, bt.err, 13))) break;
                             if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
                         }
-                        if (!ok) break;
-                        continue;
-                    }
-                    constexpr int kSub = 4 / G;         // sub-blocks of eight tokens
-#pragma unroll 1
-                    for (int sb = 0; sb < kSub; ++sb) {
-                        uint64_t b[4][4];
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            if (sb == 0 && !(ok = wait_bar(&ctl->t_full[j], n, ctl, bt.err, 13))) break;
-                            tc_fence_after();
-                            // eight tokens' columns, 16 at a time (8 for G = 1)
-                            constexpr int kCols = G == 1 ? 8 : 16;
-#pragma unroll
-                            for (int x = 0; x < 8 * G; x += kCols) {
-                                float v[kCols];
-                                tmem_ldn(ta + j * 128 + sb * 8 * G + x, v);
-                                tmem_wait_ld(v);
-                                if (sb == kSub - 1 && x + kCols == 8 * G) {   // registers hold the rest
-                                    tc_fence_before();
-                                    __syncwarp();
-                                    if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
-                                }
-                                head_sums<G>(v, cc, b[j] + x / (2 * G));
-                            }
-                        }
-                        if (!ok) break;
-                        if (!all_valid) {
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const bool valid = pos + j >= 0 && pos + j < T;
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) b[j][i] = valid ? b[j][i] : 0ull;
-                            }
-                        }
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            float x0[4], x1[4], o0[4], o1[4];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                unpack2(b[j][i], x0[j], x1[j]);
-                                us[j] += x0[j] + x1[j];
-                            }
-                            pool4<PH>(x0, o0);
-                            pool4<PH>(x1, o1);
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                if (P2) {
-                                    ns[j] = fmaf(o0[j], o0[j], fmaf(o1[j], o1[j], ns[j]));
-                                } else if (p_inf) {   // p = infinity: largest pooled value
-                                    ns[j] = fmaxf(ns[j], fmaxf(o0[j], o1[j]));
-                                } else {
-                                    ns[j] += pow_p(o0[j], bt.p) + pow_p(o1[j], bt.p);
-                                }
-                            }
-                        }
+                    } else if (all_valid) {
+                        round(std::false_type{});
+                    } else {
+                        round(std::true_type{});
                     }
                     if (!ok) break;
                 }
@@ -938,7 +975,6 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
     } else {
         // ---------------- warp 3: the column quarters' sums of a block, added in a fixed order ----------------
         const float4* xch = reinterpret_cast<const float4*>(sm.epi) + lane;   // [column quarter][U, N][lane quarter][lane]
-        const bool p_inf = !P2 && bt.p_inf;
         const int nS = bt.nL * bt.Hkv;
         bool ok = true;
         float* part = nullptr;                   // U partials of the current group and row chunk
@@ -953,9 +989,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                 nc = sd.n_blk2;
             }
             if (!(ok = wait_bar(&ctl->xb, (uint32_t)u & 1, ctl, bt.err, 14))) break;
-#pragma unroll
-            for (int sp = 0; sp < 4; ++sp) {
-                const int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
+            for (int sp = 0; sp < nw; ++sp) {
+                const int pos = un.c * kOutW * nw + kOutW * sp - kMargin + 4 * lane;
                 float4 x[4], y[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
@@ -969,7 +1004,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                 if (lane >= 1 && lane <= 30 && pos < T) {   // rows are padded to a multiple of four positions
                     *reinterpret_cast<float4*>(part + pos) = add(add(x[0], x[1]), add(x[2], x[3]));
                     *reinterpret_cast<float4*>(part + nST + pos) =
-                        p_inf ? mx(mx(y[0], y[1]), mx(y[2], y[3])) : add(add(y[0], y[1]), add(y[2], y[3]));
+                        P == kPowInf ? mx(mx(y[0], y[1]), mx(y[2], y[3])) : add(add(y[0], y[1]), add(y[2], y[3]));
                 }
             }
             __syncwarp();
@@ -1041,33 +1076,37 @@ size_t smem2_bytes(int d, int rows, int kbufs) {
     return 1024 + (size_t)rows * (d * 2 + 32) + 128 * 32 + (size_t)kbufs * 4 * kTileRows * d * 2 + 512 + 4 * 8 * 128 * 4;
 }
 
-template <int D, int G, int PH, bool P2>
+template <int D, int G, int PH, int P>
 cudaError_t launch_accum(const TcBatch& tb, int grid, cudaStream_t st) {
     const size_t smem = smem2_bytes(D, tb.rows2, tb.kbufs);
     static std::atomic<uint64_t> done{0};
-    const cudaError_t e = allow_smem(k_accum_tc<D, G, PH, P2>, done);
+    const cudaError_t e = allow_smem(k_accum_tc<D, G, PH, P>, done);
     if (e != cudaSuccess) return e;
-    k_accum_tc<D, G, PH, P2><<<grid, kThreadsTc, smem, st>>>(tb);
+    k_accum_tc<D, G, PH, P><<<grid, kThreadsTc, smem, st>>>(tb);
     return cudaGetLastError();
 }
 
-template <int D, int G, bool P2>
+template <int D, int G, int P>
 cudaError_t launch_accum_gp(const TcBatch& tb, int grid, cudaStream_t st) {
     switch (tb.ph) {
-        case 0: return launch_accum<D, G, 0, P2>(tb, grid, st);
-        case 1: return launch_accum<D, G, 1, P2>(tb, grid, st);
-        case 2: return launch_accum<D, G, 2, P2>(tb, grid, st);
-        case 3: return launch_accum<D, G, 3, P2>(tb, grid, st);
+        case 0: return launch_accum<D, G, 0, P>(tb, grid, st);
+        case 1: return launch_accum<D, G, 1, P>(tb, grid, st);
+        case 2: return launch_accum<D, G, 2, P>(tb, grid, st);
+        case 3: return launch_accum<D, G, 3, P>(tb, grid, st);
     }
     return cudaErrorInvalidValue;
 }
 
+template <int D, int G>
+cudaError_t launch_accum_g(const TcBatch& tb, int grid, cudaStream_t st) {
+    if (tb.p == 2.f) return launch_accum_gp<D, G, kPowSquare>(tb, grid, st);
+    return tb.p_inf ? launch_accum_gp<D, G, kPowInf>(tb, grid, st) : launch_accum_gp<D, G, kPowAny>(tb, grid, st);
+}
+
 template <int D>
 cudaError_t launch_accum_d(const TcBatch& tb, int grid, cudaStream_t st) {
-    const bool p2 = tb.p == 2.f;
-    if (tb.G == 4) return p2 ? launch_accum_gp<D, 4, true>(tb, grid, st) : launch_accum_gp<D, 4, false>(tb, grid, st);
-    if (tb.G == 2) return p2 ? launch_accum_gp<D, 2, true>(tb, grid, st) : launch_accum_gp<D, 2, false>(tb, grid, st);
-    return p2 ? launch_accum_gp<D, 1, true>(tb, grid, st) : launch_accum_gp<D, 1, false>(tb, grid, st);
+    if (tb.G == 4) return launch_accum_g<D, 4>(tb, grid, st);
+    return tb.G == 2 ? launch_accum_g<D, 2>(tb, grid, st) : launch_accum_g<D, 1>(tb, grid, st);
 }
 
 template <int D, int NH>
@@ -1094,6 +1133,28 @@ int pass_grid(int64_t units, int num_sms, int n_rc) {
     int g = num_sms;
     if (n_rc > 1 && n_rc <= g) g = g / n_rc * n_rc;
     return (int)(units < g ? units : g);
+}
+
+// Lane quarters of a pass-2 block: four, unless the grid has so few units that fewer positions a
+// unit spread them better over the SMs (a unit costs about its quarters and one more, so 32 groups
+// of 2106 positions take two units of 240 positions an SM and not two of 480 on eight of them).
+// A position's sums do not depend on it.
+int pass2_quarters(const ScoreSender* s, int n, int G, int nS, int num_sms) {
+    int best = 4;
+    int64_t cost = INT64_MAX;
+    for (int nw = 4; nw >= 1; nw /= 2) {
+        int64_t units = 0;
+        for (int i = 0; i < n; ++i) {
+            const int64_t halves = ((int64_t)s[i].m * G + kRowHalf - 1) / kRowHalf;
+            units += nS * ((halves + kHalves2 - 1) / kHalves2) * ((s[i].T + kOutW * nw - 1) / (kOutW * nw));
+        }
+        const int64_t c = (units + num_sms - 1) / num_sms * (nw + 1);
+        if (c < cost) {
+            cost = c;
+            best = nw;
+        }
+    }
+    return best;
 }
 
 }  // namespace
@@ -1156,6 +1217,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
         tb->max_rc1 = tb->max_rc2 = 1;
         tb->weight1 = tb->weight2 = 0;
         tb->paged = 0;
+        tb->nw = pass2_quarters(&b.s[firsts.back()], nb, G, nS, num_sms);
         int rows1 = kRowHalf, rows2 = kRowHalf;
         int64_t staged = 0;
         const int b_first = firsts.back();
@@ -1195,7 +1257,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             d.R = s.m * G;
             d.halves = (d.R + kRowHalf - 1) / kRowHalf;
             d.n_chunk1 = (int32_t)(4 * ((s.T + kChunk1 - 1) / kChunk1));   // one partial per (chunk, column quarter)
-            d.n_blk2 = (int32_t)((s.T + kOut2 - 1) / kOut2);
+            d.n_blk2 = (int32_t)((s.T + kOutW * tb->nw - 1) / (kOutW * tb->nw));
             d.n_rc1 = (d.halves + kHalves1 - 1) / kHalves1;
             d.n_rc2 = (d.halves + kHalves2 - 1) / kHalves2;
             d.stats = b.stats + s.stats_off;

@@ -39,6 +39,10 @@ CASES = [
     ((1, 8, 2, 128), [1030, 1025, 5, 129], 100, dict(self_keys=True)),
     ((1, 8, 2, 128), [1, 2, 3, 5, 119, 120, 121, 122, 480, 481, 482, 483], 5, {}),
     ((1, 8, 2, 64), [1, 3, 121, 479, 480, 483], 66, dict(pool_width=1)),
+    # few units: blocks of one, two and four lane quarters (2, 8 and 32 groups)
+    ((1, 2, 2, 128), [1000], 20, dict(pool_width=1, p=3.0)),
+    ((2, 16, 4, 128), [2106], 24, dict(p=3.0)),
+    ((8, 8, 4, 128), [2400], 24, dict(pool_width=1, p=float("inf"))),
 ]
 
 
