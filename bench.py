@@ -68,6 +68,14 @@ def workload_bytes_flops(spec, keep):
     return tot_b, score_b, compact_b, tot_f
 
 
+def partial_bytes(spec, Ts):
+    """Bytes of the second pass's partial sums: two fp32 per position and KV group (the sums over
+    the query tokens of b and of Pool(b)^p) for every 256 query rows of a group."""
+    sh = spec.shape
+    chunks = math.ceil(spec.m * sh.n_q_heads // sh.n_kv_heads / 256)
+    return sum(2 * chunks * sh.n_layers * sh.n_kv_heads * T * 4 for T in Ts)
+
+
 def workload_config(spec, keep, paged: int = 0, ws: int = 1):
     """The keys that define the workload of a bench line; both arms report the same dict."""
     sh = spec.shape
@@ -491,9 +499,9 @@ def time_workload(name: str, ws: int, rank: int, dev, use_graph: bool):
            "warmup": warmup, "config": workload_config(spec, keep, 0, ws),
            "hbm_gbs": tot_b / step_s / 1e9, "hbm_frac": tot_b / step_s / 1e9 / hbm_peak,
            "algorithmic_bytes_per_step": tot_b,
-           "roofline": dict(kernel_roofline(score_b + sum(3 * spec.shape.n_layers * spec.shape.n_kv_heads * T * 4
-                                                          for T in f.Ts), flops / 2, accum, hbm_peak, tc_peak,
-                                            "%s bf16 %s (cuBLAS)" % (src, peak_kind)), kernel="k_accum_tc"),
+           "roofline": dict(kernel_roofline(score_b + partial_bytes(spec, f.Ts), flops / 2, accum, hbm_peak,
+                                            tc_peak, "%s bf16 %s (cuBLAS)" % (src, peak_kind)),
+                            kernel="k_accum_tc"),
            "roofline_step": {"t_hbm_us": tot_b / (hbm_peak * 1e9) * 1e6,
                              "t_tensor_us": flops / (tc_peak * 1e12) * 1e6,
                              "frac": max(tot_b / (hbm_peak * 1e9), flops / (tc_peak * 1e12)) / step_s},
@@ -783,8 +791,9 @@ def run_ours(args):
     tokens_per_rank = sum(f.Ts)
     def launches(n):
         # per call group of <= 64 senders: statistics, combine and accumulation per sub-batch of
-        # <= 32 senders (paged caches: also a de-page launch, and sub-batches end where the staging
-        # buffer is full), then one finalize launch; one select and one compact launch per group
+        # <= 32 senders (paged caches: sub-batches end where the staging buffer is full, and pages of
+        # fewer than 8 rows take a de-page launch each), then one finalize launch; one select and one
+        # compact launch per group
         sb = math.ceil(n / 64)
         if not args.paged:
             tc = sum(math.ceil(min(64, n - 64 * b) / 32) for b in range(sb))
@@ -793,7 +802,7 @@ def run_ours(args):
         stage = max(e, min(n * e, 1 << 30))
         per = max(1, min(32, stage // e))
         tc = sum(math.ceil(min(64, n - 64 * b) / per) for b in range(sb))
-        return 4 * tc + sb + sb + sb
+        return (3 if args.paged >= 8 else 4) * tc + sb + sb + sb
 
     waves = [min(wave, n_send - a) for a in range(0, n_send, wave)] if wave else [n_send]
     launches_per_step = sum(launches(n) for n in waves)
@@ -801,7 +810,7 @@ def run_ours(args):
     hbm_peak, tc_peak, tc_sus, src = peaks()
     tot_b, score_b, compact_b, flops = workload_bytes_flops(spec, keep)
     pass_flops = flops / 2                                   # one QK^T pass
-    part_bytes = sum(3 * spec.shape.n_layers * spec.shape.n_kv_heads * T * 4 for T in f.Ts)
+    part_bytes = partial_bytes(spec, f.Ts)
     step_s = ms / args.steps / 1e3
 
     # e2e: the whole step through the C-ABI with every sender cache kept in pinned host memory.

@@ -70,9 +70,11 @@ typedef struct cb_ctx cb_ctx; /* opaque; owns device scratch only */
  *   pool_width         Pool window, odd, 1..15 (7 in the paper; 1 disables pooling)
  *   span_width         span width for selection, 1..256 (16 in the paper; 1 ranks positions)
  *   n_sink, n_latent   forced positions: the first n_sink and the last n_latent (1 and 40)
- *   score_kernel       0: automatic (tcgen05 tensor-core passes when head_dim = 128,
- *                      pool_width <= 7 and max_query_tokens * G <= 512, else the mma.sync
- *                      passes); 1: mma.sync passes; 2: tcgen05 passes (CB_ESHAPE if unsupported)
+ *   score_kernel       0: automatic (tcgen05 tensor-core passes when pool_width <= 7, except for
+ *                      small senders of head_dim 64, which take less time on the mma.sync
+ *                      passes; else the mma.sync passes); 1: mma.sync passes; 2: tcgen05 passes
+ *                      (CB_ESHAPE unless head_dim = 128, pool_width <= 7 and
+ *                      max_query_tokens * G <= 512)
  */
 typedef struct {
     int32_t n_layers, n_q_heads, n_kv_heads, head_dim;
@@ -152,8 +154,9 @@ cb_status cb_create(const cb_config *cfg, cb_ctx **out);
  * sender state against many receiver queries (multi-query serving: Sec. 5, Discussion, notes
  * that one completed sender state can be scored for several receiver queries), each pair
  * exactly as if it were scored alone.
- * Paged senders (cb_kv.pages) on the tcgen05 passes are first copied into a contiguous staging
- * buffer of the context (the copy is timed with pass 1).  The first call that needs more room
+ * Paged senders (cb_kv.pages) on the tcgen05 passes are copied into a contiguous staging buffer of
+ * the context for the second pass: by pass 1 itself from pages of at least 8 rows, ahead of it from
+ * shorter ones (the copy is timed with pass 1).  The first call that needs more room
  * than the buffer has allocates it anew, which waits for the device: make such a call before
  * capturing cb_score in a CUDA graph.  Its size is that of the largest paged cache of the call,
  * or of all of them up to 2 GiB, whichever is larger (senders beyond it are scored in later

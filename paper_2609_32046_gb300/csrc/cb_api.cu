@@ -394,7 +394,7 @@ cb_status cb_score(cb_ctx* ctx, int32_t n, const cb_kv* senders, const cb_query*
     cudaStream_t strm = reinterpret_cast<cudaStream_t>(stream);
     const int nS = c.n_layers * c.n_kv_heads;
     if (ctx->use_tc) {
-        // paged senders are copied into a contiguous staging buffer for the tensor-map passes:
+        // paged senders are copied into a contiguous staging buffer for the second pass:
         // room for the largest one, and for the rest up to kStageBudget elements per sub-batch
         int64_t largest = 0, sum = 0;
         for (int i = 0; i < n; ++i)

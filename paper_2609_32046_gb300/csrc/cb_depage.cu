@@ -1,10 +1,11 @@
-// Contiguous copy of paged sender caches (the tcgen05 score passes read K through TMA tensor
-// maps, whose fixed tile shape a page boundary inside a tile would break).
+// Contiguous copy of paged sender caches with pages of fewer than 8 rows, which the tcgen05 score
+// passes would have to load by too many small TMA boxes (4-row boxes take 442 us for the K of 36
+// layers and T = 8192 where this copy takes 183; longer pages are read, and copied, by pass 1).
 //
 // Position t of a paged sender is row t mod P of page pages[t / P] (the block table); the copy
 // is K[l][g][t][:] in the plain [nL][Hkv][T][d] layout.  Consecutive threads take consecutive
 // 16-byte pieces of the rows of one position, heads next, positions last, so reads follow a
-// vLLM page ([row][head][d] contiguous) and writes are whole 256-byte rows.  Each thread moves
+// vLLM page ([row][head][d] contiguous) and writes are whole rows.  Each thread moves
 // kUnroll pieces with all loads issued before the stores.  A block-table entry outside the
 // pool is never dereferenced: its rows are written as zeros and the error word records it.
 #include <cstdint>

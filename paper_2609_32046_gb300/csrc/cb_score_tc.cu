@@ -30,12 +30,13 @@
 // from L2.
 //
 // Warp roles (640 threads, one CTA per SM, persistent over a contiguous range of work
-// units): warp 0 producer, warps 1 and 2 MMA issuers (warp 1 owns TMEM), warp 3 writes pass
-// 2's sums, warps 4-19 epilogue
-// (warp w reads TMEM lanes 32*(w%4)..+31; the four warps of a lane quarter share a buffer's
-// columns).  K tiles flow through a ring of smem stages; TMEM holds a ring of four 128-column
-// accumulator buffers, each drained by all sixteen epilogue warps: the MMA runs up to four buffers
-// ahead.
+// units): warp 0 producer, warps 1 and 2 MMA issuers (warp 1 owns TMEM), warp 3 pass 1's stores of
+// staged pages and pass 2's sums, warps 4-19 epilogue (warp w reads TMEM lanes 32*(w%4)..+31; the
+// four warps of a lane quarter share a buffer's columns).  K tiles flow through a ring of smem
+// stages; TMEM holds a ring of four 128-column accumulator buffers, each drained by all sixteen
+// epilogue warps: the MMA runs up to four buffers ahead.  Two issuers, because one thread that
+// waits, fences and commits for every tile issues a 128 x 128 x 16 step in 76.5 cycles and two in
+// 64.1, the tensor core's own rate.
 // Every mbarrier wait is bounded (1 s); on a timeout the kernel records kErrTimeout, drains
 // its copies and MMAs, frees TMEM and returns.
 #include <algorithm>
@@ -365,6 +366,11 @@ __device__ __forceinline__ void stats_block(const float (&v)[32], uint64_t cc, u
 // positions; it keeps the offset and sum of exp2 of its rows over the chunk and writes them as
 // partial (chunk, quarter); the combine kernel merges all partials of a group s.  The two MMA
 // issuers take alternate buffers.
+// Bound by the epilogue, whose loop of TMEM load, exp2 and packed adds takes 115 us alone for 36
+// layers, T = 8192, 256 rows (exp2 alone 100); the K loads alone take 102 (89 at the copy rate).
+// 124 us together, against 130 with two accumulator tiles of two epilogue groups each and one
+// issuer; 3 x T = 16384 with 512 rows 1216 against 1448 us.  Chunks of 512, 640 or 768 positions
+// take 119 to 122 us, but the combine kernel 2 to 4 more, and longer at 512 rows.
 template <int D, int NH>
 __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constant__ TcBatch bt) {
     constexpr int kTile = kTileRows * D * 2;
@@ -716,11 +722,16 @@ __device__ __forceinline__ void head_sums(const float (&v)[C], uint64_t cc, uint
 
 // Epilogue: lane quarter w = warp % 4 of block c covers positions 480 c + 120 w - 4 .. + 127; its
 // lane i holds positions 4 i .. 4 i + 3 of them, one in each of the block's four tiles.  Lanes 1
-// to 30 are outputs, lanes 0 and 31 their Pool margin.  The four warps of
-// a lane quarter take 32 columns (query rows) each of every buffer; their sums meet in
-// shared memory at the end of the block, where warp 3 does the adding: an epilogue warp that
-// waited for its three neighbours would hold up the next block's buffers (28 us of this pass).  MMA issuer i fills
-// the buffers of tiles i and i + 2.
+// to 30 are outputs, lanes 0 and 31 their Pool margin.  The four warps of a lane quarter take 32
+// columns (query rows) each of every buffer; their sums meet in shared memory at the end of the
+// block, where warp 3 does the adding: an epilogue warp that waited for its three neighbours would
+// hold up the next block's buffers (28 us of this pass).  MMA issuer i fills the buffers of tiles i
+// and i + 2.
+// Bound by the epilogue: 138 us alone for 36 layers, T = 8192, 256 rows (of about 3700 cycles for
+// four buffers, exp2 takes 2420 and Pool 780), 155 with the K loads (+12) and the MMA (+5).
+// Against one position a thread, tiles of 104 outputs in 128 rows and Pool through a shuffle for
+// every position and shift: 155 against 170 us; 3 x T = 16384 with 512 rows 1627 against 1867;
+// d = 64, 256 rows, T = 8192, where the mma.sync kernel ran, 137 against 769.
 // P: how N adds up the pooled values.  kPowSquare p = 2, kPowAny another p, kPowInf maxima (an
 // instantiation each: choosing inside the loops spilled registers).
 enum { kPowSquare, kPowAny, kPowInf };
