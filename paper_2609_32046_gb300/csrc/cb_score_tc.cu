@@ -21,7 +21,7 @@
 //               logits (a / G), the head mean b and the sums over tokens stay in registers; Pool
 //               over positions needs the neighbouring lanes' prefix and suffix maxima only.  A
 //               block's four lane quarters cover 128 positions each, 120 of them outputs (480 a
-//               block; blocks of two or one quarters where there are few).
+//               block).
 //
 // Rows: a group's m * G query rows, padded to 128, are processed in row chunks of up to 512
 // (pass 1) or 256 rows (pass 2) whose Q fits in shared memory; a row chunk is the outermost part
@@ -70,6 +70,7 @@ constexpr int kRowHalf = 128;           // query rows of one accumulator buffer
 constexpr int kHalves1 = 4, kHalves2 = 2;        // most 128-row halves of a row chunk (pass 1, pass 2)
 constexpr int kMargin = 4;              // pass-2 positions before/after a lane quarter's outputs
 constexpr int kOutW = 128 - 2 * kMargin;         // 120 output positions per pass-2 lane quarter
+constexpr int kOut2 = 4 * kOutW;                 // 480 output positions per pass-2 block
 constexpr uint32_t kTmemCols = 512;
 constexpr uint64_t kWaitNs = 1000000000ull;      // 1 s per wait
 constexpr uint32_t kPollNs = 1000000u;           // longest suspension of one poll (woken at completion)
@@ -106,7 +107,6 @@ struct TcBatch {
     int32_t nL, Hq, Hkv, G, log2g;
     int32_t stages1, rows1;       // pass 1: K ring stages, Q rows held
     int32_t kbufs, rows2;         // pass 2: K blocks in flight (1 or 2, four tiles each), Q rows held
-    int32_t nw;                   // pass 2: lane quarters in use, 120 output positions each (4; fewer when units are few)
     int32_t max_rc1, max_rc2;
     float sl2e, p;
     int32_t p_inf, ph;
@@ -732,6 +732,9 @@ __device__ __forceinline__ void head_sums(const float (&v)[C], uint64_t cc, uint
 // Against one position a thread, tiles of 104 outputs in 128 rows and Pool through a shuffle for
 // every position and shift: 155 against 170 us; 3 x T = 16384 with 512 rows 1627 against 1867;
 // d = 64, 256 rows, T = 8192, where the mma.sync kernel ran, 137 against 769.
+// Blocks of fewer lane quarters gain nothing where there are fewer blocks than SMs (16.2 us either
+// way for 32 groups of T = 2106): a lane quarter's warps share one scheduler, so a block takes as
+// long with one quarter as with four.
 // P: how N adds up the pooled values.  kPowSquare p = 2, kPowAny another p, kPowInf maxima (an
 // instantiation each: choosing inside the loops spilled registers).
 enum { kPowSquare, kPowAny, kPowInf };
@@ -757,7 +760,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
     const uint32_t tmem = ctl->tmem_base;
     const int n_units = ctl->units;
     Unit un = ctl->first;
-    const int slots = 4 * bt.kbufs, nw = bt.nw;
+    const int slots = 4 * bt.kbufs;
 
     if (warp == 0) {
         if (elect_one()) {
@@ -782,18 +785,18 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                     load_q<D, 2>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0);
                     ++qn;
                 }
-                const int32_t t0 = un.c * kOutW * nw - kMargin;
+                const int32_t t0 = un.c * kOut2 - kMargin;
                 // the 5D map serves every tile (a change of map costs the TMA unit time: 150 against
                 // 115 us for the loads of this pass with a map a tile); the maps of the single tiles
                 // are for a last block that ends on one of the last T mod 4 positions
                 const int32_t i0 = t0 / 4;
-                const bool whole = t0 + kOutW * nw + 2 * kMargin <= T / 4 * 4 || T % 4 == 0;
+                const bool whole = t0 + kOut2 + 2 * kMargin <= T / 4 * 4 || T % 4 == 0;
                 for (int j = 0; j < 4; ++j) {
                     if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 9))) break;
                     // lane quarter w: positions t0 + 120 w + j + 4 i, i = 0 .. 31 (t0 a multiple of four)
                     uint8_t* dst = sm.k + (size_t)st * kTile;
-                    mbar_arrive_expect_tx(&ctl->k_full[st], kTile / 4 * nw);
-                    if (whole && nw == 4) {
+                    mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
+                    if (whole) {
                         // (unrolled, one map: the issue time of these loads is on the path of the next block)
 #pragma unroll
                         for (int w = 0; w < 4; ++w)
@@ -802,13 +805,10 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                                 tma_load_5d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[4], &ctl->k_full[st], 64 * kb,
                                             i0 + kOutW / 4 * w, j, g, l);
                     } else {
-                        for (int w = 0; w < nw; ++w)
-                            for (int kb = 0; kb < D / 64; ++kb) {
-                                uint8_t* box = dst + kb * kTileRows * 128 + w * 32 * 128;
-                                const int32_t iw = i0 + kOutW / 4 * w;
-                                if (whole) tma_load_5d(box, &mp.k[4], &ctl->k_full[st], 64 * kb, iw, j, g, l);
-                                else tma_load_4d(box, &mp.k[j], &ctl->k_full[st], 64 * kb, iw, g, l);
-                            }
+                        for (int w = 0; w < 4; ++w)
+                            for (int kb = 0; kb < D / 64; ++kb)
+                                tma_load_4d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[j], &ctl->k_full[st], 64 * kb,
+                                            i0 + kOutW / 4 * w, g, l);
                     }
                     ++kt;
                     if (++st == slots) { st = 0; ph ^= 1u; }
@@ -877,11 +877,11 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
             const int nh = rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0;
             const int R = sd.R - h0 * kRowHalf;  // query rows from the row chunk's first on
             const int T = (int)sd.T, nc = sd.n_blk2, run = min(left, nc - un.c);
-            int pos = un.c * kOutW * nw + kOutW * sp - kMargin + 4 * lane;
+            int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
             left -= run;
             un.c += run - 1;
             next_unit<2>(bt, un, nc);
-            for (int k = 0; k < run && ok; ++k, pos += kOutW * nw) {
+            for (int k = 0; k < run && ok; ++k, pos += kOut2) {
                 const int first = pos - 4 * lane;
                 const bool all_valid = first >= 0 && first + 128 <= T;
                 float us[4] = {0.f, 0.f, 0.f, 0.f}, ns[4] = {0.f, 0.f, 0.f, 0.f};   // per position: sums over tokens
@@ -961,7 +961,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                     }
                 };
                 for (int h = 0; h < nh; ++h, n ^= 1) {
-                    if (h * kRowHalf + 32 * q >= R || sp >= nw) {   // padding columns, or no positions
+                    if (h * kRowHalf + 32 * q >= R) {   // padding columns
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             if (!(ok = wait_bar(&ctl->t_full[j], n, ctl, bt.err, 13))) break;
@@ -1000,8 +1000,9 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                 nc = sd.n_blk2;
             }
             if (!(ok = wait_bar(&ctl->xb, (uint32_t)u & 1, ctl, bt.err, 14))) break;
-            for (int sp = 0; sp < nw; ++sp) {
-                const int pos = un.c * kOutW * nw + kOutW * sp - kMargin + 4 * lane;
+#pragma unroll
+            for (int sp = 0; sp < 4; ++sp) {
+                const int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
                 float4 x[4], y[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
@@ -1146,28 +1147,6 @@ int pass_grid(int64_t units, int num_sms, int n_rc) {
     return (int)(units < g ? units : g);
 }
 
-// Lane quarters of a pass-2 block: four, unless the grid has so few units that fewer positions a
-// unit spread them better over the SMs (a unit costs about its quarters and one more, so 32 groups
-// of 2106 positions take two units of 240 positions an SM and not two of 480 on eight of them).
-// A position's sums do not depend on it.
-int pass2_quarters(const ScoreSender* s, int n, int G, int nS, int num_sms) {
-    int best = 4;
-    int64_t cost = INT64_MAX;
-    for (int nw = 4; nw >= 1; nw /= 2) {
-        int64_t units = 0;
-        for (int i = 0; i < n; ++i) {
-            const int64_t halves = ((int64_t)s[i].m * G + kRowHalf - 1) / kRowHalf;
-            units += nS * ((halves + kHalves2 - 1) / kHalves2) * ((s[i].T + kOutW * nw - 1) / (kOutW * nw));
-        }
-        const int64_t c = (units + num_sms - 1) / num_sms * (nw + 1);
-        if (c < cost) {
-            cost = c;
-            best = nw;
-        }
-    }
-    return best;
-}
-
 }  // namespace
 
 bool tc_path_supported(int head_dim, int G, int pool_half) {
@@ -1228,7 +1207,6 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
         tb->max_rc1 = tb->max_rc2 = 1;
         tb->weight1 = tb->weight2 = 0;
         tb->paged = 0;
-        tb->nw = pass2_quarters(&b.s[firsts.back()], nb, G, nS, num_sms);
         int rows1 = kRowHalf, rows2 = kRowHalf;
         int64_t staged = 0;
         const int b_first = firsts.back();
@@ -1268,7 +1246,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             d.R = s.m * G;
             d.halves = (d.R + kRowHalf - 1) / kRowHalf;
             d.n_chunk1 = (int32_t)(4 * ((s.T + kChunk1 - 1) / kChunk1));   // one partial per (chunk, column quarter)
-            d.n_blk2 = (int32_t)((s.T + kOutW * tb->nw - 1) / (kOutW * tb->nw));
+            d.n_blk2 = (int32_t)((s.T + kOut2 - 1) / kOut2);
             d.n_rc1 = (d.halves + kHalves1 - 1) / kHalves1;
             d.n_rc2 = (d.halves + kHalves2 - 1) / kHalves2;
             d.stats = b.stats + s.stats_off;
