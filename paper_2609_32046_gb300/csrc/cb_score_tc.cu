@@ -65,10 +65,11 @@ constexpr int kEpi0 = 4;                    // first epilogue warp (TMEM lane qu
 constexpr int kMaxStages = 8;
 constexpr int kTileRows = 128;          // K rows per tile
 constexpr int kMinPageShift = 3;        // shortest pages pass 1 reads itself: 8 rows, one swizzle atom
-constexpr int kChunk1 = kStatsChunkTc;  // pass-1 positions per chunk
+constexpr int kChunk1 = kStatsChunkTc;  // pass-1 positions per chunk, or twice as many (stats_chunk)
 constexpr int kRowHalf = 128;           // query rows of one accumulator buffer
 constexpr int kHalves1 = 4, kHalves2 = 2;        // most 128-row halves of a row chunk (pass 1, pass 2)
 constexpr int kMargin = 4;              // pass-2 positions before/after a lane quarter's outputs
+constexpr int64_t kLongChunkUnits = 1024;  // pass-1 units from which chunks are twice as long
 constexpr int kOutW = 128 - 2 * kMargin;         // 120 output positions per pass-2 lane quarter
 constexpr int kOut2 = 4 * kOutW;                 // 480 output positions per pass-2 block
 constexpr uint32_t kTmemCols = 512;
@@ -97,6 +98,7 @@ struct TcSender {
     int32_t n_blk2;       // pass-2 blocks of positions
     int32_t n_rc1, n_rc2; // row chunks of each pass
     int32_t m_self;       // query tokens whose own keys join the softmax (m or 0)
+    int32_t chunk1;       // pass-1 positions per chunk
     const int32_t* pages; // block table of a paged sender that pass 1 reads itself, else null
     int32_t n_pages, page_shift;
 };
@@ -346,8 +348,8 @@ __device__ __forceinline__ void mma_d(uint32_t d_tmem, uint32_t a_lo, uint32_t a
 // logit up to 2^127 above it is exact; one so far above it that exp2 or the sum overflows leaves
 // an infinite sum, and the combine kernel recomputes that row's statistics from Q and K.  (The
 // maximum of the first block in place of its first logit makes the buffers that hold one wait for
-// the maximum: 788 against 729 cycles a buffer.)  The packed adds leave the loop bound by exp2 (584 cycles for a
-// 128 x 128 buffer, 603 with scalar adds, against 512 for its exp2 alone).
+// the maximum: 788 against 729 cycles a buffer.)  The packed adds leave the loop bound by exp2 (584
+// cycles for a 128 x 128 buffer, 603 with scalar adds, against 512 for its exp2 alone).
 __device__ __forceinline__ void stats_block(const float (&v)[32], uint64_t cc, uint64_t nm, uint64_t& p0, uint64_t& p1) {
 #pragma unroll
     for (int q = 0; q < 16; q += 2) {
@@ -366,8 +368,9 @@ __device__ __forceinline__ void stats_block(const float (&v)[32], uint64_t cc, u
 // positions; it keeps the offset and sum of exp2 of its rows over the chunk and writes them as
 // partial (chunk, quarter); the combine kernel merges all partials of a group s.  The two MMA
 // issuers take alternate buffers.
-// Bound by the epilogue, whose loop of TMEM load, exp2 and packed adds takes 115 us alone for 36
-// layers, T = 8192, 256 rows (exp2 alone 100); the K loads alone take 102 (89 at the copy rate).
+// Bound by the epilogue, whose waits, TMEM loads, exp2 and packed adds take 115 us without the K
+// loads for 36 layers, T = 8192, 256 rows (64 at the rate of exp2 alone); the K loads without the
+// epilogue take 102 (89 at the copy rate).
 // 124 us together, against 130 with two accumulator tiles of two epilogue groups each and one
 // issuer; 3 x T = 16384 with 512 rows 1216 against 1448 us.  Chunks of 512, 640 or 768 positions
 // take 119 to 122 us, but the combine kernel 2 to 4 more, and longer at 512 rows.
@@ -401,7 +404,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
             int st = 0;               // ring slot of the next K tile and its phase parity
             uint32_t ph = 0;
             bool ok = true;
-            int nc = 0, l = 0, g = 0, n_self = 0;
+            int nc = 0, l = 0, g = 0, n_self = 0, chunk = 0;
             int64_t T = 0;
             const int32_t* pages = nullptr;
             int32_t n_pages = 0, ps = 0;
@@ -410,6 +413,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                 if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
                     const TcSender& sd = bt.s[un.i];
                     nc = n_c<1>(sd);
+                    chunk = sd.chunk1;
                     n_self = self_tiles(sd);
                     pages = sd.pages;
                     n_pages = sd.n_pages;
@@ -422,8 +426,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                     load_q<D, 1>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0);
                     ++qn;
                 }
-                const int64_t c0 = (int64_t)un.c * kChunk1;
-                const int nt = (int)((min((int64_t)kChunk1, T - c0) + kTileRows - 1) / kTileRows);
+                const int64_t c0 = (int64_t)un.c * chunk;
+                const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows);
                 const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
                 for (int tile = 0; tile < n_tiles; ++tile) {
                     const bool self = tile >= nt;
@@ -488,12 +492,13 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
             // wait gives up, sets the abort flag and every role of this CTA leaves
             if (bt.stall && blockIdx.x == 0) ok = wait_bar(&ctl->stall, 0, ctl, bt.err, 6);
             uint32_t nh = 0;
-            int nc = 0, n_self = 0;
+            int nc = 0, n_self = 0, chunk = 0;
             int64_t T = 0;
             for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
                 if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
                     const TcSender& sd = bt.s[un.i];
                     nc = n_c<1>(sd);
+                    chunk = sd.chunk1;
                     n_self = self_tiles(sd);
                     T = sd.T;
                     nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - rc_begin(sd.halves, sd.n_rc1, un.rc);
@@ -501,8 +506,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                     if (!(ok = wait_bar(&ctl->q_full, qn & 1, ctl, bt.err, 2))) break;
                     ++qn;
                 }
-                const int64_t c0 = (int64_t)un.c * kChunk1;
-                const int nt = (int)((min((int64_t)kChunk1, T - c0) + kTileRows - 1) / kTileRows) +
+                const int64_t c0 = (int64_t)un.c * chunk;
+                const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows) +
                                (un.c + 1 == nc ? n_self : 0);
                 for (int tile = 0; tile < nt; ++tile) {
                     if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
@@ -531,21 +536,22 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
             uint32_t ph = 0;
             int prev = -1;            // slot of the tile before, whose stores may still read it
             bool ok = true;
-            int nc = 0, l = 0, g = 0, n_self = 0;
+            int nc = 0, l = 0, g = 0, n_self = 0, chunk = 0;
             int64_t T = 0;
             bool store = false;
             for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
                 if (u == 0 || un.c == 0) {
                     const TcSender& sd = bt.s[un.i];
                     nc = n_c<1>(sd);
+                    chunk = sd.chunk1;
                     n_self = self_tiles(sd);
                     T = sd.T;
                     l = un.s / bt.Hkv;
                     g = un.s % bt.Hkv;
                     store = sd.pages && un.rc == 0;   // once for all row chunks
                 }
-                const int64_t c0 = (int64_t)un.c * kChunk1;
-                const int nt = (int)((min((int64_t)kChunk1, T - c0) + kTileRows - 1) / kTileRows);
+                const int64_t c0 = (int64_t)un.c * chunk;
+                const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows);
                 const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
                 for (int tile = 0; tile < n_tiles; ++tile) {
                     if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
@@ -619,14 +625,14 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
             const int nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0;
             const int R = sd.R, rows = R - h0 * kRowHalf - L;   // rows: query rows from the thread's first on
             const int m_self = sd.m_self, tok = (h0 * kRowHalf + L) >> bt.log2g;   // the thread's first row's token
-            const int T = (int)sd.T, nc = n_c<1>(sd), run = min(left, nc - un.c);
-            int c = un.c;
-            float2* dst = sd.stats + ((int64_t)un.s * sd.n_chunk1 + 4 * c + q) * R + h0 * kRowHalf + L;
+            const int chunk = sd.chunk1, nc = n_c<1>(sd), run = min(left, nc - un.c);
+            int rest = (int)sd.T - un.c * chunk;   // positions from the chunk's first on
+            float2* dst = sd.stats + ((int64_t)un.s * sd.n_chunk1 + 4 * un.c + q) * R + h0 * kRowHalf + L;
             left -= run;
             un.c += run - 1;
             next_unit<1>(bt, un, nc);
-            for (int k = 0; k < run && ok; ++k, ++c, dst += 4 * (int64_t)R) {
-                const int len = min(kChunk1, T - c * kChunk1);
+            for (int k = 0; k < run && ok; ++k, rest -= chunk, dst += 4 * (int64_t)R) {
+                const int len = min(chunk, rest);
 #pragma unroll
                 for (int h = 0; h < NH; ++h) { M[h] = -INFINITY; S[h] = 0; }
                 int t0 = 0;
@@ -634,7 +640,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                 constexpr std::true_type yes{};
                 for (; t0 + kTileRows <= len && ok; t0 += kTileRows) tile(no, no, 32, t0 == 0, nh, 0);
                 if (t0 < len && ok) tile(yes, no, len - t0 - 32 * q, t0 == 0, nh, 0);
-                if (m_self > 0 && c + 1 == nc)   // the query tokens' own keys join the last chunk
+                if (m_self > 0 && rest <= chunk)   // the query tokens' own keys join the last chunk
                     for (int u0 = 32 * q; u0 - 32 * q < m_self && ok; u0 += kTileRows)
                         tile(yes, yes, m_self - u0, false, nh, tok + 1 - u0);
                 if (!ok) break;
@@ -731,7 +737,7 @@ __device__ __forceinline__ void head_sums(const float (&v)[C], uint64_t cc, uint
 // four buffers, exp2 takes 2420 and Pool 780), 155 with the K loads (+12) and the MMA (+5).
 // Against one position a thread, tiles of 104 outputs in 128 rows and Pool through a shuffle for
 // every position and shift: 155 against 170 us; 3 x T = 16384 with 512 rows 1627 against 1867;
-// d = 64, 256 rows, T = 8192, where the mma.sync kernel ran, 137 against 769.
+// 24 layers, 2 x T = 7001, 200 rows of d = 64, where the mma.sync kernel ran, 137 against 769.
 // Blocks of fewer lane quarters gain nothing where there are fewer blocks than SMs (16.2 us either
 // way for 32 groups of T = 2106): a lane quarter's warps share one scheduler, so a block takes as
 // long with one quarter as with four.
@@ -1138,6 +1144,18 @@ cudaError_t launch_stats_d(const TcBatch& tb, int grid, cudaStream_t st) {
     return launch_stats<D, kHalves1>(tb, grid, st);
 }
 
+// Positions of a pass-1 chunk of a sender of T positions and nS groups.  Chunks of 2048 positions
+// leave half as many partials to write and merge as chunks of 1024, but units too few to spread
+// evenly over the SMs unless there are many.  The combine kernel takes 10.7 against 12.4 us for 288
+// groups, T = 8192 (1152 units), 44 against 73 for three senders of T = 16384 with 512 rows, 13
+// against 19 for 64 groups, T = 65536 (2048 units; pass 1 208 against 204 there, the same
+// elsewhere); below the line pass 1 loses more: 135 against 126 us for 192 groups, 2 x T = 7001
+// (768 units a sender), 146 against 139 for 96 groups, T = 6001 (288).  The rule reads the sender
+// alone, so its scores do not depend on the call's others.
+int32_t stats_chunk(int64_t T, int nS) {
+    return nS * ((T + 2 * kChunk1 - 1) / (2 * kChunk1)) >= kLongChunkUnits ? 2 * kChunk1 : kChunk1;
+}
+
 // CTAs of a pass of `units` units: one an SM, a multiple of the row-chunk count when every sender
 // has the same one (CTAs k, k + grid / n_rc, ... then walk the same K tiles in step, so that a
 // tile comes from DRAM once and from L2 for the other row chunks).
@@ -1245,7 +1263,8 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             d.m_self = s.kself ? s.m : 0;
             d.R = s.m * G;
             d.halves = (d.R + kRowHalf - 1) / kRowHalf;
-            d.n_chunk1 = (int32_t)(4 * ((s.T + kChunk1 - 1) / kChunk1));   // one partial per (chunk, column quarter)
+            d.chunk1 = stats_chunk(s.T, nS);
+            d.n_chunk1 = (int32_t)(4 * ((s.T + d.chunk1 - 1) / d.chunk1));   // one partial per (chunk, column quarter)
             d.n_blk2 = (int32_t)((s.T + kOut2 - 1) / kOut2);
             d.n_rc1 = (d.halves + kHalves1 - 1) / kHalves1;
             d.n_rc2 = (d.halves + kHalves2 - 1) / kHalves2;

@@ -39,7 +39,7 @@ CASES = [
     ((1, 8, 2, 128), [1030, 1025, 5, 129], 100, dict(self_keys=True)),
     ((1, 8, 2, 128), [1, 2, 3, 5, 119, 120, 121, 122, 480, 481, 482, 483], 5, {}),
     ((1, 8, 2, 64), [1, 3, 121, 479, 480, 483], 66, dict(pool_width=1)),
-    # few units: blocks of one, two and four lane quarters (2, 8 and 32 groups)
+    # fewer blocks than SMs
     ((1, 2, 2, 128), [1000], 20, dict(pool_width=1, p=3.0)),
     ((2, 16, 4, 128), [2106], 24, dict(p=3.0)),
     ((8, 8, 4, 128), [2400], 24, dict(pool_width=1, p=float("inf"))),
@@ -63,6 +63,25 @@ def test_scores(case):
         assert_scores_close(f.scores[i].cpu().numpy(), ref["S"], rtol=RTOL)
         check_sender(f, i, s.K, s.V, w.queries[s.task], p=extra.get("p", 2.0), pool_w=extra.get("pool_width", 7),
                      Kself=kself)
+
+
+@pytest.mark.parametrize("own", [False, True])
+def test_long_chunks(own):
+    """1024 groups, enough for chunks of 2048 positions: one with and without a second half, and two;
+    the query tokens' own keys join the last."""
+    nL, H, d, m, Ts = 64, 16, 64, 5, [130, 1024, 1030, 2049]
+    gen = torch.Generator().manual_seed(7)
+    draw = lambda *s: torch.randn(*s, generator=gen).bfloat16()
+    K, Q, own_k = draw(nL, H, max(Ts), d), draw(nL, m, H, d), draw(nL, m, H, d) if own else None
+    c = cb.CacheBack(nL, H, H, d, m, max(Ts), len(Ts))
+    Kd, Qd = K.cuda(), Q.cuda()
+    out = [torch.empty(T, device="cuda") for T in Ts]
+    c.score([Kd[:, :, :T] for T in Ts], [Qd] * len(Ts), out, Kselfs=None if not own else [own_k.cuda()] * len(Ts))
+    c.sync_status()
+    assert c.score_path() == 2
+    for T, got in zip(Ts, out):
+        ref = oracle_scores(oracle.default(), K[:, :, :T].contiguous(), Q, Kself=own_k)
+        assert_scores_close(got.cpu().numpy(), ref["S"], rtol=RTOL)
 
 
 def test_senders_of_different_query_lengths_equal_single_calls():
