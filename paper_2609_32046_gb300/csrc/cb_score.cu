@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(kCombThreads) k_combine(const __grid_constant_
     }
     if (row < R) {
         // A chunk partial whose sum left fp32 range makes the row's sum infinite (pass 1 of the
-        // tensor-memory path offsets each chunk by the maximum of its first 32 logits, so a logit
+        // tensor-memory path offsets each chunk by its first logit, so a logit
         // far larger later in the chunk overflows exp2).  Such rows, rare, are recomputed here
         // from Q and K directly: position t on chain t mod 4.
         bool bad = false;
@@ -616,9 +616,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_accum(const __grid_constant__ S
 // values, which come by shuffles from the neighbouring lanes, so the first and last HQ quads of a
 // tile (HQ = 1 for pool widths up to 9, else 2) are its Pool margin: 16 quads read, 56 (48)
 // positions written.  A batch of groups' loads is issued before they are added: the partials come
-// mostly from DRAM, so the kernel needs many bytes in flight, and with 288 groups a thread has
-// all of its nine groups' loads in flight at once.  The 32 slice sums of every position are then
-// added as a tree in shared memory (the rounding of these sums is most of a score's error: 4.5e-7
+// mostly from DRAM, whose latency bounds the kernel (12.7 us for 19 MB of 288 groups, T = 8192).
+// Rows padded to 16 bytes let ragged lengths load as wide: T = 8191 32 -> 12.5 us.  The 32 slice
+// sums of every position are then added as a tree in shared memory (the rounding of these sums is most of a score's error: 4.5e-7
 // with the slices added in turn), U is pooled and C and S written.  Each sum has a fixed order, so
 // the scores are deterministic.
 constexpr int kFinQuads = 16;
@@ -650,9 +650,10 @@ __device__ __forceinline__ void pool_quads(const float (&x)[4], int ph, float (&
     }
 }
 
-// BATCH: groups of a slice loaded before they are added: 9 (all of 288 groups) while the grid is
-// about one block an SM; 3, whose smaller register footprint fits two blocks an SM, so that one
-// block's loads are in flight while the other adds, for more blocks; 2 for up to 64 groups.
+// BATCH: groups of a slice loaded before they are added: 3, whose register footprint fits two blocks
+// an SM, so that one block's loads are in flight while the other adds (41 us for 8 senders of T =
+// 8192 and 288 groups; all nine of a slice's groups at once 56, two at a time 43; one sender 12.7 us
+// either way); 2 for up to 64 groups, of which a slice has two (T = 65536: 20 us against 21).
 template <int BATCH, int HQ>
 __global__ void __launch_bounds__(kFinThreads) k_finalize(const __grid_constant__ ScoreBatch bt) {
     __shared__ float su[kFinSlices][kFinSpan];
@@ -770,15 +771,11 @@ cudaError_t launch_finalize_b(const ScoreBatch& b, int64_t maxT, cudaStream_t st
     return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(const ScoreBatch& b, cudaStream_t st, int num_sms) {
-    int64_t maxT = 0, tiles = 0;
-    for (int i = 0; i < b.n; ++i) {
-        maxT = b.s[i].T > maxT ? b.s[i].T : maxT;
-        tiles += (b.s[i].T + fin_out(1) - 1) / fin_out(1);
-    }
+cudaError_t launch_finalize(const ScoreBatch& b, cudaStream_t st) {
+    int64_t maxT = 0;
+    for (int i = 0; i < b.n; ++i) maxT = b.s[i].T > maxT ? b.s[i].T : maxT;
     const int per_slice = (b.n_layers * b.n_kv_heads + kFinSlices - 1) / kFinSlices;
-    if (per_slice <= 2) return launch_finalize_b<2>(b, maxT, st);
-    return tiles <= num_sms + num_sms / 4 ? launch_finalize_b<9>(b, maxT, st) : launch_finalize_b<3>(b, maxT, st);
+    return per_slice <= 2 ? launch_finalize_b<2>(b, maxT, st) : launch_finalize_b<3>(b, maxT, st);
 }
 
 // Rows of all senders of a batch; few rows (long senders, few groups) take four threads a row.
@@ -848,7 +845,7 @@ cudaError_t launch_dg(const ScoreBatch& b, cudaStream_t st, int num_sms) {
     stage_mark(b.timer, kStageCombine, st);
     k_accum<D, G><<<(unsigned)nblk2, kThreads, smem2, st>>>(b);
     stage_mark(b.timer, kStageAccum, st);
-    launch_finalize(b, st, num_sms);
+    launch_finalize(b, st);
     stage_mark(b.timer, kStageFinalize, st);
     return cudaGetLastError();
 }
@@ -865,7 +862,7 @@ cudaError_t launch_score(ScoreBatch& b, cudaStream_t st, int num_sms, int* path_
         if (e != cudaErrorNotSupported) {
             *path_out = 2;
             if (e == cudaSuccess) {
-                launch_finalize(b, st, num_sms);
+                launch_finalize(b, st);
                 stage_mark(b.timer, kStageFinalize, st);
                 e = cudaGetLastError();
             }
