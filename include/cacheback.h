@@ -160,7 +160,11 @@ cb_status cb_create(const cb_config *cfg, cb_ctx **out);
  * than the buffer has allocates it anew, which waits for the device: make such a call before
  * capturing cb_score in a CUDA graph.  Its size is that of the largest paged cache of the call,
  * or of all of them up to 2 GiB, whichever is larger (senders beyond it are scored in later
- * launches that reuse the buffer).
+ * launches that reuse the buffer).  A call inside a capture that finds too little room fails with
+ * CB_ENOMEM where head_dim = 128 and max_query_tokens * G <= 512; other shapes then record the
+ * mma.sync passes, which read the pages themselves.  A graph goes on using the buffer it was
+ * captured with: a later, larger call leaves that buffer in place until cb_destroy and takes
+ * another, so graphs stay valid and their room is held beside the new one's.
  *   n         1..max_senders;  senders, queries, scores: host arrays of n entries
  *   scores[i] device float[T_i], written; 16-byte aligned
  * Errors: CB_EINVAL (null/misaligned pointers, strides), CB_ESHAPE (T_i or m_i above the limits),

@@ -68,6 +68,8 @@ struct cb_ctx {
     float* span_keys = nullptr;
     uint16_t* stage = nullptr;      // tcgen05 passes: contiguous copies of paged senders' K (on demand)
     int64_t stage_elems = 0;
+    bool stage_captured = false;    // a captured cb_score uses `stage`: a graph holds its address
+    std::vector<uint16_t*> old_stages;   // outgrown buffers that graphs may still use, until cb_destroy
     uint32_t* err = nullptr;
     int64_t keys_per_sender = 0;
     int64_t scratch_bytes = 0;
@@ -194,6 +196,27 @@ cbk::PageMap page_map(const cb_kv& s) {
         pm.shift = sh;
     }
     return pm;
+}
+
+// A staging buffer of `want` elements; false where it cannot be had.  A graph that captured a
+// cb_score goes on writing and reading the buffer of that call, so such a buffer stays until
+// cb_destroy; another is freed first, which waits for work still using it.
+bool grow_stage(cb_ctx* ctx, int64_t want) {
+    if (ctx->stage && !ctx->stage_captured && cudaFree(ctx->stage) == cudaSuccess) {
+        ctx->scratch_bytes -= ctx->stage_elems * 2;
+        ctx->stage = nullptr;
+        ctx->stage_elems = 0;
+    }
+    uint16_t* p = nullptr;
+    const bool ok = cudaMalloc(reinterpret_cast<void**>(&p), (size_t)want * 2) == cudaSuccess;
+    cudaGetLastError();
+    if (!ok) return false;
+    if (ctx->stage) ctx->old_stages.push_back(ctx->stage);
+    ctx->stage = p;
+    ctx->stage_elems = want;
+    ctx->stage_captured = false;
+    ctx->scratch_bytes += want * 2;
+    return true;
 }
 
 template <typename T>
@@ -343,6 +366,7 @@ void cb_destroy(cb_ctx* ctx) {
         cudaFree(ctx->ones);
         cudaFree(ctx->span_keys);
         cudaFree(ctx->stage);
+        for (uint16_t* p : ctx->old_stages) cudaFree(p);
         cudaFree(ctx->err);
         delete ctx->timer;
     }
@@ -405,26 +429,16 @@ cb_status cb_score(cb_ctx* ctx, int32_t n, const cb_kv* senders, const cb_query*
             }
         const int64_t want = largest > (sum < cbk::kStageBudget ? sum : cbk::kStageBudget)
                                  ? largest : (sum < cbk::kStageBudget ? sum : cbk::kStageBudget);
-        if (want > ctx->stage_elems) {
+        if (want > 0) {
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(strm, &cap) != cudaSuccess) cudaGetLastError();
+            const bool capturing = cap != cudaStreamCaptureStatusNone;
             // Shapes that score_kernel = 2 does not name can also read pages directly (the mma.sync
             // passes), so they neither allocate inside a stream capture nor fail for want of memory.
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-            if (!ctx->tc_stage_must && cudaStreamIsCapturing(strm, &cap) != cudaSuccess) cudaGetLastError();
-            if (ctx->tc_stage_must || cap == cudaStreamCaptureStatusNone) {
-                cudaFree(ctx->stage);   // waits for work still using it
-                ctx->scratch_bytes -= ctx->stage_elems * 2;
-                ctx->stage = nullptr;
-                ctx->stage_elems = 0;
-                if (cudaMalloc(reinterpret_cast<void**>(&ctx->stage), (size_t)want * 2) == cudaSuccess) {
-                    ctx->stage_elems = want;
-                    ctx->scratch_bytes += want * 2;
-                } else {
-                    cudaGetLastError();
-                    ctx->stage = nullptr;
-                    if (ctx->tc_stage_must)
-                        return fail(ctx, CB_ENOMEM, "cannot allocate %lld bytes to stage paged caches", (long long)want * 2);
-                }
-            }
+            if (want > ctx->stage_elems && (ctx->tc_stage_must || !capturing) && !grow_stage(ctx, want) &&
+                ctx->tc_stage_must)
+                return fail(ctx, CB_ENOMEM, "cannot allocate %lld bytes to stage paged caches", (long long)want * 2);
+            ctx->stage_captured |= capturing;
         }
     }
     // the senders of the tcgen05 passes, then those of the mma.sync passes

@@ -159,3 +159,43 @@ def test_bad_page_arguments_are_rejected():
         out = (ctypes.c_void_p * 1)(S.data_ptr())
         st = c.lib.cb_score(c.h, 1, kva, qa, out, torch.cuda.current_stream().cuda_stream)
         assert st == cb.CB_EINVAL, (field, value, st)
+
+
+# (d, m): shapes that must be staged, and shapes whose pages the mma.sync passes can read as well
+@pytest.mark.parametrize("d,m", [(128, 16), (64, 70)])
+def test_captured_graph_outlives_a_larger_call(d, m):
+    """A graph keeps the staging buffer it was captured with: a later call with a larger paged cache
+    takes another, and replays of the graph still give the first call's scores, also when new
+    allocations have filled whatever room was given back."""
+    w = synth.custom_workload(synth.Shape(2, 8, 2, d), [600, 3000], m, seed=d, n_planted_spans=2)
+    Q = w.queries[0].cuda()
+    small, large = (_page(s.K.cuda(), s.V.cuda(), 16, 1, 3) for s in w.senders)
+    c = make_cb(w.spec.shape, 3000, m, 1)
+    S, SL = torch.empty(600, device="cuda"), torch.empty(3000, device="cuda")
+    st = torch.cuda.Stream()
+    c.score([small], [Q], [S], st)              # sizes the staging buffer
+    c.sync_status(st)
+    want = S.clone()
+    before = c.scratch_bytes
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        c.score([small], [Q], [S], st)
+    assert c.score_path() == 2 and c.scratch_bytes == before
+    for T in (1000, 3000):                      # the second replaces a buffer that no graph uses
+        c.score([cb.PagedKV(large.k_pool, large.v_pool, large.pages, T)], [Q], [SL], st)
+        c.sync_status(st)
+        assert c.score_path() == 2
+    nS = 4
+    assert c.scratch_bytes == before + nS * 3000 * d * 2
+    size = nS * 600 * d * 2
+    filler = [torch.full((size,), 0x7f, dtype=torch.uint8, device="cuda") for _ in range(8)]
+    for _ in range(2):
+        S.zero_()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(st):
+            g.replay()
+        c.sync_status(st)
+        assert torch.equal(S.view(torch.int32), want.view(torch.int32))
+    assert all(bool((f == 0x7f).all()) for f in filler)
+    del g
+    c.close()
