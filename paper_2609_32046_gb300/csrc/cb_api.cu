@@ -200,8 +200,12 @@ cbk::PageMap page_map(const cb_kv& s) {
 
 // A staging buffer of `want` elements; false where it cannot be had.  A graph that captured a
 // cb_score goes on writing and reading the buffer of that call, so such a buffer stays until
-// cb_destroy; another is freed first, which waits for work still using it.
-bool grow_stage(cb_ctx* ctx, int64_t want) {
+// cb_destroy; another is freed first, which waits for work still using it.  Unless the call's own
+// stream is being captured, cudaFree and cudaMalloc are let through while some other stream is (the
+// mode is the thread's own, and put back).
+bool grow_stage(cb_ctx* ctx, int64_t want, bool capturing) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (!capturing) cudaThreadExchangeStreamCaptureMode(&mode);
     if (ctx->stage && !ctx->stage_captured && cudaFree(ctx->stage) == cudaSuccess) {
         ctx->scratch_bytes -= ctx->stage_elems * 2;
         ctx->stage = nullptr;
@@ -209,6 +213,7 @@ bool grow_stage(cb_ctx* ctx, int64_t want) {
     }
     uint16_t* p = nullptr;
     const bool ok = cudaMalloc(reinterpret_cast<void**>(&p), (size_t)want * 2) == cudaSuccess;
+    if (!capturing) cudaThreadExchangeStreamCaptureMode(&mode);
     cudaGetLastError();
     if (!ok) return false;
     if (ctx->stage) ctx->old_stages.push_back(ctx->stage);
@@ -435,7 +440,7 @@ cb_status cb_score(cb_ctx* ctx, int32_t n, const cb_kv* senders, const cb_query*
             const bool capturing = cap != cudaStreamCaptureStatusNone;
             // Shapes that score_kernel = 2 does not name can also read pages directly (the mma.sync
             // passes), so they neither allocate inside a stream capture nor fail for want of memory.
-            if (want > ctx->stage_elems && (ctx->tc_stage_must || !capturing) && !grow_stage(ctx, want) &&
+            if (want > ctx->stage_elems && (ctx->tc_stage_must || !capturing) && !grow_stage(ctx, want, capturing) &&
                 ctx->tc_stage_must)
                 return fail(ctx, CB_ENOMEM, "cannot allocate %lld bytes to stage paged caches", (long long)want * 2);
             ctx->stage_captured |= capturing;

@@ -19,7 +19,7 @@ import torch
 import oracle
 import paper_2609_32046_gb300 as cb
 import synth
-from gpu_helpers import check_sender, make_cb
+from gpu_helpers import assert_scores_close, check_sender, make_cb
 
 pytestmark = pytest.mark.gpu
 
@@ -199,3 +199,28 @@ def test_captured_graph_outlives_a_larger_call(d, m):
     assert all(bool((f == 0x7f).all()) for f in filler)
     del g
     c.close()
+
+
+def test_growth_leaves_another_streams_capture_alone():
+    """A paged call on one stream sizes the staging buffer while another stream is being captured (in
+    the default mode, which forbids allocations to every thread that does not say otherwise)."""
+    w = synth.custom_workload(synth.Shape(2, 8, 2, 64), [600, 900], 70, seed=8, n_planted_spans=2)
+    Q = w.queries[0].cuda()
+    caches = [_page(s.K.cuda(), s.V.cuda(), 16, 1, 4) for s in w.senders]
+    out = [torch.empty(s.T, device="cuda") for s in w.senders]
+    c = make_cb(w.spec.shape, 900, 70, 1)
+    side, x = torch.cuda.Stream(), torch.zeros(16, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        x.add_(1)
+        for kv, S in zip(caches, out):          # the first allocates, the second also frees
+            c.score([kv], [Q], [S], side)
+            assert c.score_path() == 2
+        x.add_(1)
+    g.replay()
+    c.sync_status(side)
+    torch.cuda.synchronize()
+    assert bool((x == 2).all())
+    for s, S in zip(w.senders, out):
+        assert_scores_close(S.cpu().numpy(), oracle.default().score(s.K, w.queries[0])["S"])
