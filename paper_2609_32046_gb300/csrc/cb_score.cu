@@ -422,10 +422,8 @@ __global__ void __launch_bounds__(kCombThreads) k_combine(const __grid_constant_
             self_keys_staged<64, NC>(sd, l, g, r_tok, c0l, qrow, bt.scale_log2e, row < R, M, L, ks_sm);
     }
     if (row < R) {
-        // A chunk partial whose sum left fp32 range makes the row's sum infinite (pass 1 of the
-        // tensor-memory path offsets each chunk by its first logit, so a logit
-        // far larger later in the chunk overflows exp2).  Such rows, rare, are recomputed here
-        // from Q and K directly: position t on chain t mod 4.
+        // Logits that are infinite or NaN leave sums that are.  Such rows are recomputed here from Q
+        // and K directly: position t on chain t mod 4.
         bool bad = false;
 #pragma unroll
         for (int k = 0; k < NC; ++k) bad = bad || !(L[k] <= FLT_MAX);

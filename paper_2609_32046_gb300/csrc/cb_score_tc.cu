@@ -69,6 +69,7 @@ constexpr int kChunk1 = kStatsChunkTc;  // pass-1 positions per chunk, or twice 
 constexpr int kRowHalf = 128;           // query rows of one accumulator buffer
 constexpr int kHalves1 = 4, kHalves2 = 2;        // most 128-row halves of a row chunk (pass 1, pass 2)
 constexpr int kMargin = 4;              // pass-2 positions before/after a lane quarter's outputs
+constexpr float kRaise = 8.f;           // pass 1, second run: a logit this far (log2 domain) above a row's offset raises it
 constexpr int64_t kLongChunkUnits = 1024;  // pass-1 units from which chunks are twice as long
 constexpr int kOutW = 128 - 2 * kMargin;         // 120 output positions per pass-2 lane quarter
 constexpr int kOut2 = 4 * kOutW;                 // 480 output positions per pass-2 block
@@ -137,6 +138,7 @@ struct Ctl {
     uint64_t xb, xe;        // pass 2: a block's sums written by the epilogue and read by warp 3
     int32_t units;          // this CTA's units, the first of which is `first`
     Unit first;
+    int32_t redo_lo, redo_hi;   // pass 1: first and last of them with a sum out of range
     uint32_t tmem_base;
     int abort;
 };
@@ -304,6 +306,8 @@ __device__ __forceinline__ void init_ctl(Ctl* ctl, int k_releasers, uint64_t wai
     mbar_init(&ctl->stall, 1);
     ctl->wait_ns = wait_ns;
     ctl->abort = 0;
+    ctl->redo_lo = INT32_MAX;
+    ctl->redo_hi = -1;
     fence_barrier_init();
 }
 
@@ -342,15 +346,12 @@ __device__ __forceinline__ void mma_d(uint32_t d_tmem, uint32_t a_lo, uint32_t a
                   idesc, k > 0 ? 1u : 0u);
 }
 
-// 32 columns of pass 1 for this lane's row: sum of exp2(c z - m), m the row's offset (log2
-// domain): its first logit of the chunk, or -FLT_MAX where the warp's first block holds no
-// position, in which case neither do the chunk's others.  The sum holds that logit's 1, and any
-// logit up to 2^127 above it is exact; one so far above it that exp2 or the sum overflows leaves
-// an infinite sum, and the combine kernel recomputes that row's statistics from Q and K.  (The
-// maximum of the first block in place of its first logit makes the buffers that hold one wait for
-// the maximum: 788 against 729 cycles a buffer.)  The packed adds leave the loop bound by exp2 (584
-// cycles for a 128 x 128 buffer, 603 with scalar adds, against 512 for its exp2 alone).
-__device__ __forceinline__ void stats_block(const float (&v)[32], uint64_t cc, uint64_t nm, uint64_t& p0, uint64_t& p1) {
+// 32 columns of pass 1 for this lane's row: sum of exp2(c z - m), m the row's offset (log2 domain).
+// The packed adds leave the loop bound by exp2 (584 cycles for a 128 x 128 buffer, 603 with scalar
+// adds, against 512 for its exp2 alone).
+__device__ __forceinline__ uint64_t stats_block(const float (&v)[32], uint64_t cc, float m) {
+    const uint64_t nm = pack2(-m, -m);
+    uint64_t p0 = 0, p1 = 0;
 #pragma unroll
     for (int q = 0; q < 16; q += 2) {
         float a0, a1, b0, b1;
@@ -359,15 +360,152 @@ __device__ __forceinline__ void stats_block(const float (&v)[32], uint64_t cc, u
         p0 = fadd2(p0, pack2(ex2(a0), ex2(a1)));
         p1 = fadd2(p1, pack2(ex2(b0), ex2(b1)));
     }
+    return fadd2(p0, p1);
 }
 
 // ===========================================================================
 // pass 1
 // ===========================================================================
+// Epilogue of pass 1 over the CTA's units: offset and sum of each row.  `n`: accumulator buffers
+// consumed so far.  RISE: the second run, which replaces the sums that were out of range.
+template <int NH, bool RISE>
+__device__ __forceinline__ void stats_rows(const TcBatch& bt, Ctl* ctl, uint32_t tmem, uint32_t& n) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int q = (warp - kEpi0) >> 2;       // column quarter: positions 32 q .. +31 of each tile
+    const int sp = warp & 3;                 // TMEM lane quarter
+    const int L = sp * 32 + lane;
+    const uint32_t ta = tmem + ((uint32_t)(sp * 32) << 16) + 32 * q;
+    const float c = bt.sl2e;
+    Unit un = ctl->first;
+    const uint64_t cc = pack2(c, c);
+    float M[NH];                             // per half: offset (log2 domain) and sum of exp2(c z - offset)
+    uint64_t S[NH];
+    bool ok = true;
+    // One tile, one buffer a half: load its 32 columns, hand the buffer back, sum.  PART: `nvalid` of
+    // the columns hold a position.  SELF: the columns are query tokens' own keys, of which row
+    // (token r, head) has those up to r: `nvalid` there, `tok0` of them for the thread's first row
+    // and one more for each token after its own.  FIRST: the chunk's first tile sets the offset to the
+    // largest of its first 8 logits, or to -FLT_MAX where it has none (then the row's first self keys set
+    // it).  RISE (the second run): the largest of all 32, and a logit more than kRaise above the offset
+    // raises it.
+    // (In the first run the largest of 32 costs 3 us of 124, a maximum in every buffer 14, a look at
+    // every buffer's sum 9 to 18.)
+    auto tile = [&](auto part, auto self, auto first, int nvalid, int nh, int tok0) {
+        constexpr bool PART = decltype(part)::value, SELF = decltype(self)::value;
+        constexpr bool FIRST = decltype(first)::value;
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            if (h >= nh) break;
+            const uint32_t buf = n & 3;
+            if (!(ok = wait_bar(&ctl->t_full[buf], (n >> 2) & 1, ctl, bt.err, 5))) break;
+            ++n;
+            tc_fence_after();
+            float v[32];
+            tmem_ld32(ta + buf * 128, v);
+            tmem_wait_ld(v);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->t_empty[buf]);
+            if (PART) {
+                const int nv = SELF ? min(nvalid, tok0 + (h * kRowHalf >> bt.log2g)) : nvalid;
+#pragma unroll
+                for (int e = 0; e < 32; ++e) v[e] = e < nv ? v[e] : -INFINITY;
+            }
+            if (RISE) {
+                const float m = max_tree1(v) * c;
+                if (FIRST) {
+                    M[h] = fmaxf(m, -FLT_MAX);
+                } else if (m > M[h] + kRaise) {
+                    const float f = ex2(M[h] - m);
+                    S[h] = fmul2(S[h], pack2(f, f));
+                    M[h] = m;
+                }
+            } else if (FIRST || (SELF && M[h] == -FLT_MAX)) {
+                const float m = fmax3(fmax3(v[0], v[1], v[2]), fmax3(v[3], v[4], v[5]), fmaxf(v[6], v[7]));
+                M[h] = fmaxf(m * c, -FLT_MAX);
+            }
+            S[h] = fadd2(S[h], stats_block(v, cc, M[h]));
+        }
+    };
+    for (int left = ctl->units; left > 0 && ok;) {
+        // the run of chunks of one group and row chunk (nothing but positions changes in it)
+        const TcSender& sd = bt.s[un.i];
+        const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
+        const int nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0;
+        const int R = sd.R, rows = R - h0 * kRowHalf - L;   // rows: query rows from the thread's first on
+        const int m_self = sd.m_self, tok = (h0 * kRowHalf + L) >> bt.log2g;   // the thread's first row's token
+        const int chunk = sd.chunk1, nc = n_c<1>(sd), len_run = min(left, nc - un.c);
+        int rest = (int)sd.T - un.c * chunk;   // positions from the chunk's first on
+        float2* dst = sd.stats + ((int64_t)un.s * sd.n_chunk1 + 4 * un.c + q) * R + h0 * kRowHalf + L;
+        left -= len_run;
+        un.c += len_run - 1;
+        next_unit<1>(bt, un, nc);
+        for (int k = 0; k < len_run && ok; ++k, rest -= chunk, dst += 4 * (int64_t)R) {
+            const int len = min(chunk, rest);
+#pragma unroll
+            for (int h = 0; h < NH; ++h) { M[h] = -INFINITY; S[h] = 0; }
+            int t0 = 0;
+            constexpr std::false_type no{};
+            constexpr std::true_type yes{};
+            if (len >= kTileRows) {
+                tile(no, no, yes, 32, nh, 0);
+                for (t0 = kTileRows; t0 + kTileRows <= len && ok; t0 += kTileRows) tile(no, no, no, 32, nh, 0);
+                if (t0 < len && ok) tile(yes, no, no, len - t0 - 32 * q, nh, 0);
+            } else {
+                tile(yes, no, yes, len - 32 * q, nh, 0);
+            }
+            if (m_self > 0 && rest <= chunk)   // the query tokens' own keys join the last chunk
+                for (int u0 = 32 * q; u0 - 32 * q < m_self && ok; u0 += kTileRows)
+                    tile(yes, yes, no, m_self - u0, nh, tok + 1 - u0);
+            if (!ok) break;
+            // this warp's partial statistics for the chunk: slot 4 c + q (rows of positions past T
+            // are (-FLT_MAX, 0), which adds nothing); the combine kernel merges all slots
+#pragma unroll
+            for (int h = 0; h < NH; ++h) {
+                if (h >= nh || h * kRowHalf >= rows) break;
+                float s0, s1;
+                unpack2(S[h], s0, s1);
+                // The combine kernel scales sums by powers of two down to 2^-126, below which exp2 is zero, and
+                // the largest of a row's offsets has a sum of at least one.  A large sum's exponent goes into
+                // the offset (what that rounds off, back into the sum), so that what is scaled to zero is nothing.
+                float m = M[h], x = s0 + s1;
+                if (x > 0x1p30f && x <= FLT_MAX) {
+                    const int e = (__float_as_int(x) >> 23) - 127;
+                    const float m1 = m + (float)e;
+                    x = __int_as_float(__float_as_int(x) - (e << 23)) * ex2(m - (m1 - (float)e));
+                    m = m1;
+                }
+                float2* at = dst + h * kRowHalf;
+                if (RISE) {
+                    if (at->y <= FLT_MAX) continue;   // in range in the first run
+                } else if (!(x <= FLT_MAX)) {
+                    const int unit = ctl->units - left - len_run + k;
+                    atomicMin(&ctl->redo_lo, unit);
+                    atomicMax(&ctl->redo_hi, unit);
+                }
+                *at = make_float2(m, x);
+            }
+        }
+    }
+}
+
+// (out of line: the first run keeps its registers)
+template <int NH>
+__device__ __noinline__ void stats_rows_again(const TcBatch& bt, Ctl* ctl, uint32_t tmem, uint32_t n) {
+    stats_rows<NH, true>(bt, ctl, tmem, n);
+}
+
 // Epilogue: thread = TMEM lane = row 128 h + lane of every half h and a quarter of each tile's
 // positions; it keeps the offset and sum of exp2 of its rows over the chunk and writes them as
 // partial (chunk, quarter); the combine kernel merges all partials of a group s.  The two MMA
 // issuers take alternate buffers.
+// A chunk's offset is the largest of its first 8 logits, so a sum is in range unless a later logit
+// lies 127 (log2 domain) above all of those: out of 6e8 normal logits, one does from a standard
+// deviation of 10 (natural units) on.  Then the CTA runs the units from its first to its last such
+// sum again with offsets that rise with the logits, and replaces those sums alone, so that they
+// depend on nothing else in the call: 36 layers, T = 8192, 256 rows take 124 us at standard deviations
+// up to 8, 142 at 10 and 254 from 14 on (recomputing such rows in the combine kernel took 14 ms and
+// more).  Stretches of marked units in place of the one range gain nothing (275 us from 14 on).
 // Bound by the epilogue, whose waits, TMEM loads, exp2 and packed adds take 115 us without the K
 // loads for 36 layers, T = 8192, 256 rows (64 at the rate of exp2 alone); the K loads without the
 // epilogue take 102 (89 at the copy rate).
@@ -380,7 +518,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
     extern __shared__ uint8_t smem_raw[];
     const Smem sm = carve<D, 1>(smem_raw, bt);
     Ctl* ctl = sm.ctl;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
         init_ctl(ctl, bt.paged ? 3 : 2, bt.wait_ns);
         my_units<1>(bt, ctl);
@@ -393,270 +531,202 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
-    const int n_units = ctl->units;
-    Unit un = ctl->first;
     const int stages = bt.stages1;
+    // what the roles carry from the first run over their units to the second
+    int64_t kt = 0;               // producer: K tiles issued
+    uint32_t qn = 0, n = 0;       // Q loads issued or consumed; accumulator buffers filled or consumed
+    int st = 0;                   // ring slot of the next K tile and its phase parity
+    uint32_t ph = 0;
+    for (int run = 0;; ++run) {
+        const int n_units = ctl->units;
+        Unit un = ctl->first;
 
-    if (warp == 0) {
-        // ---------------- TMA producer ----------------
-        if (elect_one()) {
-            int64_t kt = 0, qn = 0;   // K tiles and Q loads issued
-            int st = 0;               // ring slot of the next K tile and its phase parity
-            uint32_t ph = 0;
-            bool ok = true;
-            int nc = 0, l = 0, g = 0, n_self = 0, chunk = 0;
-            int64_t T = 0;
-            const int32_t* pages = nullptr;
-            int32_t n_pages = 0, ps = 0;
-            for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
-                const TcMaps& mp = bt.maps[un.i];
-                if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
-                    const TcSender& sd = bt.s[un.i];
-                    nc = n_c<1>(sd);
-                    chunk = sd.chunk1;
-                    n_self = self_tiles(sd);
-                    pages = sd.pages;
-                    n_pages = sd.n_pages;
-                    ps = sd.page_shift;
-                    T = sd.T;
-                    l = un.s / bt.Hkv;
-                    g = un.s % bt.Hkv;
-                    if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 0))) break;
-                    const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
-                    load_q<D, 1>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0);
-                    ++qn;
-                }
-                const int64_t c0 = (int64_t)un.c * chunk;
-                const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows);
-                const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
-                for (int tile = 0; tile < n_tiles; ++tile) {
-                    const bool self = tile >= nt;
-                    const int32_t row = self ? (tile - nt) * kTileRows : (int32_t)(c0 + tile * kTileRows);
-                    // a tile's block-table entries, all in flight together while its slot is waited for
-                    const int box = ps < 7 ? 1 << ps : kTileRows;
-                    int32_t entry[kTileRows >> kMinPageShift];
-                    if (pages && !self) {
-#pragma unroll
-                        for (int r = 0; r < kTileRows >> kMinPageShift; ++r)
-                            if (r * box < kTileRows && row + r * box < T) entry[r] = __ldg(pages + ((row + r * box) >> ps));
+        if (warp == 0) {
+            // ---------------- TMA producer ----------------
+            if (elect_one()) {
+                bool ok = true;
+                int nc = 0, l = 0, g = 0, n_self = 0, chunk = 0;
+                int64_t T = 0;
+                const int32_t* pages = nullptr;
+                int32_t n_pages = 0, ps = 0;
+                for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
+                    const TcMaps& mp = bt.maps[un.i];
+                    if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
+                        const TcSender& sd = bt.s[un.i];
+                        nc = n_c<1>(sd);
+                        chunk = sd.chunk1;
+                        n_self = self_tiles(sd);
+                        pages = sd.pages;
+                        n_pages = sd.n_pages;
+                        ps = sd.page_shift;
+                        T = sd.T;
+                        l = un.s / bt.Hkv;
+                        g = un.s % bt.Hkv;
+                        if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 0))) break;
+                        const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
+                        load_q<D, 1>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0);
+                        ++qn;
                     }
-                    if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 1))) break;
-                    mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
-                    if (pages && !self) {
-                        // one box a page (or 128 rows of one); a page past T, or outside the pool (recorded), is
-                        // the coordinate past the last page, which reads as zeros
+                    const int64_t c0 = (int64_t)un.c * chunk;
+                    const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows);
+                    const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
+                    for (int tile = 0; tile < n_tiles; ++tile) {
+                        const bool self = tile >= nt;
+                        const int32_t row = self ? (tile - nt) * kTileRows : (int32_t)(c0 + tile * kTileRows);
+                        // a tile's block-table entries, all in flight together while its slot is waited for
+                        const int box = ps < 7 ? 1 << ps : kTileRows;
+                        int32_t entry[kTileRows >> kMinPageShift];
+                        if (pages && !self) {
 #pragma unroll
-                        for (int r = 0; r < kTileRows >> kMinPageShift; ++r) {
-                            if (r * box >= kTileRows) break;
-                            int32_t pg = n_pages;
-                            if (row + r * box < T) {
-                                pg = entry[r];
-                                if (pg < 0 || pg >= n_pages) {
-                                    pg = n_pages;
-                                    atomicOr(bt.err, kErrPageIndex);
-                                }
-                            }
-                            for (int kb = 0; kb < D / 64; ++kb)
-                                tma_load_5d(sm.k + (size_t)st * kTile + (kb * kTileRows + r * box) * 128, &mp.k[0],
-                                            &ctl->k_full[st], 64 * kb, (row + r * box) & ((1 << ps) - 1), pg, g, l);
+                            for (int r = 0; r < kTileRows >> kMinPageShift; ++r)
+                                if (r * box < kTileRows && row + r * box < T) entry[r] = __ldg(pages + ((row + r * box) >> ps));
                         }
-                    } else {
-                        for (int kb = 0; kb < D / 64; ++kb)
-                            tma_load_4d(sm.k + (size_t)st * kTile + kb * kTileRows * 128, &mp.k[self ? 1 : 0],
-                                        &ctl->k_full[st], 64 * kb, row, g, l);
+                        if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 1))) break;
+                        mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
+                        if (pages && !self) {
+                            // one box a page (or 128 rows of one); a page past T, or outside the pool (recorded), is
+                            // the coordinate past the last page, which reads as zeros
+#pragma unroll
+                            for (int r = 0; r < kTileRows >> kMinPageShift; ++r) {
+                                if (r * box >= kTileRows) break;
+                                int32_t pg = n_pages;
+                                if (row + r * box < T) {
+                                    pg = entry[r];
+                                    if (pg < 0 || pg >= n_pages) {
+                                        pg = n_pages;
+                                        atomicOr(bt.err, kErrPageIndex);
+                                    }
+                                }
+                                for (int kb = 0; kb < D / 64; ++kb)
+                                    tma_load_5d(sm.k + (size_t)st * kTile + (kb * kTileRows + r * box) * 128, &mp.k[0],
+                                                &ctl->k_full[st], 64 * kb, (row + r * box) & ((1 << ps) - 1), pg, g, l);
+                            }
+                        } else {
+                            for (int kb = 0; kb < D / 64; ++kb)
+                                tma_load_4d(sm.k + (size_t)st * kTile + kb * kTileRows * 128, &mp.k[self ? 1 : 0],
+                                            &ctl->k_full[st], 64 * kb, row, g, l);
+                        }
+                        ++kt;
+                        if (++st == stages) { st = 0; ph ^= 1u; }
                     }
-                    ++kt;
-                    if (++st == stages) { st = 0; ph ^= 1u; }
                 }
+                // drain: every issued load must land before the CTA exits
+                for (int64_t k = kt - stages > 0 ? kt - stages : 0; k < kt; ++k)
+                    drain_wait(&ctl->k_full[k % stages], (uint32_t)((k / stages) & 1));
+                if (qn > 0) drain_wait(&ctl->q_full, (uint32_t)((qn - 1) & 1));
             }
-            // drain: every issued load must land before the CTA exits
-            for (int64_t k = kt - stages > 0 ? kt - stages : 0; k < kt; ++k)
-                drain_wait(&ctl->k_full[k % stages], (uint32_t)((k / stages) & 1));
-            if (qn > 0) drain_wait(&ctl->q_full, (uint32_t)((qn - 1) & 1));
-        }
-    } else if (warp <= 2) {
-        // ---------------- MMA issuers ----------------
-        if (elect_one()) {
-            const uint32_t me = (uint32_t)warp - 1;
-            uint32_t qn = 0;          // Q loads consumed
-            uint32_t n = 0;           // accumulator buffers filled by both issuers
-            int st = 0;               // ring slot of the next K tile and its phase parity
-            uint32_t ph = 0;
-            bool ok = true;
-            constexpr uint32_t idesc = idesc_bf16_f32(128, 128);
-            const uint64_t qd = smem_desc_sw128(smem_u32(sm.q));
-            const uint32_t hi = (uint32_t)(qd >> 32), q_lo = (uint32_t)qd;
-            const uint32_t k_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.k));
-            const uint32_t q_blk = (uint32_t)bt.rows1 * 128 >> 4;
-            // failure-detection test: wait on a barrier that nothing arrives on, so the bounded
-            // wait gives up, sets the abort flag and every role of this CTA leaves
-            if (bt.stall && blockIdx.x == 0) ok = wait_bar(&ctl->stall, 0, ctl, bt.err, 6);
-            uint32_t nh = 0;
-            int nc = 0, n_self = 0, chunk = 0;
-            int64_t T = 0;
-            for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
-                if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
-                    const TcSender& sd = bt.s[un.i];
-                    nc = n_c<1>(sd);
-                    chunk = sd.chunk1;
-                    n_self = self_tiles(sd);
-                    T = sd.T;
-                    nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - rc_begin(sd.halves, sd.n_rc1, un.rc);
-                    if (u > 0) umma_commit(&ctl->q_empty);
-                    if (!(ok = wait_bar(&ctl->q_full, qn & 1, ctl, bt.err, 2))) break;
-                    ++qn;
-                }
-                const int64_t c0 = (int64_t)un.c * chunk;
-                const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows) +
-                               (un.c + 1 == nc ? n_self : 0);
-                for (int tile = 0; tile < nt; ++tile) {
-                    if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
-                    const uint32_t kt_lo = k_lo + (uint32_t)st * (kTile >> 4);
-                    for (uint32_t h = (n ^ me) & 1; h < nh; h += 2) {   // the tile's buffers n + h of my parity
-                        const uint32_t x = n + h, buf = x & 3;
-                        if (!(ok = wait_bar(&ctl->t_empty[buf], ((x >> 2) & 1) ^ 1, ctl, bt.err, 4))) break;
-                        tc_fence_after();
-                        mma_d<D>(tmem + buf * 128, q_lo + h * (kRowHalf * 128 >> 4), q_blk, kt_lo, kTileRows * 128 >> 4, hi,
-                                 idesc);
-                        umma_commit(&ctl->t_full[buf]);
+        } else if (warp <= 2) {
+            // ---------------- MMA issuers ----------------
+            if (elect_one()) {
+                const uint32_t me = (uint32_t)warp - 1;
+                bool ok = true;
+                constexpr uint32_t idesc = idesc_bf16_f32(128, 128);
+                const uint64_t qd = smem_desc_sw128(smem_u32(sm.q));
+                const uint32_t hi = (uint32_t)(qd >> 32), q_lo = (uint32_t)qd;
+                const uint32_t k_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.k));
+                const uint32_t q_blk = (uint32_t)bt.rows1 * 128 >> 4;
+                // failure-detection test: wait on a barrier that nothing arrives on, so the bounded
+                // wait gives up, sets the abort flag and every role of this CTA leaves
+                if (bt.stall && blockIdx.x == 0 && run == 0) ok = wait_bar(&ctl->stall, 0, ctl, bt.err, 6);
+                uint32_t nh = 0;
+                int nc = 0, n_self = 0, chunk = 0;
+                int64_t T = 0;
+                for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
+                    if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
+                        const TcSender& sd = bt.s[un.i];
+                        nc = n_c<1>(sd);
+                        chunk = sd.chunk1;
+                        n_self = self_tiles(sd);
+                        T = sd.T;
+                        nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - rc_begin(sd.halves, sd.n_rc1, un.rc);
+                        if (u > 0) umma_commit(&ctl->q_empty);
+                        if (!(ok = wait_bar(&ctl->q_full, qn & 1, ctl, bt.err, 2))) break;
+                        ++qn;
                     }
-                    if (!ok) break;
-                    n += nh;
-                    umma_commit(&ctl->k_empty[st]);
-                    if (++st == stages) { st = 0; ph ^= 1u; }
-                }
-            }
-            umma_commit(&ctl->drain[me]);
-            drain_wait(&ctl->drain[me], 0);
-        }
-    } else if (warp < kEpi0) {
-        // ---------------- paged senders: the staged tiles on into the contiguous copy ----------------
-        if (bt.paged && elect_one()) {
-            int st = 0;               // ring slot of the next K tile and its phase parity
-            uint32_t ph = 0;
-            int prev = -1;            // slot of the tile before, whose stores may still read it
-            bool ok = true;
-            int nc = 0, l = 0, g = 0, n_self = 0, chunk = 0;
-            int64_t T = 0;
-            bool store = false;
-            for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
-                if (u == 0 || un.c == 0) {
-                    const TcSender& sd = bt.s[un.i];
-                    nc = n_c<1>(sd);
-                    chunk = sd.chunk1;
-                    n_self = self_tiles(sd);
-                    T = sd.T;
-                    l = un.s / bt.Hkv;
-                    g = un.s % bt.Hkv;
-                    store = sd.pages && un.rc == 0;   // once for all row chunks
-                }
-                const int64_t c0 = (int64_t)un.c * chunk;
-                const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows);
-                const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
-                for (int tile = 0; tile < n_tiles; ++tile) {
-                    if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
-                    if (store && tile < nt)
-                        for (int kb = 0; kb < D / 64; ++kb)
-                            tma_store_4d(&bt.maps[un.i].k[2], sm.k + (size_t)st * kTile + kb * kTileRows * 128, 64 * kb,
-                                         (int32_t)(c0 + tile * kTileRows), g, l);
-                    bulk_commit();
-                    if (prev >= 0) {
-                        bulk_wait_read<1>();
-                        mbar_arrive(&ctl->k_empty[prev]);
+                    const int64_t c0 = (int64_t)un.c * chunk;
+                    const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows) +
+                                   (un.c + 1 == nc ? n_self : 0);
+                    for (int tile = 0; tile < nt; ++tile) {
+                        if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
+                        const uint32_t kt_lo = k_lo + (uint32_t)st * (kTile >> 4);
+                        for (uint32_t h = (n ^ me) & 1; h < nh; h += 2) {   // the tile's buffers n + h of my parity
+                            const uint32_t x = n + h, buf = x & 3;
+                            if (!(ok = wait_bar(&ctl->t_empty[buf], ((x >> 2) & 1) ^ 1, ctl, bt.err, 4))) break;
+                            tc_fence_after();
+                            mma_d<D>(tmem + buf * 128, q_lo + h * (kRowHalf * 128 >> 4), q_blk, kt_lo, kTileRows * 128 >> 4, hi,
+                                     idesc);
+                            umma_commit(&ctl->t_full[buf]);
+                        }
+                        if (!ok) break;
+                        n += nh;
+                        umma_commit(&ctl->k_empty[st]);
+                        if (++st == stages) { st = 0; ph ^= 1u; }
                     }
-                    prev = st;
-                    if (++st == stages) { st = 0; ph ^= 1u; }
                 }
+                umma_commit(&ctl->q_empty);
+                umma_commit(&ctl->drain[me]);
+                drain_wait(&ctl->drain[me], (uint32_t)run);
             }
-            if (prev >= 0) {
-                bulk_wait_read<0>();
-                mbar_arrive(&ctl->k_empty[prev]);
+        } else if (warp < kEpi0) {
+            // ---------------- paged senders: the staged tiles on into the contiguous copy ----------------
+            if (bt.paged && elect_one()) {
+                int prev = -1;            // slot of the tile before, whose stores may still read it
+                bool ok = true;
+                int nc = 0, l = 0, g = 0, n_self = 0, chunk = 0;
+                int64_t T = 0;
+                bool store = false;
+                for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
+                    if (u == 0 || un.c == 0) {
+                        const TcSender& sd = bt.s[un.i];
+                        nc = n_c<1>(sd);
+                        chunk = sd.chunk1;
+                        n_self = self_tiles(sd);
+                        T = sd.T;
+                        l = un.s / bt.Hkv;
+                        g = un.s % bt.Hkv;
+                        store = sd.pages && un.rc == 0 && run == 0;   // once for all row chunks
+                    }
+                    const int64_t c0 = (int64_t)un.c * chunk;
+                    const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows);
+                    const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
+                    for (int tile = 0; tile < n_tiles; ++tile) {
+                        if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
+                        if (store && tile < nt)
+                            for (int kb = 0; kb < D / 64; ++kb)
+                                tma_store_4d(&bt.maps[un.i].k[2], sm.k + (size_t)st * kTile + kb * kTileRows * 128, 64 * kb,
+                                             (int32_t)(c0 + tile * kTileRows), g, l);
+                        bulk_commit();
+                        if (prev >= 0) {
+                            bulk_wait_read<1>();
+                            mbar_arrive(&ctl->k_empty[prev]);
+                        }
+                        prev = st;
+                        if (++st == stages) { st = 0; ph ^= 1u; }
+                    }
+                }
+                if (prev >= 0) {
+                    bulk_wait_read<0>();
+                    mbar_arrive(&ctl->k_empty[prev]);
+                }
+                bulk_wait<0>();
             }
-            bulk_wait<0>();
+        } else {
+            // ---------------- epilogue ----------------
+            if (run == 0) stats_rows<NH, false>(bt, ctl, tmem, n);
+            else stats_rows_again<NH>(bt, ctl, tmem, n);
         }
-    } else {
-        // ---------------- epilogue: running max / sum per row ----------------
-        const int q = (warp - kEpi0) >> 2;       // column quarter: positions 32 q .. +31 of each tile
-        const int sp = warp & 3;                 // TMEM lane quarter
-        const int L = sp * 32 + lane;
-        const uint32_t ta = tmem + ((uint32_t)(sp * 32) << 16) + 32 * q;
-        const float c = bt.sl2e;
-        const uint64_t cc = pack2(c, c);
-        uint32_t n = 0;                          // accumulator buffers consumed
-        float M[NH];                             // per half: offset (log2 domain) and sum of exp2(c z - offset)
-        uint64_t S[NH];
-        bool ok = true;
-        // One tile, one buffer a half: load its 32 columns, hand the buffer back, sum.  PART: `nvalid` of
-        // the columns hold a position.  SELF: the columns are query tokens' own keys, of which row
-        // (token r, head) has those up to r: `nvalid` there, `tok0` of them for the thread's first row
-        // and one more for each token after its own.  The first tile of a chunk sets the offset to its
-        // first logit, or to -FLT_MAX where it has none (then the first self key of the row sets it).
-        auto tile = [&](auto part, auto self, int nvalid, bool first, int nh, int tok0) {
-            constexpr bool PART = decltype(part)::value, SELF = decltype(self)::value;
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                if (h >= nh) break;
-                const uint32_t buf = n & 3;
-                if (!(ok = wait_bar(&ctl->t_full[buf], (n >> 2) & 1, ctl, bt.err, 5))) break;
-                ++n;
-                tc_fence_after();
-                float v[32];
-                tmem_ld32(ta + buf * 128, v);
-                tmem_wait_ld(v);
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->t_empty[buf]);
-                if (PART) {
-                    const int nv = SELF ? min(nvalid, tok0 + (h * kRowHalf >> bt.log2g)) : nvalid;
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) v[e] = e < nv ? v[e] : -INFINITY;
-                }
-                if (first || (SELF && M[h] == -FLT_MAX)) M[h] = fmaxf(v[0] * c, -FLT_MAX);
-                const uint64_t nm = pack2(-M[h], -M[h]);
-                uint64_t p0 = 0, p1 = 0;
-                stats_block(v, cc, nm, p0, p1);
-                S[h] = fadd2(S[h], fadd2(p0, p1));
-            }
-        };
-        for (int left = n_units; left > 0 && ok;) {
-            // the run of chunks of one group and row chunk (nothing but positions changes in it)
-            const TcSender& sd = bt.s[un.i];
-            const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
-            const int nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0;
-            const int R = sd.R, rows = R - h0 * kRowHalf - L;   // rows: query rows from the thread's first on
-            const int m_self = sd.m_self, tok = (h0 * kRowHalf + L) >> bt.log2g;   // the thread's first row's token
-            const int chunk = sd.chunk1, nc = n_c<1>(sd), run = min(left, nc - un.c);
-            int rest = (int)sd.T - un.c * chunk;   // positions from the chunk's first on
-            float2* dst = sd.stats + ((int64_t)un.s * sd.n_chunk1 + 4 * un.c + q) * R + h0 * kRowHalf + L;
-            left -= run;
-            un.c += run - 1;
-            next_unit<1>(bt, un, nc);
-            for (int k = 0; k < run && ok; ++k, rest -= chunk, dst += 4 * (int64_t)R) {
-                const int len = min(chunk, rest);
-#pragma unroll
-                for (int h = 0; h < NH; ++h) { M[h] = -INFINITY; S[h] = 0; }
-                int t0 = 0;
-                constexpr std::false_type no{};
-                constexpr std::true_type yes{};
-                for (; t0 + kTileRows <= len && ok; t0 += kTileRows) tile(no, no, 32, t0 == 0, nh, 0);
-                if (t0 < len && ok) tile(yes, no, len - t0 - 32 * q, t0 == 0, nh, 0);
-                if (m_self > 0 && rest <= chunk)   // the query tokens' own keys join the last chunk
-                    for (int u0 = 32 * q; u0 - 32 * q < m_self && ok; u0 += kTileRows)
-                        tile(yes, yes, m_self - u0, false, nh, tok + 1 - u0);
-                if (!ok) break;
-                // this warp's partial statistics for the chunk: slot 4 c + q (rows of positions past T
-                // are (-FLT_MAX, 0), which adds nothing); the combine kernel merges all slots
-#pragma unroll
-                for (int h = 0; h < NH; ++h) {
-                    float s0, s1;
-                    unpack2(S[h], s0, s1);
-                    if (h < nh && h * kRowHalf < rows) dst[h * kRowHalf] = make_float2(M[h], s0 + s1);
-                }
-            }
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        if (run == 1 || ctl->redo_hi < 0 || ctl->abort) break;
+        if (threadIdx.x == 0) {
+            Unit f = ctl->first;
+            for (int u = 0; u < ctl->redo_lo; ++u) next_unit<1>(bt, f, n_c<1>(bt.s[f.i]));
+            ctl->first = f;
+            ctl->units = ctl->redo_hi - ctl->redo_lo + 1;
         }
+        __syncthreads();
     }
-    tc_fence_before();
-    __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, kTmemCols);
 }
 

@@ -297,9 +297,8 @@ def test_results_do_not_depend_on_the_score_sms():
 @pytest.mark.parametrize("kernel", [1, 2], ids=["mma_sync", "tcgen05"])
 @pytest.mark.parametrize("scale", [70.0, 150.0], ids=["large_finite", "overflowing"])
 def test_extreme_logit_rows(kernel, scale):
-    """One query row meets keys far above the rest of its chunk: c*z - m about 100 log2 units stays
-    in fp32 range on the fast path, about 210 overflows pass 1's exp2 and the combine kernel
-    recomputes that row's statistics from Q and K.  Scores must still match the oracle."""
+    """One query row meets keys far above the rest of its chunk: about 100 log2 units, within the
+    range of exp2 in fp32, and about 210, beyond it.  Scores must still match the oracle."""
     w = synth.custom_workload(synth.Shape(2, 8, 2, 128), [700], 8, seed=77, n_planted_spans=2)
     s = w.senders[0]
     K, V, Q = s.K.clone(), s.V, w.queries[0]
