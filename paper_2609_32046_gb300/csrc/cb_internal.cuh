@@ -102,7 +102,7 @@ struct ScoreBatch {
     StageTimer* timer;        // host-side; null unless stage timing is enabled
     float2* stats;            // pass-1 partial (max, sum) in log2 domain
     float* offs;              // per-row log2 offsets (max + log2(sum) + log2(G))
-    uint16_t* ext;            // tcgen05 passes: -offset / scale_log2e per row as three bf16 terms
+    uint16_t* ext;            // tcgen05 passes: (centre - offset) / scale_log2e per row as three bf16 terms
                               // (hi, mid, lo, then 13 zeros; -1e30 on padding rows), else null
     const uint16_t* ones;     // tcgen05 passes: [128][16] bf16, columns 0-2 = 1, the rest 0
     float* part;              // per-group partials: sums over tokens of b and of Pool(b)^p
@@ -130,6 +130,18 @@ struct DepageBatch {
     DepageSender s[kMaxDepage];
 };
 
+// A whole number near the offset (log2 domain) that rows of a sender of T positions usually have:
+// the tcgen05 pass 2 adds the offset less this inside the contraction, whose sums are truncated
+// at an ulp of their largest term, and subtracts this in 32 bits.  With the whole offset inside,
+// that ulp is 2^-17 for T = 8192 and the logits of all rows are off by half of it, one way; with
+// nearly all of it outside (0 in place of 3) rows of one large weight are off by as much.  Errors of
+// scores against 64 bits: 36 layers, T = 8192, 4.0e-7 -> 1.9e-7; d = 64, 24 layers, T = 7001, 2.9e-7 ->
+// 2.1e-7 (mma.sync passes 2.6e-7).
+__host__ __device__ inline int offset_centre(int64_t T, int G) {
+    int n = (G == 4 ? 2 : G - 1) - 3;
+    for (int64_t t = T; t > 1; t >>= 1) ++n;
+    return n;
+}
 constexpr int kExtCols = 16;   // one bf16 K-step: the extra contraction column block of pass 2
 
 // Query rows padded to the 128-row granule of the tcgen05 passes.

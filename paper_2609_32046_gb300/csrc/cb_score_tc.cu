@@ -15,7 +15,7 @@
 //               the sum of exp2 over a chunk of positions.  The query tokens' own keys, where a
 //               call has them, are further tiles of the last chunk under a causal mask.
 //   k_accum_tc  pass 2, D = K_tile Q_s^T (+ one more K-step of ones x the rows' offset terms,
-//               so TMEM holds z - offset / scale): TMEM lane = position, column = row (r, h).
+//               so TMEM holds z - (offset - centre) / scale, centre a whole number): TMEM lane = position, column = row (r, h).
 //               A block of positions is four tiles: tile j holds every fourth position from j on,
 //               so a thread owns four neighbouring positions, one of each tile.  exp2 of its
 //               logits (a / G), the head mean b and the sums over tokens stay in registers; Pool
@@ -775,15 +775,15 @@ __device__ __forceinline__ float sum4(const float* e) {
     return p + q;
 }
 
-// Head sums of C / G tokens from their C columns: a / G = exp2(c z - offset) per column, summed
-// over each token's G heads, as pairs of tokens (2 i, 2 i + 1).
+// Head sums of C / G tokens from their C columns: a / G = exp2(c D - centre) per column, `nc` minus
+// the centre, summed over each token's G heads, as pairs of tokens (2 i, 2 i + 1).
 template <int G, int C>
-__device__ __forceinline__ void head_sums(const float (&v)[C], uint64_t cc, uint64_t* b) {
+__device__ __forceinline__ void head_sums(const float (&v)[C], uint64_t cc, uint64_t nc, uint64_t* b) {
     float e[C];
 #pragma unroll
     for (int q = 0; q < C / 2; ++q) {
         float a0, a1;
-        unpack2(fmul2(pack2(v[2 * q], v[2 * q + 1]), cc), a0, a1);
+        unpack2(ffma2(pack2(v[2 * q], v[2 * q + 1]), cc, nc), a0, a1);
         e[2 * q] = ex2(a0);
         e[2 * q + 1] = ex2(a1);
     }
@@ -927,8 +927,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                         tc_fence_after();
                         mma_d<D>(tmem + j * 128, k_lo + (uint32_t)(st0 + j) * (kTile >> 4), kTileRows * 128 >> 4,
                                  q_lo + h * (kRowHalf * 128 >> 4), q_blk, hi, idesc);
-                        // one more K-step: ones (positions) x offset terms (rows) adds -offset / scale to
-                        // every logit, so the epilogue needs only exp2(scale * D)
+                        // one more K-step: ones (positions) x offset terms (rows) adds (centre - offset) / scale
+                        // to every logit, so the epilogue needs only exp2(scale * D - centre)
                         umma_bf16(tmem + j * 128, ones_desc, desc64(ext_lo + h * (kRowHalf * 32 >> 4), ext_hi), idesc, 1u);
                         umma_commit(&ctl->t_full[j]);
                         if (h == nh - 1) umma_commit(&ctl->k_empty[st0 + j]);
@@ -953,6 +953,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
             const int nh = rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0;
             const int R = sd.R - h0 * kRowHalf;  // query rows from the row chunk's first on
             const int T = (int)sd.T, nc = sd.n_blk2, run = min(left, nc - un.c);
+            const float cen = (float)offset_centre(T, G);
+            const uint64_t ncen = pack2(-cen, -cen);
             int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
             left -= run;
             un.c += run - 1;
@@ -1013,7 +1015,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                                     if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
                                 }
                                 uint64_t* bx = bc[j] + x / (2 * G);
-                                head_sums<G>(v, cc, bx);
+                                head_sums<G>(v, cc, ncen, bx);
                                 if (EDGE) {
                                     const bool valid = pos + j >= 0 && pos + j < T;
 #pragma unroll
