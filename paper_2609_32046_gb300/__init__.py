@@ -199,12 +199,20 @@ class Chain:
             raise ValueError("hop of %d positions exceeds the chain capacity %d" % (b, self.capacity))
         return self.K[self.cur][:, :, a:b], self.V[self.cur][:, :, a:b]
 
-    def _append(self, K_new, V_new):
-        """K_new and V_new into the current buffer after the message: one launch of the compaction
+    def _append(self, K_new, V_new, stream=None):
+        """K_new and V_new, as the current stream has them, into the current buffer after the message: one launch of the compaction
         kernel, which moves 16-byte pieces of every row of both at 0.96 of the copy bandwidth (two
-        strided tensor copies of 8-byte words reach 0.8), where it takes the tensors; else two copies."""
+        strided tensor copies of 8-byte words reach 0.8), where it takes the tensors; else two copies.
+        `stream` is that of the hops: the copies wait for it (an earlier hop may still write or read the
+        buffer) and it waits for them."""
         import torch
         k, v = self.new_slot(K_new.shape[2])
+        cur = torch.cuda.current_stream(k.device) if k.is_cuda else None
+        if isinstance(stream, int):
+            stream = torch.cuda.ExternalStream(stream, device=k.device)
+        apart = stream is not None and cur is not None and stream.cuda_stream != cur.cuda_stream
+        if apart:
+            cur.wait_stream(stream)
         st, T = K_new.stride(), int(K_new.shape[2])
         own = {x.untyped_storage().data_ptr() for x in (*self.K, *self.V)}
         row = k.shape[3]
@@ -218,6 +226,8 @@ class Chain:
         else:
             _copy_rows(k, K_new)
             _copy_rows(v, V_new)
+        if apart:
+            stream.wait_stream(cur)
 
     def hop(self, Q, K_new=None, V_new=None, T_new: Optional[int] = None, stream=None) -> dict:
         """One hop: K_new / V_new (or T_new positions already written through new_slot) join the
@@ -225,7 +235,7 @@ class Chain:
         import torch
         if K_new is not None:
             T_new = int(K_new.shape[2])
-            self._append(K_new, V_new)
+            self._append(K_new, V_new, stream)
         T_old, T = self.T_old, self.T_old + int(T_new)
         c = self.cb.cfg
         B = chain_budget(T_old, T_new, self.keep, self.mode, self.B_max)

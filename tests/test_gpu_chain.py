@@ -82,6 +82,41 @@ def test_new_rows_join_the_message(form):
         assert torch.equal(r["K"][:, :, a:].float(), K.float()) and torch.equal(r["V"][:, :, a:].float(), V.float())
 
 
+@pytest.mark.parametrize("form", ["contiguous", "float32"])
+@pytest.mark.parametrize("handle", [False, True], ids=["stream", "handle"])
+def test_hops_on_a_stream_of_their_own(form, handle):
+    """hop(stream=...) with new rows that the current stream is still making, while earlier hops still
+    run on their stream: the same as on one stream."""
+    nL, Hkv, T, d, n = 4, 2, 300, 64, 4
+    g = torch.Generator(device="cuda").manual_seed(2)
+    draw = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    Q, KV = draw(nL, 4, 4, d), [(draw(nL, Hkv, T, d), draw(nL, Hkv, T, d)) for _ in range(n)]
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    results = []
+    for stream in (None, side):
+        c = make_cb(synth.Shape(nL, 4, Hkv, d), n * T, 4, 1)
+        chain, out = cb.Chain(c, n * T, keep=0.5, device="cuda"), []
+        torch.cuda.synchronize()
+        for K, V in KV:
+            if stream is not None:
+                with torch.cuda.stream(stream):
+                    torch.cuda._sleep(2_000_000)          # the earlier hops are not done
+                torch.cuda._sleep(4_000_000)              # nor are the new rows
+            K, V = K + 0, V + 0
+            if form == "float32":
+                K, V = K.float(), V.float()
+            r = chain.hop(Q, K, V, stream=stream.cuda_stream if handle and stream is not None else stream)
+            out.append((r["scores"], r["idx"]))
+        torch.cuda.synchronize()
+        c.sync_status(stream)
+        out.append((r["message_K"].clone(), r["message_V"].clone()))
+        results.append(out)
+    for a, b in zip(*results):
+        for x, y in zip(a, b):
+            assert torch.equal(x, y)
+
+
 def test_chain_rejects_overflow():
     shape = (1, 4, 2, 128)
     c = make_cb(synth.Shape(*shape), 200, 4, 1)
