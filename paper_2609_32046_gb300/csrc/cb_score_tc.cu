@@ -79,15 +79,15 @@ constexpr uint32_t kPollNs = 1000000u;           // longest suspension of one po
 constexpr int kMaxTcSenders = 32;         // their tensor maps fill most of the 32,764 bytes of kernel parameters
 
 struct TcMaps {
-    CUtensorMap k[5];     // pass 1: k[0] = 4D {d, T, Hkv, nL}, box {64, 128, 1, 1}; k[1] the same over the
+    CUtensorMap k[3];     // pass 1: k[0] = 4D {d, T, Hkv, nL}, box {64, 128, 1, 1}; k[1] the same over the
                           // query tokens' own keys {d, m, Hkv, nL} (senders that have them).  Of a paged
                           // sender k[0] = 5D {d, rows of a page, pages, Hkv, nL}, box {64, min(rows, 128), 1, 1, 1},
                           // and k[2] = the copy, 4D like a strided sender's.
-                          // pass 2: k[4] = 5D {d, T / 4, 4, Hkv, nL} (position 4 i + j at (i, j)), box
-                          // {64, 32, 1, 1, 1}; k[j] = 4D positions j, j + 4, ... with every one of them (the
-                          // 5D tensor lacks the last T mod 4), box {64, 32, 1, 1}
+                          // pass 2: k[0] = 5D {d, T / 4, 4, Hkv, nL} (position 4 i + j at (i, j)), box
+                          // {64, 32, 1, 1, 1}; k[1] = 4D as in pass 1 with every fourth of 128 positions in its box (the
+                          // 5D tensor lacks the last T mod 4 positions), k[2] = E, the offset terms, 3D
+                          // {16, R_pad, nS}, box {16, 128, 1}, 32-byte swizzle
     CUtensorMap q;        // 4D {d, Hq, m, nL}, box {64, G, 128 / G, 1}: 128 rows
-    CUtensorMap e;        // pass 2: 3D {16, R_pad, nS} offset terms, box {16, 128, 1}, 32-byte swizzle
 };
 
 struct TcSender {
@@ -320,7 +320,7 @@ __device__ __forceinline__ void load_q(const TcBatch& bt, const TcMaps& mp, cons
     mbar_arrive_expect_tx(&sm.ctl->q_full, (uint32_t)nh * kRowHalf * (D * 2 + (PASS == 2 ? 32 : 0)));
     for (int h = 0; h < nh; ++h) {
         if (PASS == 2)
-            tma_load_3d(sm.ext + (size_t)h * kRowHalf * 32, &mp.e, &sm.ctl->q_full, 0, (h0 + h) * kRowHalf, s);
+            tma_load_3d(sm.ext + (size_t)h * kRowHalf * 32, &mp.k[2], &sm.ctl->q_full, 0, (h0 + h) * kRowHalf, s);
         for (int kb = 0; kb < D / 64; ++kb)
             tma_load_4d(sm.q + ((size_t)kb * rows + h * kRowHalf) * 128, &mp.q, &sm.ctl->q_full, 64 * kb, g * bt.G,
                         (h0 + h) * kRowHalf / bt.G, l);
@@ -863,8 +863,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                 }
                 const int32_t t0 = un.c * kOut2 - kMargin;
                 // the 5D map serves every tile (a change of map costs the TMA unit time: 150 against
-                // 115 us for the loads of this pass with a map a tile); the maps of the single tiles
-                // are for a last block that ends on one of the last T mod 4 positions
+                // 115 us for the loads of this pass with a map a tile); a last block that ends on one of the last
+                // T mod 4 positions takes them through the other map, at half the rate
                 const int32_t i0 = t0 / 4;
                 const bool whole = t0 + kOut2 + 2 * kMargin <= T / 4 * 4 || T % 4 == 0;
                 for (int j = 0; j < 4; ++j) {
@@ -878,13 +878,13 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                         for (int w = 0; w < 4; ++w)
 #pragma unroll
                             for (int kb = 0; kb < D / 64; ++kb)
-                                tma_load_5d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[4], &ctl->k_full[st], 64 * kb,
+                                tma_load_5d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[0], &ctl->k_full[st], 64 * kb,
                                             i0 + kOutW / 4 * w, j, g, l);
                     } else {
                         for (int w = 0; w < 4; ++w)
                             for (int kb = 0; kb < D / 64; ++kb)
-                                tma_load_4d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[j], &ctl->k_full[st], 64 * kb,
-                                            i0 + kOutW / 4 * w, g, l);
+                                tma_load_4d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[1], &ctl->k_full[st], 64 * kb,
+                                            t0 + kOutW * w + j, g, l);
                     }
                     ++kt;
                     if (++st == slots) { st = 0; ph ^= 1u; }
@@ -1126,12 +1126,13 @@ PFN_cuTensorMapEncodeTiled_v12000 encoder() {
     return g_encode;
 }
 
-// bf16 tensor map of `rank` dimensions (innermost first); strides in bytes of dims 1..rank-1.
+// bf16 tensor map of `rank` dimensions (innermost first); strides in bytes of dims 1..rank-1; of
+// dimension 1 the box takes every step-th element.
 bool encode_nd(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides_bytes,
-               const cuuint32_t* box, CUtensorMapSwizzle swizzle) {
+               const cuuint32_t* box, CUtensorMapSwizzle swizzle, cuuint32_t step = 1) {
     auto fn = encoder();
     if (!fn || !base) return false;
-    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    const cuuint32_t es[5] = {1, step, 1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides_bytes, box,
               es, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -1361,21 +1362,14 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             const cuuint64_t ed[3] = {(cuuint64_t)kExtCols, rpad, (cuuint64_t)nS};
             const cuuint64_t es[2] = {(cuuint64_t)kExtCols * 2, rpad * kExtCols * 2};
             const cuuint32_t ebox[3] = {(cuuint32_t)kExtCols, kRowHalf, 1};
-            // positions (i, j) = 4 i + j of whole groups of four; and per j every fourth position from j on,
-            // ceil((T - j) / 4) of them (a sender of fewer than four positions has none in its last tiles:
-            // any valid row, masked like all past T)
+            // positions (i, j) = 4 i + j of whole groups of four (a sender of fewer than four positions has
+            // none: one row of any, which no block loads), and every fourth position up to the last
             const cuuint64_t k5d[5] = {kd[0], (cuuint64_t)(s.T / 4 > 0 ? s.T / 4 : 1), (cuuint64_t)(s.T < 4 ? s.T : 4),
                                        kd[2], kd[3]};
             const cuuint64_t k5s[4] = {4 * ks[0], ks[0], ks[1], ks[2]};
             const cuuint32_t k5box[5] = {64, 32, 1, 1, 1};
-            bool ok4 = encode_nd(&mp2.k[4], kp, 5, k5d, k5s, k5box, CU_TENSOR_MAP_SWIZZLE_128B);
-            for (int j = 0; j < 4 && s.T % 4 != 0; ++j) {
-                const int64_t first = j < s.T ? j : 0;
-                const cuuint64_t k4d[4] = {kd[0], (cuuint64_t)((s.T - first + 3) / 4), kd[2], kd[3]};
-                const cuuint64_t k4s[3] = {4 * ks[0], ks[1], ks[2]};
-                const cuuint32_t k4box[4] = {64, 32, 1, 1};
-                ok4 = ok4 && encode_4d(&mp2.k[j], kp + first * kpos, k4d, k4s, k4box);
-            }
+            bool ok4 = encode_nd(&mp2.k[0], kp, 5, k5d, k5s, k5box, CU_TENSOR_MAP_SWIZZLE_128B);
+            if (s.T % 4 != 0) ok4 = ok4 && encode_nd(&mp2.k[1], kp, 4, kd, ks, kbox, CU_TENSOR_MAP_SWIZZLE_128B, 4);
             bool ok1 = encode_4d(&mp.k[fused ? 2 : 0], kp, kd, ks, kbox);
             if (fused) {
                 const cuuint64_t rows = (cuuint64_t)1 << s.pm.shift;
@@ -1386,7 +1380,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
                 ok1 = ok1 && encode_nd(&mp.k[0], s.k, 5, pd, pst, pbox, CU_TENSOR_MAP_SWIZZLE_128B);
             }
             if (!ok1 || !ok4 || !encode_4d(&mp.q, s.q, qd, qs, qbox) || !b.ext ||
-                !encode_nd(&mp2.e, b.ext + s.ext_off, 3, ed, es, ebox, CU_TENSOR_MAP_SWIZZLE_32B)) {
+                !encode_nd(&mp2.k[2], b.ext + s.ext_off, 3, ed, es, ebox, CU_TENSOR_MAP_SWIZZLE_32B)) {
                 return cudaErrorNotSupported;
             }
             mp2.q = mp.q;
