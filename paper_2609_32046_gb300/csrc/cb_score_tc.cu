@@ -86,8 +86,8 @@ struct TcMaps {
                           // pass 2: k[0] = 5D {d, T / 4, 4, Hkv, nL} (position 4 i + j at (i, j)), box
                           // {64, 32, 1, 1, 1}; k[1] = 4D as in pass 1 with every fourth of 128 positions in its box (the
                           // 5D tensor lacks the last T mod 4 positions), k[2] = E, the offset terms, 3D
-                          // {16, R_pad, nS}, box {16, 128, 1}, 32-byte swizzle
-    CUtensorMap q;        // 4D {d, Hq, m, nL}, box {64, G, 128 / G, 1}: 128 rows
+                          // {16, R_pad, nS}, box {16, q_rows, 1}, 32-byte swizzle
+    CUtensorMap q;        // 4D {d, Hq, m, nL}, box {64, G, q_rows / G, 1}
 };
 
 struct TcSender {
@@ -95,6 +95,7 @@ struct TcSender {
     float* part;          // this sender's pass-2 partials [n_rc2][2][nS][T_pad]
     int64_t T, T_pad;
     int32_t R, halves;    // m * G query rows; 128-row halves of them
+    int32_t q_rows;       // rows loaded of a half: 128, or R rounded up to 32 where there is one half
     int32_t n_chunk1;     // pass-1 partial slots: four per chunk of positions
     int32_t n_blk2;       // pass-2 blocks of positions
     int32_t n_rc1, n_rc2; // row chunks of each pass
@@ -312,12 +313,14 @@ __device__ __forceinline__ void init_ctl(Ctl* ctl, int k_releasers, uint64_t wai
 }
 
 // Producer: the 128-row halves [h0, h0 + nh) of group s's Q (s = l * Hkv + g) into the Q region
-// (column blocks of `rows` rows).  Pass 2 also brings the rows' offset terms.
+// (column blocks of `rows` rows).  Pass 2 also brings the rows' offset terms.  Rows past the loaded ones
+// of a half hold anything: pass 1 writes nothing of theirs, pass 2's MMA does not read them.
 template <int D, int PASS>
-__device__ __forceinline__ void load_q(const TcBatch& bt, const TcMaps& mp, const Smem& sm, int s, int h0, int nh) {
+__device__ __forceinline__ void load_q(const TcBatch& bt, const TcMaps& mp, const Smem& sm, int s, int h0, int nh,
+                                       int q_rows) {
     const int l = s / bt.Hkv, g = s % bt.Hkv;
     const int rows = PASS == 1 ? bt.rows1 : bt.rows2;
-    mbar_arrive_expect_tx(&sm.ctl->q_full, (uint32_t)nh * kRowHalf * (D * 2 + (PASS == 2 ? 32 : 0)));
+    mbar_arrive_expect_tx(&sm.ctl->q_full, (uint32_t)(nh * q_rows) * (D * 2 + (PASS == 2 ? 32 : 0)));
     for (int h = 0; h < nh; ++h) {
         if (PASS == 2)
             tma_load_3d(sm.ext + (size_t)h * kRowHalf * 32, &mp.k[2], &sm.ctl->q_full, 0, (h0 + h) * kRowHalf, s);
@@ -564,7 +567,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                         g = un.s % bt.Hkv;
                         if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 0))) break;
                         const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
-                        load_q<D, 1>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0);
+                        load_q<D, 1>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0, sd.q_rows);
                         ++qn;
                     }
                     const int64_t c0 = (int64_t)un.c * chunk;
@@ -858,7 +861,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                     g = un.s % bt.Hkv;
                     if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 8))) break;
                     const int h0 = rc_begin(sd.halves, sd.n_rc2, un.rc);
-                    load_q<D, 2>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0);
+                    load_q<D, 2>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0, sd.q_rows);
                     ++qn;
                 }
                 const int32_t t0 = un.c * kOut2 - kMargin;
@@ -911,28 +914,33 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
             const uint32_t q_blk = (uint32_t)bt.rows2 * 128 >> 4;
             constexpr uint32_t idesc = idesc_bf16_f32(128, 128);
             int nc = 0, nh = 0;
+            uint32_t id_last = idesc;    // of the row chunk's last half: columns up to the last query row's 32
             for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
                 if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
                     const TcSender& sd = bt.s[un.i];
                     nc = sd.n_blk2;
-                    nh = rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - rc_begin(sd.halves, sd.n_rc2, un.rc);
+                    const int h1 = rc_begin(sd.halves, sd.n_rc2, un.rc + 1);
+                    nh = h1 - rc_begin(sd.halves, sd.n_rc2, un.rc);
+                    id_last = idesc_bf16_f32(128, min(kRowHalf, (sd.R - (h1 - 1) * kRowHalf + 31) & ~31));
                     if (u > 0) umma_commit(&ctl->q_empty);
                     if (!(ok = wait_bar(&ctl->q_full, qn & 1, ctl, bt.err, 10))) break;
                     ++qn;
                 }
-                for (int h = 0; h < nh && ok; ++h, ++n)
+                for (int h = 0; h < nh && ok; ++h, ++n) {
+                    const uint32_t id = h == nh - 1 ? id_last : idesc;
                     for (int j = me; j < 4; j += 2) {
                         if (h == 0 && !(ok = wait_bar(&ctl->k_full[st0 + j], ph, ctl, bt.err, 11))) break;
                         if (!(ok = wait_bar(&ctl->t_empty[j], (n & 1) ^ 1, ctl, bt.err, 12))) break;
                         tc_fence_after();
                         mma_d<D>(tmem + j * 128, k_lo + (uint32_t)(st0 + j) * (kTile >> 4), kTileRows * 128 >> 4,
-                                 q_lo + h * (kRowHalf * 128 >> 4), q_blk, hi, idesc);
+                                 q_lo + h * (kRowHalf * 128 >> 4), q_blk, hi, id);
                         // one more K-step: ones (positions) x offset terms (rows) adds (centre - offset) / scale
                         // to every logit, so the epilogue needs only exp2(scale * D - centre)
-                        umma_bf16(tmem + j * 128, ones_desc, desc64(ext_lo + h * (kRowHalf * 32 >> 4), ext_hi), idesc, 1u);
+                        umma_bf16(tmem + j * 128, ones_desc, desc64(ext_lo + h * (kRowHalf * 32 >> 4), ext_hi), id, 1u);
                         umma_commit(&ctl->t_full[j]);
                         if (h == nh - 1) umma_commit(&ctl->k_empty[st0 + j]);
                     }
+                }
                 st0 += 4;
                 if (st0 == slots) { st0 = 0; ph ^= 1u; }
             }
@@ -1336,6 +1344,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             d.m_self = s.kself ? s.m : 0;
             d.R = s.m * G;
             d.halves = (d.R + kRowHalf - 1) / kRowHalf;
+            d.q_rows = d.halves > 1 ? kRowHalf : (d.R + 31) & ~31;
             d.chunk1 = stats_chunk(s.T, nS);
             d.n_chunk1 = (int32_t)(4 * ((s.T + d.chunk1 - 1) / d.chunk1));   // one partial per (chunk, column quarter)
             d.n_blk2 = (int32_t)((s.T + kOut2 - 1) / kOut2);
@@ -1356,12 +1365,12 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             const cuuint32_t kbox[4] = {64, kTileRows, 1, 1};
             const cuuint64_t qd[4] = {(cuuint64_t)d_head, (cuuint64_t)b.n_q_heads, (cuuint64_t)s.m, (cuuint64_t)b.n_layers};
             const cuuint64_t qs[3] = {(cuuint64_t)s.qs_h * 2, (cuuint64_t)s.qs_t * 2, (cuuint64_t)s.qs_l * 2};
-            const cuuint32_t qbox[4] = {64, (cuuint32_t)G, (cuuint32_t)(kRowHalf / G), 1};
+            const cuuint32_t qbox[4] = {64, (cuuint32_t)G, (cuuint32_t)(d.q_rows / G), 1};
             // offset terms [nS][rows padded to 128][16] written by the combine kernel
             const cuuint64_t rpad = (cuuint64_t)d.halves * kRowHalf;
             const cuuint64_t ed[3] = {(cuuint64_t)kExtCols, rpad, (cuuint64_t)nS};
             const cuuint64_t es[2] = {(cuuint64_t)kExtCols * 2, rpad * kExtCols * 2};
-            const cuuint32_t ebox[3] = {(cuuint32_t)kExtCols, kRowHalf, 1};
+            const cuuint32_t ebox[3] = {(cuuint32_t)kExtCols, (cuuint32_t)d.q_rows, 1};
             // positions (i, j) = 4 i + j of whole groups of four (a sender of fewer than four positions has
             // none: one row of any, which no block loads), and every fourth position up to the last
             const cuuint64_t k5d[5] = {kd[0], (cuuint64_t)(s.T / 4 > 0 ? s.T / 4 : 1), (cuuint64_t)(s.T < 4 ? s.T : 4),
