@@ -22,6 +22,8 @@ LIB_NAME = "libcacheback.so"
 LIB_PATH = os.path.join(PKG, LIB_NAME)
 SOURCES = ["cb_api.cu", "cb_score.cu", "cb_score_tc.cu", "cb_select.cu", "cb_compact.cu", "cb_gather.cu", "cb_rope.cu",
            "cb_depage.cu"]
+# files compiled in several parts at the same time: a macro and its values
+PARTS = {"cb_score_tc.cu": ("CB_TC_PART", (0, 64, 128))}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
                      "-I", INCLUDE, "-I", CSRC]
@@ -48,9 +50,20 @@ def up_to_date() -> bool:
     return all(os.path.getmtime(p) <= t for p in _deps())
 
 
-def _compile(src: str, verbose: bool) -> str:
-    obj = os.path.join(BUILD_DIR, os.path.splitext(src)[0] + ".o")
-    cmd = [nvcc(), *NVCC_FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+def _units() -> list:
+    """(source, object name, extra flags) of every compilation."""
+    out = []
+    for src in SOURCES:
+        stem = os.path.splitext(src)[0]
+        macro, values = PARTS.get(src, (None, ()))
+        out += [(src, "%s_%d" % (stem, v), ["-D%s=%d" % (macro, v)]) for v in values] or [(src, stem, [])]
+    return out
+
+
+def _compile(unit: tuple, verbose: bool) -> str:
+    src, stem, flags = unit
+    obj = os.path.join(BUILD_DIR, stem + ".o")
+    cmd = [nvcc(), *NVCC_FLAGS, *flags, "-c", os.path.join(CSRC, src), "-o", obj]
     if verbose:
         cmd.insert(1, "-Xptxas=-v")
     res = subprocess.run(cmd, capture_output=True, text=True)
@@ -65,8 +78,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and up_to_date():
         return LIB_PATH
     os.makedirs(BUILD_DIR, exist_ok=True)
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        objs = list(ex.map(lambda s: _compile(s, verbose), SOURCES))
+    units = _units()
+    with cf.ThreadPoolExecutor(max_workers=len(units)) as ex:
+        objs = list(ex.map(lambda u: _compile(u, verbose), units))
     tmp = LIB_PATH + ".tmp%d" % os.getpid()
     cmd = [nvcc(), *ARCH, "-shared", "-o", tmp, *objs]
     res = subprocess.run(cmd, capture_output=True, text=True)

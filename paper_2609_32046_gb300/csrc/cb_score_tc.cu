@@ -55,7 +55,7 @@
 #include "cb_sm100.cuh"
 
 namespace cbk {
-namespace {
+namespace tc {   // (not anonymous: the parts of this file, below, share it)
 using namespace sm100;
 
 constexpr int kWarpsTc = 20;                // 0 TMA, 1 and 2 MMA, 3 pass 2's sums, 4..19 epilogue
@@ -78,6 +78,9 @@ constexpr uint64_t kWaitNs = 1000000000ull;      // 1 s per wait
 constexpr uint32_t kPollNs = 1000000u;           // longest suspension of one poll (woken at completion)
 constexpr int kMaxTcSenders = 32;         // their tensor maps fill most of the 32,764 bytes of kernel parameters
 
+// Rows up to which a half's columns go to the warps in eights (pass 2).
+__host__ __device__ constexpr int few_rows(int G) { return G == 1 ? 96 : 64; }
+
 struct TcMaps {
     CUtensorMap k[3];     // pass 1: k[0] = 4D {d, T, Hkv, nL}, box {64, 128, 1, 1}; k[1] the same over the
                           // query tokens' own keys {d, m, Hkv, nL} (senders that have them).  Of a paged
@@ -99,6 +102,7 @@ struct TcSender {
     int32_t n_chunk1;     // pass-1 partial slots: four per chunk of positions
     int32_t n_blk2;       // pass-2 blocks of positions
     int32_t n_rc1, n_rc2; // row chunks of each pass
+    int32_t share;        // log2 of the lane quarters of a pass-2 block that hold the same positions
     int32_t m_self;       // query tokens whose own keys join the softmax (m or 0)
     int32_t chunk1;       // pass-1 positions per chunk
     const int32_t* pages; // block table of a paged sender that pass 1 reads itself, else null
@@ -116,6 +120,7 @@ struct TcBatch {
     int32_t p_inf, ph;
     int64_t weight1, weight2;     // work of each pass: 128-row halves over all units
     uint64_t wait_ns;     // limit of one bounded mbarrier wait
+    int32_t few;          // some sender needs the pass-2 instantiation FEW
     int32_t paged;        // some sender has `pages`: warp 3 of pass 1 stores its tiles
     int32_t stall;        // 1: CTA 0's pass-1 MMA issuer first waits on a barrier nothing arrives on
     uint32_t* err;
@@ -154,7 +159,7 @@ __device__ __forceinline__ uint64_t now_ns() {
 // Bounded wait: true when the phase completed, false on abort (set by anyone) or timeout.
 // `tag` names the wait in the device error word (bit 8 + tag) when it times out.  The polling is
 // out of line: the epilogue loops stay small enough for the instruction cache.
-__device__ __noinline__ bool wait_poll(uint64_t* bar, uint32_t parity, Ctl* ctl, uint32_t* err, int tag) {
+static __device__ __noinline__ bool wait_poll(uint64_t* bar, uint32_t parity, Ctl* ctl, uint32_t* err, int tag) {
     const uint64_t t0 = now_ns();
     for (uint32_t i = 1; i < (1u << 30); ++i) {
         if (mbar_try_wait_hint(bar, parity, kPollNs)) return true;
@@ -816,9 +821,11 @@ __device__ __forceinline__ void head_sums(const float (&v)[C], uint64_t cc, uint
 // long with one quarter as with four.
 // P: how N adds up the pooled values.  kPowSquare p = 2, kPowAny another p, kPowInf maxima (an
 // instantiation each: choosing inside the loops spilled registers).
+// FEW: some sender of the batch has a half of few query rows (few_rows) or lane quarters that share
+// positions (an instantiation each: the others' loops are 2 % faster without the code for those).
 enum { kPowSquare, kPowAny, kPowInf };
 
-template <int D, int G, int PH, int P>
+template <int D, int G, int PH, int P, bool FEW>
 __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constant__ TcBatch bt) {
     constexpr int kTile = kTileRows * D * 2;
     extern __shared__ uint8_t smem_raw[];
@@ -850,13 +857,14 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
             // the ones columns of the offset K-step, once per CTA
             mbar_arrive_expect_tx(&ctl->o_full, 128 * 32);
             tma_load_2d(sm.ones, &bt.omap, &ctl->o_full, 0, 0);
-            int nc = 0, l = 0, g = 0, T = 0;
+            int nc = 0, l = 0, g = 0, T = 0, share = 0;
             for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
                 const TcMaps& mp = bt.maps[un.i];
                 if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
                     const TcSender& sd = bt.s[un.i];
                     nc = sd.n_blk2;
                     T = (int)sd.T;
+                    share = FEW ? sd.share : 0;
                     l = un.s / bt.Hkv;
                     g = un.s % bt.Hkv;
                     if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 8))) break;
@@ -872,7 +880,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                 const bool whole = t0 + kOut2 + 2 * kMargin <= T / 4 * 4 || T % 4 == 0;
                 for (int j = 0; j < 4; ++j) {
                     if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 9))) break;
-                    // lane quarter w: positions t0 + 120 w + j + 4 i, i = 0 .. 31 (t0 a multiple of four)
+                    // lane quarter w: positions t0 + 120 (w >> share) + j + 4 i, i = 0 .. 31 (t0 a multiple of four)
                     uint8_t* dst = sm.k + (size_t)st * kTile;
                     mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
                     if (whole) {
@@ -882,12 +890,12 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
 #pragma unroll
                             for (int kb = 0; kb < D / 64; ++kb)
                                 tma_load_5d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[0], &ctl->k_full[st], 64 * kb,
-                                            i0 + kOutW / 4 * w, j, g, l);
+                                            i0 + kOutW / 4 * (w >> share), j, g, l);
                     } else {
                         for (int w = 0; w < 4; ++w)
                             for (int kb = 0; kb < D / 64; ++kb)
                                 tma_load_4d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[1], &ctl->k_full[st], 64 * kb,
-                                            t0 + kOutW * w + j, g, l);
+                                            t0 + kOutW * (w >> share) + j, g, l);
                     }
                     ++kt;
                     if (++st == slots) { st = 0; ph ^= 1u; }
@@ -963,7 +971,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
             const int T = (int)sd.T, nc = sd.n_blk2, run = min(left, nc - un.c);
             const float cen = (float)offset_centre(T, G);
             const uint64_t ncen = pack2(-cen, -cen);
-            int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
+            const int share = FEW ? sd.share : 0;
+            int pos = un.c * kOut2 + kOutW * (sp >> share) - kMargin + 4 * lane;
             left -= run;
             un.c += run - 1;
             next_unit<2>(bt, un, nc);
@@ -990,34 +999,33 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
 #pragma unroll
                     for (int j = 0; j < 4; ++j) add_n(j, o0[j], o1[j]);
                 };
-                // One round of the four buffers.  EDGE: positions outside [0, T) are masked.  For d = 128 a
-                // buffer's 32 columns are read one after the other (eight tokens at a time for G < 4, 16
-                // columns a load) and go back to the MMA, which takes as long as the reading, before the
-                // next buffer's.  For d = 64 the MMA takes half that, so buffers can be held longer: four
-                // tokens' columns at a time, the exp2 of a chunk's four tiles interleaved with Pool of the
-                // chunk before it (143 -> 137 us for d64; d = 128 156 -> 168).  Unpooled sums (PH = 0) need no
+                // One round of the four buffers: chunks c0, c0 + step, ... below c1 of the columns from `t` on, TOK
+                // tokens each.  EDGE: positions outside [0, T) are masked.  LAP: exp2 of a chunk's four
+                // tiles interleaved with Pool of the chunk before it.  Unpooled sums (PH = 0) need no
                 // neighbours and are taken load by load.
-                auto round = [&](auto edge) {
-                    constexpr bool EDGE = decltype(edge)::value, LAP = D == 64 && PH > 0;
-                    constexpr int kTok = LAP ? 4 : 8, kChunks = 32 / (kTok * G), kPairs = kTok / 2;
+                auto round = [&](auto edge, auto lap, auto tok, uint32_t t, int c0, int c1, int step) {
+                    constexpr bool EDGE = decltype(edge)::value, LAP = decltype(lap)::value;
+                    constexpr int kTok = decltype(tok)::value, kChunks = 32 / (kTok * G), kPairs = kTok / 2;
                     constexpr int kCols = kTok * G < 16 ? kTok * G : 16;   // columns of a load
                     uint64_t b[LAP ? 2 : 1][4][kPairs];
 #pragma unroll(LAP ? kChunks : 1)
-                    for (int c = 0; c < kChunks; ++c) {
+                    for (int c = LAP ? 0 : c0; c < (LAP || kChunks == 1 ? kChunks : c1); c += LAP || kChunks == 1 ? 1 : step) {
                         auto& bc = b[LAP ? c & 1 : 0];
+                        const bool begin = LAP || kChunks == 1 ? c == 0 : c == c0;
+                        const bool end = LAP || kChunks == 1 ? c == kChunks - 1 : c + step >= c1;
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            if (c == 0) {
+                            if (begin) {
                                 if (!(ok = wait_bar(&ctl->t_full[j], n, ctl, bt.err, 13))) return;
                                 tc_fence_after();
                             }
 #pragma unroll
                             for (int x = 0; x < kTok * G; x += kCols) {
                                 float v[kCols];
-                                tmem_ldn(ta + j * 128 + c * kTok * G + x, v);
+                                tmem_ldn(t + j * 128 + c * kTok * G + x, v);
                                 if (LAP && c > 0 && (j & 1)) pool_pair(b[LAP ? (c & 1) ^ 1 : 0], j >> 1);
                                 tmem_wait_ld(v);
-                                if (c == kChunks - 1 && x + kCols == kTok * G) {   // registers hold the rest
+                                if (end && x + kCols == kTok * G) {   // registers hold the rest
                                     tc_fence_before();
                                     __syncwarp();
                                     if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
@@ -1047,16 +1055,36 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                     }
                 };
                 for (int h = 0; h < nh; ++h, n ^= 1) {
-                    if (h * kRowHalf + 32 * q >= R) {   // padding columns
+                    // A half of more than few_rows(G) rows: 32 columns a warp.  For d = 128 a buffer's are read one after the
+                    // other (eight tokens at a time for G < 4, 16 columns a load) and go back to the MMA,
+                    // which takes as long as the reading, before the next buffer's.  For d = 64 the MMA takes half
+                    // that, so buffers can be held longer: four tokens' columns at a time, interleaved with
+                    // Pool (143 -> 137 us for d64; d = 128 156 -> 168).
+                    // Fewer rows, or lane quarters that share positions: in eights of columns, as many for each of the
+                    // four warps of a lane quarter, of which lane quarters with the same positions take turns.
+                    const int rows = R - h * kRowHalf;
+                    constexpr bool kLap = D == 64 && PH > 0;
+                    constexpr std::integral_constant<int, kLap ? 4 : 8> tok{};
+                    constexpr std::integral_constant<int, 8 / G> tok8{};
+                    constexpr std::bool_constant<kLap> lap{};
+                    constexpr std::false_type no{};
+                    constexpr std::true_type yes{};
+                    constexpr int kChunks = 32 / (tok.value * G);
+                    const bool wide = !FEW || (rows > few_rows(G) && share == 0);
+                    const int eights = min(4, (rows + 31) >> 5), col = 8 * eights * q;
+                    const int c0 = sp & ((1 << share) - 1), c1 = min(eights, (rows - col + 7) >> 3);
+                    if (wide ? 32 * q >= rows : c0 >= c1) {   // no columns
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             if (!(ok = wait_bar(&ctl->t_full[j], n, ctl, bt.err, 13))) break;
                             if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
                         }
-                    } else if (all_valid) {
-                        round(std::false_type{});
-                    } else {
-                        round(std::true_type{});
+                    } else if (wide) {
+                        if (all_valid) round(no, lap, tok, ta, 0, kChunks, 1);
+                        else round(yes, lap, tok, ta, 0, kChunks, 1);
+                    } else if (FEW) {
+                        if (all_valid) round(no, no, tok8, ta - 32 * q + col, c0, c1, 1 << share);
+                        else round(yes, no, tok8, ta - 32 * q + col, c0, c1, 1 << share);
                     }
                     if (!ok) break;
                 }
@@ -1076,7 +1104,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
         bool ok = true;
         float* part = nullptr;                   // U partials of the current group and row chunk
         int64_t nST = 0;                         // distance between the U and N partials
-        int T = 0, nc = 0;
+        int T = 0, nc = 0, share = 0;
         for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
             if (u == 0 || un.c == 0) {
                 const TcSender& sd = bt.s[un.i];
@@ -1084,25 +1112,31 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                 part = sd.part + 2 * un.rc * nST + (int64_t)un.s * sd.T_pad;
                 T = (int)sd.T;
                 nc = sd.n_blk2;
+                share = FEW ? sd.share : 0;
             }
             if (!(ok = wait_bar(&ctl->xb, (uint32_t)u & 1, ctl, bt.err, 14))) break;
+            auto add = [](float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
+            auto mx = [](float4 a, float4 b) {
+                return make_float4(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z), fmaxf(a.w, b.w));
+            };
+            auto add_n = [&](float4 a, float4 b) { return P == kPowInf ? mx(a, b) : add(a, b); };
+            float4 su, sn;                       // of the lane quarters so far that share positions
 #pragma unroll
             for (int sp = 0; sp < 4; ++sp) {
-                const int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
                 float4 x[4], y[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     x[k] = xch[(8 * k + sp) * 32];
                     y[k] = xch[(8 * k + 4 + sp) * 32];
                 }
-                auto add = [](float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
-                auto mx = [](float4 a, float4 b) {
-                    return make_float4(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z), fmaxf(a.w, b.w));
-                };
-                if (lane >= 1 && lane <= 30 && pos < T) {   // rows are padded to a multiple of four positions
-                    *reinterpret_cast<float4*>(part + pos) = add(add(x[0], x[1]), add(x[2], x[3]));
-                    *reinterpret_cast<float4*>(part + nST + pos) =
-                        P == kPowInf ? mx(mx(y[0], y[1]), mx(y[2], y[3])) : add(add(y[0], y[1]), add(y[2], y[3]));
+                const float4 u4 = add(add(x[0], x[1]), add(x[2], x[3])), n4 = add_n(add_n(y[0], y[1]), add_n(y[2], y[3]));
+                const int part_of = sp & ((1 << share) - 1);
+                su = part_of == 0 ? u4 : add(su, u4);
+                sn = part_of == 0 ? n4 : add_n(sn, n4);
+                const int pos = un.c * kOut2 + kOutW * (sp >> share) - kMargin + 4 * lane;
+                if (part_of == (1 << share) - 1 && lane >= 1 && lane <= 30 && pos < T) {   // rows are padded to four
+                    *reinterpret_cast<float4*>(part + pos) = su;
+                    *reinterpret_cast<float4*>(part + nST + pos) = sn;
                 }
             }
             __syncwarp();
@@ -1115,42 +1149,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
 }
 
 // ---------------------------------------------------------------------------
-// host side
+// launches
 // ---------------------------------------------------------------------------
-PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
-std::once_flag g_encode_once;
-
-PFN_cuTensorMapEncodeTiled_v12000 encoder() {
-    std::call_once(g_encode_once, [] {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-        else
-            cudaGetLastError();
-    });
-    return g_encode;
-}
-
-// bf16 tensor map of `rank` dimensions (innermost first); strides in bytes of dims 1..rank-1; of
-// dimension 1 the box takes every step-th element.
-bool encode_nd(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides_bytes,
-               const cuuint32_t* box, CUtensorMapSwizzle swizzle, cuuint32_t step = 1) {
-    auto fn = encoder();
-    if (!fn || !base) return false;
-    const cuuint32_t es[5] = {1, step, 1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides_bytes, box,
-              es, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-bool encode_4d(CUtensorMap* m, const void* base, const cuuint64_t dims[4], const cuuint64_t strides_bytes[3],
-               const cuuint32_t box[4]) {
-    return encode_nd(m, base, 4, dims, strides_bytes, box, CU_TENSOR_MAP_SWIZZLE_128B);
-}
-
 constexpr size_t kSmemMax = 227 * 1024;
 
 // Raises a kernel's dynamic shared-memory limit to the SM's, once per device (`done`: a bit each;
@@ -1167,22 +1167,27 @@ cudaError_t allow_smem(K kernel, std::atomic<uint64_t>& done) {
     return e;
 }
 
-size_t smem1_bytes(int d, int rows, int stages) {
+inline size_t smem1_bytes(int d, int rows, int stages) {
     return 1024 + (size_t)rows * d * 2 + (size_t)stages * kTileRows * d * 2 + 512;
 }
 
-size_t smem2_bytes(int d, int rows, int kbufs) {
+inline size_t smem2_bytes(int d, int rows, int kbufs) {
     return 1024 + (size_t)rows * (d * 2 + 32) + 128 * 32 + (size_t)kbufs * 4 * kTileRows * d * 2 + 512 + 4 * 8 * 128 * 4;
+}
+
+template <int D, int G, int PH, int P, bool FEW>
+cudaError_t launch_accum_few(const TcBatch& tb, int grid, cudaStream_t st) {
+    const size_t smem = smem2_bytes(D, tb.rows2, tb.kbufs);
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = allow_smem(k_accum_tc<D, G, PH, P, FEW>, done);
+    if (e != cudaSuccess) return e;
+    k_accum_tc<D, G, PH, P, FEW><<<grid, kThreadsTc, smem, st>>>(tb);
+    return cudaGetLastError();
 }
 
 template <int D, int G, int PH, int P>
 cudaError_t launch_accum(const TcBatch& tb, int grid, cudaStream_t st) {
-    const size_t smem = smem2_bytes(D, tb.rows2, tb.kbufs);
-    static std::atomic<uint64_t> done{0};
-    const cudaError_t e = allow_smem(k_accum_tc<D, G, PH, P>, done);
-    if (e != cudaSuccess) return e;
-    k_accum_tc<D, G, PH, P><<<grid, kThreadsTc, smem, st>>>(tb);
-    return cudaGetLastError();
+    return tb.few ? launch_accum_few<D, G, PH, P, true>(tb, grid, st) : launch_accum_few<D, G, PH, P, false>(tb, grid, st);
 }
 
 template <int D, int G, int P>
@@ -1223,6 +1228,65 @@ cudaError_t launch_stats_d(const TcBatch& tb, int grid, cudaStream_t st) {
     if (tb.rows1 <= kRowHalf) return launch_stats<D, 1>(tb, grid, st);
     if (tb.rows1 <= 2 * kRowHalf) return launch_stats<D, 2>(tb, grid, st);
     return launch_stats<D, kHalves1>(tb, grid, st);
+}
+
+// This file is compiled in three parts, at the same time: with CB_TC_PART = 64 and 128 the kernels of
+// that head dimension, with 0 everything else (without it, all in one).
+#if !defined(CB_TC_PART) || CB_TC_PART == 64
+template cudaError_t launch_stats_d<64>(const TcBatch&, int, cudaStream_t);
+template cudaError_t launch_accum_d<64>(const TcBatch&, int, cudaStream_t);
+#else
+extern template cudaError_t launch_stats_d<64>(const TcBatch&, int, cudaStream_t);
+extern template cudaError_t launch_accum_d<64>(const TcBatch&, int, cudaStream_t);
+#endif
+#if !defined(CB_TC_PART) || CB_TC_PART == 128
+template cudaError_t launch_stats_d<128>(const TcBatch&, int, cudaStream_t);
+template cudaError_t launch_accum_d<128>(const TcBatch&, int, cudaStream_t);
+#else
+extern template cudaError_t launch_stats_d<128>(const TcBatch&, int, cudaStream_t);
+extern template cudaError_t launch_accum_d<128>(const TcBatch&, int, cudaStream_t);
+#endif
+}  // namespace tc
+
+#if !defined(CB_TC_PART) || CB_TC_PART == 0
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+namespace {
+using namespace tc;
+
+PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
+std::once_flag g_encode_once;
+
+PFN_cuTensorMapEncodeTiled_v12000 encoder() {
+    std::call_once(g_encode_once, [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+        else
+            cudaGetLastError();
+    });
+    return g_encode;
+}
+
+// bf16 tensor map of `rank` dimensions (innermost first); strides in bytes of dims 1..rank-1; of
+// dimension 1 the box takes every step-th element.
+bool encode_nd(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides_bytes,
+               const cuuint32_t* box, CUtensorMapSwizzle swizzle, cuuint32_t step = 1) {
+    auto fn = encoder();
+    if (!fn || !base) return false;
+    const cuuint32_t es[5] = {1, step, 1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides_bytes, box,
+              es, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool encode_4d(CUtensorMap* m, const void* base, const cuuint64_t dims[4], const cuuint64_t strides_bytes[3],
+               const cuuint32_t box[4]) {
+    return encode_nd(m, base, 4, dims, strides_bytes, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 // Positions of a pass-1 chunk of a sender of T positions and nS groups.  Chunks of 2048 positions
@@ -1305,7 +1369,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
         tb->err = err;
         tb->max_rc1 = tb->max_rc2 = 1;
         tb->weight1 = tb->weight2 = 0;
-        tb->paged = 0;
+        tb->paged = tb->few = 0;
         int rows1 = kRowHalf, rows2 = kRowHalf;
         int64_t staged = 0;
         const int b_first = firsts.back();
@@ -1348,6 +1412,8 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             d.chunk1 = stats_chunk(s.T, nS);
             d.n_chunk1 = (int32_t)(4 * ((s.T + d.chunk1 - 1) / d.chunk1));   // one partial per (chunk, column quarter)
             d.n_blk2 = (int32_t)((s.T + kOut2 - 1) / kOut2);
+            d.share = s.T <= kOutW ? 2 : (s.T <= 2 * kOutW ? 1 : 0);
+            tb->few |= d.share > 0 || d.R - (d.halves - 1) * kRowHalf <= few_rows(G);
             d.n_rc1 = (d.halves + kHalves1 - 1) / kHalves1;
             d.n_rc2 = (d.halves + kHalves2 - 1) / kHalves2;
             d.stats = b.stats + s.stats_off;
@@ -1457,5 +1523,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
     }
     return e;
 }
+
+#endif
 
 }  // namespace cbk

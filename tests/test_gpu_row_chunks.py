@@ -65,6 +65,34 @@ def test_scores(case):
                      Kself=kself)
 
 
+@pytest.mark.parametrize("pool_width,p", [(7, 2.0), (1, 3.0), (5, float("inf"))])
+@pytest.mark.parametrize("G", [1, 2, 4])
+def test_few_rows_and_short_senders(G, pool_width, p):
+    """Pass 2 hands a half's columns to the warps in eights up to 64 rows (96 for G = 1), and lane
+    quarters share positions up to 240 of them: both sides of each line, in one call, beside a long
+    sender; every sender's scores are also those of a call of its own."""
+    Ts, rows = [1, 119, 120, 121, 239, 240, 241, 700], [4, 32, 36, 64, 68, 96, 100, 128, 132, 196]
+    for d in (64, 128):
+        o = oracle.default()
+        for r in rows:
+            m = r // G
+            if d == 64 and m <= 64:
+                m += 64          # (fewer tokens: the mma.sync passes)
+            w = synth.custom_workload(synth.Shape(1, 2 * G, 2, d), Ts, m, seed=r + G, n_planted_spans=1)
+            Ks, Qs = [s.K.cuda() for s in w.senders], [w.queries[s.task].cuda() for s in w.senders]
+            c = make_cb(w.spec.shape, max(Ts), m, len(Ts), pool_width=pool_width, p=p)
+            out, S = [torch.empty(T, device="cuda") for T in Ts], torch.empty(max(Ts), device="cuda")
+            c.score(Ks, Qs, out)
+            c.sync_status()
+            assert c.score_path() == 2
+            for i, s in enumerate(w.senders):
+                ref = oracle_scores(o, s.K, w.queries[s.task], p=p, pool_w=pool_width)["S"]
+                assert_scores_close(out[i].cpu().numpy(), ref, rtol=RTOL)
+                c.score([Ks[i]], [Qs[i]], [S[:Ts[i]]])
+                c.sync_status()
+                assert torch.equal(S[:Ts[i]].view(torch.int32), out[i].view(torch.int32)), (d, r, i)
+
+
 @pytest.mark.parametrize("own", [False, True])
 def test_long_chunks(own):
     """1024 groups, enough for chunks of 2048 positions: one with and without a second half, and two;
