@@ -313,8 +313,8 @@ def test_extreme_logit_rows(kernel, scale):
     check_sender(f, 0, K, V, Q)
 
 
-# Every pass-2 instantiation the tcgen05 path admits: k_accum_tc<G, pool_width / 2, p == 2>, G in
-# {1, 2, 4}, pool widths 1, 3, 5, 7 and p = 2 or not (p = 3 for the general power).
+# Pass-2 instantiations of head dimension 128 for one short sender: G in {1, 2, 4}, pool widths 1, 3, 5,
+# 7 and p = 2 or another (all of them, with p = infinity and head dimension 64: test_gpu_row_chunks.py).
 TC_INSTANCES = [(G, pw, p) for G in (1, 2, 4) for pw in (1, 3, 5, 7) for p in (2.0, 3.0)]
 
 

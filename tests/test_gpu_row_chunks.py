@@ -65,6 +65,27 @@ def test_scores(case):
                      Kself=kself)
 
 
+@pytest.mark.parametrize("few", [False, True], ids=["full", "few"])
+@pytest.mark.parametrize("G", [1, 2, 4])
+@pytest.mark.parametrize("d", [64, 128])
+def test_every_pass_2_instantiation(d, G, few):
+    """k_accum_tc<d, G, pool_width / 2, p = 2, another or infinity, few>: `few` where a sender's last 128
+    query rows are at most 64 (96 for G = 1).  T: four blocks, the last one ragged."""
+    m = {1: 65, 2: 66, 4: 66}[G] if few else {1: 100, 2: 100, 4: 90}[G]
+    T = 1501
+    w = synth.custom_workload(synth.Shape(1, 2 * G, 2, d), [T], m, seed=10 * d + G, n_planted_spans=2)
+    K, Q, S = w.senders[0].K.cuda(), w.queries[0].cuda(), torch.empty(T, device="cuda")
+    o = oracle.default()
+    for pool_width in (1, 3, 5, 7):
+        for p in (2.0, 3.0, float("inf")):
+            c = make_cb(w.spec.shape, T, m, 1, pool_width=pool_width, p=p)
+            c.score([K], [Q], [S])
+            c.sync_status()
+            assert c.score_path() == 2
+            ref = oracle_scores(o, w.senders[0].K, w.queries[0], p=p, pool_w=pool_width)["S"]
+            assert_scores_close(S.cpu().numpy(), ref, rtol=RTOL)
+
+
 @pytest.mark.parametrize("pool_width,p", [(7, 2.0), (1, 3.0), (5, float("inf"))])
 @pytest.mark.parametrize("G", [1, 2, 4])
 def test_few_rows_and_short_senders(G, pool_width, p):
@@ -193,6 +214,24 @@ def test_paged_equals_strided(d, m, P):
         assert c.score_path() == 2
     for a, b in zip(*out):
         assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+
+
+@pytest.mark.parametrize("d,P", [(64, 16), (128, 16), (128, 4)])
+def test_paged_with_own_keys_equals_strided(d, P):
+    """The query tokens' own keys after the pages' tiles of a group's last chunk."""
+    w = synth.custom_workload(synth.Shape(2, 8, 2, d), [1030, 257], 130, seed=d + 1, n_planted_spans=2)
+    Ks, Q = [s.K.cuda() for s in w.senders], w.queries[0].cuda()
+    own = synth.make_query_keys(w.spec, 5, 0)
+    out = [[torch.empty(t, device="cuda") for t in (1030, 257)] for _ in range(2)]
+    for caches, o in zip((Ks, [_paged(K, P, i) for i, K in enumerate(Ks)]), out):
+        c = make_cb(w.spec.shape, 1030, 130, 2)
+        c.score(caches, [Q, Q], o, Kselfs=[own.cuda()] * 2)
+        c.sync_status()
+        assert c.score_path() == 2
+    for i, (a, b) in enumerate(zip(*out)):
+        assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+        ref = oracle_scores(oracle.default(), w.senders[i].K, w.queries[0], Kself=own)["S"]
+        assert_scores_close(a.cpu().numpy(), ref, rtol=RTOL)
 
 
 def test_paged_first_call_inside_a_capture():
