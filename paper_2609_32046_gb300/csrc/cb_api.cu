@@ -163,8 +163,8 @@ cb_status check_source_ptr(cb_ctx* ctx, const void* p, const char* what, int i, 
 
 bool stride_ok(int64_t s) { return s > 0 && (s % 8) == 0; }
 
-// Small senders of head dimension 64 keep to the mma.sync passes: up to two waves of their blocks
-// (128 positions x 16 tokens of one group, two resident on an SM) they take less time than the
+// Small senders of head dimension 64 keep to the mma.sync passes: up to about this much work (in
+// pieces of 128 positions x 16 tokens of one group, four an SM) those take less time than the
 // tcgen05 passes, whose CTAs set up barriers and tensor memory and whose tensor maps the host
 // encodes (2 layers x 2 KV heads, m = 16: 16 against 18 us at T = 512 and 18 against 21 at 8192;
 // 24 layers x 8, T = 300, m = 8: 25 against 27; beyond the line, 16 x 8, T = 1024, m = 16: 49

@@ -616,9 +616,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_accum(const __grid_constant__ S
 // positions written.  A batch of groups' loads is issued before they are added: the partials come
 // mostly from DRAM, whose latency bounds the kernel (12.7 us for 19 MB of 288 groups, T = 8192).
 // Rows padded to 16 bytes let ragged lengths load as wide: T = 8191 32 -> 12.5 us.  The 32 slice
-// sums of every position are then added as a tree in shared memory (the rounding of these sums is most of a score's error: 4.5e-7
-// with the slices added in turn), U is pooled and C and S written.  Each sum has a fixed order, so
-// the scores are deterministic.
+// sums of every position are then added as a tree in shared memory, U is pooled and C and S
+// written.  Each sum has a fixed order, so the scores are deterministic.
 constexpr int kFinQuads = 16;
 constexpr int kFinSpan = 4 * kFinQuads;
 constexpr int kFinThreads = kFinSlices * kFinQuads;  // 512
@@ -821,7 +820,7 @@ size_t accum_smem(int max_rows) {
 }
 
 template <int D, int G>
-cudaError_t launch_dg(const ScoreBatch& b, cudaStream_t st, int num_sms) {
+cudaError_t launch_dg(const ScoreBatch& b, cudaStream_t st) {
     int64_t nblk1 = 0, nblk2 = 0;
     int max_rows = 0;
     const int nS = b.n_layers * b.n_kv_heads;
@@ -878,13 +877,13 @@ cudaError_t launch_score(ScoreBatch& b, cudaStream_t st, int num_sms, int* path_
     }
     *path_out = 1;
     if (b.head_dim == 128) {
-        if (G == 4) return launch_dg<128, 4>(b, st, num_sms);
-        if (G == 2) return launch_dg<128, 2>(b, st, num_sms);
-        if (G == 1) return launch_dg<128, 1>(b, st, num_sms);
+        if (G == 4) return launch_dg<128, 4>(b, st);
+        if (G == 2) return launch_dg<128, 2>(b, st);
+        if (G == 1) return launch_dg<128, 1>(b, st);
     } else if (b.head_dim == 64) {
-        if (G == 4) return launch_dg<64, 4>(b, st, num_sms);
-        if (G == 2) return launch_dg<64, 2>(b, st, num_sms);
-        if (G == 1) return launch_dg<64, 1>(b, st, num_sms);
+        if (G == 4) return launch_dg<64, 4>(b, st);
+        if (G == 2) return launch_dg<64, 2>(b, st);
+        if (G == 1) return launch_dg<64, 1>(b, st);
     }
     return cudaErrorInvalidValue;
 }

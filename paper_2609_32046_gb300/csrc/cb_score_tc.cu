@@ -58,7 +58,7 @@ namespace cbk {
 namespace tc {   // (not anonymous: the parts of this file, below, share it)
 using namespace sm100;
 
-constexpr int kWarpsTc = 20;                // 0 TMA, 1 and 2 MMA, 3 pass 2's sums, 4..19 epilogue
+constexpr int kWarpsTc = 20;                // 0 TMA, 1 and 2 MMA, 3 page stores (pass 1) or sums (pass 2), 4..19 epilogue
 constexpr int kThreadsTc = kWarpsTc * 32;
 constexpr int kEpiWarps = 16;
 constexpr int kEpi0 = 4;                    // first epilogue warp (TMEM lane quarter = warp % 4)
@@ -1326,9 +1326,10 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
     // pattern), nothing has been launched and the caller uses the mma.sync passes.
     std::vector<std::unique_ptr<TcBatch>> batches;
     std::vector<std::unique_ptr<TcMaps[]>> maps2;   // pass 2's tensor maps of each sub-batch
-    // Sub-batches of at most kMaxTcSenders senders; paged senders are first copied into the
-    // staging buffer (contiguous [nL][Hkv][T][d]), which each sub-batch reuses from its start,
-    // so a sub-batch also ends where its paged senders would overflow the staging.
+    // Sub-batches of at most kMaxTcSenders senders; paged senders are copied into the staging buffer
+    // (contiguous [nL][Hkv][T][d]; by pass 1, or ahead of it where pages are short), which each
+    // sub-batch reuses from its start, so a sub-batch also ends where its paged senders would
+    // overflow the staging.
     std::vector<int> firsts;
     std::vector<std::unique_ptr<DepageBatch>> depages;
     for (int b0 = 0; b0 < b.n;) {

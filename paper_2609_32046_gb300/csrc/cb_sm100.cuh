@@ -237,12 +237,9 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4]) {
 __device__ __forceinline__ void tmem_ldn(uint32_t taddr, float (&v)[4]) { tmem_ld4(taddr, v); }
 __device__ __forceinline__ void tmem_ldn(uint32_t taddr, float (&v)[8]) { tmem_ld8(taddr, v); }
 __device__ __forceinline__ void tmem_ldn(uint32_t taddr, float (&v)[16]) { tmem_ld16(taddr, v); }
-__device__ __forceinline__ void tmem_ldn(uint32_t taddr, float (&v)[32]) { tmem_ld32(taddr, v); }
 
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// The same wait, tied to the 32 registers a tcgen05.ld.32x32b.x32 wrote, so that no use of them
-// can be scheduled before the load has completed.
+// Wait for this thread's TMEM loads, tied to the 32 registers a tcgen05.ld.32x32b.x32 wrote, so
+// that no use of them can be scheduled before the load has completed.
 __device__ __forceinline__ void tmem_wait_ld(float (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
