@@ -55,8 +55,7 @@
 #include "cb_sm100.cuh"
 
 namespace cbk {
-namespace tc {   // (not anonymous: the parts of this file, below, share it)
-using namespace sm100;
+namespace tc {   // (not anonymous: the parts of this file, below, share these types)
 
 constexpr int kWarpsTc = 20;                // 0 TMA, 1 and 2 MMA, 3 page stores (pass 1) or sums (pass 2), 4..19 epilogue
 constexpr int kThreadsTc = kWarpsTc * 32;
@@ -73,13 +72,15 @@ constexpr float kRaise = 8.f;           // pass 1, second run: a logit this far 
 constexpr int64_t kLongChunkUnits = 1024;  // pass-1 units from which chunks are twice as long
 constexpr int kOutW = 128 - 2 * kMargin;         // 120 output positions per pass-2 lane quarter
 constexpr int kOut2 = 4 * kOutW;                 // 480 output positions per pass-2 block
+constexpr int kMarginN = 3, kOutNW = 32 - 2 * kMarginN, kOutN = 4 * kOutNW;   // the same of k_narrow_tc: 3, 26, 104
+constexpr int64_t kNarrowT = 3 * kOutN, kNarrowUnits = 76;   // senders of pass 2 with blocks of one tile (narrow_blocks)
 constexpr uint32_t kTmemCols = 512;
 constexpr uint64_t kWaitNs = 1000000000ull;      // 1 s per wait
 constexpr uint32_t kPollNs = 1000000u;           // longest suspension of one poll (woken at completion)
 constexpr int kMaxTcSenders = 32;         // their tensor maps fill most of the 32,764 bytes of kernel parameters
 
-// Rows up to which a half's columns go to the warps in eights (pass 2).
-__host__ __device__ constexpr int few_rows(int G) { return G == 1 ? 96 : 64; }
+// Rows up to which a half's columns go to the warps in eights (pass 2; for G = 1 and d = 128, always).
+constexpr int kFewRows = 64;
 
 struct TcMaps {
     CUtensorMap k[3];     // pass 1: k[0] = 4D {d, T, Hkv, nL}, box {64, 128, 1, 1}; k[1] the same over the
@@ -88,8 +89,8 @@ struct TcMaps {
                           // and k[2] = the copy, 4D like a strided sender's.
                           // pass 2: k[0] = 5D {d, T / 4, 4, Hkv, nL} (position 4 i + j at (i, j)), box
                           // {64, 32, 1, 1, 1}; k[1] = 4D as in pass 1 with every fourth of 128 positions in its box (the
-                          // 5D tensor lacks the last T mod 4 positions), k[2] = E, the offset terms, 3D
-                          // {16, R_pad, nS}, box {16, q_rows, 1}, 32-byte swizzle
+                          // 5D tensor lacks the last T mod 4 positions), or of a narrow sender 32 positions;
+                          // k[2] = E, the offset terms, 3D {16, R_pad, nS}, box {16, q_rows, 1}, 32-byte swizzle
     CUtensorMap q;        // 4D {d, Hq, m, nL}, box {64, G, q_rows / G, 1}
 };
 
@@ -102,7 +103,7 @@ struct TcSender {
     int32_t n_chunk1;     // pass-1 partial slots: four per chunk of positions
     int32_t n_blk2;       // pass-2 blocks of positions
     int32_t n_rc1, n_rc2; // row chunks of each pass
-    int32_t share;        // log2 of the lane quarters of a pass-2 block that hold the same positions
+    int32_t narrow;       // pass 2 takes blocks of one tile (k_narrow_tc)
     int32_t m_self;       // query tokens whose own keys join the softmax (m or 0)
     int32_t chunk1;       // pass-1 positions per chunk
     const int32_t* pages; // block table of a paged sender that pass 1 reads itself, else null
@@ -128,12 +129,26 @@ struct TcBatch {
     TcSender s[kMaxTcSenders];
 };
 
+static_assert(sizeof(TcBatch) <= 32764, "kernel parameters");
+
+// The launches of head dimension D.
+template <int D>
+cudaError_t launch_stats_d(const TcBatch& tb, int grid, cudaStream_t st);
+template <int D>
+cudaError_t launch_accum_d(const TcBatch& tb, int grid, cudaStream_t st);
+template <int D>
+cudaError_t launch_narrow_d(const TcBatch& tb, int grid, cudaStream_t st);
+}  // namespace tc
+
+namespace {
+using namespace sm100;
+using namespace tc;
+
 // One unit of work: sender i, group s, row chunk rc, position chunk (pass 1) or block (pass 2) c.
 struct Unit {
     int i, s, c, rc;
 };
 
-static_assert(sizeof(TcBatch) <= 32764, "kernel parameters");
 
 struct Ctl {
     uint64_t k_full[kMaxStages], k_empty[kMaxStages];
@@ -821,8 +836,8 @@ __device__ __forceinline__ void head_sums(const float (&v)[C], uint64_t cc, uint
 // long with one quarter as with four.
 // P: how N adds up the pooled values.  kPowSquare p = 2, kPowAny another p, kPowInf maxima (an
 // instantiation each: choosing inside the loops spilled registers).
-// FEW: some sender of the batch has a half of few query rows (few_rows) or lane quarters that share
-// positions (an instantiation each: the others' loops are 2 % faster without the code for those).
+// FEW: some sender of the batch has a half of few query rows (kFewRows; an instantiation of its own: the
+// others' loops are 2 % faster without the code for it).
 enum { kPowSquare, kPowAny, kPowInf };
 
 template <int D, int G, int PH, int P, bool FEW>
@@ -857,14 +872,13 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
             // the ones columns of the offset K-step, once per CTA
             mbar_arrive_expect_tx(&ctl->o_full, 128 * 32);
             tma_load_2d(sm.ones, &bt.omap, &ctl->o_full, 0, 0);
-            int nc = 0, l = 0, g = 0, T = 0, share = 0;
+            int nc = 0, l = 0, g = 0, T = 0;
             for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
                 const TcMaps& mp = bt.maps[un.i];
                 if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
                     const TcSender& sd = bt.s[un.i];
                     nc = sd.n_blk2;
                     T = (int)sd.T;
-                    share = FEW ? sd.share : 0;
                     l = un.s / bt.Hkv;
                     g = un.s % bt.Hkv;
                     if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 8))) break;
@@ -880,7 +894,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                 const bool whole = t0 + kOut2 + 2 * kMargin <= T / 4 * 4 || T % 4 == 0;
                 for (int j = 0; j < 4; ++j) {
                     if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 9))) break;
-                    // lane quarter w: positions t0 + 120 (w >> share) + j + 4 i, i = 0 .. 31 (t0 a multiple of four)
+                    // lane quarter w: positions t0 + 120 w + j + 4 i, i = 0 .. 31 (t0 a multiple of four)
                     uint8_t* dst = sm.k + (size_t)st * kTile;
                     mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
                     if (whole) {
@@ -890,12 +904,12 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
 #pragma unroll
                             for (int kb = 0; kb < D / 64; ++kb)
                                 tma_load_5d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[0], &ctl->k_full[st], 64 * kb,
-                                            i0 + kOutW / 4 * (w >> share), j, g, l);
+                                            i0 + kOutW / 4 * w, j, g, l);
                     } else {
                         for (int w = 0; w < 4; ++w)
                             for (int kb = 0; kb < D / 64; ++kb)
                                 tma_load_4d(dst + kb * kTileRows * 128 + w * 32 * 128, &mp.k[1], &ctl->k_full[st], 64 * kb,
-                                            t0 + kOutW * (w >> share) + j, g, l);
+                                            t0 + kOutW * w + j, g, l);
                     }
                     ++kt;
                     if (++st == slots) { st = 0; ph ^= 1u; }
@@ -971,8 +985,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
             const int T = (int)sd.T, nc = sd.n_blk2, run = min(left, nc - un.c);
             const float cen = (float)offset_centre(T, G);
             const uint64_t ncen = pack2(-cen, -cen);
-            const int share = FEW ? sd.share : 0;
-            int pos = un.c * kOut2 + kOutW * (sp >> share) - kMargin + 4 * lane;
+            int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
             left -= run;
             un.c += run - 1;
             next_unit<2>(bt, un, nc);
@@ -999,23 +1012,22 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
 #pragma unroll
                     for (int j = 0; j < 4; ++j) add_n(j, o0[j], o1[j]);
                 };
-                // One round of the four buffers: chunks c0, c0 + step, ... below c1 of the columns from `t` on, TOK
-                // tokens each.  EDGE: positions outside [0, T) are masked.  LAP: exp2 of a chunk's four
-                // tiles interleaved with Pool of the chunk before it.  Unpooled sums (PH = 0) need no
-                // neighbours and are taken load by load.
-                auto round = [&](auto edge, auto lap, auto tok, uint32_t t, int c0, int c1, int step) {
+                // One round of the four buffers: the first `chunks` chunks of the columns from `t` on, TOK tokens
+                // each.  EDGE: positions outside [0, T) are masked.  LAP: exp2 of a chunk's four tiles
+                // interleaved with Pool of the chunk before it.  Unpooled sums (PH = 0) need no neighbours and
+                // are taken load by load.
+                auto round = [&](auto edge, auto lap, auto tok, uint32_t t, int chunks) {
                     constexpr bool EDGE = decltype(edge)::value, LAP = decltype(lap)::value;
                     constexpr int kTok = decltype(tok)::value, kChunks = 32 / (kTok * G), kPairs = kTok / 2;
                     constexpr int kCols = kTok * G < 16 ? kTok * G : 16;   // columns of a load
                     uint64_t b[LAP ? 2 : 1][4][kPairs];
 #pragma unroll(LAP ? kChunks : 1)
-                    for (int c = LAP ? 0 : c0; c < (LAP || kChunks == 1 ? kChunks : c1); c += LAP || kChunks == 1 ? 1 : step) {
+                    for (int c = 0; c < (LAP || kChunks == 1 ? kChunks : chunks); ++c) {
                         auto& bc = b[LAP ? c & 1 : 0];
-                        const bool begin = LAP || kChunks == 1 ? c == 0 : c == c0;
-                        const bool end = LAP || kChunks == 1 ? c == kChunks - 1 : c + step >= c1;
+                        const bool end = c == (LAP || kChunks == 1 ? kChunks : chunks) - 1;
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            if (begin) {
+                            if (c == 0) {
                                 if (!(ok = wait_bar(&ctl->t_full[j], n, ctl, bt.err, 13))) return;
                                 tc_fence_after();
                             }
@@ -1055,36 +1067,36 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                     }
                 };
                 for (int h = 0; h < nh; ++h, n ^= 1) {
-                    // A half of more than few_rows(G) rows: 32 columns a warp.  For d = 128 a buffer's are read one after the
-                    // other (eight tokens at a time for G < 4, 16 columns a load) and go back to the MMA,
-                    // which takes as long as the reading, before the next buffer's.  For d = 64 the MMA takes half
-                    // that, so buffers can be held longer: four tokens' columns at a time, interleaved with
-                    // Pool (143 -> 137 us for d64; d = 128 156 -> 168).
-                    // Fewer rows, or lane quarters that share positions: in eights of columns, as many for each of the
-                    // four warps of a lane quarter, of which lane quarters with the same positions take turns.
+                    // A half of more than kFewRows rows: 32 columns a warp.  For d = 128 a buffer's are read one
+                    // after the other (eight tokens at a time for G < 4, 16 columns a load) and go back to the
+                    // MMA, which takes as long as the reading, before the next buffer's.  For d = 64 the MMA takes
+                    // half that, so buffers can be held longer: four tokens' columns at a time, interleaved
+                    // with Pool (143 -> 137 us for d64; d = 128 156 -> 168).
+                    // Fewer rows, or G = 1, where eight tokens fill eight columns: eights of columns, as many for each of
+                    // the four warps of a lane quarter.
                     const int rows = R - h * kRowHalf;
-                    constexpr bool kLap = D == 64 && PH > 0;
+                    constexpr bool kLap = D == 64 && PH > 0, kEights = G == 1 && !kLap;
                     constexpr std::integral_constant<int, kLap ? 4 : 8> tok{};
                     constexpr std::integral_constant<int, 8 / G> tok8{};
                     constexpr std::bool_constant<kLap> lap{};
                     constexpr std::false_type no{};
                     constexpr std::true_type yes{};
                     constexpr int kChunks = 32 / (tok.value * G);
-                    const bool wide = !FEW || (rows > few_rows(G) && share == 0);
+                    const bool wide = !kEights && (!FEW || rows > kFewRows);
                     const int eights = min(4, (rows + 31) >> 5), col = 8 * eights * q;
-                    const int c0 = sp & ((1 << share) - 1), c1 = min(eights, (rows - col + 7) >> 3);
-                    if (wide ? 32 * q >= rows : c0 >= c1) {   // no columns
+                    if (wide ? 32 * q >= rows : col >= rows) {   // no columns
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             if (!(ok = wait_bar(&ctl->t_full[j], n, ctl, bt.err, 13))) break;
                             if (lane == 0) mbar_arrive(&ctl->t_empty[j]);
                         }
                     } else if (wide) {
-                        if (all_valid) round(no, lap, tok, ta, 0, kChunks, 1);
-                        else round(yes, lap, tok, ta, 0, kChunks, 1);
-                    } else if (FEW) {
-                        if (all_valid) round(no, no, tok8, ta - 32 * q + col, c0, c1, 1 << share);
-                        else round(yes, no, tok8, ta - 32 * q + col, c0, c1, 1 << share);
+                        if (all_valid) round(no, lap, tok, ta, kChunks);
+                        else round(yes, lap, tok, ta, kChunks);
+                    } else if (FEW || kEights) {
+                        const int n8 = min(eights, (rows - col + 7) >> 3);
+                        if (all_valid) round(no, no, tok8, ta - 32 * q + col, n8);
+                        else round(yes, no, tok8, ta - 32 * q + col, n8);
                     }
                     if (!ok) break;
                 }
@@ -1104,7 +1116,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
         bool ok = true;
         float* part = nullptr;                   // U partials of the current group and row chunk
         int64_t nST = 0;                         // distance between the U and N partials
-        int T = 0, nc = 0, share = 0;
+        int T = 0, nc = 0;
         for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
             if (u == 0 || un.c == 0) {
                 const TcSender& sd = bt.s[un.i];
@@ -1112,7 +1124,6 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                 part = sd.part + 2 * un.rc * nST + (int64_t)un.s * sd.T_pad;
                 T = (int)sd.T;
                 nc = sd.n_blk2;
-                share = FEW ? sd.share : 0;
             }
             if (!(ok = wait_bar(&ctl->xb, (uint32_t)u & 1, ctl, bt.err, 14))) break;
             auto add = [](float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
@@ -1120,7 +1131,6 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                 return make_float4(fmaxf(a.x, b.x), fmaxf(a.y, b.y), fmaxf(a.z, b.z), fmaxf(a.w, b.w));
             };
             auto add_n = [&](float4 a, float4 b) { return P == kPowInf ? mx(a, b) : add(a, b); };
-            float4 su, sn;                       // of the lane quarters so far that share positions
 #pragma unroll
             for (int sp = 0; sp < 4; ++sp) {
                 float4 x[4], y[4];
@@ -1130,13 +1140,239 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                     y[k] = xch[(8 * k + 4 + sp) * 32];
                 }
                 const float4 u4 = add(add(x[0], x[1]), add(x[2], x[3])), n4 = add_n(add_n(y[0], y[1]), add_n(y[2], y[3]));
-                const int part_of = sp & ((1 << share) - 1);
-                su = part_of == 0 ? u4 : add(su, u4);
-                sn = part_of == 0 ? n4 : add_n(sn, n4);
-                const int pos = un.c * kOut2 + kOutW * (sp >> share) - kMargin + 4 * lane;
-                if (part_of == (1 << share) - 1 && lane >= 1 && lane <= 30 && pos < T) {   // rows are padded to four
-                    *reinterpret_cast<float4*>(part + pos) = su;
-                    *reinterpret_cast<float4*>(part + nST + pos) = sn;
+                const int pos = un.c * kOut2 + kOutW * sp - kMargin + 4 * lane;
+                if (lane >= 1 && lane <= 30 && pos < T) {   // rows are padded to a multiple of four positions
+                    *reinterpret_cast<float4*>(part + pos) = u4;
+                    *reinterpret_cast<float4*>(part + nST + pos) = n4;
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->xe);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(tmem, kTmemCols);
+}
+
+// Pass 2 for senders of few blocks of 480 positions: blocks of one tile, a position a lane.  Lane
+// quarter w of block c covers positions 104 c + 26 w - 3 .. + 31, lanes 3 to 28 its outputs.  Pool takes
+// two to four shuffles a value where k_accum_tc takes six for four, and 104 of a tile's 128
+// positions are outputs instead of 120, but four times as many blocks fill the SMs, and a sender of less than 480
+// positions has no lane quarters without any.
+// P is chosen inside (`mode`): these are calls of few exponentials, bound by latencies (K and Q of a
+// block arriving, its MMA, its round of exponentials one after the other).
+template <int PH>
+__device__ __forceinline__ float pool1(float x) {
+    constexpr unsigned kAll = 0xffffffffu;
+    if (PH == 0) return x;
+    const float y = fmax3(__shfl_up_sync(kAll, x, 1), x, __shfl_down_sync(kAll, x, 1));
+    if (PH == 1) return y;
+    return fmax3(__shfl_up_sync(kAll, y, PH - 1), y, __shfl_down_sync(kAll, y, PH - 1));
+}
+
+template <int D, int G, int PH>
+__global__ void __launch_bounds__(kThreadsTc, 1) k_narrow_tc(const __grid_constant__ TcBatch bt) {
+    constexpr int kTile = kTileRows * D * 2;
+    extern __shared__ uint8_t smem_raw[];
+    const Smem sm = carve<D, 2>(smem_raw, bt);
+    Ctl* ctl = sm.ctl;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        init_ctl(ctl, 2, bt.wait_ns);
+        my_units<2>(bt, ctl);
+    }
+    if (warp == 1) {
+        tmem_alloc(&ctl->tmem_base, kTmemCols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = ctl->tmem_base;
+    const int n_units = ctl->units;
+    Unit un = ctl->first;
+    const int slots = 4 * bt.kbufs;
+
+    if (warp == 0) {
+        // ---------------- TMA producer ----------------
+        if (elect_one()) {
+            int64_t kt = 0, qn = 0;   // K tiles and Q loads issued
+            int st = 0;               // slot of the next K tile and its phase parity
+            uint32_t ph = 0;
+            bool ok = true;
+            mbar_arrive_expect_tx(&ctl->o_full, 128 * 32);
+            tma_load_2d(sm.ones, &bt.omap, &ctl->o_full, 0, 0);
+            int nc = 0, l = 0, g = 0;
+            for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
+                const TcMaps& mp = bt.maps[un.i];
+                if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
+                    const TcSender& sd = bt.s[un.i];
+                    nc = sd.n_blk2;
+                    l = un.s / bt.Hkv;
+                    g = un.s % bt.Hkv;
+                    if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 8))) break;
+                    const int h0 = rc_begin(sd.halves, sd.n_rc2, un.rc);
+                    load_q<D, 2>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0, sd.q_rows);
+                    ++qn;
+                }
+                if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 9))) break;
+                mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
+                for (int w = 0; w < 4; ++w)
+                    for (int kb = 0; kb < D / 64; ++kb)
+                        tma_load_4d(sm.k + (size_t)st * kTile + kb * kTileRows * 128 + w * 32 * 128, &mp.k[1],
+                                    &ctl->k_full[st], 64 * kb, un.c * kOutN + kOutNW * w - kMarginN, g, l);
+                ++kt;
+                if (++st == slots) { st = 0; ph ^= 1u; }
+            }
+            for (int64_t k = kt - slots > 0 ? kt - slots : 0; k < kt; ++k)
+                drain_wait(&ctl->k_full[k % slots], (uint32_t)((k / slots) & 1));
+            if (qn > 0) drain_wait(&ctl->q_full, (uint32_t)((qn - 1) & 1));
+            drain_wait(&ctl->o_full, 0);
+        }
+    } else if (warp <= 2) {
+        // ---------------- MMA issuers: alternate buffers ----------------
+        if (elect_one()) {
+            const uint32_t me = (uint32_t)warp - 1;
+            uint32_t qn = 0, n = 0;      // Q loads consumed; accumulator buffers filled by both issuers
+            int st = 0;                  // slot of the next K tile and its phase parity
+            uint32_t ph = 0;
+            bool ok = wait_bar(&ctl->o_full, 0, ctl, bt.err, 15);
+            const uint64_t ones_desc = smem_desc_sw32(smem_u32(sm.ones)), ext_desc = smem_desc_sw32(smem_u32(sm.ext));
+            const uint32_t ext_hi = (uint32_t)(ext_desc >> 32), ext_lo = (uint32_t)ext_desc;
+            const uint64_t qd = smem_desc_sw128(smem_u32(sm.q));
+            const uint32_t hi = (uint32_t)(qd >> 32), q_lo = (uint32_t)qd;
+            const uint32_t k_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.k));
+            const uint32_t q_blk = (uint32_t)bt.rows2 * 128 >> 4;
+            constexpr uint32_t idesc = idesc_bf16_f32(128, 128);
+            uint32_t nh = 0, id_last = idesc;
+            int nc = 0;
+            for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
+                if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
+                    const TcSender& sd = bt.s[un.i];
+                    nc = sd.n_blk2;
+                    const int h1 = rc_begin(sd.halves, sd.n_rc2, un.rc + 1);
+                    nh = h1 - rc_begin(sd.halves, sd.n_rc2, un.rc);
+                    id_last = idesc_bf16_f32(128, min(kRowHalf, (sd.R - (h1 - 1) * kRowHalf + 31) & ~31));
+                    if (u > 0) umma_commit(&ctl->q_empty);
+                    if (!(ok = wait_bar(&ctl->q_full, qn & 1, ctl, bt.err, 10))) break;
+                    ++qn;
+                }
+                if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 11))) break;
+                for (uint32_t h = (n ^ me) & 1; h < nh; h += 2) {
+                    const uint32_t x = n + h, buf = x & 3, id = h == nh - 1 ? id_last : idesc;
+                    if (!(ok = wait_bar(&ctl->t_empty[buf], ((x >> 2) & 1) ^ 1, ctl, bt.err, 12))) break;
+                    tc_fence_after();
+                    mma_d<D>(tmem + buf * 128, k_lo + (uint32_t)st * (kTile >> 4), kTileRows * 128 >> 4,
+                             q_lo + h * (kRowHalf * 128 >> 4), q_blk, hi, id);
+                    umma_bf16(tmem + buf * 128, ones_desc, desc64(ext_lo + h * (kRowHalf * 32 >> 4), ext_hi), id, 1u);
+                    umma_commit(&ctl->t_full[buf]);
+                }
+                if (!ok) break;
+                n += nh;
+                umma_commit(&ctl->k_empty[st]);
+                if (++st == slots) { st = 0; ph ^= 1u; }
+            }
+            umma_commit(&ctl->drain[me]);
+            drain_wait(&ctl->drain[me], 0);
+        }
+    } else if (warp >= kEpi0) {
+        // ---------------- epilogue: a position a lane, a share of every buffer's columns a warp ----------------
+        const int q = (warp - kEpi0) >> 2, sp = warp & 3;   // column share, TMEM lane quarter
+        const uint32_t ta = tmem + ((uint32_t)(sp * 32) << 16);
+        float* xch = sm.epi + q * 256 + sp * 32 + lane;     // [column share][U, N][lane quarter][lane]
+        const uint64_t cc = pack2(bt.sl2e, bt.sl2e);
+        const int mode = bt.p_inf ? kPowInf : (bt.p == 2.f ? kPowSquare : kPowAny);
+        uint32_t n = 0;                          // accumulator buffers consumed
+        bool ok = true;
+        int nc = 0, nh = 0, R = 0, T = 0;
+        uint64_t ncen = 0;
+        for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
+            if (u == 0 || un.c == 0) {
+                const TcSender& sd = bt.s[un.i];
+                nc = sd.n_blk2;
+                const int h0 = rc_begin(sd.halves, sd.n_rc2, un.rc);
+                nh = rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0;
+                R = sd.R - h0 * kRowHalf;
+                T = (int)sd.T;
+                const float cen = (float)offset_centre(T, G);
+                ncen = pack2(-cen, -cen);
+            }
+            const int pos = un.c * kOutN + kOutNW * sp - kMarginN + lane;
+            const bool valid = pos >= 0 && pos < T;
+            float us = 0.f, ns = 0.f;
+            // COLS columns from `t` on: their tokens' values, Pool and the sums
+            auto take = [&](auto cols, uint32_t t, uint32_t buf, bool last) {
+                constexpr int kCols = decltype(cols)::value;
+                float v[kCols];
+                tmem_ldn(t, v);
+                tmem_wait_ld(v);
+                if (last) {   // registers hold the rest
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&ctl->t_empty[buf]);
+                }
+                uint64_t b[kCols / (2 * G)];
+                head_sums<G>(v, cc, ncen, b);
+#pragma unroll
+                for (int i = 0; i < kCols / (2 * G); ++i) {
+                    float x0, x1;
+                    unpack2(valid ? b[i] : 0ull, x0, x1);
+                    us += x0 + x1;
+                    const float o0 = pool1<PH>(x0), o1 = pool1<PH>(x1);
+                    if (mode == kPowSquare) ns = fmaf(o0, o0, fmaf(o1, o1, ns));
+                    else if (mode == kPowInf) ns = fmaxf(ns, fmaxf(o0, o1));
+                    else ns += pow_p(o0, bt.p) + pow_p(o1, bt.p);
+                }
+            };
+            for (int h = 0; h < nh; ++h, ++n) {
+                const uint32_t buf = n & 3;
+                if (!(ok = wait_bar(&ctl->t_full[buf], (n >> 2) & 1, ctl, bt.err, 13))) break;
+                tc_fence_after();
+                // eights of columns, as many for each of the four warps of a lane quarter
+                const int rows = R - h * kRowHalf, eights = min(4, (rows + 31) >> 5), col = 8 * eights * q;
+                int n8 = min(eights, (rows - col + 7) >> 3);
+                if (n8 <= 0 && lane == 0) mbar_arrive(&ctl->t_empty[buf]);   // none
+                uint32_t t = ta + buf * 128 + col;
+                for (; n8 >= 2; n8 -= 2, t += 16) take(std::integral_constant<int, 16>{}, t, buf, n8 == 2);
+                if (n8 == 1) take(std::integral_constant<int, 8>{}, t, buf, true);
+            }
+            // hand the block's sums to warp 3 (it has read the last block's long ago)
+            if (!ok || !(ok = wait_bar(&ctl->xe, ((uint32_t)u & 1) ^ 1, ctl, bt.err, 7))) break;
+            xch[0] = us;
+            xch[128] = ns;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->xb);
+        }
+    } else {
+        // ---------------- warp 3: the column shares' sums of a block, added in a fixed order ----------------
+        const float* xch = sm.epi + lane;        // [column share][U, N][lane quarter][lane]
+        const int nS = bt.nL * bt.Hkv;
+        bool ok = true;
+        float* part = nullptr;                   // U partials of the current group and row chunk
+        int64_t nST = 0;                         // distance between the U and N partials
+        int T = 0, nc = 0;
+        for (int u = 0; u < n_units && ok; ++u, next_unit<2>(bt, un, nc)) {
+            if (u == 0 || un.c == 0) {
+                const TcSender& sd = bt.s[un.i];
+                nST = (int64_t)nS * sd.T_pad;
+                part = sd.part + 2 * un.rc * nST + (int64_t)un.s * sd.T_pad;
+                T = (int)sd.T;
+                nc = sd.n_blk2;
+            }
+            if (!(ok = wait_bar(&ctl->xb, (uint32_t)u & 1, ctl, bt.err, 14))) break;
+#pragma unroll
+            for (int sp = 0; sp < 4; ++sp) {
+                float x[4], y[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    x[k] = xch[(8 * k + sp) * 32];
+                    y[k] = xch[(8 * k + 4 + sp) * 32];
+                }
+                const int pos = un.c * kOutN + kOutNW * sp - kMarginN + lane;
+                if (lane >= kMarginN && lane < kMarginN + kOutNW && pos < T) {
+                    part[pos] = (x[0] + x[1]) + (x[2] + x[3]);
+                    part[nST + pos] = bt.p_inf ? fmaxf(fmaxf(y[0], y[1]), fmaxf(y[2], y[3])) : (y[0] + y[1]) + (y[2] + y[3]);
                 }
             }
             __syncwarp();
@@ -1207,10 +1443,25 @@ cudaError_t launch_accum_g(const TcBatch& tb, int grid, cudaStream_t st) {
     return tb.p_inf ? launch_accum_gp<D, G, kPowInf>(tb, grid, st) : launch_accum_gp<D, G, kPowAny>(tb, grid, st);
 }
 
-template <int D>
-cudaError_t launch_accum_d(const TcBatch& tb, int grid, cudaStream_t st) {
-    if (tb.G == 4) return launch_accum_g<D, 4>(tb, grid, st);
-    return tb.G == 2 ? launch_accum_g<D, 2>(tb, grid, st) : launch_accum_g<D, 1>(tb, grid, st);
+template <int D, int G, int PH>
+cudaError_t launch_narrow(const TcBatch& tb, int grid, cudaStream_t st) {
+    const size_t smem = smem2_bytes(D, tb.rows2, tb.kbufs);
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = allow_smem(k_narrow_tc<D, G, PH>, done);
+    if (e != cudaSuccess) return e;
+    k_narrow_tc<D, G, PH><<<grid, kThreadsTc, smem, st>>>(tb);
+    return cudaGetLastError();
+}
+
+template <int D, int G>
+cudaError_t launch_narrow_g(const TcBatch& tb, int grid, cudaStream_t st) {
+    switch (tb.ph) {
+        case 0: return launch_narrow<D, G, 0>(tb, grid, st);
+        case 1: return launch_narrow<D, G, 1>(tb, grid, st);
+        case 2: return launch_narrow<D, G, 2>(tb, grid, st);
+        case 3: return launch_narrow<D, G, 3>(tb, grid, st);
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <int D, int NH>
@@ -1221,6 +1472,21 @@ cudaError_t launch_stats(const TcBatch& tb, int grid, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     k_stats_tc<D, NH><<<grid, kThreadsTc, smem, st>>>(tb);
     return cudaGetLastError();
+}
+
+}  // namespace
+
+namespace tc {
+template <int D>
+cudaError_t launch_accum_d(const TcBatch& tb, int grid, cudaStream_t st) {
+    if (tb.G == 4) return launch_accum_g<D, 4>(tb, grid, st);
+    return tb.G == 2 ? launch_accum_g<D, 2>(tb, grid, st) : launch_accum_g<D, 1>(tb, grid, st);
+}
+
+template <int D>
+cudaError_t launch_narrow_d(const TcBatch& tb, int grid, cudaStream_t st) {
+    if (tb.G == 4) return launch_narrow_g<D, 4>(tb, grid, st);
+    return tb.G == 2 ? launch_narrow_g<D, 2>(tb, grid, st) : launch_narrow_g<D, 1>(tb, grid, st);
 }
 
 template <int D>
@@ -1235,16 +1501,20 @@ cudaError_t launch_stats_d(const TcBatch& tb, int grid, cudaStream_t st) {
 #if !defined(CB_TC_PART) || CB_TC_PART == 64
 template cudaError_t launch_stats_d<64>(const TcBatch&, int, cudaStream_t);
 template cudaError_t launch_accum_d<64>(const TcBatch&, int, cudaStream_t);
+template cudaError_t launch_narrow_d<64>(const TcBatch&, int, cudaStream_t);
 #else
 extern template cudaError_t launch_stats_d<64>(const TcBatch&, int, cudaStream_t);
 extern template cudaError_t launch_accum_d<64>(const TcBatch&, int, cudaStream_t);
+extern template cudaError_t launch_narrow_d<64>(const TcBatch&, int, cudaStream_t);
 #endif
 #if !defined(CB_TC_PART) || CB_TC_PART == 128
 template cudaError_t launch_stats_d<128>(const TcBatch&, int, cudaStream_t);
 template cudaError_t launch_accum_d<128>(const TcBatch&, int, cudaStream_t);
+template cudaError_t launch_narrow_d<128>(const TcBatch&, int, cudaStream_t);
 #else
 extern template cudaError_t launch_stats_d<128>(const TcBatch&, int, cudaStream_t);
 extern template cudaError_t launch_accum_d<128>(const TcBatch&, int, cudaStream_t);
+extern template cudaError_t launch_narrow_d<128>(const TcBatch&, int, cudaStream_t);
 #endif
 }  // namespace tc
 
@@ -1300,6 +1570,15 @@ bool encode_4d(CUtensorMap* m, const void* base, const cuuint64_t dims[4], const
 int32_t stats_chunk(int64_t T, int nS) {
     return nS * ((T + 2 * kChunk1 - 1) / (2 * kChunk1)) >= kLongChunkUnits ? 2 * kChunk1 : kChunk1;
 }
+
+// Whether pass 2 takes a sender of T positions in blocks of one tile, given its units (blocks of 480,
+// groups and row chunks): a sender of few positions leaves lane quarters idle (20 layers x
+// 8 groups, 5 x T = 103, 6 rows: 20 against 26 us; beyond the line, 29 x 8, T = 352, 389 rows 50 against 46),
+// and units for half of 152 SMs take longer than four times as many of one tile (2 x 4 groups, T = 952,
+// 140 rows 11.5 against 14; up to 110 units, 2 senders of 2 x 8, T = 993, 397 rows 31 against 37, but 8 of
+// 5 x 2, T = 1444, 484 rows 40 against 38).  The rule reads the sender alone, so its scores do not
+// depend on the call's others.
+bool narrow_blocks(int64_t T, int64_t units) { return T <= kNarrowT || units <= kNarrowUnits; }
 
 // CTAs of a pass of `units` units: one an SM, a multiple of the row-chunk count when every sender
 // has the same one (CTAs k, k + grid / n_rc, ... then walk the same K tiles in step, so that a
@@ -1368,9 +1647,9 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
         tb->p_inf = b.p_inf;
         tb->ph = b.pool_half;
         tb->err = err;
-        tb->max_rc1 = tb->max_rc2 = 1;
-        tb->weight1 = tb->weight2 = 0;
-        tb->paged = tb->few = 0;
+        tb->max_rc1 = 1;
+        tb->weight1 = 0;
+        tb->paged = 0;
         int rows1 = kRowHalf, rows2 = kRowHalf;
         int64_t staged = 0;
         const int b_first = firsts.back();
@@ -1413,19 +1692,17 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             d.chunk1 = stats_chunk(s.T, nS);
             d.n_chunk1 = (int32_t)(4 * ((s.T + d.chunk1 - 1) / d.chunk1));   // one partial per (chunk, column quarter)
             d.n_blk2 = (int32_t)((s.T + kOut2 - 1) / kOut2);
-            d.share = s.T <= kOutW ? 2 : (s.T <= 2 * kOutW ? 1 : 0);
-            tb->few |= d.share > 0 || d.R - (d.halves - 1) * kRowHalf <= few_rows(G);
             d.n_rc1 = (d.halves + kHalves1 - 1) / kHalves1;
             d.n_rc2 = (d.halves + kHalves2 - 1) / kHalves2;
+            d.narrow = narrow_blocks(s.T, (int64_t)nS * d.n_blk2 * d.n_rc2);
+            if (d.narrow) d.n_blk2 = (int32_t)((s.T + kOutN - 1) / kOutN);
             d.stats = b.stats + s.stats_off;
             d.part = b.part + s.part_off;
             tb->max_rc1 = tb->max_rc1 > d.n_rc1 ? tb->max_rc1 : d.n_rc1;
-            tb->max_rc2 = tb->max_rc2 > d.n_rc2 ? tb->max_rc2 : d.n_rc2;
             const int r1 = (d.halves + d.n_rc1 - 1) / d.n_rc1 * kRowHalf, r2 = (d.halves + d.n_rc2 - 1) / d.n_rc2 * kRowHalf;
             rows1 = rows1 > r1 ? rows1 : r1;
             rows2 = rows2 > r2 ? rows2 : r2;
             tb->weight1 += (int64_t)nS * (d.n_chunk1 / 4) * d.halves;
-            tb->weight2 += (int64_t)nS * d.n_blk2 * d.halves;
             const cuuint64_t kd[4] = {(cuuint64_t)d_head, (cuuint64_t)s.T, (cuuint64_t)b.n_kv_heads,
                                       (cuuint64_t)b.n_layers};
             const cuuint64_t ks[3] = {(cuuint64_t)kpos * 2, (cuuint64_t)kh * 2, (cuuint64_t)kl * 2};
@@ -1444,8 +1721,14 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
                                        kd[2], kd[3]};
             const cuuint64_t k5s[4] = {4 * ks[0], ks[0], ks[1], ks[2]};
             const cuuint32_t k5box[5] = {64, 32, 1, 1, 1};
-            bool ok4 = encode_nd(&mp2.k[0], kp, 5, k5d, k5s, k5box, CU_TENSOR_MAP_SWIZZLE_128B);
-            if (s.T % 4 != 0) ok4 = ok4 && encode_nd(&mp2.k[1], kp, 4, kd, ks, kbox, CU_TENSOR_MAP_SWIZZLE_128B, 4);
+            const cuuint32_t k32box[4] = {64, 32, 1, 1};
+            bool ok4;
+            if (d.narrow) {
+                ok4 = encode_4d(&mp2.k[1], kp, kd, ks, k32box);
+            } else {
+                ok4 = encode_nd(&mp2.k[0], kp, 5, k5d, k5s, k5box, CU_TENSOR_MAP_SWIZZLE_128B);
+                if (s.T % 4 != 0) ok4 = ok4 && encode_nd(&mp2.k[1], kp, 4, kd, ks, kbox, CU_TENSOR_MAP_SWIZZLE_128B, 4);
+            }
             bool ok1 = encode_4d(&mp.k[fused ? 2 : 0], kp, kd, ks, kbox);
             if (fused) {
                 const cuuint64_t rows = (cuuint64_t)1 << s.pm.shift;
@@ -1485,14 +1768,13 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
         TcBatch* tb = batches[k].get();
         const int b0 = firsts[k];
         // row chunks in step only when all senders have the same number of them
-        int rc1 = tb->max_rc1, rc2 = tb->max_rc2;
-        int64_t units1 = 0, units2 = 0;
+        int rc1 = tb->max_rc1;
+        int64_t units1 = 0;
         for (int j = 0; j < tb->n; ++j) {
             const TcSender& d = tb->s[j];
             if (d.n_rc1 != tb->max_rc1) rc1 = 1;
-            if (d.n_rc2 != tb->max_rc2) rc2 = 1;
             units1 += (int64_t)nS * (d.n_chunk1 / 4) * d.n_rc1;
-            units2 += (int64_t)nS * d.n_blk2 * d.n_rc2;
+            b.s[b0 + j].n_rc = d.n_rc2;   // partials for the finalize kernel
         }
         stage_mark(b.timer, kStageStart, st);
         e = launch_depage(*depages[k], st, num_sms);   // timed with pass 1
@@ -1514,13 +1796,31 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             }
             stage_mark(b.timer, kStageCombine, st);
         }
-        if (e == cudaSuccess) {
-            const int g2 = pass_grid(units2, num_sms, rc2);
-            std::copy(maps2[k].get(), maps2[k].get() + tb->n, tb->maps);
-            e = d_head == 128 ? launch_accum_d<128>(*tb, g2, st) : launch_accum_d<64>(*tb, g2, st);
-            stage_mark(b.timer, kStageAccum, st);
+        // pass 2: the senders of blocks of four tiles, then those of one
+        const std::vector<TcSender> all(tb->s, tb->s + tb->n);
+        for (int narrow = 0; narrow < 2 && e == cudaSuccess; ++narrow) {
+            tb->n = tb->few = 0;
+            tb->weight2 = 0;
+            tb->max_rc2 = 1;
+            bool same_rc = true;
+            int64_t units2 = 0;
+            for (size_t j = 0; j < all.size(); ++j) {
+                const TcSender& d = all[j];
+                if (d.narrow != narrow) continue;
+                same_rc = same_rc && (tb->n == 0 || d.n_rc2 == tb->max_rc2);
+                tb->max_rc2 = tb->max_rc2 > d.n_rc2 ? tb->max_rc2 : d.n_rc2;
+                tb->weight2 += (int64_t)nS * d.n_blk2 * d.halves;
+                units2 += (int64_t)nS * d.n_blk2 * d.n_rc2;
+                tb->few |= (G > 1 || d_head == 64) && d.R - (d.halves - 1) * kRowHalf <= kFewRows;
+                tb->maps[tb->n] = maps2[k][j];
+                tb->s[tb->n++] = d;
+            }
+            if (tb->n == 0) continue;
+            const int g2 = pass_grid(units2, num_sms, same_rc ? tb->max_rc2 : 1);
+            if (narrow) e = d_head == 128 ? launch_narrow_d<128>(*tb, g2, st) : launch_narrow_d<64>(*tb, g2, st);
+            else e = d_head == 128 ? launch_accum_d<128>(*tb, g2, st) : launch_accum_d<64>(*tb, g2, st);
         }
-        for (int j = 0; j < tb->n; ++j) b.s[b0 + j].n_rc = tb->s[j].n_rc2;   // partials for the finalize kernel
+        if (e == cudaSuccess) stage_mark(b.timer, kStageAccum, st);
     }
     return e;
 }

@@ -9,6 +9,8 @@ Tolerance: a logit is a 32-bit sum of at most 128 products of bf16 values, off b
 the row's offset adds 2^-24 of itself.  A score is a mean of exponentials times the square of a
 ratio of such means, so its relative error is a few times the logits': 5e-5 bounds it.
 """
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -70,29 +72,41 @@ def test_scores(case):
 @pytest.mark.parametrize("d", [64, 128])
 def test_every_pass_2_instantiation(d, G, few):
     """k_accum_tc<d, G, pool_width / 2, p = 2, another or infinity, few>: `few` where a sender's last 128
-    query rows are at most 64 (96 for G = 1).  T: four blocks, the last one ragged."""
-    m = {1: 65, 2: 66, 4: 66}[G] if few else {1: 100, 2: 100, 4: 90}[G]
-    T = 1501
-    w = synth.custom_workload(synth.Shape(1, 2 * G, 2, d), [T], m, seed=10 * d + G, n_planted_spans=2)
-    K, Q, S = w.senders[0].K.cuda(), w.queries[0].cuda(), torch.empty(T, device="cuda")
-    o = oracle.default()
-    for pool_width in (1, 3, 5, 7):
+    query rows are at most 64.  26 groups, so that three blocks of 480 positions are more than the units
+    that go by blocks of one tile; T around the ends of blocks and lane quarters, each remainder of four.
+    Against the definition in 64 bits."""
+    m = {1: 140, 2: 66, 4: 66}[G] if few else {1: 100, 2: 100, 4: 90}[G]
+    nL, Hkv, Ts = 13, 2, [1440, 1441, 1442, 1443, 1559, 1560, 1561, 1700]
+    gen = torch.Generator(device="cuda").manual_seed(10 * d + G)
+    draw = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    K, Q = draw(nL, Hkv, max(Ts), d), draw(nL, m, Hkv * G, d)
+    q = Q.double().view(nL, m, Hkv, G, d).permute(0, 2, 1, 3, 4).reshape(nL, Hkv, m * G, d)
+    z = q @ K.double().transpose(-1, -2) / math.sqrt(d)
+    bs = [torch.softmax(z[..., :T], -1).view(nL * Hkv, m, G, T).mean(2) for T in Ts]
+    out = [torch.empty(T, device="cuda") for T in Ts]
+    for width in (1, 3, 5, 7):
+        widest = lambda x: torch.nn.functional.max_pool1d(x, width, 1, width // 2)
+        pooled = [(widest(b.sum(0).mean(0)[None])[0] / Hkv, widest(b), widest(b.mean(1))) for b in bs]
         for p in (2.0, 3.0, float("inf")):
-            c = make_cb(w.spec.shape, T, m, 1, pool_width=pool_width, p=p)
-            c.score([K], [Q], [S])
+            c = cb.CacheBack(nL, Hkv * G, Hkv, d, m, max(Ts), len(Ts), p=p, pool_width=width)
+            c.score([K[:, :, :T] for T in Ts], [Q] * len(Ts), out)
             c.sync_status()
             assert c.score_path() == 2
-            ref = oracle_scores(o, w.senders[0].K, w.queries[0], p=p, pool_w=pool_width)["S"]
-            assert_scores_close(S.cpu().numpy(), ref, rtol=RTOL)
+            for (U, N, D), got in zip(pooled, out):
+                if math.isinf(p):
+                    C = N.amax((0, 1)) / D.amax(0)
+                else:
+                    C = ((N ** p).mean(1).sum(0) / (D ** p).sum(0)) ** (1 / (p - 1))
+                assert_scores_close(got.cpu().numpy(), (U * C ** 2).cpu().numpy(), rtol=RTOL)
 
 
 @pytest.mark.parametrize("pool_width,p", [(7, 2.0), (1, 3.0), (5, float("inf"))])
 @pytest.mark.parametrize("G", [1, 2, 4])
 def test_few_rows_and_short_senders(G, pool_width, p):
-    """Pass 2 hands a half's columns to the warps in eights up to 64 rows (96 for G = 1), and lane
-    quarters share positions up to 240 of them: both sides of each line, in one call, beside a long
-    sender; every sender's scores are also those of a call of its own."""
-    Ts, rows = [1, 119, 120, 121, 239, 240, 241, 700], [4, 32, 36, 64, 68, 96, 100, 128, 132, 196]
+    """Pass 2 hands a half's columns to the warps in eights up to 64 rows, and takes senders
+    of up to 312 positions, or of few blocks of 480, in blocks of one tile (104 outputs): both sides
+    of each line, in one call; every sender's scores are also those of a call of its own."""
+    Ts, rows = [1, 26, 104, 105, 312, 313, 2100], [4, 32, 36, 64, 68, 96, 100, 128, 132, 196]
     for d in (64, 128):
         o = oracle.default()
         for r in rows:
