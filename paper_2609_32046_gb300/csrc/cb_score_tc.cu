@@ -73,7 +73,7 @@ constexpr int64_t kLongChunkUnits = 1024;  // pass-1 units from which chunks are
 constexpr int kOutW = 128 - 2 * kMargin;         // 120 output positions per pass-2 lane quarter
 constexpr int kOut2 = 4 * kOutW;                 // 480 output positions per pass-2 block
 constexpr int kMarginN = 3, kOutNW = 32 - 2 * kMarginN, kOutN = 4 * kOutNW;   // the same of k_narrow_tc: 3, 26, 104
-constexpr int64_t kNarrowT = 3 * kOutN, kNarrowUnits = 76;   // senders of pass 2 with blocks of one tile (narrow_blocks)
+constexpr int64_t kNarrowUnits = 33;             // pass-2 units up to which blocks are of one tile (narrow_blocks)
 constexpr uint32_t kTmemCols = 512;
 constexpr uint64_t kWaitNs = 1000000000ull;      // 1 s per wait
 constexpr uint32_t kPollNs = 1000000u;           // longest suspension of one poll (woken at completion)
@@ -115,7 +115,7 @@ struct TcBatch {
     int32_t n;
     int32_t nL, Hq, Hkv, G, log2g;
     int32_t stages1, rows1;       // pass 1: K ring stages, Q rows held
-    int32_t kbufs, rows2;         // pass 2: K blocks in flight (1 or 2, four tiles each), Q rows held
+    int32_t kbufs, rows2;         // pass 2: K blocks in flight (1 or 2, four tiles each; k_narrow_tc: K tiles), Q rows held
     int32_t max_rc1, max_rc2;
     float sl2e, p;
     int32_t p_inf, ph;
@@ -154,6 +154,7 @@ struct Ctl {
     uint64_t k_full[kMaxStages], k_empty[kMaxStages];
     uint64_t t_full[4], t_empty[4];   // ring of TMEM buffers of 128 columns
     uint64_t q_full, q_empty, drain[2], o_full;
+    uint64_t q2_full[2], q2_empty[2];   // k_narrow_tc's two Q buffers
     uint64_t stall;         // failure-detection test: a barrier nothing arrives on
     uint64_t wait_ns;       // limit of one bounded wait
     uint64_t xb, xe;        // pass 2: a block's sums written by the epilogue and read by warp 3
@@ -321,6 +322,10 @@ __device__ __forceinline__ void init_ctl(Ctl* ctl, int k_releasers, uint64_t wai
     mbar_init(&ctl->xe, 1);
     mbar_init(&ctl->q_full, 1);
     mbar_init(&ctl->q_empty, 2);
+    for (int b = 0; b < 2; ++b) {
+        mbar_init(&ctl->q2_full[b], 1);
+        mbar_init(&ctl->q2_empty[b], 2);
+    }
     mbar_init(&ctl->drain[0], 1);
     mbar_init(&ctl->drain[1], 1);
     mbar_init(&ctl->o_full, 1);
@@ -337,15 +342,15 @@ __device__ __forceinline__ void init_ctl(Ctl* ctl, int k_releasers, uint64_t wai
 // of a half hold anything: pass 1 writes nothing of theirs, pass 2's MMA does not read them.
 template <int D, int PASS>
 __device__ __forceinline__ void load_q(const TcBatch& bt, const TcMaps& mp, const Smem& sm, int s, int h0, int nh,
-                                       int q_rows) {
+                                       int q_rows, uint64_t* full) {
     const int l = s / bt.Hkv, g = s % bt.Hkv;
     const int rows = PASS == 1 ? bt.rows1 : bt.rows2;
-    mbar_arrive_expect_tx(&sm.ctl->q_full, (uint32_t)(nh * q_rows) * (D * 2 + (PASS == 2 ? 32 : 0)));
+    mbar_arrive_expect_tx(full, (uint32_t)(nh * q_rows) * (D * 2 + (PASS == 2 ? 32 : 0)));
     for (int h = 0; h < nh; ++h) {
         if (PASS == 2)
-            tma_load_3d(sm.ext + (size_t)h * kRowHalf * 32, &mp.k[2], &sm.ctl->q_full, 0, (h0 + h) * kRowHalf, s);
+            tma_load_3d(sm.ext + (size_t)h * kRowHalf * 32, &mp.k[2], full, 0, (h0 + h) * kRowHalf, s);
         for (int kb = 0; kb < D / 64; ++kb)
-            tma_load_4d(sm.q + ((size_t)kb * rows + h * kRowHalf) * 128, &mp.q, &sm.ctl->q_full, 64 * kb, g * bt.G,
+            tma_load_4d(sm.q + ((size_t)kb * rows + h * kRowHalf) * 128, &mp.q, full, 64 * kb, g * bt.G,
                         (h0 + h) * kRowHalf / bt.G, l);
     }
 }
@@ -587,7 +592,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
                         g = un.s % bt.Hkv;
                         if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 0))) break;
                         const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
-                        load_q<D, 1>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0, sd.q_rows);
+                        load_q<D, 1>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0, sd.q_rows,
+                                 &ctl->q_full);
                         ++qn;
                     }
                     const int64_t c0 = (int64_t)un.c * chunk;
@@ -883,7 +889,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                     g = un.s % bt.Hkv;
                     if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 8))) break;
                     const int h0 = rc_begin(sd.halves, sd.n_rc2, un.rc);
-                    load_q<D, 2>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0, sd.q_rows);
+                    load_q<D, 2>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0, sd.q_rows,
+                                 &ctl->q_full);
                     ++qn;
                 }
                 const int32_t t0 = un.c * kOut2 - kMargin;
@@ -1175,7 +1182,14 @@ template <int D, int G, int PH>
 __global__ void __launch_bounds__(kThreadsTc, 1) k_narrow_tc(const __grid_constant__ TcBatch bt) {
     constexpr int kTile = kTileRows * D * 2;
     extern __shared__ uint8_t smem_raw[];
-    const Smem sm = carve<D, 2>(smem_raw, bt);
+    Smem sm;   // [Q, offset terms] twice, ones, K tiles, Ctl, exchange of sums
+    const uint32_t q_bytes = (uint32_t)bt.rows2 * (D * 2 + 32);
+    sm.q = align1024(smem_raw);
+    sm.ext = sm.q + (size_t)bt.rows2 * D * 2;
+    sm.ones = sm.q + 2 * q_bytes;
+    sm.k = sm.ones + 128 * 32;
+    sm.ctl = reinterpret_cast<Ctl*>(sm.k + (size_t)bt.kbufs * kTile);
+    sm.epi = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(sm.ctl) + 512);
     Ctl* ctl = sm.ctl;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -1192,7 +1206,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_narrow_tc(const __grid_consta
     const uint32_t tmem = ctl->tmem_base;
     const int n_units = ctl->units;
     Unit un = ctl->first;
-    const int slots = 4 * bt.kbufs;
+    const int slots = bt.kbufs;
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
@@ -1211,9 +1225,14 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_narrow_tc(const __grid_consta
                     nc = sd.n_blk2;
                     l = un.s / bt.Hkv;
                     g = un.s % bt.Hkv;
-                    if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 8))) break;
+                    const uint32_t b = (uint32_t)qn & 1;
+                    if (!(ok = wait_bar(&ctl->q2_empty[b], (uint32_t)((qn >> 1) & 1) ^ 1u, ctl, bt.err, 8))) break;
                     const int h0 = rc_begin(sd.halves, sd.n_rc2, un.rc);
-                    load_q<D, 2>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0, sd.q_rows);
+                    Smem to = sm;
+                    to.q += b * q_bytes;
+                    to.ext += b * q_bytes;
+                    load_q<D, 2>(bt, mp, to, un.s, h0, rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0, sd.q_rows,
+                                 &ctl->q2_full[b]);
                     ++qn;
                 }
                 if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 9))) break;
@@ -1227,7 +1246,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_narrow_tc(const __grid_consta
             }
             for (int64_t k = kt - slots > 0 ? kt - slots : 0; k < kt; ++k)
                 drain_wait(&ctl->k_full[k % slots], (uint32_t)((k / slots) & 1));
-            if (qn > 0) drain_wait(&ctl->q_full, (uint32_t)((qn - 1) & 1));
+            for (int64_t k = qn - 2 > 0 ? qn - 2 : 0; k < qn; ++k) drain_wait(&ctl->q2_full[k & 1], (uint32_t)((k >> 1) & 1));
             drain_wait(&ctl->o_full, 0);
         }
     } else if (warp <= 2) {
@@ -1241,7 +1260,8 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_narrow_tc(const __grid_consta
             const uint64_t ones_desc = smem_desc_sw32(smem_u32(sm.ones)), ext_desc = smem_desc_sw32(smem_u32(sm.ext));
             const uint32_t ext_hi = (uint32_t)(ext_desc >> 32), ext_lo = (uint32_t)ext_desc;
             const uint64_t qd = smem_desc_sw128(smem_u32(sm.q));
-            const uint32_t hi = (uint32_t)(qd >> 32), q_lo = (uint32_t)qd;
+            const uint32_t hi = (uint32_t)(qd >> 32);
+            uint32_t q_lo = 0, e_lo = 0;   // of the current Q buffer
             const uint32_t k_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.k));
             const uint32_t q_blk = (uint32_t)bt.rows2 * 128 >> 4;
             constexpr uint32_t idesc = idesc_bf16_f32(128, 128);
@@ -1254,8 +1274,10 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_narrow_tc(const __grid_consta
                     const int h1 = rc_begin(sd.halves, sd.n_rc2, un.rc + 1);
                     nh = h1 - rc_begin(sd.halves, sd.n_rc2, un.rc);
                     id_last = idesc_bf16_f32(128, min(kRowHalf, (sd.R - (h1 - 1) * kRowHalf + 31) & ~31));
-                    if (u > 0) umma_commit(&ctl->q_empty);
-                    if (!(ok = wait_bar(&ctl->q_full, qn & 1, ctl, bt.err, 10))) break;
+                    if (u > 0) umma_commit(&ctl->q2_empty[(qn - 1) & 1]);
+                    if (!(ok = wait_bar(&ctl->q2_full[qn & 1], (qn >> 1) & 1, ctl, bt.err, 10))) break;
+                    q_lo = (uint32_t)qd + (qn & 1) * (q_bytes >> 4);
+                    e_lo = ext_lo + (qn & 1) * (q_bytes >> 4);
                     ++qn;
                 }
                 if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 11))) break;
@@ -1265,7 +1287,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_narrow_tc(const __grid_consta
                     tc_fence_after();
                     mma_d<D>(tmem + buf * 128, k_lo + (uint32_t)st * (kTile >> 4), kTileRows * 128 >> 4,
                              q_lo + h * (kRowHalf * 128 >> 4), q_blk, hi, id);
-                    umma_bf16(tmem + buf * 128, ones_desc, desc64(ext_lo + h * (kRowHalf * 32 >> 4), ext_hi), id, 1u);
+                    umma_bf16(tmem + buf * 128, ones_desc, desc64(e_lo + h * (kRowHalf * 32 >> 4), ext_hi), id, 1u);
                     umma_commit(&ctl->t_full[buf]);
                 }
                 if (!ok) break;
@@ -1411,6 +1433,10 @@ inline size_t smem2_bytes(int d, int rows, int kbufs) {
     return 1024 + (size_t)rows * (d * 2 + 32) + 128 * 32 + (size_t)kbufs * 4 * kTileRows * d * 2 + 512 + 4 * 8 * 128 * 4;
 }
 
+inline size_t smem_narrow_bytes(int d, int rows, int tiles) {
+    return 1024 + (size_t)2 * rows * (d * 2 + 32) + 128 * 32 + (size_t)tiles * kTileRows * d * 2 + 512 + 4 * 8 * 32 * 4;
+}
+
 template <int D, int G, int PH, int P, bool FEW>
 cudaError_t launch_accum_few(const TcBatch& tb, int grid, cudaStream_t st) {
     const size_t smem = smem2_bytes(D, tb.rows2, tb.kbufs);
@@ -1445,7 +1471,7 @@ cudaError_t launch_accum_g(const TcBatch& tb, int grid, cudaStream_t st) {
 
 template <int D, int G, int PH>
 cudaError_t launch_narrow(const TcBatch& tb, int grid, cudaStream_t st) {
-    const size_t smem = smem2_bytes(D, tb.rows2, tb.kbufs);
+    const size_t smem = smem_narrow_bytes(D, tb.rows2, tb.kbufs);
     static std::atomic<uint64_t> done{0};
     const cudaError_t e = allow_smem(k_narrow_tc<D, G, PH>, done);
     if (e != cudaSuccess) return e;
@@ -1572,13 +1598,16 @@ int32_t stats_chunk(int64_t T, int nS) {
 }
 
 // Whether pass 2 takes a sender of T positions in blocks of one tile, given its units (blocks of 480,
-// groups and row chunks): a sender of few positions leaves lane quarters idle (20 layers x
-// 8 groups, 5 x T = 103, 6 rows: 20 against 26 us; beyond the line, 29 x 8, T = 352, 389 rows 50 against 46),
-// and units for half of 152 SMs take longer than four times as many of one tile (2 x 4 groups, T = 952,
-// 140 rows 11.5 against 14; up to 110 units, 2 senders of 2 x 8, T = 993, 397 rows 31 against 37, but 8 of
-// 5 x 2, T = 1444, 484 rows 40 against 38).  The rule reads the sender alone, so its scores do not
-// depend on the call's others.
-bool narrow_blocks(int64_t T, int64_t units) { return T <= kNarrowT || units <= kNarrowUnits; }
+// groups and row chunks): a sender of few positions leaves lane quarters idle (d = 128, 20 layers x 8 groups,
+// 5 x T = 103, 6 rows: 16 against 26 us; beyond the line, 29 x 8, T = 352, 389 rows 50 against 46; d = 64, whose
+// rounds of 32 columns are better packed, beyond its line, 7 x 4, 5 x T = 212, 188 rows 17 against 16),
+// and where four times as many blocks of one tile still fit a wave of 152 SMs they take a third of the time
+// (2 x 4 groups, T = 952, 140 rows: pass 2 11.5 against 14).  The rule reads the sender alone, so its scores do
+// not depend on the call's others; many senders of few units fill the SMs together, and then blocks of
+// 480 would take up to a third less (8 of 4 x 8, T = 900, 240 rows: 64 units each, beyond the line, 34 against 39).
+bool narrow_blocks(int head_dim, int64_t T, int64_t units) {
+    return T <= (head_dim == 128 ? 3 : 2) * kOutN || units <= kNarrowUnits;
+}
 
 // CTAs of a pass of `units` units: one an SM, a multiple of the row-chunk count when every sender
 // has the same one (CTAs k, k + grid / n_rc, ... then walk the same K tiles in step, so that a
@@ -1650,7 +1679,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
         tb->max_rc1 = 1;
         tb->weight1 = 0;
         tb->paged = 0;
-        int rows1 = kRowHalf, rows2 = kRowHalf;
+        int rows1 = kRowHalf;
         int64_t staged = 0;
         const int b_first = firsts.back();
         for (int k = 0; k < nb; ++k) {
@@ -1694,14 +1723,13 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             d.n_blk2 = (int32_t)((s.T + kOut2 - 1) / kOut2);
             d.n_rc1 = (d.halves + kHalves1 - 1) / kHalves1;
             d.n_rc2 = (d.halves + kHalves2 - 1) / kHalves2;
-            d.narrow = narrow_blocks(s.T, (int64_t)nS * d.n_blk2 * d.n_rc2);
+            d.narrow = narrow_blocks(d_head, s.T, (int64_t)nS * d.n_blk2 * d.n_rc2);
             if (d.narrow) d.n_blk2 = (int32_t)((s.T + kOutN - 1) / kOutN);
             d.stats = b.stats + s.stats_off;
             d.part = b.part + s.part_off;
             tb->max_rc1 = tb->max_rc1 > d.n_rc1 ? tb->max_rc1 : d.n_rc1;
-            const int r1 = (d.halves + d.n_rc1 - 1) / d.n_rc1 * kRowHalf, r2 = (d.halves + d.n_rc2 - 1) / d.n_rc2 * kRowHalf;
+            const int r1 = (d.halves + d.n_rc1 - 1) / d.n_rc1 * kRowHalf;
             rows1 = rows1 > r1 ? rows1 : r1;
-            rows2 = rows2 > r2 ? rows2 : r2;
             tb->weight1 += (int64_t)nS * (d.n_chunk1 / 4) * d.halves;
             const cuuint64_t kd[4] = {(cuuint64_t)d_head, (cuuint64_t)s.T, (cuuint64_t)b.n_kv_heads,
                                       (cuuint64_t)b.n_layers};
@@ -1756,10 +1784,8 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             return cudaErrorNotSupported;
         }
         tb->rows1 = rows1;
-        tb->rows2 = rows2;
         tb->stages1 = 4;
         while (tb->stages1 > 2 && smem1_bytes(d_head, rows1, tb->stages1) > kSmemMax) --tb->stages1;
-        tb->kbufs = smem2_bytes(d_head, rows2, 2) <= kSmemMax ? 2 : 1;
         tb->wait_ns = b.wait_ns;
         tb->stall = batches.size() == 1 ? b.stall : 0;   // the first launch only
     }
@@ -1802,6 +1828,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             tb->n = tb->few = 0;
             tb->weight2 = 0;
             tb->max_rc2 = 1;
+            tb->rows2 = kRowHalf;
             bool same_rc = true;
             int64_t units2 = 0;
             for (size_t j = 0; j < all.size(); ++j) {
@@ -1809,6 +1836,8 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
                 if (d.narrow != narrow) continue;
                 same_rc = same_rc && (tb->n == 0 || d.n_rc2 == tb->max_rc2);
                 tb->max_rc2 = tb->max_rc2 > d.n_rc2 ? tb->max_rc2 : d.n_rc2;
+                const int r2 = (d.halves + d.n_rc2 - 1) / d.n_rc2 * kRowHalf;
+                tb->rows2 = tb->rows2 > r2 ? tb->rows2 : r2;
                 tb->weight2 += (int64_t)nS * d.n_blk2 * d.halves;
                 units2 += (int64_t)nS * d.n_blk2 * d.n_rc2;
                 tb->few |= (G > 1 || d_head == 64) && d.R - (d.halves - 1) * kRowHalf <= kFewRows;
@@ -1816,6 +1845,12 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
                 tb->s[tb->n++] = d;
             }
             if (tb->n == 0) continue;
+            if (narrow) {
+                tb->kbufs = kMaxStages;
+                while (smem_narrow_bytes(d_head, tb->rows2, tb->kbufs) > kSmemMax) --tb->kbufs;
+            } else {
+                tb->kbufs = smem2_bytes(d_head, tb->rows2, 2) <= kSmemMax ? 2 : 1;
+            }
             const int g2 = pass_grid(units2, num_sms, same_rc ? tb->max_rc2 : 1);
             if (narrow) e = d_head == 128 ? launch_narrow_d<128>(*tb, g2, st) : launch_narrow_d<64>(*tb, g2, st);
             else e = d_head == 128 ? launch_accum_d<128>(*tb, g2, st) : launch_accum_d<64>(*tb, g2, st);

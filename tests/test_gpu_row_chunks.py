@@ -67,65 +67,72 @@ def test_scores(case):
                      Kself=kself)
 
 
+def _attention_64(K, Q, Ts):
+    """b[group, token, position] in 64 bits (softmax over positions, mean over a group's heads), per T."""
+    nL, Hkv, _, d = K.shape
+    m, G = Q.shape[1], Q.shape[2] // Hkv
+    q = Q.double().view(nL, m, Hkv, G, d).permute(0, 2, 1, 3, 4).reshape(nL, Hkv, m * G, d)
+    z = q @ K.double().transpose(-1, -2) / math.sqrt(d)
+    return [torch.softmax(z[..., :T], -1).view(nL * Hkv, m, G, T).mean(2) for T in Ts]
+
+
+def _score_64(b, Hkv, width, p):
+    """Scores (alpha = 2) of b by their definition."""
+    widest = lambda x: torch.nn.functional.max_pool1d(x, width, 1, width // 2)
+    U, N, D = widest(b.sum(0).mean(0)[None])[0] / Hkv, widest(b), widest(b.mean(1))
+    if math.isinf(p):
+        return U * (N.amax((0, 1)) / D.amax(0)) ** 2
+    return U * ((N ** p).mean(1).sum(0) / (D ** p).sum(0)) ** (2 / (p - 1))
+
+
 @pytest.mark.parametrize("few", [False, True], ids=["full", "few"])
 @pytest.mark.parametrize("G", [1, 2, 4])
 @pytest.mark.parametrize("d", [64, 128])
 def test_every_pass_2_instantiation(d, G, few):
     """k_accum_tc<d, G, pool_width / 2, p = 2, another or infinity, few>: `few` where a sender's last 128
     query rows are at most 64.  26 groups, so that three blocks of 480 positions are more than the units
-    that go by blocks of one tile; T around the ends of blocks and lane quarters, each remainder of four.
-    Against the definition in 64 bits."""
+    that go by blocks of one tile; T around the ends of blocks and lane quarters, each remainder of four."""
     m = {1: 140, 2: 66, 4: 66}[G] if few else {1: 100, 2: 100, 4: 90}[G]
     nL, Hkv, Ts = 13, 2, [1440, 1441, 1442, 1443, 1559, 1560, 1561, 1700]
     gen = torch.Generator(device="cuda").manual_seed(10 * d + G)
     draw = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
     K, Q = draw(nL, Hkv, max(Ts), d), draw(nL, m, Hkv * G, d)
-    q = Q.double().view(nL, m, Hkv, G, d).permute(0, 2, 1, 3, 4).reshape(nL, Hkv, m * G, d)
-    z = q @ K.double().transpose(-1, -2) / math.sqrt(d)
-    bs = [torch.softmax(z[..., :T], -1).view(nL * Hkv, m, G, T).mean(2) for T in Ts]
-    out = [torch.empty(T, device="cuda") for T in Ts]
+    bs, out = _attention_64(K, Q, Ts), [torch.empty(T, device="cuda") for T in Ts]
     for width in (1, 3, 5, 7):
-        widest = lambda x: torch.nn.functional.max_pool1d(x, width, 1, width // 2)
-        pooled = [(widest(b.sum(0).mean(0)[None])[0] / Hkv, widest(b), widest(b.mean(1))) for b in bs]
         for p in (2.0, 3.0, float("inf")):
             c = cb.CacheBack(nL, Hkv * G, Hkv, d, m, max(Ts), len(Ts), p=p, pool_width=width)
             c.score([K[:, :, :T] for T in Ts], [Q] * len(Ts), out)
             c.sync_status()
             assert c.score_path() == 2
-            for (U, N, D), got in zip(pooled, out):
-                if math.isinf(p):
-                    C = N.amax((0, 1)) / D.amax(0)
-                else:
-                    C = ((N ** p).mean(1).sum(0) / (D ** p).sum(0)) ** (1 / (p - 1))
-                assert_scores_close(got.cpu().numpy(), (U * C ** 2).cpu().numpy(), rtol=RTOL)
+            for b, got in zip(bs, out):
+                assert_scores_close(got.cpu().numpy(), _score_64(b, Hkv, width, p).cpu().numpy(), rtol=RTOL)
 
 
-@pytest.mark.parametrize("pool_width,p", [(7, 2.0), (1, 3.0), (5, float("inf"))])
-@pytest.mark.parametrize("G", [1, 2, 4])
-def test_few_rows_and_short_senders(G, pool_width, p):
-    """Pass 2 hands a half's columns to the warps in eights up to 64 rows, and takes senders
-    of up to 312 positions, or of few blocks of 480, in blocks of one tile (104 outputs): both sides
-    of each line, in one call; every sender's scores are also those of a call of its own."""
-    Ts, rows = [1, 26, 104, 105, 312, 313, 2100], [4, 32, 36, 64, 68, 96, 100, 128, 132, 196]
-    for d in (64, 128):
-        o = oracle.default()
-        for r in rows:
-            m = r // G
-            if d == 64 and m <= 64:
-                m += 64          # (fewer tokens: the mma.sync passes)
-            w = synth.custom_workload(synth.Shape(1, 2 * G, 2, d), Ts, m, seed=r + G, n_planted_spans=1)
-            Ks, Qs = [s.K.cuda() for s in w.senders], [w.queries[s.task].cuda() for s in w.senders]
-            c = make_cb(w.spec.shape, max(Ts), m, len(Ts), pool_width=pool_width, p=p)
-            out, S = [torch.empty(T, device="cuda") for T in Ts], torch.empty(max(Ts), device="cuda")
-            c.score(Ks, Qs, out)
+@pytest.mark.parametrize("G,width,p", [(1, 7, 2.0), (1, 1, 3.0), (2, 5, 2.0), (2, 3, float("inf")), (4, 7, 3.0),
+                                       (4, 5, float("inf")), (4, 1, 2.0), (2, 7, 2.0), (1, 3, 1.5)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_few_rows_and_short_senders(d, G, width, p):
+    """Pass 2 hands a half's columns to the warps in eights up to 64 rows, and takes senders of up to 312
+    positions (d = 64: 208), or of up to 33 blocks of 480, in blocks of one tile (104 outputs): both
+    sides of each line, in one call; every sender's scores are also those of a call of its own."""
+    nL, Hkv, Ts = 9, 4, [1, 26, 104, 105, 208, 209, 312, 313, 1100]   # 36 groups
+    gen = torch.Generator(device="cuda").manual_seed(d + G)
+    draw = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    for rows in (4, 32, 36, 64, 68, 96, 100, 128, 132, 196, 264):
+        m = rows // G
+        if d == 64 and m <= 64:
+            m += 64          # (fewer tokens: the mma.sync passes)
+        K, Q = draw(nL, Hkv, max(Ts), d), draw(nL, m, Hkv * G, d)
+        c = cb.CacheBack(nL, Hkv * G, Hkv, d, m, max(Ts), len(Ts), p=p, pool_width=width)
+        out, S = [torch.empty(T, device="cuda") for T in Ts], torch.empty(max(Ts), device="cuda")
+        c.score([K[:, :, :T] for T in Ts], [Q] * len(Ts), out)
+        c.sync_status()
+        assert c.score_path() == 2
+        for b, T, got in zip(_attention_64(K, Q, Ts), Ts, out):
+            assert_scores_close(got.cpu().numpy(), _score_64(b, Hkv, width, p).cpu().numpy(), rtol=RTOL)
+            c.score([K[:, :, :T]], [Q], [S[:T]])
             c.sync_status()
-            assert c.score_path() == 2
-            for i, s in enumerate(w.senders):
-                ref = oracle_scores(o, s.K, w.queries[s.task], p=p, pool_w=pool_width)["S"]
-                assert_scores_close(out[i].cpu().numpy(), ref, rtol=RTOL)
-                c.score([Ks[i]], [Qs[i]], [S[:Ts[i]]])
-                c.sync_status()
-                assert torch.equal(S[:Ts[i]].view(torch.int32), out[i].view(torch.int32)), (d, r, i)
+            assert torch.equal(S[:T].view(torch.int32), got.view(torch.int32)), (rows, T)
 
 
 @pytest.mark.parametrize("own", [False, True])
