@@ -137,10 +137,8 @@ struct DepageBatch {
 // nearly all of it outside (0 in place of 3) rows of one large weight are off by as much.  Errors of
 // scores against 64 bits: 36 layers, T = 8192, 4.0e-7 -> 1.9e-7; d = 64, 24 layers, T = 7001, 2.9e-7 ->
 // 2.1e-7 (mma.sync passes 2.6e-7).
-__host__ __device__ inline int offset_centre(int64_t T, int G) {
-    int n = (G == 4 ? 2 : G - 1) - 3;
-    for (int64_t t = T; t > 1; t >>= 1) ++n;
-    return n;
+__device__ __forceinline__ int offset_centre(int64_t T, int G) {   // (T < 2^31)
+    return (G == 4 ? 2 : G - 1) - 3 + 31 - __clz((int)T);
 }
 constexpr int kExtCols = 16;   // one bf16 K-step: the extra contraction column block of pass 2
 

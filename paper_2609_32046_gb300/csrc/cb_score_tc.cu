@@ -79,8 +79,10 @@ constexpr uint64_t kWaitNs = 1000000000ull;      // 1 s per wait
 constexpr uint32_t kPollNs = 1000000u;           // longest suspension of one poll (woken at completion)
 constexpr int kMaxTcSenders = 32;         // their tensor maps fill most of the 32,764 bytes of kernel parameters
 
-// Rows up to which a half's columns go to the warps in eights (pass 2; for G = 1 and d = 128, always).
-constexpr int kFewRows = 64;
+// Rows up to which a sender's last half's columns go to the warps in eights (pass 2; for G = 1 and d = 128,
+// all halves'), and the most halves of such a sender: one half of ten gains less than the code
+// for it costs the others (12 layers, T = 6001, 1200 rows: 231 against 225 us).
+constexpr int kFewRows = 64, kFewHalves = 4;
 
 struct TcMaps {
     CUtensorMap k[3];     // pass 1: k[0] = 4D {d, T, Hkv, nL}, box {64, 128, 1, 1}; k[1] the same over the
@@ -104,6 +106,7 @@ struct TcSender {
     int32_t n_blk2;       // pass-2 blocks of positions
     int32_t n_rc1, n_rc2; // row chunks of each pass
     int32_t narrow;       // pass 2 takes blocks of one tile (k_narrow_tc)
+    int32_t few;          // pass 2 hands its last half's columns out in eights (FEW)
     int32_t m_self;       // query tokens whose own keys join the softmax (m or 0)
     int32_t chunk1;       // pass-1 positions per chunk
     const int32_t* pages; // block table of a paged sender that pass 1 reads itself, else null
@@ -121,7 +124,7 @@ struct TcBatch {
     int32_t p_inf, ph;
     int64_t weight1, weight2;     // work of each pass: 128-row halves over all units
     uint64_t wait_ns;     // limit of one bounded mbarrier wait
-    int32_t few;          // some sender needs the pass-2 instantiation FEW
+    int32_t few;          // some sender has `few`
     int32_t paged;        // some sender has `pages`: warp 3 of pass 1 stores its tiles
     int32_t stall;        // 1: CTA 0's pass-1 MMA issuer first waits on a barrier nothing arrives on
     uint32_t* err;
@@ -517,10 +520,209 @@ __device__ __forceinline__ void stats_rows(const TcBatch& bt, Ctl* ctl, uint32_t
     }
 }
 
+// The warps' work over the CTA's units, and where each role stands at its end, for a second run:
+// K tiles and Q loads issued or consumed, accumulator buffers filled or consumed, ring slot of the
+// next K tile and its phase parity.
+struct StatsAt {
+    int64_t kt;
+    uint32_t qn, n, ph;
+    int st;
+};
+
+template <int D, int NH, bool AGAIN>
+__device__ __forceinline__ StatsAt stats_run(const TcBatch& bt, const Smem& sm, uint32_t tmem, StatsAt at) {
+    constexpr int kTile = kTileRows * D * 2;
+    Ctl* ctl = sm.ctl;
+    const int warp = threadIdx.x >> 5;
+    const int stages = bt.stages1;
+    int64_t kt = at.kt;
+    uint32_t qn = at.qn, n = at.n, ph = at.ph;
+    int st = at.st;
+    const int n_units = ctl->units;
+    Unit un = ctl->first;
+
+    if (warp == 0) {
+        // ---------------- TMA producer ----------------
+        if (elect_one()) {
+            bool ok = true;
+            int nc = 0, l = 0, g = 0, n_self = 0, chunk = 0;
+            int64_t T = 0;
+            const int32_t* pages = nullptr;
+            int32_t n_pages = 0, ps = 0;
+            for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
+                const TcMaps& mp = bt.maps[un.i];
+                if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
+                    const TcSender& sd = bt.s[un.i];
+                    nc = n_c<1>(sd);
+                    chunk = sd.chunk1;
+                    n_self = self_tiles(sd);
+                    pages = sd.pages;
+                    n_pages = sd.n_pages;
+                    ps = sd.page_shift;
+                    T = sd.T;
+                    l = un.s / bt.Hkv;
+                    g = un.s % bt.Hkv;
+                    if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 0))) break;
+                    const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
+                    load_q<D, 1>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0, sd.q_rows,
+                             &ctl->q_full);
+                    ++qn;
+                }
+                const int64_t c0 = (int64_t)un.c * chunk;
+                const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows);
+                const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
+                for (int tile = 0; tile < n_tiles; ++tile) {
+                    const bool self = tile >= nt;
+                    const int32_t row = self ? (tile - nt) * kTileRows : (int32_t)(c0 + tile * kTileRows);
+                    // a tile's block-table entries, all in flight together while its slot is waited for
+                    const int box = ps < 7 ? 1 << ps : kTileRows;
+                    int32_t entry[kTileRows >> kMinPageShift];
+                    if (pages && !self) {
+#pragma unroll
+                        for (int r = 0; r < kTileRows >> kMinPageShift; ++r)
+                            if (r * box < kTileRows && row + r * box < T) entry[r] = __ldg(pages + ((row + r * box) >> ps));
+                    }
+                    if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 1))) break;
+                    mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
+                    if (pages && !self) {
+                        // one box a page (or 128 rows of one); a page past T, or outside the pool (recorded), is
+                        // the coordinate past the last page, which reads as zeros
+#pragma unroll
+                        for (int r = 0; r < kTileRows >> kMinPageShift; ++r) {
+                            if (r * box >= kTileRows) break;
+                            int32_t pg = n_pages;
+                            if (row + r * box < T) {
+                                pg = entry[r];
+                                if (pg < 0 || pg >= n_pages) {
+                                    pg = n_pages;
+                                    atomicOr(bt.err, kErrPageIndex);
+                                }
+                            }
+                            for (int kb = 0; kb < D / 64; ++kb)
+                                tma_load_5d(sm.k + (size_t)st * kTile + (kb * kTileRows + r * box) * 128, &mp.k[0],
+                                            &ctl->k_full[st], 64 * kb, (row + r * box) & ((1 << ps) - 1), pg, g, l);
+                        }
+                    } else {
+                        for (int kb = 0; kb < D / 64; ++kb)
+                            tma_load_4d(sm.k + (size_t)st * kTile + kb * kTileRows * 128, &mp.k[self ? 1 : 0],
+                                        &ctl->k_full[st], 64 * kb, row, g, l);
+                    }
+                    ++kt;
+                    if (++st == stages) { st = 0; ph ^= 1u; }
+                }
+            }
+            // drain: every issued load must land before the CTA exits
+            for (int64_t k = kt - stages > 0 ? kt - stages : 0; k < kt; ++k)
+                drain_wait(&ctl->k_full[k % stages], (uint32_t)((k / stages) & 1));
+            if (qn > 0) drain_wait(&ctl->q_full, (uint32_t)((qn - 1) & 1));
+        }
+    } else if (warp <= 2) {
+        // ---------------- MMA issuers ----------------
+        if (elect_one()) {
+            const uint32_t me = (uint32_t)warp - 1;
+            bool ok = true;
+            constexpr uint32_t idesc = idesc_bf16_f32(128, 128);
+            const uint64_t qd = smem_desc_sw128(smem_u32(sm.q));
+            const uint32_t hi = (uint32_t)(qd >> 32), q_lo = (uint32_t)qd;
+            const uint32_t k_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.k));
+            const uint32_t q_blk = (uint32_t)bt.rows1 * 128 >> 4;
+            // failure-detection test: wait on a barrier that nothing arrives on, so the bounded
+            // wait gives up, sets the abort flag and every role of this CTA leaves
+            if (!AGAIN && bt.stall && blockIdx.x == 0) ok = wait_bar(&ctl->stall, 0, ctl, bt.err, 6);
+            uint32_t nh = 0;
+            int nc = 0, n_self = 0, chunk = 0;
+            int64_t T = 0;
+            for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
+                if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
+                    const TcSender& sd = bt.s[un.i];
+                    nc = n_c<1>(sd);
+                    chunk = sd.chunk1;
+                    n_self = self_tiles(sd);
+                    T = sd.T;
+                    nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - rc_begin(sd.halves, sd.n_rc1, un.rc);
+                    if (u > 0) umma_commit(&ctl->q_empty);
+                    if (!(ok = wait_bar(&ctl->q_full, qn & 1, ctl, bt.err, 2))) break;
+                    ++qn;
+                }
+                const int64_t c0 = (int64_t)un.c * chunk;
+                const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows) +
+                               (un.c + 1 == nc ? n_self : 0);
+                for (int tile = 0; tile < nt; ++tile) {
+                    if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
+                    const uint32_t kt_lo = k_lo + (uint32_t)st * (kTile >> 4);
+                    for (uint32_t h = (n ^ me) & 1; h < nh; h += 2) {   // the tile's buffers n + h of my parity
+                        const uint32_t x = n + h, buf = x & 3;
+                        if (!(ok = wait_bar(&ctl->t_empty[buf], ((x >> 2) & 1) ^ 1, ctl, bt.err, 4))) break;
+                        tc_fence_after();
+                        mma_d<D>(tmem + buf * 128, q_lo + h * (kRowHalf * 128 >> 4), q_blk, kt_lo, kTileRows * 128 >> 4, hi,
+                                 idesc);
+                        umma_commit(&ctl->t_full[buf]);
+                    }
+                    if (!ok) break;
+                    n += nh;
+                    umma_commit(&ctl->k_empty[st]);
+                    if (++st == stages) { st = 0; ph ^= 1u; }
+                }
+            }
+            umma_commit(&ctl->q_empty);
+            umma_commit(&ctl->drain[me]);
+            drain_wait(&ctl->drain[me], AGAIN ? 1u : 0u);
+        }
+    } else if (warp < kEpi0) {
+        // ---------------- paged senders: the staged tiles on into the contiguous copy ----------------
+        if (bt.paged && elect_one()) {
+            int prev = -1;            // slot of the tile before, whose stores may still read it
+            bool ok = true;
+            int nc = 0, l = 0, g = 0, n_self = 0, chunk = 0;
+            int64_t T = 0;
+            bool store = false;
+            for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
+                if (u == 0 || un.c == 0) {
+                    const TcSender& sd = bt.s[un.i];
+                    nc = n_c<1>(sd);
+                    chunk = sd.chunk1;
+                    n_self = self_tiles(sd);
+                    T = sd.T;
+                    l = un.s / bt.Hkv;
+                    g = un.s % bt.Hkv;
+                    store = !AGAIN && sd.pages && un.rc == 0;   // once for all row chunks
+                }
+                const int64_t c0 = (int64_t)un.c * chunk;
+                const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows);
+                const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
+                for (int tile = 0; tile < n_tiles; ++tile) {
+                    if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
+                    if (store && tile < nt)
+                        for (int kb = 0; kb < D / 64; ++kb)
+                            tma_store_4d(&bt.maps[un.i].k[2], sm.k + (size_t)st * kTile + kb * kTileRows * 128, 64 * kb,
+                                         (int32_t)(c0 + tile * kTileRows), g, l);
+                    bulk_commit();
+                    if (prev >= 0) {
+                        bulk_wait_read<1>();
+                        mbar_arrive(&ctl->k_empty[prev]);
+                    }
+                    prev = st;
+                    if (++st == stages) { st = 0; ph ^= 1u; }
+                }
+            }
+            if (prev >= 0) {
+                bulk_wait_read<0>();
+                mbar_arrive(&ctl->k_empty[prev]);
+            }
+            bulk_wait<0>();
+        }
+    } else {
+        // ---------------- epilogue ----------------
+        stats_rows<NH, AGAIN>(bt, ctl, tmem, n);
+    }
+    return StatsAt{kt, qn, n, ph, st};
+}
+
 // (out of line: the first run keeps its registers)
-template <int NH>
-__device__ __noinline__ void stats_rows_again(const TcBatch& bt, Ctl* ctl, uint32_t tmem, uint32_t n) {
-    stats_rows<NH, true>(bt, ctl, tmem, n);
+template <int D, int NH>
+__device__ __noinline__ void stats_again(const TcBatch& bt, uint8_t* smem, uint32_t tmem, int64_t kt, uint32_t qn, uint32_t n,
+                                         uint32_t ph, int st) {
+    stats_run<D, NH, true>(bt, carve<D, 1>(smem, bt), tmem, StatsAt{kt, qn, n, ph, st});
 }
 
 // Epilogue: thread = TMEM lane = row 128 h + lane of every half h and a quarter of each tile's
@@ -542,7 +744,6 @@ __device__ __noinline__ void stats_rows_again(const TcBatch& bt, Ctl* ctl, uint3
 // take 119 to 122 us, but the combine kernel 2 to 4 more, and longer at 512 rows.
 template <int D, int NH>
 __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constant__ TcBatch bt) {
-    constexpr int kTile = kTileRows * D * 2;
     extern __shared__ uint8_t smem_raw[];
     const Smem sm = carve<D, 1>(smem_raw, bt);
     Ctl* ctl = sm.ctl;
@@ -559,201 +760,20 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_stats_tc(const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = ctl->tmem_base;
-    const int stages = bt.stages1;
-    // what the roles carry from the first run over their units to the second
-    int64_t kt = 0;               // producer: K tiles issued
-    uint32_t qn = 0, n = 0;       // Q loads issued or consumed; accumulator buffers filled or consumed
-    int st = 0;                   // ring slot of the next K tile and its phase parity
-    uint32_t ph = 0;
-    for (int run = 0;; ++run) {
-        const int n_units = ctl->units;
-        Unit un = ctl->first;
-
-        if (warp == 0) {
-            // ---------------- TMA producer ----------------
-            if (elect_one()) {
-                bool ok = true;
-                int nc = 0, l = 0, g = 0, n_self = 0, chunk = 0;
-                int64_t T = 0;
-                const int32_t* pages = nullptr;
-                int32_t n_pages = 0, ps = 0;
-                for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
-                    const TcMaps& mp = bt.maps[un.i];
-                    if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
-                        const TcSender& sd = bt.s[un.i];
-                        nc = n_c<1>(sd);
-                        chunk = sd.chunk1;
-                        n_self = self_tiles(sd);
-                        pages = sd.pages;
-                        n_pages = sd.n_pages;
-                        ps = sd.page_shift;
-                        T = sd.T;
-                        l = un.s / bt.Hkv;
-                        g = un.s % bt.Hkv;
-                        if (!(ok = wait_bar(&ctl->q_empty, (uint32_t)((qn & 1) ^ 1), ctl, bt.err, 0))) break;
-                        const int h0 = rc_begin(sd.halves, sd.n_rc1, un.rc);
-                        load_q<D, 1>(bt, mp, sm, un.s, h0, rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - h0, sd.q_rows,
-                                 &ctl->q_full);
-                        ++qn;
-                    }
-                    const int64_t c0 = (int64_t)un.c * chunk;
-                    const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows);
-                    const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
-                    for (int tile = 0; tile < n_tiles; ++tile) {
-                        const bool self = tile >= nt;
-                        const int32_t row = self ? (tile - nt) * kTileRows : (int32_t)(c0 + tile * kTileRows);
-                        // a tile's block-table entries, all in flight together while its slot is waited for
-                        const int box = ps < 7 ? 1 << ps : kTileRows;
-                        int32_t entry[kTileRows >> kMinPageShift];
-                        if (pages && !self) {
-#pragma unroll
-                            for (int r = 0; r < kTileRows >> kMinPageShift; ++r)
-                                if (r * box < kTileRows && row + r * box < T) entry[r] = __ldg(pages + ((row + r * box) >> ps));
-                        }
-                        if (!(ok = wait_bar(&ctl->k_empty[st], ph ^ 1u, ctl, bt.err, 1))) break;
-                        mbar_arrive_expect_tx(&ctl->k_full[st], kTile);
-                        if (pages && !self) {
-                            // one box a page (or 128 rows of one); a page past T, or outside the pool (recorded), is
-                            // the coordinate past the last page, which reads as zeros
-#pragma unroll
-                            for (int r = 0; r < kTileRows >> kMinPageShift; ++r) {
-                                if (r * box >= kTileRows) break;
-                                int32_t pg = n_pages;
-                                if (row + r * box < T) {
-                                    pg = entry[r];
-                                    if (pg < 0 || pg >= n_pages) {
-                                        pg = n_pages;
-                                        atomicOr(bt.err, kErrPageIndex);
-                                    }
-                                }
-                                for (int kb = 0; kb < D / 64; ++kb)
-                                    tma_load_5d(sm.k + (size_t)st * kTile + (kb * kTileRows + r * box) * 128, &mp.k[0],
-                                                &ctl->k_full[st], 64 * kb, (row + r * box) & ((1 << ps) - 1), pg, g, l);
-                            }
-                        } else {
-                            for (int kb = 0; kb < D / 64; ++kb)
-                                tma_load_4d(sm.k + (size_t)st * kTile + kb * kTileRows * 128, &mp.k[self ? 1 : 0],
-                                            &ctl->k_full[st], 64 * kb, row, g, l);
-                        }
-                        ++kt;
-                        if (++st == stages) { st = 0; ph ^= 1u; }
-                    }
-                }
-                // drain: every issued load must land before the CTA exits
-                for (int64_t k = kt - stages > 0 ? kt - stages : 0; k < kt; ++k)
-                    drain_wait(&ctl->k_full[k % stages], (uint32_t)((k / stages) & 1));
-                if (qn > 0) drain_wait(&ctl->q_full, (uint32_t)((qn - 1) & 1));
-            }
-        } else if (warp <= 2) {
-            // ---------------- MMA issuers ----------------
-            if (elect_one()) {
-                const uint32_t me = (uint32_t)warp - 1;
-                bool ok = true;
-                constexpr uint32_t idesc = idesc_bf16_f32(128, 128);
-                const uint64_t qd = smem_desc_sw128(smem_u32(sm.q));
-                const uint32_t hi = (uint32_t)(qd >> 32), q_lo = (uint32_t)qd;
-                const uint32_t k_lo = (uint32_t)smem_desc_sw128(smem_u32(sm.k));
-                const uint32_t q_blk = (uint32_t)bt.rows1 * 128 >> 4;
-                // failure-detection test: wait on a barrier that nothing arrives on, so the bounded
-                // wait gives up, sets the abort flag and every role of this CTA leaves
-                if (bt.stall && blockIdx.x == 0 && run == 0) ok = wait_bar(&ctl->stall, 0, ctl, bt.err, 6);
-                uint32_t nh = 0;
-                int nc = 0, n_self = 0, chunk = 0;
-                int64_t T = 0;
-                for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
-                    if (u == 0 || un.c == 0) {   // another group or row chunk: its Q
-                        const TcSender& sd = bt.s[un.i];
-                        nc = n_c<1>(sd);
-                        chunk = sd.chunk1;
-                        n_self = self_tiles(sd);
-                        T = sd.T;
-                        nh = rc_begin(sd.halves, sd.n_rc1, un.rc + 1) - rc_begin(sd.halves, sd.n_rc1, un.rc);
-                        if (u > 0) umma_commit(&ctl->q_empty);
-                        if (!(ok = wait_bar(&ctl->q_full, qn & 1, ctl, bt.err, 2))) break;
-                        ++qn;
-                    }
-                    const int64_t c0 = (int64_t)un.c * chunk;
-                    const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows) +
-                                   (un.c + 1 == nc ? n_self : 0);
-                    for (int tile = 0; tile < nt; ++tile) {
-                        if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
-                        const uint32_t kt_lo = k_lo + (uint32_t)st * (kTile >> 4);
-                        for (uint32_t h = (n ^ me) & 1; h < nh; h += 2) {   // the tile's buffers n + h of my parity
-                            const uint32_t x = n + h, buf = x & 3;
-                            if (!(ok = wait_bar(&ctl->t_empty[buf], ((x >> 2) & 1) ^ 1, ctl, bt.err, 4))) break;
-                            tc_fence_after();
-                            mma_d<D>(tmem + buf * 128, q_lo + h * (kRowHalf * 128 >> 4), q_blk, kt_lo, kTileRows * 128 >> 4, hi,
-                                     idesc);
-                            umma_commit(&ctl->t_full[buf]);
-                        }
-                        if (!ok) break;
-                        n += nh;
-                        umma_commit(&ctl->k_empty[st]);
-                        if (++st == stages) { st = 0; ph ^= 1u; }
-                    }
-                }
-                umma_commit(&ctl->q_empty);
-                umma_commit(&ctl->drain[me]);
-                drain_wait(&ctl->drain[me], (uint32_t)run);
-            }
-        } else if (warp < kEpi0) {
-            // ---------------- paged senders: the staged tiles on into the contiguous copy ----------------
-            if (bt.paged && elect_one()) {
-                int prev = -1;            // slot of the tile before, whose stores may still read it
-                bool ok = true;
-                int nc = 0, l = 0, g = 0, n_self = 0, chunk = 0;
-                int64_t T = 0;
-                bool store = false;
-                for (int u = 0; u < n_units && ok; ++u, next_unit<1>(bt, un, nc)) {
-                    if (u == 0 || un.c == 0) {
-                        const TcSender& sd = bt.s[un.i];
-                        nc = n_c<1>(sd);
-                        chunk = sd.chunk1;
-                        n_self = self_tiles(sd);
-                        T = sd.T;
-                        l = un.s / bt.Hkv;
-                        g = un.s % bt.Hkv;
-                        store = sd.pages && un.rc == 0 && run == 0;   // once for all row chunks
-                    }
-                    const int64_t c0 = (int64_t)un.c * chunk;
-                    const int nt = (int)((min((int64_t)chunk, T - c0) + kTileRows - 1) / kTileRows);
-                    const int n_tiles = nt + (un.c + 1 == nc ? n_self : 0);
-                    for (int tile = 0; tile < n_tiles; ++tile) {
-                        if (!(ok = wait_bar(&ctl->k_full[st], ph, ctl, bt.err, 3))) break;
-                        if (store && tile < nt)
-                            for (int kb = 0; kb < D / 64; ++kb)
-                                tma_store_4d(&bt.maps[un.i].k[2], sm.k + (size_t)st * kTile + kb * kTileRows * 128, 64 * kb,
-                                             (int32_t)(c0 + tile * kTileRows), g, l);
-                        bulk_commit();
-                        if (prev >= 0) {
-                            bulk_wait_read<1>();
-                            mbar_arrive(&ctl->k_empty[prev]);
-                        }
-                        prev = st;
-                        if (++st == stages) { st = 0; ph ^= 1u; }
-                    }
-                }
-                if (prev >= 0) {
-                    bulk_wait_read<0>();
-                    mbar_arrive(&ctl->k_empty[prev]);
-                }
-                bulk_wait<0>();
-            }
-        } else {
-            // ---------------- epilogue ----------------
-            if (run == 0) stats_rows<NH, false>(bt, ctl, tmem, n);
-            else stats_rows_again<NH>(bt, ctl, tmem, n);
-        }
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        if (run == 1 || ctl->redo_hi < 0 || ctl->abort) break;
+    const StatsAt at = stats_run<D, NH, false>(bt, sm, tmem, StatsAt{0, 0, 0, 0, 0});
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (ctl->redo_hi >= 0 && !ctl->abort) {
         if (threadIdx.x == 0) {
             Unit f = ctl->first;
             for (int u = 0; u < ctl->redo_lo; ++u) next_unit<1>(bt, f, n_c<1>(bt.s[f.i]));
             ctl->first = f;
             ctl->units = ctl->redo_hi - ctl->redo_lo + 1;
         }
+        __syncthreads();
+        stats_again<D, NH>(bt, smem_raw, tmem, at.kt, at.qn, at.n, at.ph, at.st);
+        tc_fence_before();
         __syncthreads();
     }
     if (warp == 1) tmem_dealloc(tmem, kTmemCols);
@@ -989,6 +1009,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
             const int h0 = rc_begin(sd.halves, sd.n_rc2, un.rc);
             const int nh = rc_begin(sd.halves, sd.n_rc2, un.rc + 1) - h0;
             const int R = sd.R - h0 * kRowHalf;  // query rows from the row chunk's first on
+            const bool few = FEW && sd.few;
             const int T = (int)sd.T, nc = sd.n_blk2, run = min(left, nc - un.c);
             const float cen = (float)offset_centre(T, G);
             const uint64_t ncen = pack2(-cen, -cen);
@@ -1074,7 +1095,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                     }
                 };
                 for (int h = 0; h < nh; ++h, n ^= 1) {
-                    // A half of more than kFewRows rows: 32 columns a warp.  For d = 128 a buffer's are read one
+                    // A half of more than kFewRows rows, or of a sender of many: 32 columns a warp.  For d = 128 a buffer's are read one
                     // after the other (eight tokens at a time for G < 4, 16 columns a load) and go back to the
                     // MMA, which takes as long as the reading, before the next buffer's.  For d = 64 the MMA takes
                     // half that, so buffers can be held longer: four tokens' columns at a time, interleaved
@@ -1089,7 +1110,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1) k_accum_tc(const __grid_constan
                     constexpr std::false_type no{};
                     constexpr std::true_type yes{};
                     constexpr int kChunks = 32 / (tok.value * G);
-                    const bool wide = !kEights && (!FEW || rows > kFewRows);
+                    const bool wide = !kEights && (!FEW || !few || rows > kFewRows);
                     const int eights = min(4, (rows + 31) >> 5), col = 8 * eights * q;
                     if (wide ? 32 * q >= rows : col >= rows) {   // no columns
 #pragma unroll
@@ -1724,6 +1745,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
             d.n_rc1 = (d.halves + kHalves1 - 1) / kHalves1;
             d.n_rc2 = (d.halves + kHalves2 - 1) / kHalves2;
             d.narrow = narrow_blocks(d_head, s.T, (int64_t)nS * d.n_blk2 * d.n_rc2);
+            d.few = (G > 1 || d_head == 64) && d.halves <= kFewHalves && d.R - (d.halves - 1) * kRowHalf <= kFewRows;
             if (d.narrow) d.n_blk2 = (int32_t)((s.T + kOutN - 1) / kOutN);
             d.stats = b.stats + s.stats_off;
             d.part = b.part + s.part_off;
@@ -1840,7 +1862,7 @@ cudaError_t launch_score_tc(ScoreBatch& b, cudaStream_t st, int num_sms, uint32_
                 tb->rows2 = tb->rows2 > r2 ? tb->rows2 : r2;
                 tb->weight2 += (int64_t)nS * d.n_blk2 * d.halves;
                 units2 += (int64_t)nS * d.n_blk2 * d.n_rc2;
-                tb->few |= (G > 1 || d_head == 64) && d.R - (d.halves - 1) * kRowHalf <= kFewRows;
+                tb->few |= d.few;
                 tb->maps[tb->n] = maps2[k][j];
                 tb->s[tb->n++] = d;
             }

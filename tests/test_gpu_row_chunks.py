@@ -118,7 +118,7 @@ def test_few_rows_and_short_senders(d, G, width, p):
     nL, Hkv, Ts = 9, 4, [1, 26, 104, 105, 208, 209, 312, 313, 1100]   # 36 groups
     gen = torch.Generator(device="cuda").manual_seed(d + G)
     draw = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
-    for rows in (4, 32, 36, 64, 68, 96, 100, 128, 132, 196, 264):
+    for rows in (4, 32, 36, 64, 68, 96, 100, 128, 132, 196, 264, 516):
         m = rows // G
         if d == 64 and m <= 64:
             m += 64          # (fewer tokens: the mma.sync passes)
