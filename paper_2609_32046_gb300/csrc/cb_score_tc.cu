@@ -22,6 +22,7 @@
 //               over positions needs the neighbouring lanes' prefix and suffix maxima only.  A
 //               block's four lane quarters cover 128 positions each, 120 of them outputs (480 a
 //               block).
+//   k_narrow_tc pass 2 of short senders and of few blocks: a position a lane, 104 outputs a block.
 //
 // Rows: a group's m * G query rows, padded to 128, are processed in row chunks of up to 512
 // (pass 1) or 256 rows (pass 2) whose Q fits in shared memory; a row chunk is the outermost part
@@ -734,7 +735,7 @@ __device__ __noinline__ void stats_again(const TcBatch& bt, uint8_t* smem, uint3
 // deviation of 10 (natural units) on.  Then the CTA runs the units from its first to its last such
 // sum again with offsets that rise with the logits, and replaces those sums alone, so that they
 // depend on nothing else in the call: 36 layers, T = 8192, 256 rows take 124 us at standard deviations
-// up to 8, 142 at 10 and 254 from 14 on (recomputing such rows in the combine kernel took 14 ms and
+// up to 8, 142 at 10 and 248 from 14 on (recomputing such rows in the combine kernel took 14 ms and
 // more).  Stretches of marked units in place of the one range gain nothing (275 us from 14 on).
 // Bound by the epilogue, whose waits, TMEM loads, exp2 and packed adds take 115 us without the K
 // loads for 36 layers, T = 8192, 256 rows (64 at the rate of exp2 alone); the K loads without the
