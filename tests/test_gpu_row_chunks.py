@@ -1,8 +1,8 @@
 """The tcgen05 score passes over head dimension 64, many query rows and the edges of their tiles.
 
 Pass 1 takes 128-position tiles and up to 512 query rows at a time, pass 2 blocks of 480 output
-positions (four tiles of every fourth position, the last T mod 4 positions read through maps of
-their own) and up to 256 rows at a time; rows come in halves of 128.
+positions (four tiles of every fourth position, the last T mod 4 positions read through a map of
+their own) or of 104, and up to 256 rows at a time; rows come in halves of 128.
 
 Tolerance: a logit is a 32-bit sum of at most 128 products of bf16 values, off by less than
 128 * 2^-24 * sum |q k| / sqrt(d) < 1e-4 and by about its square root's share, 1e-6, in practice;
